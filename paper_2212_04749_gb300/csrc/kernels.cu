@@ -673,51 +673,91 @@ __global__ void __launch_bounds__(128) k_step_gemm_simt2(const StepDesc d, int c
     }
 }
 
-// Steps with at most four outputs per instance (M N <= 4) and a long K:
-// each output C[i](m, n) = sum_k A[a(i)](m, k) B[b(i)](k, n) is one dot
-// product of two K-contiguous complex runs, computed by one block (16-byte
-// loads, FP32 FMA, a fixed-order block reduction), scaled by the operands'
-// power-of-two factors and stored with its instance's exponent and max.
-__global__ void __launch_bounds__(256) k_step_dot(const StepDesc d) {
-    __shared__ float2 s_part[8];
+// Steps with few outputs per instance (M N <= 32, N <= 8) and a long K (the
+// root of a plan, with its open qubits, and what is left of the ranks just
+// below it).  A unit is one instance and RM of its rows against its N
+// columns: its lanes walk the K-contiguous runs side by side, 16 bytes a
+// load, each B value used for RM rows and each A value for N columns from
+// registers (RM N <= 8 accumulators), then the lanes' sums are added in a
+// fixed order.  Bound by HBM: 8 (A + B) bytes per output row.  A GEMM tile
+// of 128 x 64 would hold RM N live outputs of 8192 and walk K serially:
+// M = 16, K = 2^15, N = 1, 256 instances (1.1 GB, 0.17 ms of HBM) took
+// 13.4 ms on the SIMT GEMM, about 0.3 ms here (the contraction that ends in
+// it 27.3 -> 14.2 ms).
+// W = 8: a block per unit (long K, or too few units to fill the chip with
+// warps); W = 1: a warp per unit.
+template <int RM, int N, int W>
+__global__ void __launch_bounds__(256) k_step_skinny(const StepDesc d, int64_t units) {
+    __shared__ float2 s_part[8][RM * N];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int mn_log = d.mb + d.nb;
-    const int64_t i = int64_t(blockIdx.x) >> mn_log;
-    const int mn = int(blockIdx.x & ((1u << mn_log) - 1));
-    const int m = mn >> d.nb, n = mn & ((1 << d.nb) - 1);
+    const int64_t u = W == 8 ? int64_t(blockIdx.x) : int64_t(blockIdx.x) * 8 + warp;
+    if (W == 1 && u >= units) return;  // a whole warp
+    constexpr int RMB = RM == 1 ? 0 : (RM == 2 ? 1 : (RM == 4 ? 2 : 3));
+    const int rbits = d.mb - RMB;  // row blocks per instance (log2)
+    const int64_t i = u >> rbits;
+    const int m0 = int(u & ((int64_t(1) << rbits) - 1)) * RM;
     const int2 ab = d.instab[i];
-    const int K = 1 << d.kb;
-    const float4 *a4 = reinterpret_cast<const float4 *>(d.A + int64_t(ab.x) * d.sA + (int64_t(m) << d.kb));
-    const float4 *b4 = reinterpret_cast<const float4 *>(d.B + int64_t(ab.y) * d.sB + (int64_t(n) << d.kb));
-    float2 acc = make_float2(0.f, 0.f), acc2 = make_float2(0.f, 0.f);
-    for (int q = tid; q < K / 2; q += 256) {
-        const float4 x = __ldg(a4 + q), y = __ldg(b4 + q);
-        cfma(acc, make_float2(x.x, x.y), make_float2(y.x, y.y));
-        cfma(acc2, make_float2(x.z, x.w), make_float2(y.z, y.w));
-    }
-    acc.x += acc2.x;
-    acc.y += acc2.y;
+    const int K2 = 1 << (d.kb - 1);  // 16-byte pieces per row
+    const float4 *a4 = reinterpret_cast<const float4 *>(d.A + int64_t(ab.x) * d.sA + (int64_t(m0) << d.kb));
+    const float4 *b4 = reinterpret_cast<const float4 *>(d.B + int64_t(ab.y) * d.sB);
+    float2 acc[RM][N];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+    for (int r = 0; r < RM; ++r)
+#pragma unroll
+        for (int n = 0; n < N; ++n) acc[r][n] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int q = W == 8 ? tid : lane; q < K2; q += 32 * W) {
+        float4 a[RM], b[N];
+#pragma unroll
+        for (int r = 0; r < RM; ++r) a[r] = __ldg(a4 + int64_t(r) * K2 + q);
+#pragma unroll
+        for (int n = 0; n < N; ++n) b[n] = __ldg(b4 + int64_t(n) * K2 + q);
+#pragma unroll
+        for (int r = 0; r < RM; ++r)
+#pragma unroll
+            for (int n = 0; n < N; ++n) {
+                cfma(acc[r][n], make_float2(a[r].x, a[r].y), make_float2(b[n].x, b[n].y));
+                cfma(acc[r][n], make_float2(a[r].z, a[r].w), make_float2(b[n].z, b[n].w));
+            }
     }
-    if (lane == 0) s_part[warp] = acc;
-    __syncthreads();
-    if (tid == 0) {
-        float2 t = s_part[0];
-        for (int w = 1; w < 8; ++w) {
-            t.x += s_part[w].x;
-            t.y += s_part[w].y;
+    float2 mine = make_float2(0.f, 0.f);  // lane j < RM N: output (row j / N, column j mod N)
+#pragma unroll
+    for (int r = 0; r < RM; ++r)
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            float2 t = acc[r][n];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+                t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+            }
+            if (lane == r * N + n) mine = t;
         }
-        const int ea = d.mxA ? exp_of(d.mxA[ab.x]) : 0;
-        const int eb = d.mxB ? exp_of(d.mxB[ab.y]) : 0;
-        const float sc = pow2f(-(ea + eb));
-        const float2 v = make_float2(t.x * sc, t.y * sc);
-        d.C[i * d.sC + dep(m, d.pCm, d.mb) + dep(n, d.pCn, d.nb)] = v;
-        if (mn == 0) d.EC[i] = d.EA[ab.x] + ea + d.EB[ab.y] + eb;
-        const uint32_t mx = absmax_bits(v);
-        if (d.mxC && mx) record_max(d.mxC + i, mx);
+    if (W == 8) {
+        if (lane < RM * N) s_part[warp][lane] = mine;
+        __syncthreads();
+        if (warp != 0) return;
+        if (lane < RM * N) {
+            mine = s_part[0][lane];
+            for (int w = 1; w < 8; ++w) {
+                mine.x += s_part[w][lane].x;
+                mine.y += s_part[w][lane].y;
+            }
+        }
+    }
+    const int ea = d.mxA ? exp_of(d.mxA[ab.x]) : 0;
+    const int eb = d.mxB ? exp_of(d.mxB[ab.y]) : 0;
+    const float sc = pow2f(-(ea + eb));
+    uint32_t mx = 0u;
+    if (lane < RM * N) {
+        const float2 v = make_float2(mine.x * sc, mine.y * sc);
+        d.C[i * d.sC + dep(m0 + lane / N, d.pCm, d.mb) + dep(lane % N, d.pCn, d.nb)] = v;
+        mx = absmax_bits(v);
+    }
+    if (lane == 0 && m0 == 0) d.EC[i] = d.EA[ab.x] + ea + d.EB[ab.y] + eb;
+    if (d.mxC) {
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0 && mx) record_max(d.mxC + i, mx);
     }
 }
 
@@ -974,12 +1014,37 @@ cudaError_t launch_step_gemm_simt(const StepDesc &d, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_step_dot(const StepDesc &d, cudaStream_t s) {
-    if (d.mb + d.nb > 2 || d.kb < 6) return cudaErrorInvalidValue;
-    const int64_t blocks = d.nInst << (d.mb + d.nb);
-    if (blocks <= 0) return cudaSuccess;
+bool step_skinny_takes(const StepDesc &d) { return d.kb >= 6 && d.nb <= 3 && d.mb + d.nb <= 5; }
+
+cudaError_t launch_step_skinny(const StepDesc &d, cudaStream_t s) {
+    if (!step_skinny_takes(d)) return cudaErrorInvalidValue;
+    const int rmb = d.mb < 3 - d.nb ? d.mb : 3 - d.nb;  // RM N <= 8
+    const int64_t units = d.nInst << (d.mb - rmb);
+    if (units <= 0) return cudaSuccess;
+    // a block per unit where its 256 lanes have several pieces each, or
+    // where one warp per unit would leave most of the chip idle
+    const bool wide = d.kb >= 12 || (d.kb >= 9 && units < 4864);
+    const int64_t blocks = wide ? units : (units + 7) / 8;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    k_step_dot<<<dim3((unsigned)blocks), 256, 0, s>>>(d);
+    const dim3 g((unsigned)blocks);
+#define TN_SKINNY(RM_, N_)                                                 \
+    do {                                                                   \
+        if (wide) k_step_skinny<RM_, N_, 8><<<g, 256, 0, s>>>(d, units);   \
+        else k_step_skinny<RM_, N_, 1><<<g, 256, 0, s>>>(d, units);        \
+    } while (0)
+    switch (4 * d.nb + rmb) {
+        case 0: TN_SKINNY(1, 1); break;
+        case 1: TN_SKINNY(2, 1); break;
+        case 2: TN_SKINNY(4, 1); break;
+        case 3: TN_SKINNY(8, 1); break;
+        case 4: TN_SKINNY(1, 2); break;
+        case 5: TN_SKINNY(2, 2); break;
+        case 6: TN_SKINNY(4, 2); break;
+        case 8: TN_SKINNY(1, 4); break;
+        case 9: TN_SKINNY(2, 4); break;
+        default: TN_SKINNY(1, 8); break;
+    }
+#undef TN_SKINNY
     return cudaGetLastError();
 }
 
