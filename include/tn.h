@@ -255,11 +255,20 @@ int tn_sample_completions(const double *amps, int64_t k, int32_t n_open, const d
  * words out_dev[0..4]: sum g, sum g^2 with g = (x - 1) / (1 + F (x - 1))
  * (the derivative of the log-likelihood in F and minus its second
  * derivative, the Fisher information), sum log(1 + F (x - 1)), sum x and
- * sum x^2 (the linear XEB F = mean(x) - 1 and its standard error).  One
- * block, fixed summation order.  TN_EINVAL for F outside [0, 1), k <= 0 or
+ * sum x^2 (the linear XEB F = mean(x) - 1 and its standard error).  Fixed
+ * summation order.  TN_EINVAL for F outside [0, 1), k <= 0 or
  * null pointers; asynchronous on `stream`. */
 int tn_pt_moments(const double *amps, int64_t k, int32_t n_qubits, double fidelity, double *out_dev,
                   void *stream);
+
+/* The same sums on every SM, with the caller's device scratch (8-byte
+ * aligned, >= tn_pt_moments_scratch_bytes(k) bytes) for the blocks'
+ * partial sums, for repeated passes over many amplitudes.  want_log = 0
+ * leaves out the logarithms (out_dev[2] = 0).  TN_ENOMEM for too little
+ * scratch, else as tn_pt_moments. */
+size_t tn_pt_moments_scratch_bytes(int64_t k);
+int tn_pt_moments_scratch(const double *amps, int64_t k, int32_t n_qubits, double fidelity, int32_t want_log,
+                          double *out_dev, void *scratch, size_t scratch_bytes, void *stream);
 
 /* Histogram of x_b = 2^n |amp_b|^2: counts_dev[j] (device, uint64, nbins + 1
  * words, caller-zeroed, accumulated into) gains the b with

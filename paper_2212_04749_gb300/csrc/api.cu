@@ -653,6 +653,24 @@ int tn_pt_moments(const double *amps, int64_t k, int32_t n_qubits, double fideli
     return TN_OK;
 }
 
+size_t tn_pt_moments_scratch_bytes(int64_t k) { return k > 0 ? tnk::pt_moments_scratch_bytes(k) : 0; }
+
+int tn_pt_moments_scratch(const double *amps, int64_t k, int32_t n_qubits, double fidelity, int32_t want_log,
+                          double *out_dev, void *scratch, size_t scratch_bytes, void *stream) {
+    if (!amps || !out_dev || !scratch || k <= 0 || n_qubits < 1 || n_qubits > 1000)
+        return set_err(TN_EINVAL, "tn_pt_moments_scratch: need k > 0, amplitudes, 5 output words and scratch");
+    if (!(fidelity >= 0.0 && fidelity < 1.0)) return set_err(TN_EINVAL, "tn_pt_moments_scratch: fidelity outside [0, 1)");
+    if (scratch_bytes < tnk::pt_moments_scratch_bytes(k))
+        return set_err(TN_ENOMEM, "tn_pt_moments_scratch: scratch needs " +
+                                      std::to_string(tnk::pt_moments_scratch_bytes(k)) + " bytes");
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    cudaError_t e = tnk::launch_pt_moments_scratch(amps, k, std::ldexp(1.0, n_qubits), fidelity, want_log != 0, out_dev,
+                                                   static_cast<double *>(scratch), st);
+    if (e != cudaSuccess) return set_err(TN_ECUDA, std::string("pt_moments: ") + cudaGetErrorString(e));
+    g_err.clear();
+    return TN_OK;
+}
+
 int tn_pt_histogram(const double *amps, int64_t k, int32_t n_qubits, double x_max, int32_t nbins,
                     uint64_t *counts_dev, void *stream) {
     if (!amps || !counts_dev || k <= 0 || n_qubits < 1 || n_qubits > 1000)

@@ -27,6 +27,8 @@
 // exponent of that maximum, and adds e to the output's exponent E.  Scaling
 // by a power of two is exact, so with and without it the FP32 results are
 // bitwise the same (barring subnormals).
+#include <cooperative_groups.h>
+
 #include "kernels.cuh"
 
 namespace tnk {
@@ -801,21 +803,58 @@ __global__ void k_extract(const float2 *__restrict__ root, const int32_t *__rest
     out[q] = make_double2(ldexp(double(v.x), E[idx]), ldexp(double(v.y), E[idx]));
 }
 
-__global__ void __launch_bounds__(1024) k_xeb(const double2 *__restrict__ amps, int64_t k, double scale,
-                                              double *__restrict__ out) {
-    __shared__ double s[1024];
-    double acc = 0.0;
-    for (int64_t p = threadIdx.x; p < k; p += 1024) {
-        const double2 a = amps[p];
-        acc += a.x * a.x + a.y * a.y;
+// Block sum of NV doubles per thread in a fixed order: lanes by xor steps,
+// then the warps in turn.  Thread v < NV returns sum v.
+template <int NV, int THREADS>
+__device__ __forceinline__ double block_sums(double (&a)[NV], double (*part)[NV]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a[v] += __shfl_xor_sync(0xffffffffu, a[v], o);
+        if (lane == 0) part[warp][v] = a[v];
     }
-    s[threadIdx.x] = acc;
     __syncthreads();
-    for (int w = 512; w > 0; w >>= 1) {
-        if (threadIdx.x < w) s[threadIdx.x] += s[threadIdx.x + w];
-        __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x < NV)
+        for (int w = 0; w < THREADS / 32; ++w) s += part[w][threadIdx.x];
+    return s;
+}
+
+// Sum over the blocks of a cluster (the whole grid), in rank order, by rank
+// 0's first NV threads through distributed shared memory.  `mine` is this
+// block's sums (thread v: sum v); returns the total there.
+template <int NV>
+__device__ __forceinline__ double cluster_sums(double mine, double *slot) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    if (threadIdx.x < NV) slot[threadIdx.x] = mine;
+    cl.sync();
+    double s = 0.0;
+    if (cl.block_rank() == 0 && threadIdx.x < NV)
+        for (unsigned r = 0; r < cl.num_blocks(); ++r) s += *cl.map_shared_rank(slot + threadIdx.x, r);
+    cl.sync();  // the blocks' shared memory is read until here
+    return s;
+}
+
+// FP64 sums over the amplitudes run on one cluster of RED_CLUSTER blocks:
+// the chip's FP64 units, two lanes per SM, bound them (48 MB of amplitudes
+// take 7 us of HBM; the sums below 5 to 50 FP64 operations each), so the
+// more SMs the better, and a cluster adds its blocks' sums in a fixed order
+// without scratch memory.
+constexpr int RED_CLUSTER = 16, RED_THREADS = 512;
+
+__global__ void __launch_bounds__(RED_THREADS) k_xeb(const double2 *__restrict__ amps, int64_t k, double scale,
+                                                     double *__restrict__ out) {
+    __shared__ double part[RED_THREADS / 32][1];
+    __shared__ double slot[1];
+    double acc[1] = {0.0};
+    for (int64_t p = int64_t(blockIdx.x) * RED_THREADS + threadIdx.x; p < k; p += int64_t(gridDim.x) * RED_THREADS) {
+        const double2 a = amps[p];
+        acc[0] += a.x * a.x + a.y * a.y;
     }
-    if (threadIdx.x == 0) out[0] = scale * s[0] - 1.0;
+    const double s = cluster_sums<1>(block_sums<1, RED_THREADS>(acc, part), slot);
+    if (blockIdx.x == 0 && threadIdx.x == 0) out[0] = scale * s - 1.0;
 }
 
 // x = N |a|^2 in FP64 with explicit round-to-nearest operations (no
@@ -829,34 +868,70 @@ __device__ __forceinline__ double pt_x(double2 a, double n_states) {
 // p(x) = e^-x (1 + F (x - 1)) of x = N |amp|^2 (fidelity F; Eq. fxeb):
 // out[0] = sum g, out[1] = sum g^2 with g = (x - 1) / (1 + F (x - 1)) (the
 // log-likelihood's first derivative and minus its second), out[2] = sum
-// log(1 + F (x - 1)), out[3] = sum x, out[4] = sum x^2.  One block, fixed
-// order.
-__global__ void __launch_bounds__(1024) k_pt_moments(const double2 *__restrict__ amps, int64_t k, double n_states,
-                                                     double fid, double *__restrict__ out) {
-    __shared__ double s[5][1024];
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, a4 = 0.0;
-    for (int64_t p = threadIdx.x; p < k; p += 1024) {
+// log(1 + F (x - 1)), out[3] = sum x, out[4] = sum x^2.  Fixed order.
+// Bound by the FP64 units: about 17 operations per amplitude, half of them
+// the division, and a logarithm for every four amplitudes: log of the
+// product of four d, each of them at least 1 - F > 0 (their separate
+// logarithms where the product leaves the range of a double).  At F = 0 g is
+// x - 1 and the logarithm 0.
+//   CLUSTER: the grid is one cluster, out holds the sums;
+//   else: any grid, block b writes its sums to out[5 b .. 5 b + 4], which
+//   k_pt_final adds up (every SM: 3 M amplitudes take 205 ms / 6 passes with
+//   one block of 1024 threads).
+template <bool CLUSTER>
+__global__ void __launch_bounds__(RED_THREADS) k_pt_moments(const double2 *__restrict__ amps, int64_t k,
+                                                            double n_states, double fid, int want_log,
+                                                            double *__restrict__ out) {
+    __shared__ double part[RED_THREADS / 32][5];
+    __shared__ double slot[5];
+    double a[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    const int64_t stride = int64_t(gridDim.x) * RED_THREADS;
+    auto add = [&](int64_t p) -> double {  // the sums but the logarithm's; returns d
         const double x = pt_x(amps[p], n_states);
-        const double d = 1.0 + fid * (x - 1.0);
-        const double g = (x - 1.0) / d;
-        a0 += g;
-        a1 += g * g;
-        a2 += log(d);
-        a3 += x;
-        a4 += x * x;
+        const double x1 = x - 1.0;
+        const double d = 1.0 + fid * x1;
+        const double g = fid == 0.0 ? x1 : x1 / d;
+        a[0] += g;
+        a[1] += g * g;
+        a[3] += x;
+        a[4] += x * x;
+        return d;
+    };
+    int64_t p = int64_t(blockIdx.x) * RED_THREADS + threadIdx.x;
+    for (; p + 3 * stride < k; p += 4 * stride) {
+        double d[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) d[j] = add(p + j * stride);
+        if (want_log && fid != 0.0) {
+            const double q = (d[0] * d[1]) * (d[2] * d[3]);
+            if (q > 1e-290 && q < 1e290) a[2] += log(q);
+            else
+                for (int j = 0; j < 4; ++j) a[2] += log(d[j]);
+        }
     }
-    s[0][threadIdx.x] = a0;
-    s[1][threadIdx.x] = a1;
-    s[2][threadIdx.x] = a2;
-    s[3][threadIdx.x] = a3;
-    s[4][threadIdx.x] = a4;
-    __syncthreads();
-    for (int w = 512; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int j = 0; j < 5; ++j) s[j][threadIdx.x] += s[j][threadIdx.x + w];
-        __syncthreads();
+    for (; p < k; p += stride) {
+        const double d = add(p);
+        if (want_log && fid != 0.0) a[2] += log(d);
     }
-    if (threadIdx.x < 5) out[threadIdx.x] = s[threadIdx.x][0];
+    const double s = block_sums<5, RED_THREADS>(a, part);
+    if (CLUSTER) {
+        const double t = cluster_sums<5>(s, slot);
+        if (blockIdx.x == 0 && threadIdx.x < 5) out[threadIdx.x] = t;
+    } else if (threadIdx.x < 5) {
+        out[5 * int64_t(blockIdx.x) + threadIdx.x] = s;
+    }
+}
+
+// out[v] = the sum of part[5 b + v] over the blocks b, warp v: lanes take
+// every 32nd block, then xor steps (a fixed order)
+__global__ void __launch_bounds__(160) k_pt_final(const double *__restrict__ part, int blocks,
+                                                  double *__restrict__ out) {
+    const int lane = threadIdx.x & 31, v = threadIdx.x >> 5;
+    double s = 0.0;
+    for (int b = lane; b < blocks; b += 32) s += part[5 * b + v];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) out[v] = s;
 }
 
 // counts[j] += #{b : j width <= x_b < (j + 1) width}, j < nbins, with
@@ -1074,9 +1149,31 @@ cudaError_t launch_extract(const float2 *root, const int32_t *E, const int32_t *
     return cudaGetLastError();
 }
 
+// one cluster as the whole grid, no more blocks than have work (a power of
+// two; a few thousand amplitudes stay on one SM)
+template <class... P, class... A>
+static cudaError_t launch_cluster(void (*fn)(P...), int64_t k, cudaStream_t s, A... args) {
+    cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn),
+                                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    unsigned blocks = 1;
+    while (blocks < unsigned(RED_CLUSTER) && int64_t(blocks) * RED_THREADS < k) blocks <<= 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(RED_THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = blocks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, fn, args...);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 cudaError_t launch_xeb(const double *amps, int64_t k, double scale, double *out, cudaStream_t s) {
-    k_xeb<<<1, 1024, 0, s>>>(reinterpret_cast<const double2 *>(amps), k, scale, out);
-    return cudaGetLastError();
+    return launch_cluster(k_xeb, k, s, reinterpret_cast<const double2 *>(amps), k, scale, out);
 }
 
 cudaError_t launch_sample(const double *amps, int64_t k, int r, const double *uniform, int64_t *picks,
@@ -1089,7 +1186,25 @@ cudaError_t launch_sample(const double *amps, int64_t k, int r, const double *un
 
 cudaError_t launch_pt_moments(const double *amps, int64_t k, double n_states, double fid, double *out,
                               cudaStream_t s) {
-    k_pt_moments<<<1, 1024, 0, s>>>(reinterpret_cast<const double2 *>(amps), k, n_states, fid, out);
+    return launch_cluster(k_pt_moments<true>, k, s, reinterpret_cast<const double2 *>(amps), k, n_states, fid, 1, out);
+}
+
+// Blocks of the scratch form: four amplitudes a thread at least, at most
+// PT_BLOCKS (two resident blocks on each of 152 SMs).
+constexpr int PT_BLOCKS = 304;
+static int pt_blocks(int64_t k) {
+    const int64_t b = (k + 4 * RED_THREADS - 1) / (4 * RED_THREADS);
+    return int(b < 1 ? 1 : (b > PT_BLOCKS ? PT_BLOCKS : b));
+}
+
+size_t pt_moments_scratch_bytes(int64_t k) { return size_t(pt_blocks(k)) * 5 * sizeof(double); }
+
+cudaError_t launch_pt_moments_scratch(const double *amps, int64_t k, double n_states, double fid, bool want_log,
+                                      double *out, double *scratch, cudaStream_t s) {
+    const int blocks = pt_blocks(k);
+    k_pt_moments<false><<<blocks, RED_THREADS, 0, s>>>(reinterpret_cast<const double2 *>(amps), k, n_states, fid,
+                                                       want_log ? 1 : 0, scratch);
+    k_pt_final<<<1, 160, 0, s>>>(scratch, blocks, out);
     return cudaGetLastError();
 }
 

@@ -86,6 +86,11 @@ cudaError_t launch_extract(const float2 *root, const int32_t *E, const int32_t *
 cudaError_t launch_xeb(const double *amps, int64_t k, double scale, double *out, cudaStream_t s);
 cudaError_t launch_pt_moments(const double *amps, int64_t k, double n_states, double fid, double *out,
                               cudaStream_t s);
+// The same sums over the whole chip, block partials in caller scratch of
+// pt_moments_scratch_bytes(k); out[2] is 0 without want_log.
+size_t pt_moments_scratch_bytes(int64_t k);
+cudaError_t launch_pt_moments_scratch(const double *amps, int64_t k, double n_states, double fid, bool want_log,
+                                      double *out, double *scratch, cudaStream_t s);
 cudaError_t launch_sample(const double *amps, int64_t k, int r, const double *uniform, int64_t *picks,
                           cudaStream_t s);
 // FP32 FMA throughput probe: `blocks` blocks of 256 threads, each thread

@@ -21,7 +21,8 @@ PRECISIONS = {"fp32": TN_FP32, "tf32": TN_TF32, "bf16x3": TN_BF16X3}
 
 EXPORTS = ("tn_options_default", "tn_network", "tn_plan", "tn_plan_query", "tn_plan_widths", "tn_plan_steps",
            "tn_plan_bind", "tn_contract", "tn_contract_slices", "tn_xeb", "tn_plan_profile",
-           "tn_plan_step_times", "tn_plan_set_kernel", "tn_plan_set_config", "tn_plan_set_tc_resident_b", "tn_plan_set_tc_pairs", "tn_plan_get_configs", "tn_pt_moments", "tn_pt_histogram", "tn_sample_completions",
+           "tn_plan_step_times", "tn_plan_set_kernel", "tn_plan_set_config", "tn_plan_set_tc_resident_b", "tn_plan_set_tc_pairs", "tn_plan_get_configs", "tn_pt_moments",
+           "tn_pt_moments_scratch_bytes", "tn_pt_moments_scratch", "tn_pt_histogram", "tn_sample_completions",
            "tn_plan_features", "tn_plan_autotune", "tn_plan_select", "tn_mlp_grad_scratch_bytes",
            "tn_mlp_forward", "tn_mlp_grad", "tn_mlp_adam", "tn_mlp_to_half", "tn_mlp_forward_f16",
            "tn_plan_check", "tn_contract_static", "tn_fma_probe", "tn_plan_batch_slices", "tn_plan_set_chain",
@@ -115,6 +116,8 @@ def load(build_if_missing: bool = False):
         "tn_contract_slices": (ctypes.c_int, [vp, ctypes.c_int, vp, i32, vp, vp]),
         "tn_xeb": (ctypes.c_int, [vp, i64, i32, vp, vp]),
         "tn_pt_moments": (ctypes.c_int, [vp, i64, i32, ctypes.c_double, vp, vp]),
+        "tn_pt_moments_scratch_bytes": (ctypes.c_size_t, [i64]),
+        "tn_pt_moments_scratch": (ctypes.c_int, [vp, i64, i32, ctypes.c_double, i32, vp, vp, ctypes.c_size_t, vp]),
         "tn_sample_completions": (ctypes.c_int, [vp, i64, i32, vp, vp, vp]),
         "tn_pt_histogram": (ctypes.c_int, [vp, i64, i32, ctypes.c_double, i32, vp, vp]),
         "tn_plan_profile": (ctypes.c_int, [vp, ctypes.c_int]),
@@ -399,6 +402,16 @@ def tn_sample_completions(amps, k, n_open, uniform, picks, stream=None):
 
 def tn_pt_moments(amps, k, n_qubits, fidelity, out, stream=None):
     _check(load().tn_pt_moments(_ptr(amps), int(k), int(n_qubits), float(fidelity), _ptr(out), _stream(stream)))
+
+
+def tn_pt_moments_scratch_bytes(k):
+    return int(load().tn_pt_moments_scratch_bytes(int(k)))
+
+
+def tn_pt_moments_scratch(amps, k, n_qubits, fidelity, out, scratch, want_log=True, stream=None):
+    nbytes = scratch.numel() * scratch.element_size()
+    _check(load().tn_pt_moments_scratch(_ptr(amps), int(k), int(n_qubits), float(fidelity), int(bool(want_log)),
+                                        _ptr(out), _ptr(scratch), int(nbytes), _stream(stream)))
 
 
 def tn_pt_histogram(amps, k, n_qubits, x_max, nbins, counts, stream=None):

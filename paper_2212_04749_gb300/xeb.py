@@ -6,8 +6,8 @@ x = 2^n |amp|^2 for comparing with that law.
 With x_b = 2^n |amp_b|^2, bitstrings drawn at fidelity F have the density
 p(x) = e^-x (1 + F (x - 1)).  The log-likelihood of F is concave; Newton's
 method on it needs sum g and sum g^2 with g = (x - 1) / (1 + F (x - 1)), which
-the library's k_pt_moments kernel reduces on the device in FP64 (one launch
-per iteration); the scalar update runs here.  The error bar is the inverse
+the library's k_pt_moments kernel reduces on the device in FP64 (one pass
+over the amplitudes per iteration); the scalar update runs here.  The error bar is the inverse
 square root of the Fisher information sum g^2 at the maximum.
 """
 
@@ -26,9 +26,13 @@ def porter_thomas_fit(amps, k, n_qubits, stream=None, iters=60, tol=1e-13):
     import torch
 
     out = torch.empty(5, dtype=torch.float64, device=amps.device)
+    scratch = torch.empty(tn.tn_pt_moments_scratch_bytes(k), dtype=torch.uint8, device=amps.device)
+    if isinstance(stream, torch.cuda.Stream):  # the kernels run there, not on the stream these were made on
+        out.record_stream(stream)
+        scratch.record_stream(stream)
 
-    def moments(f):
-        tn.tn_pt_moments(amps, k, n_qubits, f, out, stream=stream)
+    def moments(f, log=False):
+        tn.tn_pt_moments_scratch(amps, k, n_qubits, f, out, scratch, want_log=log, stream=stream)
         return out.cpu().numpy()  # synchronises with the launch
 
     top = 1.0 - 1e-12
@@ -43,7 +47,7 @@ def porter_thomas_fit(amps, k, n_qubits, stream=None, iters=60, tol=1e-13):
         f = nf
         if done:
             break
-    s = moments(f)
+    s = moments(f, log=True)
     var = max(s[4] / k - mean * mean, 0.0)
     return {"fidelity": float(f), "stderr": float(1.0 / math.sqrt(s[1])), "loglik": float(s[2] - s[3]),
             "linear": float(mean - 1.0), "linear_stderr": float(math.sqrt(var / k)), "iterations": it}

@@ -91,3 +91,33 @@ def test_fit_on_contracted_amplitudes():
               f"linear {r['linear']:.4f} +- {r['linear_stderr']:.4f}")
         assert abs(r["fidelity"] - f_true) < 4 * r["stderr"] + 1e-6
         assert abs(r["linear"] - f_true) < 4 * r["linear_stderr"]
+
+
+@pytest.mark.parametrize("k", [1, 511, 512, 2047, 2049, 8193, 20481, 1300003])
+@pytest.mark.parametrize("f", [0.0, 0.37, 1.0 - 2.0 ** -53])
+def test_moments_scratch_form_and_xeb_at_block_edges(k, f):
+    # one block, part of a cluster, whole clusters, every SM; groups of four
+    # amplitudes and their remainders; products of four 1 + F (x - 1) of
+    # 1e-16 (x = 0 at F = 1 - 2^-53) and beyond the range of a double
+    torch, tn = require_cuda()
+    n = 20
+    a = _amps(k, n, 3)
+    a[: k // 7] = 0.0
+    a[k // 7: k // 5] *= 1e60
+    d = _dev(torch, a)
+    x = oxeb.x_values(a, n)
+    ref = oxeb.pt_moments(x, f)
+    out = torch.full((5,), float("nan"), dtype=torch.float64, device="cuda")
+    scratch = torch.empty(tn.tn_pt_moments_scratch_bytes(k), dtype=torch.uint8, device="cuda")
+    for log in (True, False):
+        tn.tn_pt_moments_scratch(d, k, n, f, out, scratch, want_log=log)
+        got = out.cpu().numpy()
+        want = ref if log else np.where(np.arange(5) == 2, 0.0, ref)
+        assert np.all(np.abs(got - want) <= 1e-11 * np.maximum(np.abs(want), 1.0)), (f, log, got, want)
+    tn.tn_pt_moments(d, k, n, f, out)
+    assert np.all(np.abs(out.cpu().numpy() - ref) <= 1e-11 * np.maximum(np.abs(ref), 1.0))
+    tn.tn_xeb(d, k, n, out)
+    want = np.sum(np.abs(a) ** 2) * 2.0 ** n / k - 1.0
+    assert abs(out[0].item() - want) <= 1e-12 * max(abs(want), 1.0)
+    with pytest.raises(tn.TnError):
+        tn.tn_pt_moments_scratch(d, k, n, f, out, scratch[:-1])
