@@ -876,8 +876,9 @@ __device__ __forceinline__ double pt_x(double2 a, double n_states) {
 // x - 1 and the logarithm 0.
 //   CLUSTER: the grid is one cluster, out holds the sums;
 //   else: any grid, block b writes its sums to out[5 b .. 5 b + 4], which
-//   k_pt_final adds up (every SM: 3 M amplitudes take 205 ms / 6 passes with
-//   one block of 1024 threads).
+//   k_pt_final adds up (every SM).
+// The fit of 3 M amplitudes with XEB and histogram: 1.10 ms, about 0.13 ms a
+// pass; with one block of 1024 threads and a logarithm each 205.7 ms.
 template <bool CLUSTER>
 __global__ void __launch_bounds__(RED_THREADS) k_pt_moments(const double2 *__restrict__ amps, int64_t k,
                                                             double n_states, double fid, int want_log,
@@ -956,29 +957,86 @@ __global__ void k_pt_hist(const double2 *__restrict__ amps, int64_t k, double n_
 // Row p's batch a[p 2^r .. p 2^r + 2^r): with u = uniform[p] in [0, 1), the
 // smallest x whose running sum of |a_x|^2 exceeds u times the batch total
 // (2^r - 1 if none does); FP64, correctly rounded operations in x order.
-__global__ void k_sample(const double2 *__restrict__ amps, int64_t k, int r, const double *__restrict__ uniform,
-                         int64_t *__restrict__ picks) {
-    const int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (p >= k) return;
-    const double2 *a = amps + (p << r);
-    const int64_t n = int64_t(1) << r;
-    double tot = 0.0;
-    for (int64_t x = 0; x < n; ++x) {
-        const double2 v = a[x];
-        tot = __dadd_rn(tot, __dadd_rn(__dmul_rn(v.x, v.x), __dmul_rn(v.y, v.y)));
-    }
-    const double thr = __dmul_rn(uniform[p], tot);
-    double c = 0.0;
-    int64_t pick = n - 1;
-    for (int64_t x = 0; x < n; ++x) {
-        const double2 v = a[x];
-        c = __dadd_rn(c, __dadd_rn(__dmul_rn(v.x, v.x), __dmul_rn(v.y, v.y)));
-        if (c > thr) {
-            pick = x;
-            break;
+//
+// The running sum is a chain of dependent additions by definition, one row
+// per lane (a warp instruction on the FP64 units costs the same for one lane
+// as for 32).  A block takes 32 rows: four warps read the amplitudes in
+// tiles of 32 rows x SAMP_T completions, coalesced, and leave |a|^2 in shared
+// memory one tile ahead of warp 0, which adds up its row per lane.  It keeps
+// the sum after each of at most SAMP_SEG segments; sums never decrease, so
+// the first segment whose sum exceeds the threshold holds the pick, and only
+// that segment is read again (8192 rows x 1024: 134 MB, 20 us of HBM, 33 M
+// FP64 operations; one thread per row reading its own row twice took 632 us).
+constexpr int SAMP_T = 32, SAMP_SEG = 64, SAMP_THREADS = 160;
+
+__global__ void __launch_bounds__(SAMP_THREADS) k_sample(const double2 *__restrict__ amps, int64_t k, int r,
+                                                         const double *__restrict__ uniform,
+                                                         int64_t *__restrict__ picks) {
+    __shared__ double s_p[2][32][SAMP_T + 1];
+    __shared__ double s_ck[SAMP_SEG][32];  // running sum after each segment
+    __shared__ int s_x0[32];               // first completion of the row's segment
+    const int tid = threadIdx.x, lane = tid & 31;
+    const bool adder = tid < 32;
+    const int64_t row0 = int64_t(blockIdx.x) * 32;
+    const int n = 1 << r;
+    const int tb = r < 5 ? r : 5, T = 1 << tb;            // completions per tile
+    const int seg = n / SAMP_SEG > T ? n / SAMP_SEG : T;  // completions per segment
+    constexpr int PER = 32 * SAMP_T / (SAMP_THREADS - 32);  // entries per loading thread
+    // One pass over `tiles` tiles of every row, the first at completion
+    // x0(row); the adder warp calls add(p, completion within the pass) in order.
+    auto pass = [&](int tiles, auto x0, auto add) {
+        double2 v[PER];
+        auto load = [&](int t) {
+#pragma unroll
+            for (int j = 0; j < PER; ++j) {
+                const int e = (tid - 32) + j * (SAMP_THREADS - 32);
+                const int row = e >> tb, x = e & (T - 1);
+                v[j] = make_double2(0.0, 0.0);
+                if (row < 32 && row0 + row < k) v[j] = amps[((row0 + row) << r) + x0(row) + t * T + x];
+            }
+        };
+        if (!adder) load(0);
+        for (int t = 0; t < tiles; ++t) {
+            if (!adder) {
+#pragma unroll
+                for (int j = 0; j < PER; ++j) {
+                    const int e = (tid - 32) + j * (SAMP_THREADS - 32);
+                    if (e < (32 << tb))
+                        s_p[t & 1][e >> tb][e & (T - 1)] = __dadd_rn(__dmul_rn(v[j].x, v[j].x), __dmul_rn(v[j].y, v[j].y));
+                }
+                if (t + 1 < tiles) load(t + 1);
+            }
+            __syncthreads();  // tile t is in place; its buffer's tile t - 2 has been added up
+            if (adder)
+                for (int x = 0; x < T; ++x) add(s_p[t & 1][lane][x], t * T + x);
         }
+        __syncthreads();
+    };
+    double c = 0.0;
+    pass(n / T, [](int) { return 0; }, [&](double p, int x) {
+        c = __dadd_rn(c, p);
+        if (((x + 1) & (seg - 1)) == 0) s_ck[x / seg][lane] = c;
+    });
+    double thr = 0.0, c1 = 0.0;
+    int x0 = 0, pick = n - 1;
+    if (adder) {
+        thr = __dmul_rn(row0 + lane < k ? uniform[row0 + lane] : 0.0, c);
+        int j = 0;
+        while (j + 1 < n / seg && !(s_ck[j][lane] > thr)) ++j;  // the last segment if none exceeds it
+        x0 = j * seg;
+        c1 = j > 0 ? s_ck[j - 1][lane] : 0.0;
+        s_x0[lane] = x0;
     }
-    picks[p] = pick;
+    __syncthreads();
+    bool found = false;
+    pass(seg / T, [&](int row) { return s_x0[row]; }, [&](double p, int x) {
+        c1 = __dadd_rn(c1, p);
+        if (!found && c1 > thr) {
+            pick = x0 + x;
+            found = true;
+        }
+    });
+    if (adder && row0 + lane < k) picks[row0 + lane] = pick;
 }
 
 // FP32 fused multiply-add throughput probe: each thread runs 8 independent
@@ -1179,8 +1237,10 @@ cudaError_t launch_xeb(const double *amps, int64_t k, double scale, double *out,
 cudaError_t launch_sample(const double *amps, int64_t k, int r, const double *uniform, int64_t *picks,
                           cudaStream_t s) {
     if (k == 0) return cudaSuccess;
-    k_sample<<<dim3((unsigned)((k + 127) / 128)), 128, 0, s>>>(reinterpret_cast<const double2 *>(amps), k, r,
-                                                               uniform, picks);
+    const int64_t blocks = (k + 31) / 32;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    k_sample<<<dim3((unsigned)blocks), SAMP_THREADS, 0, s>>>(reinterpret_cast<const double2 *>(amps), k, r, uniform,
+                                                             picks);
     return cudaGetLastError();
 }
 

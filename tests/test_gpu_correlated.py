@@ -101,3 +101,24 @@ def test_pipeline_with_open_qubits(case20):
     got = dict(contract_batches(c, batches, ssa, sl, "fp32", ws, open_qubits=open_q))
     for i, b in enumerate(batches):
         assert rel_l2(got[i], sv.correlated_amplitudes(c, b, open_q)) <= 1e-5
+
+
+@pytest.mark.parametrize("rows,n_open", [(1, 0), (33, 0), (65, 1), (31, 4), (32, 5), (33, 6), (100, 10), (3, 12), (2, 16)])
+def test_samples_over_tiles_and_segments(rows, n_open):
+    # rows per block (32), completions per tile (32) and per segment; numbers
+    # at 0 and next to 1, rows of zeros, infinities and NaN
+    torch, tn = require_cuda()
+    rng = np.random.default_rng(rows + 64 * n_open)
+    a = rng.normal(size=(rows, 1 << n_open)) + 1j * rng.normal(size=(rows, 1 << n_open))
+    u = rng.random(rows)
+    u[:: 5], u[1:: 7] = 0.0, 1.0 - 2.0 ** -53
+    if rows > 8:
+        a[3], a[4, -1], a[5, 0], a[6, : 1 << n_open >> 1] = 0.0, np.inf, np.nan, 0.0
+    d = torch.from_numpy(a.reshape(-1).view(np.float64).copy()).cuda()
+    picks = torch.full((rows + 1,), -5, dtype=torch.int64, device="cuda")
+    tn.tn_sample_completions(d, rows, n_open, torch.from_numpy(u).cuda(), picks)
+    p = a.real * a.real + a.imag * a.imag
+    c = np.cumsum(p, axis=1)
+    hit = c > (u * c[:, -1])[:, None]
+    ref = np.where(hit.any(1), hit.argmax(1), (1 << n_open) - 1)
+    assert np.array_equal(picks[:rows].cpu().numpy(), ref) and picks[rows].item() == -5
