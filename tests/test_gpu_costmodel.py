@@ -113,6 +113,36 @@ def test_fp16_inference_matches_oracle():
     assert np.max(err) <= 3e-2 * max(1.0, np.max(np.abs(ref)))
 
 
+@pytest.mark.parametrize("n", [1, 31, 33, 255, 257, 4864, 4865, 78000])
+def test_row_tiles_and_their_remainders(n):
+    # rows per tile (32), per FP16 block (256), one chunk per SM (152 x 32)
+    # and several tiles a chunk; FP16 parameters on an odd address
+    torch, tn = require_cuda()
+    p = _params(8).astype(np.float32)
+    X, t = _data(n, 11)
+    X, t = X.astype(np.float32), t.astype(np.float32)
+    dp, dX = _dev(torch, p), _dev(torch, X)
+    ref = omlp.forward(p.astype(np.float64), X.astype(np.float64), D, H)
+    y = torch.full((n + 1,), 7.0, dtype=torch.float32, device="cuda")
+    tn.tn_mlp_forward(dp, dX, n, y)
+    assert rel_l2(y[:n].cpu().numpy(), ref) <= 1e-6 and y[n].item() == 7.0
+    q = torch.zeros(tn.TN_MLP_NPARAMS + 1, dtype=torch.int16, device="cuda")
+    for off in (0, 1):
+        tn.tn_mlp_to_half(dp, q[off:])
+        tn.tn_mlp_forward_f16(q[off:], dX, n, y)
+        err = np.abs(y[:n].cpu().numpy() - ref)
+        assert np.max(err) <= 3e-2 * max(1.0, np.max(np.abs(ref))) and y[n].item() == 7.0
+    g, loss = torch.empty(tn.TN_MLP_NPARAMS, device="cuda"), torch.empty(1, device="cuda")
+    scratch = torch.empty(tn.tn_mlp_grad_scratch_bytes(n), dtype=torch.uint8, device="cuda")
+    tn.tn_mlp_grad(dp, dX, _dev(torch, t), n, g, loss, scratch)
+    gref, L = omlp.grad(p.astype(np.float64), X.astype(np.float64), t.astype(np.float64), D, H)
+    assert abs(loss.item() - L) <= 2e-6 * L
+    # FP32 sums: 1e-6; a unit whose z lies within FP32 rounding of 0 (about
+    # 256 n 1e-7 of the 256 n) may be on in one and off in the other, each a
+    # row's share 1 / n of one unit's gradient: held to 1e-4 as above
+    assert rel_l2(g.cpu().numpy(), gref) <= 1e-4
+
+
 def test_training_fits_a_smooth_target():
     torch, tn = require_cuda()
     from paper_2212_04749_gb300.costmodel import Trainer
