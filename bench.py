@@ -52,7 +52,7 @@ import numpy as np  # noqa: E402
 
 METRIC = "amplitudes/sec & TFLOP/s (frac of peak), mixed vs FP32 at stated amp error"
 UNIT = "amplitudes/s"
-FAMILIES = {0: "k_step_row", 1: "k_step_gemm_simt", 2: "k_step_gemm_tc", 3: "k_chain"}
+FAMILIES = {0: "k_step_row", 1: "k_step_gemm_simt", 2: "k_step_gemm_tc", 3: "k_chain", 4: "k_small_steps"}
 TOL = {"fp32": 1e-5, "bf16x3": 1e-3, "tf32": 1e-3}
 
 
@@ -779,7 +779,7 @@ def run_ours(args, world, rank, local):
         "correlated_batches": correlated,
         "fused_chains": fusion,
         "e2e": e2e,
-        "gpu_launches": int(info["launches_per_call"]) * args.steps,
+        "gpu_launches": plan.tn_plan_launches() * args.steps,
         "clocks": clocks,
     }
     if rank == 0:

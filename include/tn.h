@@ -117,7 +117,8 @@ typedef struct {
     int64_t workspace_bytes;      /* device bytes tn_plan_bind needs */
     int64_t peak_tensor_bytes;    /* largest intermediate set (all instances) */
     int64_t upload_bytes;         /* host-to-device bytes tn_plan_bind copies */
-    int64_t launches_per_call;    /* kernels one full tn_contract launches */
+    int64_t launches_per_call;    /* steps (a fused chain: one) that one full tn_contract
+                                     runs, + leaf fill and sum per batch */
     int32_t n_open;               /* open output qubits (tn_options.open_mask) */
     int32_t n_chains;             /* fused chains (tn_options.fuse) */
     int64_t amps_per_row;         /* 2^n_open complex amplitudes per input row */
@@ -149,6 +150,12 @@ int tn_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k,
  * workspace tn_plan_bind needs and the batch partition of the slices
  * (SM Sec. IV.B).  TN_EINVAL for null arguments. */
 int tn_plan_query(tn_plan_t plan, tn_plan_info *info);
+
+/* Kernels that one full tn_contract launches now: tn_plan_info's
+ * launches_per_call less what small steps save by sharing launches (see
+ * tn_plan_step_times, family 4); helper launches inside a step (a packed B)
+ * are not counted.  Host only. */
+int tn_plan_launches(tn_plan_t plan, int64_t *launches);
 
 /* Per-node reuse widths w_v (distinct projections of the bitstrings onto
  * the node's output qubits) and per-instance ranks, 2T-1 entries each; the
@@ -306,7 +313,12 @@ int tn_plan_set_kernel(tn_plan_t plan, int32_t step, int32_t kernel);
 #define TN_NCONFIG 4
 
 /* Set step `step` to configuration `config` (-1: the plan's own choice).
+ * A step given a configuration (>= 0) then runs by itself even if it is small
+ * (see tn_plan_step_times, family 4); config + TN_CONFIG_TUNED, with config as
+ * tn_plan_get_configs returned it for a tuned plan of the same shape, leaves
+ * small steps together, as tn_plan_autotune and tn_plan_select do.
  * TN_EINVAL for a configuration the step's shape does not allow. */
+#define TN_CONFIG_TUNED 16
 int tn_plan_set_config(tn_plan_t plan, int32_t step, int32_t config);
 
 /* Tensor-core form of the grouped GEMM.  enable = 1 (the default): where B
@@ -329,10 +341,12 @@ int tn_plan_set_tc_pairs(tn_plan_t plan, int32_t enable);
 
 /* Fused chains (tn_options.fuse; SM Sec. V.C fuses a run of steps so that
  * only its last output leaves fast memory).  A chain runs fused (enable = 1,
- * the default: one kernel, intermediates never stored) or as its separate
+ * one kernel, intermediates never stored) or as its separate
  * steps (0: each step with its own configuration, its intermediate written
  * to the slot the plan keeps for it); both give the same values up to
- * rounding.  tn_plan_autotune decides per chain by timing both.  TN_EINVAL
+ * rounding.  A chain for which nothing was chosen runs fused, or, if all its
+ * steps are small, among the plan's merged small steps (tn_plan_get_chains:
+ * 1).  tn_plan_autotune decides per chain by timing both.  TN_EINVAL
  * for a chain outside [0, n_chains). */
 int tn_plan_set_chain(tn_plan_t plan, int32_t chain, int32_t enable);
 /* Whether each chain runs fused (n entries, 1 or 0). */
@@ -365,7 +379,8 @@ int tn_plan_features(tn_plan_t plan, int precision, int32_t config, float *feat,
  * afterwards).  Fused chains: the configurations are timed with every
  * chain run as separate steps; then each chain is timed fused and kept
  * fused only where that beats the sum of its steps' best times
- * (tn_plan_set_chain).  Needs a bound workspace; synchronises `stream`. */
+ * (tn_plan_set_chain); chains of small steps only run among the plan's
+ * merged small steps.  Needs a bound workspace; synchronises `stream`. */
 int tn_plan_autotune(tn_plan_t plan, int precision, int32_t reps, const uint8_t *step_mask, double *amps_scratch,
                      double *times, void *stream);
 
@@ -373,7 +388,8 @@ int tn_plan_autotune(tn_plan_t plan, int precision, int32_t reps, const uint8_t 
  * configuration) with the FP16 network params16 (device, TN_MLP_NPARAMS
  * halves, see tn_mlp_to_half), set each step to its predicted fastest
  * configuration, and flag in uncertain (host, n_steps int32, may be NULL)
- * the steps whose two best predictions lie within `margin` (log2 units):
+ * the steps, other than small ones that share launches, whose two best
+ * predictions lie within `margin` (log2 units):
  * those are the steps to hand to tn_plan_autotune (its step_mask) as the
  * fallback.  scratch: device buffer of at least
  * n_steps * TN_NCONFIG * (TN_NFEAT + 1) * 4 bytes.  Synchronises `stream`. */
@@ -420,7 +436,9 @@ int tn_plan_check(tn_plan_t plan, void *stream);
  * synchronises the events); ms has n_steps entries.  kernel (may be NULL)
  * receives the kernel family each step last ran: 0 per-row SIMT, 1 tiled
  * SIMT GEMM, 2 tensor-core GEMM, 3 fused chain (the chain's time is booked
- * on its last step). */
+ * on its last step), 4 small steps (at most 2^18 complex multiply-adds and
+ * 2^14 outputs each, no kernel set for them by tn_plan_set_config) that share one launch (its
+ * time is booked on the last of them). */
 int tn_plan_profile(tn_plan_t plan, int enable);
 int tn_plan_step_times(tn_plan_t plan, double *ms, int32_t *kernel, int32_t n);
 

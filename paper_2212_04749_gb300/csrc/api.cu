@@ -51,8 +51,16 @@ struct PlanObj {
     size_t ev_used = 0;
     std::vector<int32_t> step_kernel;     // kernel family each step ran last (0 row, 1 SIMT GEMM, 2 TC GEMM)
     std::vector<int32_t> config_override; // per step: -1 plan choice, else a configuration (tn.h)
-    std::vector<uint8_t> chain_on;        // per fused chain: run as one kernel (1) or as its steps (0)
-    bool chain_fused(int c) const { return c >= 0 && (c >= (int)chain_on.size() || chain_on[c] != 0); }
+    // per fused chain: run as one kernel (1), as its steps (0), or not chosen
+    // (-1: one kernel, unless all its steps are small: those share the merged
+    // launches, which cost less than a kernel of their own)
+    std::vector<int8_t> chain_on;
+    std::vector<uint8_t> chain_small;     // all steps of the chain are small
+    int chain_state(int c) const { return c < (int)chain_on.size() ? chain_on[c] : -1; }
+    bool chain_enabled(int c) const { return c >= 0 && chain_state(c) != 0; }
+    bool chain_fused(int c) const {
+        return c >= 0 && (chain_state(c) > 0 || (chain_state(c) < 0 && !(merge_small && chain_small[c])));
+    }
     struct GraphKey {
         int precision;
         int64_t lo, hi;
@@ -61,11 +69,25 @@ struct PlanObj {
             return std::tie(precision, lo, hi, amps) < std::tie(o.precision, o.lo, o.hi, o.amps);
         }
     };
+    // Launch order of the steps that a slice batch of one recompute level
+    // runs (64: every step).
+    struct Sched {
+        struct Item {
+            int step;   // group < 0: this step's launch (a fused chain's last step: the chain)
+            int group;  // else: the small steps of groups[group], one launch
+        };
+        std::vector<Item> items;
+        std::vector<tnk::SmallArgs> groups;
+    };
+    std::map<int, Sched> scheds;  // by level; dropped with the graphs
+    bool merge_small = true;                      // small steps run together (off while the autotuner times them singly)
+    std::vector<uint8_t> pinned;                  // per step: the caller chose its kernel (tn_plan_set_config)
     std::map<GraphKey, cudaGraphExec_t> graphs;  // captured tn_contract launch sequences
     cudaStream_t cap_stream = nullptr;           // private stream the sequences are captured on
     void drop_graphs() {
         for (auto &kv : graphs) cudaGraphExecDestroy(kv.second);
         graphs.clear();
+        scheds.clear();
     }
     int64_t last_batches = 0;
 };
@@ -189,6 +211,38 @@ void build_descs(PlanObj *o) {
     }
 }
 
+// The steps as small.cu sees them (those that are not small stay empty).
+std::vector<tnk::SmallDesc> small_descs(const PlanObj *o) {
+    static_assert(sizeof(tnk::SmallDesc) == tnp::SMALL_DESC_BYTES, "room in the workspace");
+    std::vector<tnk::SmallDesc> v(o->P.steps.size());
+    for (size_t s = 0; s < v.size(); ++s) {
+        const tnk::StepDesc &d = o->desc[s];
+        tnk::SmallDesc &r = v[s];
+        std::memset(&r, 0, sizeof(r));
+        if (!o->P.steps[s].small) continue;
+        r.A = d.A;
+        r.B = d.B;
+        r.C = d.C;
+        r.instab = d.instab;
+        r.EA = d.EA;
+        r.EB = d.EB;
+        r.EC = d.EC;
+        r.mxA = d.mxA;
+        r.mxB = d.mxB;
+        r.mxC = d.mxC;
+        r.sA = d.sA;
+        r.sB = d.sB;
+        r.sC = d.sC;
+        r.kb = (int8_t)d.kb;
+        r.nb = (int8_t)d.nb;
+        r.mnb = (int8_t)(d.mb + d.nb);
+        r.outputs = (int32_t)(d.nInst << (d.mb + d.nb));
+        for (int j = 0; j < d.nb; ++j) r.pC[j] = d.pCn[j];
+        for (int j = 0; j < d.mb; ++j) r.pC[d.nb + j] = d.pCm[j];
+    }
+    return v;
+}
+
 // Configurations (tn.h): 0, 1 per-row kernel (schedule 0, 1); 2, 3 grouped
 // GEMM (schedule 0, 1).
 bool config_allowed(const tnp::Step &S, int c) {
@@ -204,9 +258,6 @@ int effective_config(const PlanObj *o, int s) {
 int run_step(PlanObj *o, int s, int precision, cudaStream_t st) {
     const tnp::Step &S = o->P.steps[s];
     if (o->chain_fused(S.chain)) {  // fused chain: runs whole at its last step
-        if ((int)o->step_kernel.size() <= s) o->step_kernel.resize(o->P.steps.size(), -1);
-        o->step_kernel[s] = 3;
-        if (!S.chain_last) return TN_OK;
         const cudaError_t e = tnk::launch_chain(o->chain_desc[S.chain], st);
         if (e != cudaSuccess)
             return set_err(TN_ECUDA, "fused chain at step " + std::to_string(s) + ": " + cudaGetErrorString(e));
@@ -234,11 +285,139 @@ int run_step(PlanObj *o, int s, int precision, cudaStream_t st) {
         fam = 1;
         e = tnk::launch_step_gemm_simt(d, st);
     }
-    if ((int)o->step_kernel.size() <= s) o->step_kernel.resize(o->P.steps.size(), -1);
     o->step_kernel[s] = fam;
     if (e != cudaSuccess)
         return set_err(TN_ECUDA, "step " + std::to_string(s) + ": " + cudaGetErrorString(e));
     return TN_OK;
+}
+
+int run_group(PlanObj *o, tnk::SmallArgs g, cudaStream_t st) {
+    g.descs = at<const tnk::SmallDesc>(o, o->P.off_small);
+    for (int j = 0; j < g.n_steps; ++j) o->step_kernel[g.step[j]] = 4;
+    const cudaError_t e = tnk::launch_small(g, st);
+    if (e != cudaSuccess) return set_err(TN_ECUDA, std::string("small steps: ") + cudaGetErrorString(e));
+    return TN_OK;
+}
+
+// Whether step s may share a launch with other small steps.
+bool merges(const PlanObj *o, int s) {
+    return o->merge_small && o->P.steps[s].small && !(s < (int)o->pinned.size() && o->pinned[s]);
+}
+
+// Launch order for a slice batch of recompute level lv (64: every step).
+// The steps keep the plan's order except that small ones move: they wait
+// until a step that does not merge needs one of them, and then every small
+// step whose operands exist runs in the same launch, in phases.  Two steps
+// keep their order where the later reads what the earlier writes, or writes
+// memory that the earlier reads or writes (the workspace gives a slot to
+// another node after its last reader in the plan's order).
+PlanObj::Sched make_schedule(const PlanObj *o, int lv) {
+    PlanObj::Sched R;
+    const tnp::Plan &P = o->P;
+    struct Node {
+        int step, write;
+        std::vector<int> reads;
+        bool small;
+    };
+    std::vector<Node> L;
+    for (int s = 0; s < (int)P.steps.size(); ++s) {
+        const tnp::Step &S = P.steps[s];
+        if (S.level > lv) continue;
+        Node n{s, S.node, {}, false};
+        if (o->chain_fused(S.chain)) {
+            if (!S.chain_last) continue;
+            const tnp::Chain &c = P.chains[S.chain];
+            n.reads.push_back(P.steps[c.steps[0]].a);
+            for (int q : c.steps) n.reads.push_back(P.steps[q].b);
+        } else {
+            n.reads = {S.a, S.b};
+            n.small = merges(o, s);
+        }
+        L.push_back(n);
+    }
+    const int nl = (int)L.size();
+    auto overlap = [&](int u, int v) {
+        const tnp::Node &x = P.nodes[u], &y = P.nodes[v];
+        return x.buf.data < y.buf.data + y.n_inst * (int64_t(8) << y.rank) &&
+               y.buf.data < x.buf.data + x.n_inst * (int64_t(8) << x.rank);
+    };
+    std::vector<std::vector<int>> after(nl);  // edges to later items
+    std::vector<int> open(nl, 0);             // unfinished items before
+    for (int q = 0; q < nl; ++q)
+        for (int p = 0; p < q; ++p) {
+            bool dep = overlap(L[q].write, L[p].write);
+            for (int r : L[q].reads) dep = dep || r == L[p].write;
+            for (int r : L[p].reads) dep = dep || overlap(L[q].write, r);
+            if (dep) {
+                after[p].push_back(q);
+                ++open[q];
+            }
+        }
+    std::vector<char> done(nl, 0);
+    auto finish = [&](int q) {
+        done[q] = 1;
+        for (int t : after[q]) --open[t];
+    };
+    int left = nl, next_big = 0;
+    while (left > 0) {
+        while (next_big < nl && (done[next_big] || L[next_big].small)) ++next_big;
+        if (next_big < nl && open[next_big] == 0) {
+            R.items.push_back({L[next_big].step, -1});
+            finish(next_big);
+            --left;
+            continue;
+        }
+        tnk::SmallArgs g;
+        std::memset(&g, 0, sizeof(g));
+        int last = -1;
+        while (g.n_phases < tnk::SMALL_MAX_PHASES && g.n_steps < tnk::SMALL_MAX_STEPS) {
+            std::vector<int> ready;
+            int64_t outputs = 0;
+            for (int q = 0; q < nl && g.n_steps + (int)ready.size() < tnk::SMALL_MAX_STEPS; ++q)
+                if (!done[q] && L[q].small && open[q] == 0) {
+                    ready.push_back(q);
+                    const tnp::Step &S = P.steps[L[q].step];
+                    outputs += P.nodes[S.node].n_inst << (S.mb + S.nb);
+                }
+            if (ready.empty()) break;
+            // lanes per output: as many as leave the phase within 4096 threads
+            int lanes = 0;
+            while (lanes < 5 && (outputs << (lanes + 1)) <= 4096) ++lanes;
+            int64_t warps = 0;
+            for (int q : ready) {
+                const tnp::Step &S = P.steps[L[q].step];
+                const int lg = std::min(lanes, std::max(S.kb - 1, 0));
+                // a warp takes 32 lanes of outputs, four times as many where
+                // the step fills the cluster's 128 warps four times over
+                const int64_t w = (((P.nodes[S.node].n_inst << (S.mb + S.nb)) << lg) + 31) / 32;
+                const bool four = w >= 512;
+                g.four[g.n_steps] = four;
+                warps += four ? (w + 3) / 4 : w;
+                g.step[g.n_steps] = (uint16_t)L[q].step;
+                g.lanes_log2[g.n_steps] = (uint8_t)lg;
+                g.wend[g.n_steps] = (int32_t)warps;
+                last = std::max(last, L[q].step);
+                ++g.n_steps;
+            }
+            for (int q : ready) finish(q);
+            left -= (int)ready.size();
+            g.max_warps = std::max<int32_t>(g.max_warps, (int32_t)std::min<int64_t>(warps, 1 << 20));
+            g.phase_end[g.n_phases++] = (uint16_t)g.n_steps;
+        }
+        if (g.n_steps == 1) {
+            R.items.push_back({last, -1});
+        } else {
+            R.items.push_back({last, (int)R.groups.size()});
+            R.groups.push_back(g);
+        }
+    }
+    return R;
+}
+
+const PlanObj::Sched &schedule(PlanObj *o, int lv) {
+    auto it = o->scheds.find(lv);
+    if (it == o->scheds.end()) it = o->scheds.emplace(lv, make_schedule(o, lv)).first;
+    return it->second;
 }
 
 // Cost-model features of step s under configuration c (tn.h, TN_NFEAT).
@@ -294,7 +473,9 @@ void step_features(const tnp::Plan &P, int s, int precision, int c, float *f) {
 template <class F>
 int run_batches(PlanObj *o, int precision, int64_t b_lo, int64_t b_hi, cudaStream_t st, F per_batch) {
     tnp::Plan &P = o->P;
-    const int nst = (int)P.steps.size();
+    o->step_kernel.resize(P.steps.size(), -1);
+    for (size_t s = 0; s < P.steps.size(); ++s)
+        if (o->chain_fused(P.steps[s].chain)) o->step_kernel[s] = 3;
     o->ev_used = 0;
     o->ev_step.clear();
     const auto *jobs = at<const tnk::FillJobD>(o, P.off_fill_jobs);
@@ -305,8 +486,9 @@ int run_batches(PlanObj *o, int precision, int64_t b_lo, int64_t b_hi, cudaStrea
         if (clear) CU(cudaMemsetAsync(o->ws + P.off_emax, 0, clear, st));
         cudaError_t e = tnk::launch_fill(jobs, P.n_fill_jobs, highs, b, at<float2>(o, 0), st);
         if (e != cudaSuccess) return set_err(TN_ECUDA, std::string("leaf fill: ") + cudaGetErrorString(e));
-        for (int s = 0; s < nst; ++s) {
-            if (b != b_lo && P.steps[s].level > lv) continue;
+        const PlanObj::Sched &order = schedule(o, lv);
+        for (const PlanObj::Sched::Item &it : order.items) {
+            const int s = it.step;
             if (o->profile) {
                 while (o->ev.size() < 2 * (o->ev_used + 1)) {
                     cudaEvent_t ev;
@@ -315,7 +497,11 @@ int run_batches(PlanObj *o, int precision, int64_t b_lo, int64_t b_hi, cudaStrea
                 }
                 CU(cudaEventRecord(o->ev[2 * o->ev_used], st));
             }
-            if (int rc = run_step(o, s, precision, st)) return rc;
+            if (it.group >= 0) {
+                if (int rc = run_group(o, order.groups[it.group], st)) return rc;
+            } else if (int rc = run_step(o, s, precision, st)) {
+                return rc;
+            }
             if (o->profile) {
                 CU(cudaEventRecord(o->ev[2 * o->ev_used + 1], st));
                 o->ev_step.push_back(s);
@@ -325,7 +511,6 @@ int run_batches(PlanObj *o, int precision, int64_t b_lo, int64_t b_hi, cudaStrea
         if (int rc = per_batch(b)) return rc;
     }
     o->last_batches = b_hi - b_lo;
-    (void)nst;
     return TN_OK;
 }
 
@@ -388,6 +573,11 @@ int tn_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int32_
     } catch (const std::bad_alloc &) {
         return set_err(TN_ENOMEM, "tn_plan: host allocation failed");
     }
+    for (const tnp::Chain &c : o->P.chains) {
+        bool all = true;
+        for (int q : c.steps) all = all && o->P.steps[q].small;
+        o->chain_small.push_back(all ? 1 : 0);
+    }
     *out = reinterpret_cast<tn_plan_t>(o.release());
     g_err.clear();
     return TN_OK;
@@ -418,11 +608,23 @@ int tn_plan_query(tn_plan_t plan, tn_plan_info *info) {
     info->upload_bytes = up;
     const PlanObj *po = reinterpret_cast<const PlanObj *>(plan);
     double steps_run = 0;
-    for (const tnp::Step &st : P.steps) steps_run += (!po->chain_fused(st.chain) || st.chain_last) ? st.runs : 0.0;
+    for (const tnp::Step &st : P.steps) steps_run += (!po->chain_enabled(st.chain) || st.chain_last) ? st.runs : 0.0;
     info->launches_per_call = (int64_t)steps_run + 2 * P.n_batches;  // + leaf fill and accumulate per batch
     info->n_open = (int32_t)P.open_qubits.size();
     info->n_chains = (int32_t)P.chains.size();
     info->amps_per_row = int64_t(1) << P.open_qubits.size();
+    return TN_OK;
+}
+
+int tn_plan_launches(tn_plan_t plan, int64_t *launches) {
+    if (!plan || !launches) return set_err(TN_EINVAL, "tn_plan_launches: null argument");
+    const PlanObj *o = reinterpret_cast<const PlanObj *>(plan);
+    // the first batch runs every step, n_batches >> (l + 1) later ones those of level l and below
+    const int64_t nb = o->P.n_batches;
+    int64_t n = 2 * nb + (int64_t)make_schedule(o, 64).items.size();
+    for (int l = 0; (nb >> (l + 1)) > 0; ++l) n += (nb >> (l + 1)) * (int64_t)make_schedule(o, l).items.size();
+    *launches = n;
+    g_err.clear();
     return TN_OK;
 }
 
@@ -509,6 +711,7 @@ int tn_plan_bind(tn_plan_t plan, void *workspace, size_t bytes, void *stream) {
     CU(tnk::init_kernels());
     CU(tnk::init_chain_kernel());
     CU(tnk::init_simt_kernels());
+    CU(tnk::init_small_kernel());
     o->drop_graphs();
     o->ws = static_cast<uint8_t *>(workspace);
     o->ws_bytes = bytes;
@@ -518,8 +721,11 @@ int tn_plan_bind(tn_plan_t plan, void *workspace, size_t bytes, void *stream) {
     }
     o->err_flag = at<int32_t>(o, o->P.off_scratch);
     CU(cudaMemsetAsync(o->err_flag, 0, 4, st));
-    CU(cudaStreamSynchronize(st));
     build_descs(o);
+    const std::vector<tnk::SmallDesc> small = small_descs(o);
+    CU(cudaMemcpyAsync(o->ws + o->P.off_small, small.data(), small.size() * sizeof(tnk::SmallDesc),
+                       cudaMemcpyHostToDevice, st));
+    CU(cudaStreamSynchronize(st));
     g_err.clear();
     return TN_OK;
 }
@@ -742,11 +948,16 @@ int tn_plan_set_config(tn_plan_t plan, int32_t step, int32_t config) {
     PlanObj *o = reinterpret_cast<PlanObj *>(plan);
     const tnp::Plan &P = o->P;
     if (step < 0 || step >= (int32_t)P.steps.size()) return set_err(TN_EINVAL, "tn_plan_set_config: bad step");
+    const bool tuned = config >= TN_CONFIG_TUNED;
+    if (tuned) config -= TN_CONFIG_TUNED;
     if (config < -1 || config >= TN_NCONFIG) return set_err(TN_EINVAL, "tn_plan_set_config: bad configuration");
     if (config >= 0 && !config_allowed(P.steps[step], config))
         return set_err(TN_EINVAL, "tn_plan_set_config: per-row kernel needs N <= 16 and K*N <= 256");
     o->config_override.resize(P.steps.size(), -1);
     o->config_override[step] = config;
+    // a step whose kernel was chosen runs by itself even if it is small
+    o->pinned.resize(P.steps.size(), 0);
+    o->pinned[step] = !tuned && config >= 0;
     o->drop_graphs();
     return TN_OK;
 }
@@ -755,7 +966,7 @@ int tn_plan_set_chain(tn_plan_t plan, int32_t chain, int32_t enable) {
     if (!plan) return set_err(TN_EINVAL, "tn_plan_set_chain: null plan");
     PlanObj *o = reinterpret_cast<PlanObj *>(plan);
     if (chain < 0 || chain >= (int32_t)o->P.chains.size()) return set_err(TN_EINVAL, "tn_plan_set_chain: bad chain");
-    o->chain_on.resize(o->P.chains.size(), 1);
+    o->chain_on.resize(o->P.chains.size(), -1);
     o->chain_on[chain] = enable ? 1 : 0;
     o->drop_graphs();
     return TN_OK;
@@ -764,7 +975,7 @@ int tn_plan_set_chain(tn_plan_t plan, int32_t chain, int32_t enable) {
 int tn_plan_get_chains(tn_plan_t plan, int32_t *enabled, int32_t n) {
     if (!plan || (n > 0 && !enabled)) return set_err(TN_EINVAL, "tn_plan_get_chains: null argument");
     PlanObj *o = reinterpret_cast<PlanObj *>(plan);
-    for (int32_t c = 0; c < n && c < (int32_t)o->P.chains.size(); ++c) enabled[c] = o->chain_fused(c) ? 1 : 0;
+    for (int32_t c = 0; c < n && c < (int32_t)o->P.chains.size(); ++c) enabled[c] = o->chain_enabled(c) ? 1 : 0;
     return TN_OK;
 }
 
@@ -818,10 +1029,20 @@ int tn_plan_autotune(tn_plan_t plan, int precision, int32_t reps, const uint8_t 
     std::vector<double> best(size_t(ns) * TN_NCONFIG, NAN), ms(ns);
     const bool prof = o->profile;
     o->profile = true;  // CUDA events around every step launch
+    // Every step in a launch of its own; with a mask, the steps that are not
+    // timed share launches as ever.
+    const std::vector<uint8_t> prev_pinned = o->pinned;
+    if (step_mask) {
+        o->pinned.resize(ns, 0);
+        for (int s = 0; s < ns; ++s) o->pinned[s] |= step_mask[s] != 0;
+    } else {
+        o->merge_small = false;
+    }
     o->config_override.assign(ns, -1);
     const int nchains = (int)P.chains.size();
-    const std::vector<uint8_t> prev_chain = o->chain_on;
+    const std::vector<int8_t> prev_chain = o->chain_on;
     o->chain_on.assign(nchains, 0);  // configurations are timed on the separate steps
+    o->drop_graphs();
     int rc = TN_OK;
     for (int c = 0; c < TN_NCONFIG && rc == TN_OK; ++c) {
         bool any = false;
@@ -861,11 +1082,14 @@ int tn_plan_autotune(tn_plan_t plan, int precision, int32_t reps, const uint8_t 
         }
         o->config_override[s] = pick;
     }
+    o->merge_small = true;
+    o->pinned = prev_pinned;
     // fused chains: each kept fused only where its kernel beats the sum of
     // its steps' best times (the chain's time is booked on its last step)
     // (with a step mask only some steps were timed: the chains keep their
     // previous setting)
     if (rc != TN_OK || step_mask) o->chain_on = prev_chain;
+    o->drop_graphs();
     if (rc == TN_OK && nchains > 0 && !step_mask) {
         std::vector<double> unfused(nchains, 0.0), fused(nchains, NAN);
         for (int s = 0; s < ns; ++s) {
@@ -878,7 +1102,8 @@ int tn_plan_autotune(tn_plan_t plan, int precision, int32_t reps, const uint8_t 
             }
             unfused[c] += std::isnan(bt) ? 0.0 : bt;
         }
-        o->chain_on.assign(nchains, 1);
+        for (int c = 0; c < nchains; ++c) o->chain_on[c] = o->chain_small[c] ? 0 : 1;
+        o->drop_graphs();
         o->profile = true;
         for (int r = 0; r <= reps && rc == TN_OK; ++r) {
             rc = tn_contract(plan, precision, 0, P.n_batches > 0 ? 1 : 0, amps_scratch, stream);
@@ -895,6 +1120,10 @@ int tn_plan_autotune(tn_plan_t plan, int precision, int32_t reps, const uint8_t 
         o->profile = prof;
         for (int c = 0; c < nchains; ++c) o->chain_on[c] = (!std::isnan(fused[c]) && fused[c] < unfused[c]) ? 1 : 0;
         if (rc != TN_OK) o->chain_on = prev_chain;
+        // (chains of small steps only stay among the plan's other small steps
+        // in their merged launches: a phase there costs a tenth of a kernel)
+        for (int c = 0; c < nchains; ++c)
+            if (rc == TN_OK && o->chain_small[c]) o->chain_on[c] = 0;
     }
     o->drop_graphs();
     if (times) std::copy(best.begin(), best.end(), times);
@@ -943,7 +1172,8 @@ int tn_plan_select(tn_plan_t plan, int precision, const uint16_t *params16, floa
             }
         }
         o->config_override[s] = b1;
-        if (uncertain) uncertain[s] = (have2 && y2 - y1 < margin) ? 1 : 0;
+        // (a small step that shares a launch runs the same whatever is chosen)
+        if (uncertain) uncertain[s] = (have2 && y2 - y1 < margin && !merges(o, s)) ? 1 : 0;
     }
     o->drop_graphs();
     g_err.clear();

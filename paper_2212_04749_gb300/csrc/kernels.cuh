@@ -152,6 +152,40 @@ size_t chain_smem_bytes(const ChainDesc &d);
 cudaError_t init_chain_kernel();
 cudaError_t launch_chain(ChainDesc d, cudaStream_t s);
 
+// Small steps, many to a launch (small.cu).  A step as the kernel sees it;
+// one per step in the workspace, written when it is bound.
+struct SmallDesc {
+    const float2 *A, *B;
+    float2 *C;
+    const int2 *instab;           // per output instance: {A instance, B instance}
+    const int32_t *EA, *EB;
+    int32_t *EC;
+    const uint32_t *mxA, *mxB;    // null: no rescale
+    uint32_t *mxC;
+    int64_t sA, sB, sC;           // elements per instance
+    int32_t outputs;              // instances << (mb + nb)
+    int8_t kb, nb, mnb, pad_;     // mnb = mb + nb
+    int8_t pC[24];                // C address bit of output bit j: the n bits, then the m bits
+    int8_t pad2_[24];
+};
+static_assert(sizeof(SmallDesc) == 160, "tnp::SMALL_DESC_BYTES");
+// One launch: steps in phases; the steps of a phase depend on earlier phases
+// only.
+constexpr int SMALL_MAX_STEPS = 256, SMALL_MAX_PHASES = 64;
+struct SmallArgs {
+    const SmallDesc *descs;       // of the whole plan
+    int32_t n_steps, n_phases;
+    int32_t max_warps;            // warps that the widest phase can use
+    int32_t wend[SMALL_MAX_STEPS];       // warps of the phase's steps up to and with this one
+    uint16_t step[SMALL_MAX_STEPS];
+    uint8_t lanes_log2[SMALL_MAX_STEPS]; // lanes that share one output's K sum
+    uint8_t four[SMALL_MAX_STEPS];       // a warp takes 4 x 32 lanes of outputs
+    uint16_t phase_end[SMALL_MAX_PHASES];
+};
+static_assert(sizeof(SmallArgs) <= 4096, "kernel parameters");
+cudaError_t init_small_kernel();
+cudaError_t launch_small(const SmallArgs &a, cudaStream_t s);
+
 // Cost-model MLP (mlp.cu); sizes and parameter layout in include/tn.h.
 size_t mlp_grad_scratch_bytes(int64_t n);
 cudaError_t mlp_forward(const float *params, const float *X, int64_t n, float *y, cudaStream_t s);

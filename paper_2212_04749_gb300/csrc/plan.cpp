@@ -461,6 +461,8 @@ struct Builder {
             // A on average); everything else is a GEMM over instance groups
             const double cols_per_a = std::ldexp(double(nd.n_inst) / double(st.n_groups), st.nb);
             st.kernel = (st.nb <= 4 && st.kb + st.nb <= 8 && cols_per_a < 16.0) ? 0 : 1;
+            st.small = macs * double(nd.n_inst) <= SMALL_MACS && st.kb <= SMALL_MAX_KB &&
+                       std::ldexp(double(nd.n_inst), nd.rank) <= SMALL_OUTPUTS;
         }
         for (int s = 0; s < (int)P.steps.size(); ++s) {
             P.nodes[P.steps[s].a].last_use = s;
@@ -652,8 +654,9 @@ struct Builder {
         }
     }
 
-    // Workspace layout; returns total bytes.
-    int64_t layout_workspace(bool emit) {
+    // Workspace layout; returns total bytes.  own_slots: the outputs of small
+    // steps share no memory with other intermediates.
+    int64_t layout_workspace(bool emit, bool own_slots = false) {
         Plan &p = P;
         if (emit) p.uploads.clear();
         int64_t off = 0;
@@ -918,6 +921,15 @@ struct Builder {
                 push_upload(p, c.off_tab, tab);
             }
         }
+        p.off_small = take(int64_t(p.steps.size()) * SMALL_DESC_BYTES);
+        std::vector<char> own(NN, 0);
+        if (own_slots)
+            for (const Step &st : p.steps) {
+                Node &nd = p.nodes[st.node];
+                if (!st.small || nd.persistent) continue;
+                own[st.node] = 1;
+                nd.buf.data = take(nd.n_inst * (int64_t(8) << nd.rank));
+            }
         // transient intermediates: first-fit over one full pass of the steps
         Arena ar;
         ar.base = ar.top = ar.high = off;
@@ -927,10 +939,10 @@ struct Builder {
             const Step &st = p.steps[s];
             Node &nd = p.nodes[st.node];
             const int64_t bytes = nd.n_inst * (int64_t(8) << nd.rank);
-            if (!nd.persistent) nd.buf.data = ar.alloc(bytes);
+            if (!nd.persistent && !own[st.node]) nd.buf.data = ar.alloc(bytes);
             for (int c : {st.a, st.b}) {
                 Node &ch = p.nodes[c];
-                if (ch.persistent || ch.last_use != s) continue;
+                if (ch.persistent || own[c] || ch.last_use != s) continue;
                 ar.release(ch.buf.data, ch.n_inst * (int64_t(8) << ch.rank));
             }
             p.peak_tensor_bytes = std::max(p.peak_tensor_bytes, bytes);
@@ -1233,9 +1245,23 @@ bool make_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int
     // the loop's last schedule() was for `chosen` (layout_workspace(false)
     // only sets offsets that the final layout recomputes)
     B.find_chains();
-    for (Node &nd : P.nodes) { nd.buf = NodeBuf(); }
-    P.peak_tensor_bytes = 0;
-    P.ws_bytes = B.layout_workspace(true);
+    auto layout = [&](bool emit, bool own_slots) {
+        for (Node &nd : P.nodes) nd.buf = NodeBuf();
+        P.peak_tensor_bytes = 0;
+        return B.layout_workspace(emit, own_slots);
+    };
+    // own slots for the small steps' outputs, unless they would take a plan
+    // above a limit that it meets without them
+    int64_t slots = 0;
+    for (const Step &st : P.steps)
+        if (st.small) slots += Arena::align(P.nodes[st.node].n_inst * (int64_t(8) << P.nodes[st.node].rank));
+    bool own_slots = slots <= SMALL_SLOTS_MAX;
+    if (own_slots) {
+        const int64_t without = layout(false, false), with = layout(false, true);
+        for (int64_t limit : {P.opt.workspace_limit, int64_t(TN_STATIC_SCRATCH_BYTES)})
+            if (without <= limit && with > limit) own_slots = false;
+    }
+    P.ws_bytes = layout(true, own_slots);
     if (B.bad_offsets) {
         code = TN_EUNSUPPORTED;
         err = "internal error: workspace layout self-check failed";

@@ -107,11 +107,25 @@ struct Step {
     int64_t n_pair_tiles = 0;
     int64_t off_pair_tab = -1;
     int kernel = 0;          // 0 = per-row SIMT, 1 = tiled SIMT GEMM, 2 = tensor-core GEMM
+    bool small = false;      // little work: may run with others in one launch (small.cu)
     int chain = -1;          // fused chain holding this step (-1: none)
     bool chain_last = false; // the chain runs at its last step; the others launch nothing
     double flops = 0;        // executed per pass: 8 * n_inst * 2^{mb+kb+nb}
     double bytes = 0;        // A + B reads and C write per pass
 };
+
+// A step of at most SMALL_MACS complex multiply-adds and SMALL_OUTPUTS outputs
+// costs its launch and its chain of dependent loads, about 5 us, whatever it
+// computes; such steps run together, many to a launch, on one cluster of 16
+// blocks (small.cu).  There 2^18 multiply-adds, or four outputs for each of
+// its 4096 threads, are about 2 us of loads; steps of 2^17 outputs, whose
+// instance pairs and operands 16 SMs fetch at 2 TB/s, took 12 us.
+constexpr double SMALL_MACS = 262144.0, SMALL_OUTPUTS = 16384.0;
+constexpr int SMALL_MAX_KB = 10;
+constexpr int64_t SMALL_DESC_BYTES = 160;
+// Their outputs get slots of their own, so that no order of them overwrites
+// one still in use, where these slots add little to the workspace.
+constexpr int64_t SMALL_SLOTS_MAX = int64_t(32) << 20;
 
 // A fused chain (SM Sec. V.C): steps s_1..s_L where each step's A operand is
 // the previous step's output, instance counts do not grow, and every side
@@ -174,6 +188,7 @@ struct Plan {
     int64_t off_emax = -1, emax_bytes = 0;  // max words of every node, by level
     std::vector<int64_t> emax_prefix;       // [lv]: bytes covering the nodes of level <= lv
     int64_t off_scratch = -1;               // 256 bytes of device scratch (error word)
+    int64_t off_small = -1;                 // per step: descriptor for small.cu, written at bind time
     int64_t off_bpack = -1, bpack_bytes = 0; // tensor cores: room for one step's B packed in MMA form
     // host images uploaded at bind time: (offset, bytes)
     std::vector<std::pair<int64_t, std::vector<uint8_t>>> uploads;

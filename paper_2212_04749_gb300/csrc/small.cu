@@ -1,0 +1,190 @@
+// Small steps, many to a launch.
+//
+// Below a few 10^5 multiply-adds a pairwise step costs what any launch
+// costs: the launch itself, its wait for the previous step and four or five
+// dependent loads, about 5 us, and a contraction has tens to hundreds of such
+// steps (the merges of leaf tensors and the tail near the root).  Here one
+// cluster of up to 16 blocks runs a list of them: the steps are sorted into
+// phases on the host, a phase's steps depend on earlier phases only and run
+// side by side, and a cluster barrier between phases takes the place of the
+// launch.  A phase costs its barrier and two round trips to L2 (the instance
+// pair, then maxima, A and B together).
+//
+// An output C[i](m, n) is one sum over k, split over 2^lanes_log2
+// neighbouring lanes where a step has fewer outputs than the cluster has
+// threads, in FP32 FMA; rescale and exponents as in the other step kernels.
+// Operands written by an earlier phase of the same launch come from other
+// SMs, so they are read past L1 (ld.global.cg).
+#include <cooperative_groups.h>
+
+#include "kernels.cuh"
+
+namespace tnk {
+
+namespace {
+
+constexpr int SM_THREADS = 256, SM_WARPS = SM_THREADS / 32;
+constexpr int SM_CLUSTER = 16;
+
+__device__ __forceinline__ int sm_exp(uint32_t bits) {
+    if (bits == 0u) return 0;
+    const int e = int((bits >> 23) & 0xffu) - 127;
+    return max(-126, min(126, e));
+}
+
+__device__ __forceinline__ void sm_cfma(float2 &acc, float2 a, float2 b) {
+    acc.x = fmaf(a.x, b.x, acc.x);
+    acc.x = fmaf(-a.y, b.y, acc.x);
+    acc.y = fmaf(a.x, b.y, acc.y);
+    acc.y = fmaf(a.y, b.x, acc.y);
+}
+
+// U x 32 lanes of one step (lane groups of 2^lg lanes, one output each), U
+// outputs a lane at once so that their loads are in flight together.
+template <int U>
+__device__ __forceinline__ void small_outputs(const SmallDesc &d, int lg, int first, int lane) {
+    const int sub = lane & ((1 << lg) - 1);
+    bool valid[U];
+    int i[U], mn[U];
+    int2 ab[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int o = (first + 32 * u + lane) >> lg;
+        valid[u] = o < d.outputs;
+        const int oc = valid[u] ? o : 0;
+        i[u] = oc >> d.mnb;
+        mn[u] = oc & ((1 << d.mnb) - 1);
+        ab[u] = __ldg(d.instab + i[u]);
+    }
+    uint32_t ma[U], mb[U];
+    const float2 *a[U], *b[U];
+    float2 acc[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        ma[u] = d.mxA ? __ldcg(d.mxA + ab[u].x) : 0u;
+        mb[u] = d.mxB ? __ldcg(d.mxB + ab[u].y) : 0u;
+        a[u] = d.A + int64_t(ab[u].x) * d.sA + (int64_t(mn[u] >> d.nb) << d.kb);
+        b[u] = d.B + int64_t(ab[u].y) * d.sB + (int64_t(mn[u] & ((1 << d.nb) - 1)) << d.kb);
+        acc[u] = make_float2(0.f, 0.f);
+    }
+    if (d.kb == 0) {
+        float2 x[U], y[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            x[u] = __ldcg(a[u]);
+            y[u] = __ldcg(b[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) sm_cfma(acc[u], x[u], y[u]);
+    } else {
+        const int pieces = 1 << (d.kb - 1);
+#pragma unroll(U == 1 ? 4 : 2)
+        for (int q = sub; q < pieces; q += 1 << lg) {
+            float4 x[U], y[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                x[u] = __ldcg(reinterpret_cast<const float4 *>(a[u]) + q);
+                y[u] = __ldcg(reinterpret_cast<const float4 *>(b[u]) + q);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                sm_cfma(acc[u], make_float2(x[u].x, x[u].y), make_float2(y[u].x, y[u].y));
+                sm_cfma(acc[u], make_float2(x[u].z, x[u].w), make_float2(y[u].z, y[u].w));
+            }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        for (int s = 1; s < (1 << lg); s <<= 1) {  // lg is the same for the warp
+            acc[u].x += __shfl_xor_sync(0xffffffffu, acc[u].x, s);
+            acc[u].y += __shfl_xor_sync(0xffffffffu, acc[u].y, s);
+        }
+        const int ea = sm_exp(ma[u]), eb = sm_exp(mb[u]);
+        // 2^-(ea + eb), in two factors where it is no normal number
+        const int e1 = max(-126, min(126, ea + eb)), e2 = ea + eb - e1;
+        const float sc = __int_as_float((127 - e1) << 23);
+        float2 v = make_float2(acc[u].x * sc, acc[u].y * sc);
+        if (e2) {
+            const float s2 = __int_as_float((127 - e2) << 23);
+            v.x *= s2;
+            v.y *= s2;
+        }
+        uint32_t mx = 0u;
+        if (valid[u] && sub == 0) {
+            int64_t c = int64_t(i[u]) * d.sC;
+            for (int j = 0; j < d.mnb; ++j) c += int64_t((mn[u] >> j) & 1) << d.pC[j];
+            d.C[c] = v;
+            if (mn[u] == 0) d.EC[i[u]] = __ldcg(d.EA + ab[u].x) + ea + __ldcg(d.EB + ab[u].y) + eb;
+            mx = __float_as_uint(fmaxf(fabsf(v.x), fabsf(v.y)));
+        }
+        if (d.mxC) {
+            if (d.mnb + lg >= 5) {  // one instance for the 32 lanes
+                mx = __reduce_max_sync(0xffffffffu, mx);
+                if (lane == 0 && mx) atomicMax(d.mxC + i[u], mx);
+            } else if (mx) {
+                atomicMax(d.mxC + i[u], mx);
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(SM_THREADS) k_small_steps(const __grid_constant__ SmallArgs p) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    SmallDesc *sd = reinterpret_cast<SmallDesc *>(sm_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int PIECES = int(sizeof(SmallDesc) / 16);
+    for (int e = tid; e < p.n_steps * PIECES; e += SM_THREADS) {
+        const int s = e / PIECES, q = e - s * PIECES;
+        reinterpret_cast<uint4 *>(sd + s)[q] = __ldg(reinterpret_cast<const uint4 *>(p.descs + p.step[s]) + q);
+    }
+    __syncthreads();
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int nw = int(gridDim.x) * SM_WARPS, gw = int(blockIdx.x) + warp * int(gridDim.x);
+    int s0 = 0;
+    for (int ph = 0; ph < p.n_phases; ++ph) {
+        const int s1 = p.phase_end[ph];
+        if (ph > 0) cl.sync();  // release / acquire: the last phase's outputs, maxima and exponents are visible
+        int s = s0;
+        for (int w = gw; w < p.wend[s1 - 1]; w += nw) {
+            while (w >= p.wend[s]) ++s;
+            const int local = w - (s > s0 ? p.wend[s - 1] : 0);
+            if (p.four[s]) small_outputs<4>(sd[s], p.lanes_log2[s], local * 128, lane);
+            else small_outputs<1>(sd[s], p.lanes_log2[s], local * 32, lane);
+        }
+        s0 = s1;
+    }
+}
+
+}  // namespace
+
+cudaError_t init_small_kernel() {
+    cudaError_t e = cudaFuncSetAttribute(k_small_steps, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int(SMALL_MAX_STEPS * sizeof(SmallDesc)));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_small_steps, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+cudaError_t launch_small(const SmallArgs &a, cudaStream_t s) {
+    if (a.n_steps < 1 || a.n_steps > SMALL_MAX_STEPS || a.n_phases < 1 || a.n_phases > SMALL_MAX_PHASES)
+        return cudaErrorInvalidValue;
+    // as many blocks as the widest phase has work for: a barrier over fewer
+    // blocks is shorter
+    unsigned blocks = 1;
+    while (blocks < unsigned(SM_CLUSTER) && int(blocks) * SM_WARPS < a.max_warps) blocks <<= 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(SM_THREADS);
+    cfg.dynamicSmemBytes = size_t(a.n_steps) * sizeof(SmallDesc);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = blocks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_small_steps, a);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace tnk

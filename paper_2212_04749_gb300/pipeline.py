@@ -22,6 +22,7 @@ from concurrent.futures import ThreadPoolExecutor
 import numpy as np
 
 from . import tn
+from .tn import TN_CONFIG_TUNED
 
 
 def contract_batches(circ, batches, tree_ssa, sliced, precision, workspace, stream=None, configs=None, chains=None,
@@ -92,7 +93,7 @@ def contract_batches(circ, batches, tree_ssa, sliced, precision, workspace, stre
                 futs[j] = ex.submit(plan_of, j, done.get(j % nws))
             if configs is not None:
                 for s, c in enumerate(configs):
-                    p.tn_plan_set_config(s, int(c))
+                    p.tn_plan_set_config(s, int(c) + (TN_CONFIG_TUNED if c >= 0 else 0))
             if chains is not None:
                 for c, on in enumerate(chains):
                     p.tn_plan_set_chain(c, int(on))

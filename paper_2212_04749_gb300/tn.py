@@ -19,7 +19,8 @@ TN_OK, TN_EINVAL, TN_ENOMEM, TN_ECUDA, TN_ETIMEOUT, TN_EUNSUPPORTED, TN_ESTATE =
 TN_FP32, TN_TF32, TN_BF16X3 = 0, 1, 2
 PRECISIONS = {"fp32": TN_FP32, "tf32": TN_TF32, "bf16x3": TN_BF16X3}
 
-EXPORTS = ("tn_options_default", "tn_network", "tn_plan", "tn_plan_query", "tn_plan_widths", "tn_plan_steps",
+EXPORTS = ("tn_options_default", "tn_network", "tn_plan", "tn_plan_query", "tn_plan_launches",
+           "tn_plan_widths", "tn_plan_steps",
            "tn_plan_bind", "tn_contract", "tn_contract_slices", "tn_xeb", "tn_plan_profile",
            "tn_plan_step_times", "tn_plan_set_kernel", "tn_plan_set_config", "tn_plan_set_tc_resident_b", "tn_plan_set_tc_pairs", "tn_plan_get_configs", "tn_pt_moments",
            "tn_pt_moments_scratch_bytes", "tn_pt_moments_scratch", "tn_pt_histogram", "tn_sample_completions",
@@ -31,6 +32,7 @@ TN_STATIC_SCRATCH_BYTES = 64 << 20
 TN_PT_MAX_BINS = 8192
 TN_MAX_OPEN = 16
 TN_NCONFIG = 4
+TN_CONFIG_TUNED = 16
 TN_NFEAT = TN_MLP_IN = 24
 TN_MLP_HIDDEN = 128
 TN_MLP_NPARAMS = TN_MLP_HIDDEN * TN_MLP_IN + TN_MLP_HIDDEN + TN_MLP_HIDDEN * TN_MLP_HIDDEN + 2 * TN_MLP_HIDDEN + 1
@@ -109,6 +111,7 @@ def load(build_if_missing: bool = False):
         "tn_plan": (ctypes.c_int, [ctypes.POINTER(tn_circuit), vp, i64, vp, vp, i32,
                                    ctypes.POINTER(tn_options), ctypes.POINTER(vp)]),
         "tn_plan_query": (ctypes.c_int, [vp, ctypes.POINTER(tn_plan_info)]),
+        "tn_plan_launches": (ctypes.c_int, [vp, ctypes.POINTER(i64)]),
         "tn_plan_widths": (ctypes.c_int, [vp, vp, vp, vp]),
         "tn_plan_bind": (ctypes.c_int, [vp, vp, ctypes.c_size_t, vp]),
         "tn_plan_steps": (ctypes.c_int, [vp, vp, i32]),
@@ -247,6 +250,11 @@ class Plan:
         return {f: getattr(info, f) for f, _ in tn_plan_info._fields_}
 
     info = property(tn_plan_query)
+
+    def tn_plan_launches(self):
+        n = ctypes.c_int64()
+        _check(self._lib.tn_plan_launches(self.h, ctypes.byref(n)))
+        return n.value
 
     def tn_plan_widths(self):
         n = self.info["n_nodes"]
