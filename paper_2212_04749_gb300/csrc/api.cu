@@ -122,7 +122,7 @@ void build_descs(PlanObj *o) {
         d.nOutB = B.n_out;
         d.nOut = nd.n_out;
         d.nInst = nd.n_inst;
-        d.nInstB = B.n_inst;
+        d.nInstB = d.packBn = B.n_inst;
         d.EA = at<const int32_t>(o, A.buf.E);
         d.EB = at<const int32_t>(o, B.buf.E);
         d.EC = at<int32_t>(o, nd.buf.E);
@@ -255,16 +255,66 @@ int effective_config(const PlanObj *o, int s) {
     return o->P.steps[s].kernel == 0 ? 0 : 2;
 }
 
-int run_step(PlanObj *o, int s, int precision, cudaStream_t st) {
+// The slice instance of node nd that low slice bits sigma select: the bits
+// of its own batched edges, compressed.
+int64_t slice_instance(const tnp::Node &nd, int64_t sigma) {
+    int64_t r = 0;
+    for (size_t j = 0; j < nd.slices_low.size(); ++j) r |= ((sigma >> nd.slices_low[j]) & 1) << j;
+    return r;
+}
+
+// Narrow a step to the output instances of one slice: the groups that hold
+// them (a group that reaches beyond them is computed whole; its other
+// instances are then never read).
+void apply_window(const PlanObj *o, const tnp::Step &S, int64_t sigma, tnk::StepDesc &d) {
+    const tnp::Node &nd = o->P.nodes[S.node], &B = o->P.nodes[S.b];
+    const int64_t i0 = slice_instance(nd, sigma) * nd.n_out, i1 = i0 + nd.n_out;
+    const auto &gf = S.group_first;
+    const int64_t g0 = std::upper_bound(gf.begin(), gf.end(), i0) - gf.begin() - 1;
+    const int64_t g1 = std::lower_bound(gf.begin(), gf.end(), i1) - gf.begin();
+    const auto &ct = S.col_tiles;
+    const int64_t t0 = std::lower_bound(ct.begin(), ct.end(), g0 << 20) - ct.begin();
+    const int64_t t1 = std::lower_bound(ct.begin(), ct.end(), g1 << 20) - ct.begin();
+    d.inst0 = i0;
+    d.nInst = nd.n_out;
+    d.gfirst += g0;
+    d.n_groups = g1 - g0;
+    d.trec += t0;
+    d.ctab += t0;
+    d.n_ctab = t1 - t0;
+    d.tile0 = t0;
+    if (d.ptab) {
+        int64_t p0 = 0, p1 = 0;
+        for (int64_t g = 0; g < g1; ++g) {
+            const int64_t n = gf[g + 1] - gf[g];
+            (g < g0 ? p0 : p1) += n + (n & 1);
+        }
+        d.ptab += p0;
+        d.ptile0 = p0;
+        d.n_ptab = p1;
+    }
+    d.packB0 = slice_instance(B, sigma) * B.n_out;
+    d.packBn = B.n_out;
+}
+
+// sigma >= 0: only the output instances of that slice of the pass
+int run_step(PlanObj *o, int s, int precision, int64_t sigma, cudaStream_t st) {
     const tnp::Step &S = o->P.steps[s];
     if (o->chain_fused(S.chain)) {  // fused chain: runs whole at its last step
-        const cudaError_t e = tnk::launch_chain(o->chain_desc[S.chain], st);
+        tnk::ChainDesc c = o->chain_desc[S.chain];
+        if (sigma >= 0) {
+            const tnp::Node &nd = o->P.nodes[S.node];
+            c.inst0 = slice_instance(nd, sigma) * nd.n_out;
+            c.n_inst = nd.n_out;
+        }
+        const cudaError_t e = tnk::launch_chain(c, st);
         if (e != cudaSuccess)
             return set_err(TN_ECUDA, "fused chain at step " + std::to_string(s) + ": " + cudaGetErrorString(e));
         return TN_OK;
     }
     const int cfg = effective_config(o, s);
     tnk::StepDesc d = o->desc[s];
+    if (sigma >= 0) apply_window(o, S, sigma, d);
     d.sched = cfg & 1;
     d.tc_resident_b = o->tc_resident_b ? 1 : 0;
     d.tc_pair = o->tc_pair ? 1 : 0;
@@ -467,47 +517,60 @@ void step_features(const tnp::Plan &P, int s, int precision, int c, float *f) {
     f[i++] = lg(double(nd.n_inst) * std::ldexp(1.0, S.mb)) / 64.f;
 }
 
-// Batches [b_lo, b_hi) in order.  The first batch of the call runs every
-// step; batch b > b_lo re-runs only the steps whose sliced edges changed
-// from batch b-1 (level <= ctz(b)).  `per_batch(b)` runs after each batch.
-template <class F>
-int run_batches(PlanObj *o, int precision, int64_t b_lo, int64_t b_hi, cudaStream_t st, F per_batch) {
-    tnp::Plan &P = o->P;
+void start_launches(PlanObj *o) {
+    const tnp::Plan &P = o->P;
     o->step_kernel.resize(P.steps.size(), -1);
     for (size_t s = 0; s < P.steps.size(); ++s)
         if (o->chain_fused(P.steps[s].chain)) o->step_kernel[s] = 3;
     o->ev_used = 0;
     o->ev_step.clear();
+}
+
+// One pass over slice batch b: the steps of level <= lv (64: all), the
+// others keep what an earlier pass left.  sigma >= 0: one slice of the batch.
+int run_pass(PlanObj *o, int precision, int64_t b, int lv, int64_t sigma, cudaStream_t st) {
+    tnp::Plan &P = o->P;
     const auto *jobs = at<const tnk::FillJobD>(o, P.off_fill_jobs);
     const auto *highs = at<const tnk::LeafHighD>(o, P.off_leaf_high);
+    const int64_t clear = lv >= 64 ? P.emax_bytes : P.emax_prefix[lv];
+    if (clear) CU(cudaMemsetAsync(o->ws + P.off_emax, 0, clear, st));
+    cudaError_t e = tnk::launch_fill(jobs, P.n_fill_jobs, highs, b, at<float2>(o, 0), st);
+    if (e != cudaSuccess) return set_err(TN_ECUDA, std::string("leaf fill: ") + cudaGetErrorString(e));
+    const PlanObj::Sched &order = schedule(o, lv);
+    for (const PlanObj::Sched::Item &it : order.items) {
+        const int s = it.step;
+        if (o->profile) {
+            while (o->ev.size() < 2 * (o->ev_used + 1)) {
+                cudaEvent_t ev;
+                CU(cudaEventCreate(&ev));
+                o->ev.push_back(ev);
+            }
+            CU(cudaEventRecord(o->ev[2 * o->ev_used], st));
+        }
+        // merged small steps compute every slice of the pass
+        if (it.group >= 0) {
+            if (int rc = run_group(o, order.groups[it.group], st)) return rc;
+        } else if (int rc = run_step(o, s, precision, sigma, st)) {
+            return rc;
+        }
+        if (o->profile) {
+            CU(cudaEventRecord(o->ev[2 * o->ev_used + 1], st));
+            o->ev_step.push_back(s);
+            o->ev_used++;
+        }
+    }
+    return TN_OK;
+}
+
+// Batches [b_lo, b_hi) in order.  The first batch of the call runs every
+// step; batch b > b_lo re-runs only the steps whose sliced edges changed
+// from batch b-1 (level <= ctz(b)).  `per_batch(b)` runs after each batch.
+template <class F>
+int run_batches(PlanObj *o, int precision, int64_t b_lo, int64_t b_hi, cudaStream_t st, F per_batch) {
+    start_launches(o);
     for (int64_t b = b_lo; b < b_hi; ++b) {
         const int lv = (b == b_lo) ? 64 : __builtin_ctzll((unsigned long long)b);
-        const int64_t clear = (b == b_lo) ? P.emax_bytes : P.emax_prefix[lv];
-        if (clear) CU(cudaMemsetAsync(o->ws + P.off_emax, 0, clear, st));
-        cudaError_t e = tnk::launch_fill(jobs, P.n_fill_jobs, highs, b, at<float2>(o, 0), st);
-        if (e != cudaSuccess) return set_err(TN_ECUDA, std::string("leaf fill: ") + cudaGetErrorString(e));
-        const PlanObj::Sched &order = schedule(o, lv);
-        for (const PlanObj::Sched::Item &it : order.items) {
-            const int s = it.step;
-            if (o->profile) {
-                while (o->ev.size() < 2 * (o->ev_used + 1)) {
-                    cudaEvent_t ev;
-                    CU(cudaEventCreate(&ev));
-                    o->ev.push_back(ev);
-                }
-                CU(cudaEventRecord(o->ev[2 * o->ev_used], st));
-            }
-            if (it.group >= 0) {
-                if (int rc = run_group(o, order.groups[it.group], st)) return rc;
-            } else if (int rc = run_step(o, s, precision, st)) {
-                return rc;
-            }
-            if (o->profile) {
-                CU(cudaEventRecord(o->ev[2 * o->ev_used + 1], st));
-                o->ev_step.push_back(s);
-                o->ev_used++;
-            }
-        }
+        if (int rc = run_pass(o, precision, b, lv, -1, st)) return rc;
         if (int rc = per_batch(b)) return rc;
     }
     o->last_batches = b_hi - b_lo;
@@ -810,19 +873,50 @@ int tn_contract_slices(tn_plan_t plan, int precision, const int64_t *slice_ids, 
     const float2 *root = at<const float2>(o, R.buf.data);
     const int32_t *E = at<const int32_t>(o, R.buf.E);
     const int32_t *uniq = at<const int32_t>(o, P.off_uniq);
-    for (auto &kv : by_batch) {
-        const int64_t b = kv.first;
-        int rc = run_batches(o, precision, b, b + 1, st, [&](int64_t) -> int {
-            for (int32_t i : kv.second) {
-                const int64_t sigma = internal[i] % per;
-                cudaError_t e = tnk::launch_extract(root, E, uniq, P.k, sigma, R.n_out, R.rank,
-                                                    partials + (2 * P.k * i << R.rank), st);
-                if (e != cudaSuccess) return set_err(TN_ECUDA, std::string("extract: ") + cudaGetErrorString(e));
+    // A pass computes the 2^m_low slices of a batch side by side; where at
+    // most half of them are asked for, a pass per slice computes just the
+    // instances of that slice (a step's time goes with its instances: 16
+    // slices of grid6x7_m10, 8 to a pass, took 19 ms each as whole passes).
+    // Steps that no value of a sliced edge changed for since the last pass
+    // keep their results: pass p re-runs the levels up to the highest of a
+    // node that depends on a changed one.
+    start_launches(o);
+    int64_t b_prev = -1, s_prev = -1;  // s_prev = -1: a whole pass
+    auto pass = [&](int64_t b, int64_t sigma) -> int {
+        int lv = 64;
+        if (b_prev >= 0) {
+            lv = b == b_prev ? -1 : 63 - __builtin_clzll((unsigned long long)(b ^ b_prev));
+            for (const tnp::Node &nd : P.nodes) {
+                if (nd.slices_low.empty()) continue;
+                const bool same = sigma < 0 ? s_prev < 0
+                                            : s_prev >= 0 && slice_instance(nd, sigma) == slice_instance(nd, s_prev);
+                if (!same) lv = std::max(lv, nd.level);
             }
-            return TN_OK;
-        });
-        if (rc) return rc;
+        }
+        b_prev = b;
+        s_prev = sigma;
+        return lv >= 0 ? run_pass(o, precision, b, lv, sigma, st) : TN_OK;
+    };
+    auto extract = [&](int32_t i) -> int {
+        cudaError_t e = tnk::launch_extract(root, E, uniq, P.k, internal[i] % per, R.n_out, R.rank,
+                                            partials + (2 * P.k * i << R.rank), st);
+        if (e != cudaSuccess) return set_err(TN_ECUDA, std::string("extract: ") + cudaGetErrorString(e));
+        return TN_OK;
+    };
+    for (auto &kv : by_batch) {
+        std::map<int64_t, std::vector<int32_t>> by_slice;
+        for (int32_t i : kv.second) by_slice[internal[i] % per].push_back(i);
+        const bool whole = 2 * (int64_t)by_slice.size() > per;
+        if (whole)
+            if (int rc = pass(kv.first, -1)) return rc;
+        for (auto &ks : by_slice) {
+            if (!whole)
+                if (int rc = pass(kv.first, ks.first)) return rc;
+            for (int32_t i : ks.second)
+                if (int rc = extract(i)) return rc;
+        }
     }
+    o->last_batches = (int64_t)by_batch.size();
     g_err.clear();
     return TN_OK;
 }

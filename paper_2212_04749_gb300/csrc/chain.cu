@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(CH_THREADS) k_chain(const ChainDesc d) {
     __shared__ uint32_t s_mx;
     __shared__ int32_t s_tab[CH_MAXL + 1], s_e[CH_MAXL + 1], s_E[CH_MAXL + 1];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t inst = int64_t(blockIdx.x) / d.oblocks;
+    const int64_t inst = d.inst0 + int64_t(blockIdx.x) / d.oblocks;
     const int64_t ob = int64_t(blockIdx.x) % d.oblocks;
     const int L = d.L;
     if (tid <= L) s_tab[tid] = d.tab[inst * (L + 1) + tid];

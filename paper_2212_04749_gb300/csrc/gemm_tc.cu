@@ -432,12 +432,13 @@ struct TileIter {
     }
     __device__ __forceinline__ void init(const StepDesc &d, int64_t T, int64_t mtiles) {
         if (pp) {
-            const int2 q = __ldg(d.ptab + T / mtiles);  // {group's first column tile, its first padded one}
-            f = q.x;
+            // {group's first column tile, its first padded one}, of the whole step
+            const int2 q = __ldg(d.ptab + T / mtiles);
+            f = q.x - d.tile0;
             rec = __ldg(d.trec + f);  // column offset 0
             nct = unit_tiles(d, rec);
             nctp = nct + (nct & 1);
-            const int64_t local = T - int64_t(q.y) * mtiles;
+            const int64_t local = T - (q.y - d.ptile0) * mtiles;
             mt = int(local / nctp);
             ct = int(local - int64_t(mt) * nctp);
             fetch_next(d);
@@ -1535,7 +1536,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
 template <int PREC, bool RM = false>
 __global__ void __launch_bounds__(256) k_pack_b(const StepDesc d, int nch) {
     const int tid = threadIdx.x, bcol = tid & 63, kqb = tid >> 6;
-    const int64_t blk = blockIdx.x;
+    const int64_t blk = blockIdx.x + ((d.packB0 * nch) << (d.nb - 6));
     const int c = int(blk % nch);
     const int64_t ct_all = blk / nch;  // ib * (N / 64) + column tile
     const int64_t ib = ct_all >> (d.nb - 6);
@@ -1561,7 +1562,7 @@ __global__ void __launch_bounds__(256) k_pack_b(const StepDesc d, int nch) {
 template <int PREC>
 __global__ void __launch_bounds__(256) k_pack_b_pair(const StepDesc d, int nch) {
     const int tid = threadIdx.x, bcol = tid & 63, kqb = tid >> 6;
-    const int64_t blk = blockIdx.x;
+    const int64_t blk = blockIdx.x + ((d.packB0 * nch) << (d.nb - 7));
     const int c = int(blk % nch);
     const int64_t cp_all = blk / nch;  // ib * (N / 128) + pair
     const int64_t ib = cp_all >> (d.nb - 7);
@@ -1717,7 +1718,7 @@ cudaError_t launch_step_gemm_tc(const StepDesc &d, const CUtensorMap *a_map, int
     if (ndict == 0 && (nbset == 0 || unit_chunks < 64) && d.tc_resident_b && pack > 0 && d.bpack &&
         pack <= d.bpack_bytes) {
         const int nch = int(((int64_t(1) << d.kb) + TBK - 1) / TBK);
-        const int64_t blocks = pack / (TBNR * TBKR * 4);
+        const int64_t blocks = (d.packBn * nch) << (d.nb - 6);
         if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
         // BF16x3, schedule 0, N >= 64: column tiles in pairs (a row tile's
         // consecutive tiles; N >= 128 gives every group an even count, with

@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(ROW_THREADS) k_step_row(const StepDesc d, int 
             const int64_t gid = int64_t(blockIdx.x) * rows_per_block + (int64_t(it) * 8 + warp) * R + sub;
             const bool valid = gid < total;
             const int64_t gr = valid ? gid : 0;
-            const int64_t i = gr >> mb, m = gr & (M - 1);
+            const int64_t i = d.inst0 + (gr >> mb), m = gr & (M - 1);
             const int2 ab = d.instab[i];
             const int ea = d.mxA ? exp_of(d.mxA[ab.x]) : 0;
             const int eb = d.mxB ? exp_of(d.mxB[ab.y]) : 0;
@@ -696,7 +696,7 @@ __global__ void __launch_bounds__(256) k_step_skinny(const StepDesc d, int64_t u
     if (W == 1 && u >= units) return;  // a whole warp
     constexpr int RMB = RM == 1 ? 0 : (RM == 2 ? 1 : (RM == 4 ? 2 : 3));
     const int rbits = d.mb - RMB;  // row blocks per instance (log2)
-    const int64_t i = u >> rbits;
+    const int64_t i = d.inst0 + (u >> rbits);
     const int m0 = int(u & ((int64_t(1) << rbits) - 1)) * RM;
     const int2 ab = d.instab[i];
     const int K2 = 1 << (d.kb - 1);  // 16-byte pieces per row

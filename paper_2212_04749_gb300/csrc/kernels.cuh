@@ -46,6 +46,12 @@ struct StepDesc {
                                   // {group's first column tile, its first padded one} (else null)
     int64_t n_ptab;
     const int2 *instab;           // per output instance: {A instance, B instance}
+    // A window of the output instances (tn_contract_slices: one slice's): the
+    // first instance, and the first column tile (padded column tile) of the
+    // group tables above, which point at the window's first group.  All 0
+    // for a whole step.
+    int64_t inst0, tile0, ptile0;
+    int64_t packB0, packBn;       // B instances that a packed B has to hold
     uint8_t *bpack;               // tensor cores: scratch for B packed in MMA form (null: none)
     int64_t bpack_bytes;
     int8_t pAm[40];
@@ -140,7 +146,8 @@ struct ChainDesc {
     int32_t *EC;
     const int32_t *tab;           // per C_L instance: a_1, b_1 .. b_L
     const unsigned char *idx;     // index tables (plan.hpp, Chain::off_idx)
-    int64_t n_inst;               // C_L instances
+    int64_t n_inst;               // C_L instances to compute
+    int64_t inst0;                // the first of them
     int64_t oblocks;              // blocks per instance (set by the launcher)
     int32_t L, tin, no, tmax;     // steps, A_1 tile bits, outside bits, largest tile bits
     int32_t kb[CH_MAXL], nb[CH_MAXL], tb[CH_MAXL];
