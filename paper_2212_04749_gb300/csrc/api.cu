@@ -59,8 +59,13 @@ struct PlanObj {
     int chain_state(int c) const { return c < (int)chain_on.size() ? chain_on[c] : -1; }
     bool chain_enabled(int c) const { return c >= 0 && chain_state(c) != 0; }
     bool chain_fused(int c) const {
-        return c >= 0 && (chain_state(c) > 0 || (chain_state(c) < 0 && !(merge_small && chain_small[c])));
+        if (c < 0) return false;
+        if (!P.opt.fuse)  // not asked for: not where the caller chose a step's kernel
+            for (int s : P.chains[c].steps)
+                if (s < (int)pinned.size() && pinned[s]) return false;
+        return chain_state(c) > 0 || (chain_state(c) < 0 && !(merge_small && chain_small[c]));
     }
+    int reported_chains() const { return P.opt.fuse ? (int)P.chains.size() : 0; }
     struct GraphKey {
         int precision;
         int64_t lo, hi;
@@ -175,7 +180,16 @@ void build_descs(PlanObj *o) {
         cd.EA = at<const int32_t>(o, A1.buf.E);
         cd.EC = at<int32_t>(o, CL.buf.E);
         cd.tab = at<const int32_t>(o, c.off_tab);
-        cd.idx = at<const unsigned char>(o, c.off_idx);
+        cd.lo = at<const unsigned char>(o, c.off_lo);
+        cd.threads = c.threads;
+        static_assert(tnk::CH_ROUNDS == tnp::CHAIN_ROUNDS && tnk::CH_MAXT == tnp::CHAIN_MAX_TILE_BITS &&
+                          tnk::CH_MAXL == tnp::CHAIN_MAX_STEPS, "the planner's chain is the kernel's");
+        for (int i = 0; i < tnk::CH_ROUNDS; ++i) {
+            for (size_t b = 0; b + 1 < c.in_pos.size(); ++b)
+                if (((int64_t(i) * c.threads) >> b) & 1) cd.inhi[i] += int64_t(1) << c.in_pos[b + 1];
+            for (size_t b = 0; b + 1 < c.out_pos.size(); ++b)
+                if (((int64_t(i) * c.threads) >> b) & 1) cd.outhi[i] += int64_t(1) << c.out_pos[b + 1];
+        }
         cd.n_inst = CL.n_inst;
         cd.L = L;
         cd.tin = c.tin;
@@ -191,7 +205,21 @@ void build_descs(PlanObj *o) {
             cd.nb[j] = st.nb;
             cd.tb[j] = c.tbits[j];
             cd.tmax = std::max(cd.tmax, c.tbits[j]);
-            for (int b = 0; b < c.tbits[j]; ++b) cd.code[j][b] = c.code[j][b];
+            // columns in the kernel's order: the n bit at the output's lowest
+            // address bit first, if there is one
+            const size_t nb = c.cpos[j].size();
+            for (size_t b = 0; b < nb; ++b) cd.nperm[j][b] = (int8_t)b;
+            for (size_t b = 1; b < nb; ++b)
+                if (c.cpos[j][b] == 0) std::swap(cd.nperm[j][0], cd.nperm[j][b]);
+            for (size_t b = 0; b < nb; ++b) cd.cpos[j][b] = c.cpos[j][cd.nperm[j][b]];
+            for (int i = 0; i < tnk::CH_ROUNDS; ++i) {
+                int r = 0, n = 0;
+                for (size_t b = 0; b < c.rpos[j].size(); ++b)
+                    if (((int64_t(i) * c.threads) >> b) & 1) r |= 1 << c.rpos[j][b];
+                for (size_t b = 0; b < nb && b < 4; ++b) n |= ((i >> b) & 1) << cd.cpos[j][b];
+                cd.rowhi[j][i] = (int16_t)tnp::chain_swz(r);
+                cd.col[j][i] = (int16_t)tnp::chain_swz(n);
+            }
         }
         for (int b = 0; b < c.tin; ++b) cd.in_pos[b] = c.in_pos[b];
         for (size_t b = 0; b < c.out_pos.size(); ++b) cd.out_pos[b] = c.out_pos[b];
@@ -671,10 +699,11 @@ int tn_plan_query(tn_plan_t plan, tn_plan_info *info) {
     info->upload_bytes = up;
     const PlanObj *po = reinterpret_cast<const PlanObj *>(plan);
     double steps_run = 0;
-    for (const tnp::Step &st : P.steps) steps_run += (!po->chain_enabled(st.chain) || st.chain_last) ? st.runs : 0.0;
+    for (const tnp::Step &st : P.steps)
+        steps_run += (!P.opt.fuse || !po->chain_enabled(st.chain) || st.chain_last) ? st.runs : 0.0;
     info->launches_per_call = (int64_t)steps_run + 2 * P.n_batches;  // + leaf fill and accumulate per batch
     info->n_open = (int32_t)P.open_qubits.size();
-    info->n_chains = (int32_t)P.chains.size();
+    info->n_chains = po->reported_chains();
     info->amps_per_row = int64_t(1) << P.open_qubits.size();
     return TN_OK;
 }
@@ -734,8 +763,8 @@ int tn_plan_steps(tn_plan_t plan, tn_step_info *out, int32_t n) {
         r.b_run_k = run(st.pBk);
         r.b_run_n = run(st.pBn);
         r.n_groups = st.n_groups;
-        r.chain = st.chain;
-        r.chain_last = st.chain_last ? 1 : 0;
+        r.chain = P.opt.fuse ? st.chain : -1;
+        r.chain_last = P.opt.fuse && st.chain_last ? 1 : 0;
         for (int j = 0; j < 40; ++j) r.c_pos_m[j] = j < st.mb ? st.pCm[j] : -1;
         for (int j = 0; j < 24; ++j) r.c_pos_n[j] = j < st.nb ? st.pCn[j] : -1;
         int64_t mg = 0;
@@ -1059,7 +1088,7 @@ int tn_plan_set_config(tn_plan_t plan, int32_t step, int32_t config) {
 int tn_plan_set_chain(tn_plan_t plan, int32_t chain, int32_t enable) {
     if (!plan) return set_err(TN_EINVAL, "tn_plan_set_chain: null plan");
     PlanObj *o = reinterpret_cast<PlanObj *>(plan);
-    if (chain < 0 || chain >= (int32_t)o->P.chains.size()) return set_err(TN_EINVAL, "tn_plan_set_chain: bad chain");
+    if (chain < 0 || chain >= o->reported_chains()) return set_err(TN_EINVAL, "tn_plan_set_chain: bad chain");
     o->chain_on.resize(o->P.chains.size(), -1);
     o->chain_on[chain] = enable ? 1 : 0;
     o->drop_graphs();
@@ -1069,7 +1098,7 @@ int tn_plan_set_chain(tn_plan_t plan, int32_t chain, int32_t enable) {
 int tn_plan_get_chains(tn_plan_t plan, int32_t *enabled, int32_t n) {
     if (!plan || (n > 0 && !enabled)) return set_err(TN_EINVAL, "tn_plan_get_chains: null argument");
     PlanObj *o = reinterpret_cast<PlanObj *>(plan);
-    for (int32_t c = 0; c < n && c < (int32_t)o->P.chains.size(); ++c) enabled[c] = o->chain_enabled(c) ? 1 : 0;
+    for (int32_t c = 0; c < n && c < o->reported_chains(); ++c) enabled[c] = o->chain_enabled(c) ? 1 : 0;
     return TN_OK;
 }
 

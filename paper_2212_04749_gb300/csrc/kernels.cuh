@@ -132,8 +132,9 @@ cudaError_t launch_step_gemm_tc(const StepDesc &d, const CUtensorMap *a_map, int
 // Fused chain of small-operand steps (chain.cu); the planner's Chain as the
 // kernel sees it.
 constexpr int CH_MAXL = 6;    // steps
-constexpr int CH_MAXT = 10;   // tile bits
+constexpr int CH_MAXT = 12;   // tile bits
 constexpr int CH_MAXO = 40;   // outside bits
+constexpr int CH_ROUNDS = 16;
 constexpr int CH_MAX_SMEM = 160 * 1024;
 struct ChainDesc {
     const float2 *A;              // A_1
@@ -145,13 +146,19 @@ struct ChainDesc {
     const int32_t *EA, *EB[CH_MAXL];
     int32_t *EC;
     const int32_t *tab;           // per C_L instance: a_1, b_1 .. b_L
-    const unsigned char *idx;     // index tables (plan.hpp, Chain::off_idx)
     int64_t n_inst;               // C_L instances to compute
     int64_t inst0;                // the first of them
     int64_t oblocks;              // blocks per instance (set by the launcher)
+    const unsigned char *lo;      // the threads' index parts (plan.hpp, Chain::off_lo)
+    int32_t threads;              // of a block
     int32_t L, tin, no, tmax;     // steps, A_1 tile bits, outside bits, largest tile bits
     int32_t kb[CH_MAXL], nb[CH_MAXL], tb[CH_MAXL];
-    int8_t code[CH_MAXL][CH_MAXT];      // per output tile bit: 0x80 | n bit, or A tile bit
+    int8_t cpos[CH_MAXL][8];            // output tile bit of each column bit, and B's n bit that it is
+    int8_t nperm[CH_MAXL][8];
+    // index parts of a thread's rounds (entries / threads of them) and of the
+    // columns, swizzled tile indexes or element offsets
+    int64_t inhi[CH_ROUNDS], outhi[CH_ROUNDS];
+    int16_t rowhi[CH_MAXL][CH_ROUNDS], col[CH_MAXL][CH_ROUNDS];
     int8_t in_pos[CH_MAXT], out_pos[CH_MAXT];
     int8_t o_in[CH_MAXO], o_out[CH_MAXO];
 };

@@ -510,19 +510,28 @@ struct Builder {
             c.o_out_pos.push_back(int8_t(at.back()));
             opos.push_back(at);
         }
-        // widen the tiles: the lowest outside bits (by address in A_1) join
-        // every tile as pass-through rows, until the largest tile reaches
-        // 2^dt entries, so that a warp has enough rows to spread over lanes
+        // widen the tiles: outside bits join every tile as pass-through rows up
+        // to 2^12 entries (fewer where that would leave less than 512 tiles),
+        // the lowest address bits of A_1 and of C_L first, so that tiles are
+        // read and written in contiguous runs
         {
             int widest = A1.rank - (int)opos.size();
             for (int j = 0; j < L; ++j)
                 widest = std::max(widest, P.nodes[P.steps[ch[j]].node].rank - (int)opos.size());
             if (widest > dt) return false;
-            int extra = std::min(dt - widest, (int)opos.size());
+            const int64_t ni = P.nodes[P.steps[ch[L - 1]].node].n_inst;
+            int all = A1.rank;
+            while ((int64_t(1) << (all - A1.rank)) < ni) ++all;
+            const int target = std::max(widest, std::min(CHAIN_MAX_TILE_BITS, all - 9));
+            int extra = std::min(target - widest, (int)opos.size());
+            auto key = [&](size_t q) {
+                const int in = c.o_in_pos[q], out = c.o_out_pos[q];
+                return in < 4 ? in : (out < 4 ? 4 + out : 8 + std::min(in, out));
+            };
             while (extra-- > 0) {
                 size_t lo = 0;
                 for (size_t q = 1; q < opos.size(); ++q)
-                    if (c.o_in_pos[q] < c.o_in_pos[lo]) lo = q;
+                    if (key(q) < key(lo)) lo = q;
                 opos.erase(opos.begin() + lo);
                 c.o_in_pos.erase(c.o_in_pos.begin() + lo);
                 c.o_out_pos.erase(c.o_out_pos.begin() + lo);
@@ -534,7 +543,7 @@ struct Builder {
         for (int p = 0; p < A1.rank; ++p)
             if (std::find(c.o_in_pos.begin(), c.o_in_pos.end(), p) == c.o_in_pos.end()) prev.push_back(p);
         c.tin = (int)prev.size();
-        if (c.tin > dt) return false;
+        if (c.tin > CHAIN_MAX_TILE_BITS) return false;
         for (int p : prev) c.in_pos.push_back(int8_t(p));
         for (int j = 0; j < L; ++j) {
             const Step &st = P.steps[ch[j]];
@@ -545,86 +554,67 @@ struct Builder {
                 for (const auto &at : opos) outside = outside || at[j] == p;
                 if (!outside) cur.push_back(p);
             }
-            if ((int)cur.size() > dt) return false;
-            std::vector<int8_t> code;
-            for (int p : cur) {
-                int8_t v = -1;
+            if ((int)cur.size() > CHAIN_MAX_TILE_BITS) return false;
+            std::vector<int8_t> rpos(std::max(st.mb, 0), -1), cpos(st.nb, -1);
+            for (size_t b = 0; b < cur.size(); ++b) {
+                const int p = cur[b];
+                bool found = false;
                 for (int i = 0; i < st.nb; ++i)
-                    if (st.pCn[i] == p) v = int8_t(0x80 | i);
-                for (int i = 0; i < st.mb && v == -1; ++i)
+                    if (st.pCn[i] == p) {
+                        cpos[i] = int8_t(b);
+                        found = true;
+                    }
+                for (int i = 0; i < st.mb && !found; ++i)
                     if (st.pCm[i] == p) {
                         const int pa = st.kb + i;  // address bit in A
                         const auto it = std::find(prev.begin(), prev.end(), pa);
                         if (it == prev.end()) return false;  // cannot happen: non-outside m bits are tile bits
-                        v = int8_t(it - prev.begin());
+                        rpos[(it - prev.begin()) - st.kb] = int8_t(b);
+                        found = true;
                     }
-                if (v == -1) return false;
-                code.push_back(v);
+                if (!found) return false;
             }
             // the contracted bits are the lowest tile bits of A
             for (int k = 0; k < st.kb; ++k)
                 if (k >= (int)prev.size() || prev[k] != k) return false;
+            rpos.resize(cur.size() - st.nb);  // rows: the input tile's bits above K
             c.tbits.push_back((int)cur.size());
-            c.code.push_back(code);
+            c.rpos.push_back(rpos);
+            c.cpos.push_back(cpos);
             prev = cur;
         }
         for (int p : prev) c.out_pos.push_back(int8_t(p));
-        // index tables
-        c.inoff.assign(size_t(1) << c.tin, 0);
-        for (size_t e = 0; e < c.inoff.size(); ++e)
-            for (int b = 0; b < c.tin; ++b)
-                if ((e >> b) & 1) c.inoff[e] += int64_t(1) << c.in_pos[b];
-        c.outoff.assign(size_t(1) << c.tbits.back(), 0);
-        for (size_t t = 0; t < c.outoff.size(); ++t)
-            for (size_t b = 0; b < c.out_pos.size(); ++b)
-                if ((t >> b) & 1) c.outoff[t] += int64_t(1) << c.out_pos[b];
-        c.rowin.assign(L, {});
-        c.rowout.assign(L, {});
-        c.colout.assign(L, {});
-        for (int j = 0; j < L; ++j) {
-            const Step &st = P.steps[ch[j]];
-            const int tb = c.tbits[j];
-            const int rows = 1 << (tb - st.nb);
-            c.rowin[j].assign(rows, 0);
-            c.rowout[j].assign(rows, 0);
-            for (int r = 0; r < rows; ++r) {
-                int qb = 0;
-                for (int b = 0; b < tb; ++b) {
-                    const int cd = c.code[j][b];
-                    if (cd & 0x80) continue;  // n bit
-                    if ((r >> qb) & 1) {
-                        c.rowin[j][r] |= 1 << cd;
-                        c.rowout[j][r] |= 1 << b;
-                    }
-                    ++qb;
-                }
-            }
-            c.colout[j].assign(size_t(1) << st.nb, 0);
-            for (int n = 0; n < (1 << st.nb); ++n)
-                for (int b = 0; b < tb; ++b) {
-                    const int cd = c.code[j][b];
-                    if ((cd & 0x80) && ((n >> (cd & 0x7f)) & 1)) c.colout[j][n] |= 1 << b;
-                }
-        }
         return true;
     }
 
-    // Fused chains (opt.fuse): greedy, in step order.
-    void find_chains() {
+    void drop_chains() {
         P.chains.clear();
-        for (Step &st : P.steps) {
-            st.chain = -1;
-            st.chain_last = false;
+        for (int s = 0; s < (int)P.steps.size(); ++s) {
+            P.steps[s].chain = -1;
+            P.steps[s].chain_last = false;
+            P.nodes[P.steps[s].a].last_use = s;
+            P.nodes[P.steps[s].b].last_use = s;
         }
-        if (!P.opt.fuse) return;
-        const int dt = std::max(1, std::min(P.opt.fuse_max_bits > 0 ? P.opt.fuse_max_bits : 7, CHAIN_MAX_TILE_BITS));
+    }
+
+    // Fused chains: greedy, in step order.
+    void find_chains() {
+        drop_chains();
+        const int want = P.opt.fuse_max_bits > 0 ? P.opt.fuse_max_bits : 7;
+        const int dt = P.opt.fuse ? std::max(1, std::min(want, CHAIN_MAX_BITS)) : CHAIN_MAX_BITS;
         const int ns = (int)P.steps.size();
         std::vector<int> consumer(P.nodes.size(), -1);
         for (int s = 0; s < ns; ++s) {
             consumer[P.steps[s].a] = s;
             consumer[P.steps[s].b] = s;
         }
-        auto small = [](const Step &st) { return st.kb + st.nb <= 8; };
+        auto small = [&](const Step &st) {
+            if (P.opt.fuse) return st.kb + st.nb <= 8;
+            const Node &A = P.nodes[st.a], &C = P.nodes[st.node];
+            return st.kernel == 0 && st.kb >= 1 && st.kb + st.nb <= 5 && st.kb <= 4 && st.nb <= 4 && A.rank >= CHAIN_MAX_BITS &&
+                   C.rank >= CHAIN_MAX_BITS &&
+                   std::ldexp(double(C.n_inst), C.rank) >= std::ldexp(1.0, AUTO_CHAIN_MIN_LOG2);
+        };
         for (int s = 0; s < ns; ++s) {
             if (P.steps[s].chain >= 0 || !small(P.steps[s])) continue;
             std::vector<int> ch{s};
@@ -756,7 +746,10 @@ struct Builder {
         // fill jobs (one per leaf instance)
         std::vector<LeafHigh> highs;
         std::vector<FillJob> jobs;
-        for (int v = 0; v < T; ++v) {
+        std::vector<int32_t> job_leaf;
+        p.n_fill_jobs = 0;
+        for (int v = 0; v < T; ++v) p.n_fill_jobs += p.nodes[v].n_inst;
+        for (int v = 0; v < T && emit; ++v) {
             const Node &nd = p.nodes[v];
             LeafHigh hh{};
             const std::vector<int> &sj = leaf_sl[v];
@@ -786,6 +779,7 @@ struct Builder {
                     j.leaf_high = hidx;
                     j.n = int32_t(1) << nd.rank;
                     jobs.push_back(j);
+                    job_leaf.push_back(v);
                 }
             }
         }
@@ -799,9 +793,8 @@ struct Builder {
             if (j.src < p.off_leaf_full / 8 || j.src + hmax + j.n > p.off_leaf_full / 8 + full_elems)
                 bad_offsets = true;
         }
-        p.n_fill_jobs = (int64_t)jobs.size();
-        p.off_fill_jobs = take(int64_t(jobs.size()) * sizeof(FillJob));
-        p.off_leaf_high = take(int64_t(highs.size()) * sizeof(LeafHigh));
+        p.off_fill_jobs = take(p.n_fill_jobs * int64_t(sizeof(FillJob)));
+        p.off_leaf_high = take(int64_t(T) * int64_t(sizeof(LeafHigh)));
         if (emit) {
             push_upload(p, p.off_fill_jobs, jobs);
             push_upload(p, p.off_leaf_high, highs);
@@ -891,21 +884,28 @@ struct Builder {
             const int64_t ni = p.nodes[last.node].n_inst;
             const int L = (int)c.steps.size();
             c.off_tab = take(ni * (L + 1) * 4);
-            {
-                std::vector<uint8_t> blob;
-                auto put = [&](const void *src, size_t n) {
-                    const uint8_t *b = static_cast<const uint8_t *>(src);
-                    blob.insert(blob.end(), b, b + n);
-                };
-                put(c.inoff.data(), c.inoff.size() * 8);
-                put(c.outoff.data(), c.outoff.size() * 8);
-                for (int j = 0; j < L; ++j) {
-                    put(c.rowin[j].data(), c.rowin[j].size() * 4);
-                    put(c.rowout[j].data(), c.rowout[j].size() * 4);
-                    put(c.colout[j].data(), c.colout[j].size() * 4);
+            int tmax = c.tin;
+            for (int t : c.tbits) tmax = std::max(tmax, t);
+            c.threads = chain_threads(tmax);
+            c.off_lo = take(int64_t(c.threads) * (16 + 2 * L));
+            if (emit) {
+                std::vector<uint8_t> blob(size_t(c.threads) * (16 + 2 * L));
+                int64_t *in = reinterpret_cast<int64_t *>(blob.data()), *out = in + c.threads;
+                int16_t *row = reinterpret_cast<int16_t *>(out + c.threads);
+                for (int t = 0; t < c.threads; ++t) {
+                    in[t] = out[t] = 0;
+                    for (int b = 0; b + 1 < c.tin; ++b)
+                        if ((t >> b) & 1) in[t] += int64_t(1) << c.in_pos[b + 1];
+                    for (int b = 0; b + 1 < (int)c.out_pos.size(); ++b)
+                        if ((t >> b) & 1) out[t] += int64_t(1) << c.out_pos[b + 1];
+                    for (int j = 0; j < L; ++j) {
+                        int r = 0;
+                        for (size_t b = 0; b < c.rpos[j].size(); ++b)
+                            if ((t >> b) & 1) r |= 1 << c.rpos[j][b];
+                        row[j * c.threads + t] = int16_t(chain_swz(r));
+                    }
                 }
-                c.off_idx = take((int64_t)blob.size());
-                if (emit) push_upload(p, c.off_idx, blob);
+                push_upload(p, c.off_lo, blob);
             }
             if (emit) {
                 std::vector<int32_t> tab(size_t(ni) * (L + 1));
@@ -935,15 +935,18 @@ struct Builder {
         ar.base = ar.top = ar.high = off;
         p.peak_tensor_bytes = 0;
         const int nst = (int)p.steps.size();
+        // by last reader: a step, or for a chain's operands the chain's last
+        std::vector<std::vector<int>> dying(nst);
+        for (int v = 0; v < NN; ++v)
+            if (p.nodes[v].last_use >= 0) dying[p.nodes[v].last_use].push_back(v);
         for (int s = 0; s < nst; ++s) {
             const Step &st = p.steps[s];
             Node &nd = p.nodes[st.node];
             const int64_t bytes = nd.n_inst * (int64_t(8) << nd.rank);
             if (!nd.persistent && !own[st.node]) nd.buf.data = ar.alloc(bytes);
-            for (int c : {st.a, st.b}) {
+            for (int c : dying[s]) {
                 Node &ch = p.nodes[c];
-                if (ch.persistent || own[c] || ch.last_use != s) continue;
-                ar.release(ch.buf.data, ch.n_inst * (int64_t(8) << ch.rank));
+                if (!ch.persistent && !own[c]) ar.release(ch.buf.data, ch.n_inst * (int64_t(8) << ch.rank));
             }
             p.peak_tensor_bytes = std::max(p.peak_tensor_bytes, bytes);
         }
@@ -954,14 +957,10 @@ struct Builder {
             if (nd.buf.data < 0 || nd.buf.data + nd.n_inst * (int64_t(8) << nd.rank) > total) bad_offsets = true;
             if (nd.buf.E < 0 || nd.buf.mx < 0) bad_offsets = true;
         }
-        for (const FillJob &j : jobs) {
-            bool inside = false;
-            for (int v = 0; v < T && !inside; ++v) {
-                const Node &nd = p.nodes[v];
-                const int64_t b0 = nd.buf.data / 8, b1 = b0 + nd.n_inst * (int64_t(1) << nd.rank);
-                inside = j.dst >= b0 && j.dst + j.n <= b1;
-            }
-            if (!inside) bad_offsets = true;
+        for (size_t q = 0; q < jobs.size(); ++q) {
+            const Node &nd = p.nodes[job_leaf[q]];
+            const int64_t b0 = nd.buf.data / 8, b1 = b0 + nd.n_inst * (int64_t(1) << nd.rank);
+            if (jobs[q].dst < b0 || jobs[q].dst + jobs[q].n > b1) bad_offsets = true;
         }
         return total;
     }
@@ -1250,6 +1249,27 @@ bool make_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int
         P.peak_tensor_bytes = 0;
         return B.layout_workspace(emit, own_slots);
     };
+    // chains that were not asked for, unless keeping their inputs to their
+    // ends takes a plan above a limit that it meets without them
+    if (!P.opt.fuse && !P.chains.empty()) {
+        const int64_t with = layout(false, false);
+        const std::vector<Chain> chains = P.chains;
+        std::vector<int> last(NN);
+        for (int v = 0; v < NN; ++v) last[v] = P.nodes[v].last_use;
+        B.drop_chains();
+        const int64_t without = layout(false, false);
+        bool keep = true;
+        for (int64_t limit : {P.opt.workspace_limit, int64_t(TN_STATIC_SCRATCH_BYTES)})
+            if (without <= limit && with > limit) keep = false;
+        if (keep) {
+            P.chains = chains;
+            for (size_t c = 0; c < chains.size(); ++c) {
+                for (int q : chains[c].steps) P.steps[q].chain = (int)c;
+                P.steps[chains[c].steps.back()].chain_last = true;
+            }
+            for (int v = 0; v < NN; ++v) P.nodes[v].last_use = last[v];
+        }
+    }
     // own slots for the small steps' outputs, unless they would take a plan
     // above a limit that it meets without them
     int64_t slots = 0;
@@ -1273,7 +1293,7 @@ bool make_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int
         const Node &nd = P.nodes[st.node];
         P.flops_exec += st.flops * st.runs;
         double bytes = st.bytes;
-        if (st.chain >= 0) {  // a chain's intermediates are never stored
+        if (P.opt.fuse && st.chain >= 0) {  // a chain's intermediates are never stored
             const double inner = 8.0 * double(nd.n_inst) * std::ldexp(1.0, nd.rank);
             if (!st.chain_last) bytes -= inner;  // C_j of a non-final step
             if (P.steps[P.chains[st.chain].steps[0]].node != st.node) {

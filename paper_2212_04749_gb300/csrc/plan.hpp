@@ -130,12 +130,18 @@ constexpr int64_t SMALL_SLOTS_MAX = int64_t(32) << 20;
 // A fused chain (SM Sec. V.C): steps s_1..s_L where each step's A operand is
 // the previous step's output, instance counts do not grow, and every side
 // operand B_j is small.  It runs as one kernel at s_L: per output instance
-// and per value of the "outside" bits O (A_1's free bits that no chain step
+// and per value of the "outside" bits O (free bits of A_1 that no chain step
 // touches), a tile of A_1 (its other bits) is loaded once, multiplied by
 // B_1 .. B_L in shared memory, and written to C_L; the intermediates
-// C_1 .. C_{L-1} are never stored.
+// C_1 .. C_{L-1} are never stored.  The bits that the chain touches are at
+// most dt (tn_options.fuse_max_bits); tiles then take in further free bits.
 constexpr int CHAIN_MAX_STEPS = 6;
-constexpr int CHAIN_MAX_TILE_BITS = 10;
+constexpr int CHAIN_MAX_BITS = 10;       // dt
+constexpr int CHAIN_MAX_TILE_BITS = 12;  // 2^12 entries: two buffers of 32 KB, three blocks an SM
+// Without tn_options.fuse, chains of steps that only stream a large tensor
+// (K, N <= 16, K N <= 32, at least 2^14 entries) run the same way: unfused
+// each of them reads and writes the whole tensor again.
+constexpr int AUTO_CHAIN_MIN_LOG2 = 14;
 struct Chain {
     std::vector<int> steps;            // s_1 .. s_L
     int tin = 0;                       // tile bits of A_1
@@ -144,17 +150,24 @@ struct Chain {
     std::vector<int8_t> in_pos;        // address bit in A_1 of each A_1 tile bit (ascending)
     std::vector<int8_t> o_in_pos, o_out_pos;  // address bit of each outside bit in A_1 and C_L
     std::vector<int8_t> out_pos;       // address bit in C_L of each C_L tile bit (ascending)
-    std::vector<std::vector<int8_t>> code;  // per step, per output tile bit: 0x80|i (n bit i) or r (A tile bit r)
+    std::vector<std::vector<int8_t>> rpos, cpos;  // per step: output tile bit of each row bit, of each n bit
     int64_t off_tab = -1;              // int32 per C_L instance: a_1, b_1 .. b_L
-    // index tables, uploaded at off_idx (int64 inoff[2^tin], int64
-    // outoff[2^tL], then per step int32 rowin[R_j], rowout[R_j], colout[N_j]):
-    // address offset in A_1 of each input tile entry, in C_L of each output
-    // tile entry, and per step the input / output tile index of each row
-    // (R_j = 2^(tbits_j - nb_j)) and the output tile bits of each column
-    std::vector<int64_t> inoff, outoff;
-    std::vector<std::vector<int32_t>> rowin, rowout, colout;
-    int64_t off_idx = -1;
+    // Index parts of the kernel's threads, uploaded at off_lo: int64 offset
+    // in A_1 and in C_L of 16-byte unit t of a tile, then per step the int16
+    // (swizzled) output index of row t, for t below the block's threads.
+    int threads = 0;
+    int64_t off_lo = -1;
 };
+// Tile entries per thread, and the block's threads for tiles of 2^tmax.
+constexpr int CHAIN_ROUNDS = 16;
+inline int chain_threads(int tmax) {
+    const int n = (1 << tmax) / CHAIN_ROUNDS;
+    return n < 32 ? 32 : (n > 256 ? 256 : n);
+}
+// Entry i of a tile buffer sits at chain_swz(i): 16-byte units XOR-permuted so
+// that threads whose entries lie a power of two apart use different banks;
+// linear over GF(2).
+constexpr int chain_swz(int i) { return i ^ ((((i >> 4) ^ (i >> 7)) & 7) << 1); }
 
 struct Plan {
     Network net;
@@ -171,7 +184,7 @@ struct Plan {
     int64_t n_batches = 1;
     std::vector<Node> nodes;          // 2T-1
     std::vector<Step> steps;          // SSA order
-    std::vector<Chain> chains;        // fused chains (opt.fuse)
+    std::vector<Chain> chains;        // fused chains (opt.fuse; else the ones of AUTO_CHAIN_MIN_LOG2, not reported)
     int n_static_steps = 0;
     int root = -1;
     int max_rank = 0;
