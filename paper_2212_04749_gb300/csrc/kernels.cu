@@ -675,6 +675,148 @@ __global__ void __launch_bounds__(128) k_step_gemm_simt2(const StepDesc d, int c
     }
 }
 
+// Steps with a long row and few columns per A instance (K >= 32, K N <= 256,
+// M >= 128), grouped: a block takes 128 rows of a group's A instance and up to
+// 16 of the group's concatenated columns (the instances that share it), so A
+// is read once for 16 columns.  Chunks of 8 complex k of A (128 rows x 64
+// bytes) and B arrive by cp.async in three stages; a thread holds 4 rows x 4
+// columns, rows 32 apart, and reads both operands 16 bytes at a time (128 FMA
+// for 8 loads, B's as broadcasts).  A warp takes four columns, which four
+// rotates with the block so that tiles of fewer columns load all four
+// schedulers; the other warps only copy.  Bound by HBM (A) and the FMA rate
+// at about the same time for 8 columns; a block lives for little more than
+// its latencies, so six of them share an SM.  The per-row kernel held a row
+// of 64 in two lanes' registers, read B from shared memory for every row and
+// instance again and loaded 32 bytes a row at a time: 4.47 ms on 2^8 x 64 x 2
+// with 64448 A instances of 4 (9.5 GB, 1.40 ms of HBM), 2.61 ms here.
+constexpr int NBM = 128, NBN = 16, NBK = 8, NLD = NBK + 2, NST = 3;
+constexpr size_t NARROW_SMEM = size_t(NST) * (NBM + NBN) * NLD * sizeof(float2);
+
+__global__ void __launch_bounds__(128, 6) k_step_narrow(const StepDesc d, int subs, int mtiles) {
+    extern __shared__ __align__(16) float2 sn[];
+    __shared__ int64_t s_bbase[NBN], s_cbase[NBN];
+    __shared__ int32_t s_e[NBN];
+    __shared__ uint32_t s_mx[NBN];
+    __shared__ int8_t s_pCm[40];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int64_t bid = blockIdx.x;
+    const int sub = int(bid % subs);
+    const int64_t rest = bid / subs;
+    const int mt = int(rest % mtiles);
+    // {first instance, count, A instance, first column} of 64 columns
+    const int4 rec = __ldg(d.trec + rest / mtiles);
+    const int N = 1 << d.nb, K = 1 << d.kb;
+    const int64_t M = int64_t(1) << d.mb;
+    const int c0 = rec.w + sub * NBN;  // column of the group
+    const int left = min(rec.y << d.nb, rec.w + 64) - c0;
+    if (left <= 0) return;  // uniform across the block
+    const int ncols = min(left, NBN);
+    const int64_t m0 = int64_t(mt) * NBM;
+    const float2 *A = d.A + int64_t(rec.z) * d.sA + (m0 << d.kb);
+    const int nchunk = K / NBK;
+    float2 *sa = sn, *sb = sn + NST * NBM * NLD;
+    auto issue_a = [&](int ch) {  // 16-byte pieces, four a row (M >= 128: every row exists)
+#pragma unroll
+        for (int e = tid; e < NBM * NBK / 2; e += 128) {
+            const int r = e >> 2, q = e & 3;
+            cp_async16_zfill(static_cast<uint32_t>(__cvta_generic_to_shared(sa + ((ch % NST) * NBM + r) * NLD + 2 * q)),
+                             A + (int64_t(r) << d.kb) + ch * NBK + 2 * q, true);
+        }
+    };
+    auto issue_b = [&](int ch) {
+        if (tid < NBN * NBK / 2) {
+            const int c = tid >> 2, q = tid & 3;
+            const bool v = s_bbase[c] >= 0;
+            cp_async16_zfill(static_cast<uint32_t>(__cvta_generic_to_shared(sb + ((ch % NST) * NBN + c) * NLD + 2 * q)),
+                             v ? d.B + s_bbase[c] + ch * NBK + 2 * q : d.B, v);
+        }
+    };
+    auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+    issue_a(0);
+    issue_a(1);
+    if (tid < 40) s_pCm[tid] = d.pCm[tid];
+    if (tid < NBN) {
+        s_mx[tid] = 0u;
+        s_bbase[tid] = -1;
+        if (tid < ncols) {
+            const int inst = rec.x + ((c0 + tid) >> d.nb);
+            const int n = (c0 + tid) & (N - 1);
+            const int ib = d.instab[inst].y;
+            const int ea = d.mxA ? exp_of(d.mxA[rec.z]) : 0, eb = d.mxB ? exp_of(d.mxB[ib]) : 0;
+            s_bbase[tid] = int64_t(ib) * d.sB + (int64_t(n) << d.kb);
+            s_cbase[tid] = int64_t(inst) * d.sC + dep(n, d.pCn, d.nb);
+            s_e[tid] = ea + eb;
+            if (n == 0 && mt == 0) d.EC[inst] = d.EA[rec.z] + ea + d.EB[ib] + eb;
+        }
+    }
+    __syncthreads();
+    issue_b(0);
+    commit();
+    issue_b(1);
+    commit();
+    const int cg = ((tid >> 5) + int(bid)) & 3;
+    const bool works = 4 * cg < ncols;  // the same for a warp
+    float2 acc[4][4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) acc[x][y] = make_float2(0.f, 0.f);
+    for (int ch = 0; ch < nchunk; ++ch) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();  // chunk ch is in place; every warp is done with chunk ch - 1
+        if (ch + 2 < nchunk) {
+            issue_a(ch + 2);
+            issue_b(ch + 2);
+        }
+        commit();
+        if (works) {
+            const float2 *a_s = sa + ((ch % NST) * NBM + lane) * NLD, *b_s = sb + ((ch % NST) * NBN + 4 * cg) * NLD;
+#pragma unroll
+            for (int kk = 0; kk < NBK; kk += 2) {
+                float4 a[4], b[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) a[x] = *reinterpret_cast<const float4 *>(a_s + 32 * x * NLD + kk);
+#pragma unroll
+                for (int y = 0; y < 4; ++y) b[y] = *reinterpret_cast<const float4 *>(b_s + y * NLD + kk);
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) {
+                        cfma(acc[x][y], make_float2(a[x].x, a[x].y), make_float2(b[y].x, b[y].y));
+                        cfma(acc[x][y], make_float2(a[x].z, a[x].w), make_float2(b[y].z, b[y].w));
+                    }
+            }
+        }
+    }
+    if (works) {
+        int64_t off[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) off[x] = dep(m0 + lane + 32 * x, s_pCm, d.mb);
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+            const int c = 4 * cg + y;
+            if (c >= ncols) break;  // the same for a warp
+            const float sc = pow2f(-s_e[c]);
+            float2 *C = d.C + s_cbase[c];
+            uint32_t mx = 0u;
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const float2 v = make_float2(acc[x][y].x * sc, acc[x][y].y * sc);
+                C[off[x]] = v;
+                mx = max(mx, absmax_bits(v));
+            }
+            if (d.mxC) {
+                mx = __reduce_max_sync(0xffffffffu, mx);
+                if (lane == 0 && mx) atomicMax(&s_mx[c], mx);
+            }
+        }
+    }
+    if (d.mxC) {
+        __syncthreads();
+        if (tid < ncols && s_mx[tid]) record_max(d.mxC + rec.x + ((c0 + tid) >> d.nb), s_mx[tid]);
+    }
+}
+
 // Steps with few outputs per instance (M N <= 32, N <= 8) and a long K (the
 // root of a plan, with its open qubits, and what is left of the ranks just
 // below it).  A unit is one instance and RM of its rows against its N
@@ -1068,6 +1210,10 @@ cudaError_t launch_fill(const FillJobD *jobs, int64_t njobs, const LeafHighD *hi
     return cudaGetLastError();
 }
 
+// Rows of 32 and more go to k_step_narrow, the shorter ones stay in a few
+// lanes' registers.
+constexpr int NARROW_MIN_KB = 5;
+
 // Lanes per row of the row kernel: as few as keep a lane's share of the
 // row's K * N products within 64 (fewer cross-lane sums per output), at
 // least K / 32 (a lane holds at most 32 complex A values) and at most 8
@@ -1083,6 +1229,16 @@ static int row_lanes(int kb, int nb) {
 
 cudaError_t launch_step_row(const StepDesc &d, cudaStream_t s) {
     if (d.kb + d.nb > 8 || d.nb > 4 || d.mb > 40) return cudaErrorInvalidValue;
+    if (d.kb >= NARROW_MIN_KB && d.mb >= 7) {
+        const int64_t cols = int64_t(d.max_group) << d.nb;
+        const int subs = cols >= 64 ? 4 : int((cols + NBN - 1) / NBN);
+        const int64_t mtiles = (int64_t(1) << d.mb) / NBM;
+        const int64_t nblk = d.n_ctab * subs * mtiles;
+        if (nblk <= 0) return cudaSuccess;
+        if (nblk > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+        k_step_narrow<<<dim3((unsigned)nblk), 128, NARROW_SMEM, s>>>(d, subs, (int)mtiles);
+        return cudaGetLastError();
+    }
     const int K = 1 << d.kb;
     const int L = row_lanes(d.kb, d.nb);
     const int R = 32 / L;
@@ -1182,6 +1338,9 @@ cudaError_t launch_step_skinny(const StepDesc &d, cudaStream_t s) {
 }
 
 cudaError_t init_simt_kernels() {
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_step_narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, int(NARROW_SMEM));
+    if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_step_gemm_simt2, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SIMT2_SMEM));
 }
 
