@@ -256,6 +256,19 @@ struct Builder {
             oa.clear();
             ob.clear();
             oi[v].resize(ku);
+            if (na == 1 || nb == 1) {
+                // one side without a choice: the other's instances, each once
+                const int32_t n = std::max(na, nb);
+                oa.resize(n);
+                ob.resize(n);
+                for (int32_t x = 0; x < n; ++x) {
+                    oa[x] = na == 1 ? 0 : x;
+                    ob[x] = na == 1 ? x : 0;
+                }
+                oi[v] = na == 1 ? kb : ka;
+                nd.n_out = n;
+                continue;
+            }
             if (int64_t(na) * nb <= (int64_t(1) << 16)) {
                 // few possible pairs: a table over all of them, scanned in
                 // (A, B) order
@@ -482,23 +495,23 @@ struct Builder {
                 int32_t(int64_t(sgB[sg]) * P.nodes[st.b].n_out + otB[bt])};
     }
 
-    // Bit maps of a candidate chain (see Chain); false if a tile exceeds
-    // 2^dt entries.
-    bool chain_bits(const std::vector<int> &ch, int dt, Chain &c) const {
+    // Bit maps of a candidate chain (see Chain); false if it touches more
+    // than dt bits.  With build = false only that is decided.
+    bool chain_bits(const std::vector<int> &ch, int dt, Chain &c, bool build) const {
         const int L = (int)ch.size();
         const Step &s1 = P.steps[ch[0]];
         const Node &A1 = P.nodes[s1.a];
-        c = Chain();
         // follow every free bit of A_1 through the chain; the ones no step
         // contracts are the outside bits
-        std::vector<std::vector<int>> opos;  // per outside bit: its address bit in C_1 .. C_L
+        std::vector<std::array<int8_t, CHAIN_MAX_STEPS>> opos;  // per outside bit: its address bit in C_1 .. C_L
+        std::vector<int8_t> in_pos;                             // and in A_1
         for (int i = 0; i < s1.mb; ++i) {
             int idx = i;
             bool alive = true;
-            std::vector<int> at;
+            std::array<int8_t, CHAIN_MAX_STEPS> at{};
             for (int j = 0; j < L && alive; ++j) {
                 const int p = P.steps[ch[j]].pCm[idx];
-                at.push_back(p);
+                at[j] = int8_t(p);
                 if (j + 1 < L) {
                     const int kn = P.steps[ch[j + 1]].kb;
                     if (p < kn) alive = false;
@@ -506,19 +519,21 @@ struct Builder {
                 }
             }
             if (!alive) continue;
-            c.o_in_pos.push_back(int8_t(s1.kb + i));
-            c.o_out_pos.push_back(int8_t(at.back()));
+            in_pos.push_back(int8_t(s1.kb + i));
             opos.push_back(at);
         }
+        int widest = A1.rank - (int)opos.size();
+        for (int j = 0; j < L; ++j) widest = std::max(widest, P.nodes[P.steps[ch[j]].node].rank - (int)opos.size());
+        if (widest > dt) return false;
+        if (!build) return true;
+        c = Chain();
+        c.o_in_pos = in_pos;
+        for (const auto &at : opos) c.o_out_pos.push_back(at[L - 1]);
         // widen the tiles: outside bits join every tile as pass-through rows up
         // to 2^12 entries (fewer where that would leave less than 512 tiles),
         // the lowest address bits of A_1 and of C_L first, so that tiles are
         // read and written in contiguous runs
         {
-            int widest = A1.rank - (int)opos.size();
-            for (int j = 0; j < L; ++j)
-                widest = std::max(widest, P.nodes[P.steps[ch[j]].node].rank - (int)opos.size());
-            if (widest > dt) return false;
             const int64_t ni = P.nodes[P.steps[ch[L - 1]].node].n_inst;
             int all = A1.rank;
             while ((int64_t(1) << (all - A1.rank)) < ni) ++all;
@@ -628,11 +643,10 @@ struct Builder {
                 if (P.nodes[nst.node].n_inst != P.nodes[last.node].n_inst || P.nodes[last.node].persistent) break;
                 std::vector<int> trial = ch;
                 trial.push_back(nx);
-                if (!chain_bits(trial, dt, c)) break;
+                if (!chain_bits(trial, dt, c, false)) break;
                 ch = trial;
             }
-            if (ch.size() < 2) continue;
-            chain_bits(ch, dt, c);
+            if (ch.size() < 2 || !chain_bits(ch, dt, c, true)) continue;
             c.steps = ch;
             for (int q : ch) P.steps[q].chain = (int)P.chains.size();
             P.steps[ch.back()].chain_last = true;
@@ -968,6 +982,39 @@ struct Builder {
 
 }  // namespace
 
+namespace {
+
+// Join uploads that lie close together (what is between them holds nothing
+// yet): a copy costs some microseconds, and a plan has several hundred
+// tables.
+void join_uploads(Plan &p) {
+    auto &u = p.uploads;
+    std::sort(u.begin(), u.end(), [](const auto &a, const auto &b) { return a.first < b.first; });
+    constexpr int64_t GAP = 16384;
+    std::vector<std::pair<int64_t, std::vector<uint8_t>>> joined;
+    for (size_t i = 0; i < u.size();) {
+        size_t j = i;
+        int64_t end = u[i].first + (int64_t)u[i].second.size();
+        while (j + 1 < u.size() && u[j + 1].first - end <= GAP) {
+            ++j;
+            end = u[j].first + (int64_t)u[j].second.size();
+        }
+        if (j == i) {
+            joined.push_back(std::move(u[i]));
+        } else {
+            std::vector<uint8_t> bytes(size_t(end - u[i].first), 0);
+            for (size_t q = i; q <= j; ++q)
+                if (!u[q].second.empty())
+                    std::memcpy(bytes.data() + (u[q].first - u[i].first), u[q].second.data(), u[q].second.size());
+            joined.emplace_back(u[i].first, std::move(bytes));
+        }
+        i = j + 1;
+    }
+    u.swap(joined);
+}
+
+}  // namespace
+
 bool make_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int32_t *ssa,
                const int32_t *sliced, int32_t n_sliced, const tn_options *opt, Plan &P,
                std::string &err, int &code) {
@@ -1200,6 +1247,7 @@ bool make_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int
     int lo = 0, hi = std::min(n_sliced, 20);
     if (P.opt.slice_batch_log2 >= 0) lo = hi = std::min(P.opt.slice_batch_log2, n_sliced);
     int chosen = -1;
+    int64_t plain = 0;  // workspace bytes of `chosen` without chains and own slots
     // Cheap bounds before building a candidate's tables: every instance
     // costs ~48 bytes of host tables (instance maps, group and tile records),
     // and the tensors kept across slice batches (a node whose parent is
@@ -1230,7 +1278,7 @@ bool make_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int
     for (int ml = hi; ml >= lo; --ml) {
         if (ml > lo && surely_too_big(ml)) continue;
         if (!B.schedule(ml)) return false;
-        const int64_t ws = B.layout_workspace(false);
+        const int64_t ws = plain = B.layout_workspace(false);
         if (ws <= P.opt.workspace_limit || ml == lo) {
             chosen = ml;
             if (ws > P.opt.workspace_limit && P.opt.slice_batch_log2 < 0) {
@@ -1249,39 +1297,26 @@ bool make_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int
         P.peak_tensor_bytes = 0;
         return B.layout_workspace(emit, own_slots);
     };
-    // chains that were not asked for, unless keeping their inputs to their
-    // ends takes a plan above a limit that it meets without them
-    if (!P.opt.fuse && !P.chains.empty()) {
-        const int64_t with = layout(false, false);
-        const std::vector<Chain> chains = P.chains;
-        std::vector<int> last(NN);
-        for (int v = 0; v < NN; ++v) last[v] = P.nodes[v].last_use;
-        B.drop_chains();
-        const int64_t without = layout(false, false);
-        bool keep = true;
+    // Chains that were not asked for, and own slots for the small steps'
+    // outputs: unless keeping a chain's inputs to its end, or the slots, take
+    // a plan above a limit that it meets without them.
+    auto crosses = [&](int64_t without, int64_t with) {
         for (int64_t limit : {P.opt.workspace_limit, int64_t(TN_STATIC_SCRATCH_BYTES)})
-            if (without <= limit && with > limit) keep = false;
-        if (keep) {
-            P.chains = chains;
-            for (size_t c = 0; c < chains.size(); ++c) {
-                for (int q : chains[c].steps) P.steps[q].chain = (int)c;
-                P.steps[chains[c].steps.back()].chain_last = true;
-            }
-            for (int v = 0; v < NN; ++v) P.nodes[v].last_use = last[v];
-        }
+            if (without <= limit && with > limit) return true;
+        return false;
+    };
+    if (!P.chains.empty()) {
+        const int64_t with = layout(false, false);
+        if (!P.opt.fuse && crosses(plain, with)) B.drop_chains();
+        else plain = with;
     }
-    // own slots for the small steps' outputs, unless they would take a plan
-    // above a limit that it meets without them
     int64_t slots = 0;
     for (const Step &st : P.steps)
         if (st.small) slots += Arena::align(P.nodes[st.node].n_inst * (int64_t(8) << P.nodes[st.node].rank));
-    bool own_slots = slots <= SMALL_SLOTS_MAX;
-    if (own_slots) {
-        const int64_t without = layout(false, false), with = layout(false, true);
-        for (int64_t limit : {P.opt.workspace_limit, int64_t(TN_STATIC_SCRATCH_BYTES)})
-            if (without <= limit && with > limit) own_slots = false;
-    }
+    const bool own_slots = slots > 0 && slots <= SMALL_SLOTS_MAX;
     P.ws_bytes = layout(true, own_slots);
+    if (own_slots && crosses(plain, P.ws_bytes)) P.ws_bytes = layout(true, false);
+    join_uploads(P);
     if (B.bad_offsets) {
         code = TN_EUNSUPPORTED;
         err = "internal error: workspace layout self-check failed";

@@ -22,7 +22,7 @@ from concurrent.futures import ThreadPoolExecutor
 import numpy as np
 
 from . import tn
-from .tn import TN_CONFIG_TUNED
+from .tn import TN_CONFIG_TUNED, circuit_struct
 
 
 def contract_batches(circ, batches, tree_ssa, sliced, precision, workspace, stream=None, configs=None, chains=None,
@@ -49,6 +49,8 @@ def contract_batches(circ, batches, tree_ssa, sliced, precision, workspace, stre
     n = len(batches)
     if n == 0:
         return
+    if hasattr(circ, "to_arrays"):
+        circ = circuit_struct(circ)  # once for all batches
     spaces = list(workspace) if isinstance(workspace, (list, tuple)) else [workspace]
     if not spaces:
         raise ValueError("workspace: at least one buffer")

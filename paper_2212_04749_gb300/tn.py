@@ -186,9 +186,9 @@ def circuit_struct(circ):
     """Marshal an ``rqc.Circuit`` into a ``tn_circuit`` (keeps the arrays alive)."""
     q0, q1, layer, m = circ.to_arrays()
     arr = (tn_gate * len(q0))()
-    for i in range(len(q0)):
-        arr[i].q0, arr[i].q1, arr[i].layer = int(q0[i]), int(q1[i]), int(layer[i])
-        ctypes.memmove(arr[i].m, m[i].ctypes.data, 32 * 8)
+    if len(q0):
+        rec = np.frombuffer(arr, np.dtype([("q0", "i4"), ("q1", "i4"), ("layer", "i4"), ("pad", "i4"), ("m", "f8", 32)]))
+        rec["q0"], rec["q1"], rec["layer"], rec["m"] = q0, q1, layer, m
     c = tn_circuit(circ.n_qubits, len(q0), arr)
     c._keep = arr
     return c
@@ -219,13 +219,14 @@ def tn_network(circ):
 
 class Plan:
     """A tn_plan handle: host planning in the constructor, device work after
-    :meth:`tn_plan_bind`."""
+    :meth:`tn_plan_bind`.  circ: an ``rqc.Circuit``, or what
+    :func:`circuit_struct` made of one (several plans of one circuit)."""
 
     def __init__(self, circ, bits, tree_ssa, sliced=(), **opts):
         lib = load()
         self._lib = lib
         self.n_qubits = circ.n_qubits
-        c = circuit_struct(circ)
+        c = circ if isinstance(circ, tn_circuit) else circuit_struct(circ)
         self._bits = np.ascontiguousarray(bits, np.uint8)
         self.k = self._bits.shape[0]
         ssa = np.ascontiguousarray(np.asarray(tree_ssa, np.int32).reshape(-1, 2))
@@ -237,6 +238,8 @@ class Plan:
                            len(sl), ctypes.byref(o), ctypes.byref(h)))
         self.h = h.value
         self.n_sliced = len(sl)
+        info = self.tn_plan_query()  # these never change
+        self._amps_per_row, self._n_batches = info["amps_per_row"], info["n_batches"]
         self._ws = None
 
     def __del__(self):
@@ -303,9 +306,9 @@ class Plan:
     def tn_contract(self, amps, precision=TN_FP32, batch_lo=0, batch_hi=None, stream=None):
         if isinstance(precision, str):
             precision = PRECISIONS[precision]
-        self._check_amps(amps, self.k * self.info["amps_per_row"], "tn_contract")
+        self._check_amps(amps, self.k * self._amps_per_row, "tn_contract")
         if batch_hi is None:
-            batch_hi = self.info["n_batches"]
+            batch_hi = self._n_batches
         _check(self._lib.tn_contract(self.h, int(precision), int(batch_lo), int(batch_hi), _ptr(amps),
                                      _stream(stream)))
 
@@ -322,7 +325,7 @@ class Plan:
         plans above TN_STATIC_SCRATCH_BYTES are rejected)."""
         if isinstance(precision, str):
             precision = PRECISIONS[precision]
-        self._check_amps(amps, self.k * self.info["amps_per_row"], "tn_contract_static")
+        self._check_amps(amps, self.k * self._amps_per_row, "tn_contract_static")
         _check(self._lib.tn_contract_static(self.h, int(precision), _ptr(amps), _stream(stream)))
 
     def tn_plan_set_kernel(self, step, kernel):
