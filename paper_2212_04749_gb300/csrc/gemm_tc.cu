@@ -690,25 +690,29 @@ __device__ __forceinline__ void tmem_gather16(uint32_t (&r)[32], uint32_t tb, co
 
 // Max-|component| of a warp block (16 complex columns; r: this lane's 32
 // accumulator values as float bits) over runs of RUN columns (one instance
-// each): folded in registers, one warp reduction per run, scaled by the
-// run's power of two (exact; SCALED: the values carry it already) and merged
-// into the slot's entry at the run's first column.  Columns past the tile's
-// valid ones hold zeros and merge nothing.
+// each): folded in registers, one warp reduction per run, whose result the
+// run's own lane keeps; then the runs' lanes scale theirs by the run's power
+// of two (exact; SCALED: the values carry it already) and merge them into the
+// slot's entries at the runs' first columns in one instruction.  (Lane 0
+// merging one run after the other, each behind its branch and its load of
+// the scale, cost 28 % of the 2^12 x 64 x 4 step, runs of 4: 3.50 ms a pass
+// against 2.52 without the fold.)  Columns past the tile's valid ones hold
+// zeros and merge nothing.
 template <int NC, int RUN, bool SCALED>
 __device__ __forceinline__ void fold_max16(const uint32_t (&r)[32], EpiMeta &em, int c0, int lane) {
-    uint32_t a[NC];
+    uint32_t mine = 0u;
 #pragma unroll
-    for (int j = 0; j < NC; ++j)
-        a[j] = __float_as_uint(fmaxf(fabsf(__uint_as_float(r[2 * j])), fabsf(__uint_as_float(r[2 * j + 1]))));
+    for (int q = 0; q < NC / RUN; ++q) {
+        float m = 0.f;  // |x| as float and as bits order alike
 #pragma unroll
-    for (int s = 1; s < RUN; s <<= 1)
-#pragma unroll
-        for (int j = 0; j < NC; j += 2 * s) a[j] = max(a[j], a[j + s]);
-#pragma unroll
-    for (int j = 0; j < NC; j += RUN) {
-        const uint32_t m = __reduce_max_sync(0xffffffffu, a[j]);
-        if (lane == 0 && m)
-            atomicMax(&em.mx[c0 + j], SCALED ? m : __float_as_uint(__uint_as_float(m) * em.sc[c0 + j]));
+        for (int j = q * RUN; j < (q + 1) * RUN; ++j)
+            m = fmaxf(m, fmaxf(fabsf(__uint_as_float(r[2 * j])), fabsf(__uint_as_float(r[2 * j + 1]))));
+        const uint32_t w = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+        mine = lane == q ? w : mine;
+    }
+    if (mine) {  // lanes below NC / RUN
+        const int c = c0 + lane * RUN;
+        atomicMax(&em.mx[c], SCALED ? mine : __float_as_uint(__uint_as_float(mine) * em.sc[c]));
     }
 }
 
