@@ -312,7 +312,9 @@ int tn_plan_set_kernel(tn_plan_t plan, int32_t step, int32_t kernel);
  * allows (K >= 8, 64 <= M < 2^31), on the CUDA cores otherwise. */
 #define TN_NCONFIG 4
 
-/* Set step `step` to configuration `config` (-1: the plan's own choice).
+/* Set step `step` to configuration `config` (-1: the plan's own choice: 0 or
+ * 2, on the tensor cores 3 where a group's resident B would leave the stream
+ * of A too little of the shared memory).
  * A step given a configuration (>= 0) then runs by itself even if it is small
  * (see tn_plan_step_times, family 4); config + TN_CONFIG_TUNED, with config as
  * tn_plan_get_configs returned it for a tuned plan of the same shape, leaves

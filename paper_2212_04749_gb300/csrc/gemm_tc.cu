@@ -1620,6 +1620,19 @@ int tc_resident_b_chunks(const StepDesc &d) {
     return n >= 1 && n <= BRES_MAX_B ? int(n) : 0;
 }
 
+int tc_rule_schedule(const StepDesc &d) {
+    // Schedule 0 reads A once per row tile, but a group's whole B resident in
+    // more than 6 of the pool's 11 slots leaves the A stream fewer than 5: one
+    // column tile's then (2^12 x 64 x 4 with groups of 32, 8 chunks against 4:
+    // 3.49 -> 3.10 ms a pass; 2^20 x 32 x 256, 8 against 2: 0.664 -> 0.653)
+    StepDesc t = d;
+    t.sched = 0;
+    const int all = tc_dictionary_chunks(t) > 0 ? 0 : tc_resident_b_chunks(t);
+    t.sched = 1;
+    const int one = tc_resident_b_chunks(t);
+    return all > 6 && one > 0 && one <= 6 ? 1 : 0;
+}
+
 namespace {
 int g_num_sms = 0;
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;

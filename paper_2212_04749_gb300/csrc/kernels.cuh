@@ -117,6 +117,8 @@ int tc_resident_b_chunks(const StepDesc &d);
 // tile keeps them resident for the whole launch (a dictionary): the chunk
 // count, else 0.
 int tc_dictionary_chunks(const StepDesc &d);
+// The schedule of a tensor-core step for which none was chosen.
+int tc_rule_schedule(const StepDesc &d);
 // Bytes of the packed-B form of a step (every B instance in the MMA layout,
 // 16 KB per 64 columns x 16 complex k), 0 if the step cannot take it.
 int64_t tc_packed_b_bytes(const StepDesc &d);
