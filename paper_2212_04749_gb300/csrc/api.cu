@@ -459,17 +459,17 @@ PlanObj::Sched make_schedule(const PlanObj *o, int lv) {
                     outputs += P.nodes[S.node].n_inst << (S.mb + S.nb);
                 }
             if (ready.empty()) break;
-            // lanes per output: as many as leave the phase within 4096 threads
+            // lanes per output: as many as leave the phase within 8192 threads
             int lanes = 0;
-            while (lanes < 5 && (outputs << (lanes + 1)) <= 4096) ++lanes;
+            while (lanes < 5 && (outputs << (lanes + 1)) <= 8192) ++lanes;
             int64_t warps = 0;
             for (int q : ready) {
                 const tnp::Step &S = P.steps[L[q].step];
                 const int lg = std::min(lanes, std::max(S.kb - 1, 0));
                 // a warp takes 32 lanes of outputs, four times as many where
-                // the step fills the cluster's 128 warps four times over
+                // the step fills the cluster's 256 warps four times over
                 const int64_t w = (((P.nodes[S.node].n_inst << (S.mb + S.nb)) << lg) + 31) / 32;
-                const bool four = w >= 512;
+                const bool four = w >= 1024;
                 g.four[g.n_steps] = four;
                 warps += four ? (w + 3) / 4 : w;
                 g.step[g.n_steps] = (uint16_t)L[q].step;

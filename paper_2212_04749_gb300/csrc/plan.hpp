@@ -117,8 +117,8 @@ struct Step {
 // A step of at most SMALL_MACS complex multiply-adds and SMALL_OUTPUTS outputs
 // costs its launch and its chain of dependent loads, about 5 us, whatever it
 // computes; such steps run together, many to a launch, on one cluster of 16
-// blocks (small.cu).  There 2^18 multiply-adds, or four outputs for each of
-// its 4096 threads, are about 2 us of loads; steps of 2^17 outputs, whose
+// blocks (small.cu).  There 2^18 multiply-adds, or two outputs for each of
+// its 8192 threads, are about 2 us of loads; steps of 2^17 outputs, whose
 // instance pairs and operands 16 SMs fetch at 2 TB/s, took 12 us.
 constexpr double SMALL_MACS = 262144.0, SMALL_OUTPUTS = 16384.0;
 constexpr int SMALL_MAX_KB = 10;
