@@ -200,7 +200,7 @@ struct Builder {
     std::vector<std::vector<int32_t>> oi;  // node -> per distinct bitstring out-instance
     std::vector<int> slice_of;             // bond edge -> internal slice index (-1: not sliced)
     bool bad_offsets = false;              // set by layout_workspace's self-check
-    std::vector<std::vector<int>> low_bits; // per node: bonds its consumer contracts (edge-id order)
+    std::vector<std::vector<int>> low_bits; // per node: bonds its consumer contracts, in address order
     std::vector<std::vector<int>> tails;    // per node: its other bonds, in its consumer's row/column order
 
     bool fail(int c, const std::string &msg) {
@@ -397,7 +397,7 @@ struct Builder {
             P.steps.push_back(st);
         }
         // Layouts.  Every node is stored with the bonds its consumer contracts
-        // (L = its open bonds shared with its sibling, in edge-id order) as
+        // (L = its open bonds shared with its sibling, in low_bits' order) as
         // the lowest address bits, so that both operands of every step are
         // K-major with the same k order; the producing step's epilogue writes
         // that layout directly.  Leaves got theirs in make_plan.
@@ -1151,23 +1151,40 @@ bool make_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int
         low_bits[a] = kset;
         low_bits[b] = kset;
     }
-    // Address order above the contracted bonds: the bonds the grandparent's
-    // step contracts first, then the rest, each in edge-id order.  That is
-    // the consumer's row (resp. column) order, so every operand is
-    // row-affine: address = k + 2^kb * m.
-    std::vector<std::vector<int>> tails(NN);
-    for (int v = 0; v < NN; ++v) {
-        const int p = P.nodes[v].parent;
-        auto has = [](const std::vector<int> &s, int e) { return std::binary_search(s.begin(), s.end(), e); };
-        std::vector<int> rest;
-        for (int e : open[v]) {
-            if (has(low_bits[v], e)) continue;
-            if (p >= 0 && has(low_bits[p], e)) tails[v].push_back(e);
-            else rest.push_back(e);
-        }
-        tails[v].insert(tails[v].end(), rest.begin(), rest.end());
+    // Order of the contracted bonds: those that the larger operand's own step
+    // takes from its rows come first, then its columns' (each in edge-id
+    // order), so that consecutive rows of that step, a warp's lanes, store to
+    // consecutive addresses.
+    auto rows_of = [&](int v) {  // child of v that holds the rows of its step
+        const int l = P.nodes[v].left, r = P.nodes[v].right;
+        return Builder::a_is_left(P.nodes[l], P.nodes[r]) ? l : r;
+    };
+    for (int v = T; v < NN; ++v) {
+        const int big = rows_of(v);
+        if (big < T) continue;
+        const std::vector<int> &rows = open[rows_of(big)];
+        std::vector<int> &k = low_bits[P.nodes[v].left];
+        std::stable_partition(k.begin(), k.end(),
+                              [&](int e) { return std::binary_search(rows.begin(), rows.end(), e); });
+        low_bits[P.nodes[v].right] = k;
     }
-    // leaf layouts: the contracted bonds first (edge-id order), then the tail
+    // Address order above the contracted bonds: the order that the consumer's
+    // output gives them (the root: edge-id order).  That is the consumer's
+    // row (resp. column) order, so every operand is row-affine: address =
+    // k + 2^kb * m, and the rows' addresses in the output rise with m.
+    std::vector<std::vector<int>> tails(NN);
+    for (int v = NN - 1; v >= 0; --v) {
+        const int p = P.nodes[v].parent;
+        auto has = [](const std::vector<int> &s, int e) { return std::find(s.begin(), s.end(), e) != s.end(); };
+        if (p < 0) {
+            tails[v] = open[v];
+            continue;
+        }
+        for (const std::vector<int> *part : {&low_bits[p], &tails[p]})
+            for (int e : *part)
+                if (std::binary_search(open[v].begin(), open[v].end(), e) && !has(low_bits[v], e)) tails[v].push_back(e);
+    }
+    // leaf layouts: the contracted bonds first, then the tail
     for (int v = 0; v < T; ++v) {
         Node &nd = P.nodes[v];
         nd.layout = low_bits[v];
