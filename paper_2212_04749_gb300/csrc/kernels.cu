@@ -676,23 +676,37 @@ __global__ void __launch_bounds__(128) k_step_gemm_simt2(const StepDesc d, int c
 }
 
 // Steps with a long row and few columns per A instance (K >= 32, K N <= 256,
-// M >= 128), grouped: a block takes 128 rows of a group's A instance and up to
-// 16 of the group's concatenated columns (the instances that share it), so A
-// is read once for 16 columns.  Chunks of 8 complex k of A (128 rows x 64
-// bytes) and B arrive by cp.async in three stages; a thread holds 4 rows x 4
-// columns, rows 32 apart, and reads both operands 16 bytes at a time (128 FMA
-// for 8 loads, B's as broadcasts).  A warp takes four columns, which four
-// rotates with the block so that tiles of fewer columns load all four
-// schedulers; the other warps only copy.  Bound by HBM (A) and the FMA rate
-// at about the same time for 8 columns; a block lives for little more than
-// its latencies, so six of them share an SM.  The per-row kernel held a row
-// of 64 in two lanes' registers, read B from shared memory for every row and
-// instance again and loaded 32 bytes a row at a time: 4.47 ms on 2^8 x 64 x 2
-// with 64448 A instances of 4 (9.5 GB, 1.40 ms of HBM), 2.61 ms here.
-constexpr int NBM = 128, NBN = 16, NBK = 8, NLD = NBK + 2, NST = 3;
-constexpr size_t NARROW_SMEM = size_t(NST) * (NBM + NBN) * NLD * sizeof(float2);
+// M >= 128), grouped: a block takes 128 rows of a group's A instance and all
+// of the group's concatenated columns (the instances that share it), 8 or 16
+// at a time, so A is read once for most groups and from L2 for the others'
+// further columns.  Chunks of 8 complex k of A (128 rows x 64 bytes) and B
+// arrive by cp.async in three stages; a thread holds 2 or 4 rows x 4 columns,
+// rows 32 apart, and reads both operands 16 bytes at a time (64 FMA for 6
+// loads or 128 for 8, B's as broadcasts).  Groups of 8 columns on average
+// take tiles of 8, on which all four warps work; with tiles of 16 two of them
+// would only copy (38.3 against 39.8 ms of the step below).  In tiles of 16
+// the four columns of a warp rotate with the block, so that tiles with fewer
+// load all four schedulers.  Bound by HBM (A) and the FMA rate at about the
+// same time for 8 columns; a block lives for little more than its latencies,
+// so six of them share an SM.  The per-row kernel held a row of 64 in two
+// lanes' registers, read B from shared memory for every row and instance
+// again and loaded 32 bytes a row at a time: 4.47 ms on 2^8 x 64 x 2 with
+// 64448 A instances of 1 to 10 (9.5 GB, 1.40 ms of HBM), 2.40 ms here (1.9
+// without the FMAs).
+constexpr int NBK = 8, NLD = NBK + 2, NST = 3;
 
-__global__ void __launch_bounds__(128, 6) k_step_narrow(const StepDesc d, int subs, int mtiles) {
+// WR x WC warps, a warp 32 RX rows x 4 columns
+template <int WR, int WC, int RX>
+struct NarrowTile {
+    static constexpr int ROWS = 32 * WR * RX, COLS = 4 * WC, THREADS = 32 * WR * WC;
+    static constexpr size_t SMEM = size_t(NST) * (ROWS + COLS) * NLD * sizeof(float2);
+};
+
+template <int WR, int WC, int RX, int BLOCKS>
+__global__ void __launch_bounds__(32 * WR * WC, BLOCKS) k_step_narrow(const StepDesc d, int mtiles) {
+    using T = NarrowTile<WR, WC, RX>;
+    constexpr int NBM = T::ROWS, NBN = T::COLS, NT = T::THREADS;
+    static_assert(NT >= 40 && NBN * NBK / 2 <= NT, "threads of the set-up");
     extern __shared__ __align__(16) float2 sn[];
     __shared__ int64_t s_bbase[NBN], s_cbase[NBN];
     __shared__ int32_t s_e[NBN];
@@ -700,24 +714,19 @@ __global__ void __launch_bounds__(128, 6) k_step_narrow(const StepDesc d, int su
     __shared__ int8_t s_pCm[40];
     const int tid = threadIdx.x, lane = tid & 31;
     const int64_t bid = blockIdx.x;
-    const int sub = int(bid % subs);
-    const int64_t rest = bid / subs;
-    const int mt = int(rest % mtiles);
+    const int mt = int(bid % mtiles);
     // {first instance, count, A instance, first column} of 64 columns
-    const int4 rec = __ldg(d.trec + rest / mtiles);
+    const int4 rec = __ldg(d.trec + bid / mtiles);
     const int N = 1 << d.nb, K = 1 << d.kb;
     const int64_t M = int64_t(1) << d.mb;
-    const int c0 = rec.w + sub * NBN;  // column of the group
-    const int left = min(rec.y << d.nb, rec.w + 64) - c0;
-    if (left <= 0) return;  // uniform across the block
-    const int ncols = min(left, NBN);
+    const int cend = min(rec.y << d.nb, rec.w + 64);  // columns of the group
     const int64_t m0 = int64_t(mt) * NBM;
     const float2 *A = d.A + int64_t(rec.z) * d.sA + (m0 << d.kb);
     const int nchunk = K / NBK;
     float2 *sa = sn, *sb = sn + NST * NBM * NLD;
-    auto issue_a = [&](int ch) {  // 16-byte pieces, four a row (M >= 128: every row exists)
+    auto issue_a = [&](int ch) {  // 16-byte pieces, four a row (M >= NBM: every row exists)
 #pragma unroll
-        for (int e = tid; e < NBM * NBK / 2; e += 128) {
+        for (int e = tid; e < NBM * NBK / 2; e += NT) {
             const int r = e >> 2, q = e & 3;
             cp_async16_zfill(static_cast<uint32_t>(__cvta_generic_to_shared(sa + ((ch % NST) * NBM + r) * NLD + 2 * q)),
                              A + (int64_t(r) << d.kb) + ch * NBK + 2 * q, true);
@@ -732,88 +741,93 @@ __global__ void __launch_bounds__(128, 6) k_step_narrow(const StepDesc d, int su
         }
     };
     auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
-    issue_a(0);
-    issue_a(1);
     if (tid < 40) s_pCm[tid] = d.pCm[tid];
-    if (tid < NBN) {
-        s_mx[tid] = 0u;
-        s_bbase[tid] = -1;
-        if (tid < ncols) {
-            const int inst = rec.x + ((c0 + tid) >> d.nb);
-            const int n = (c0 + tid) & (N - 1);
-            const int ib = d.instab[inst].y;
-            const int ea = d.mxA ? exp_of(d.mxA[rec.z]) : 0, eb = d.mxB ? exp_of(d.mxB[ib]) : 0;
-            s_bbase[tid] = int64_t(ib) * d.sB + (int64_t(n) << d.kb);
-            s_cbase[tid] = int64_t(inst) * d.sC + dep(n, d.pCn, d.nb);
-            s_e[tid] = ea + eb;
-            if (n == 0 && mt == 0) d.EC[inst] = d.EA[rec.z] + ea + d.EB[ib] + eb;
-        }
-    }
-    __syncthreads();
-    issue_b(0);
-    commit();
-    issue_b(1);
-    commit();
-    const int cg = ((tid >> 5) + int(bid)) & 3;
-    const bool works = 4 * cg < ncols;  // the same for a warp
-    float2 acc[4][4];
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] = make_float2(0.f, 0.f);
-    for (int ch = 0; ch < nchunk; ++ch) {
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-        __syncthreads();  // chunk ch is in place; every warp is done with chunk ch - 1
-        if (ch + 2 < nchunk) {
-            issue_a(ch + 2);
-            issue_b(ch + 2);
-        }
-        commit();
-        if (works) {
-            const float2 *a_s = sa + ((ch % NST) * NBM + lane) * NLD, *b_s = sb + ((ch % NST) * NBN + 4 * cg) * NLD;
-#pragma unroll
-            for (int kk = 0; kk < NBK; kk += 2) {
-                float4 a[4], b[4];
-#pragma unroll
-                for (int x = 0; x < 4; ++x) a[x] = *reinterpret_cast<const float4 *>(a_s + 32 * x * NLD + kk);
-#pragma unroll
-                for (int y = 0; y < 4; ++y) b[y] = *reinterpret_cast<const float4 *>(b_s + y * NLD + kk);
-#pragma unroll
-                for (int x = 0; x < 4; ++x)
-#pragma unroll
-                    for (int y = 0; y < 4; ++y) {
-                        cfma(acc[x][y], make_float2(a[x].x, a[x].y), make_float2(b[y].x, b[y].y));
-                        cfma(acc[x][y], make_float2(a[x].z, a[x].w), make_float2(b[y].z, b[y].w));
-                    }
+    for (int c0 = rec.w; c0 < cend; c0 += NBN) {  // the same for a block
+        if (c0 > rec.w) __syncthreads();  // the stages and the columns' records are reused
+        const int ncols = min(cend - c0, NBN);
+        issue_a(0);
+        issue_a(1);
+        if (tid < NBN) {
+            s_mx[tid] = 0u;
+            s_bbase[tid] = -1;
+            if (tid < ncols) {
+                const int inst = rec.x + ((c0 + tid) >> d.nb);
+                const int n = (c0 + tid) & (N - 1);
+                const int ib = d.instab[inst].y;
+                const int ea = d.mxA ? exp_of(d.mxA[rec.z]) : 0, eb = d.mxB ? exp_of(d.mxB[ib]) : 0;
+                s_bbase[tid] = int64_t(ib) * d.sB + (int64_t(n) << d.kb);
+                s_cbase[tid] = int64_t(inst) * d.sC + dep(n, d.pCn, d.nb);
+                s_e[tid] = ea + eb;
+                if (n == 0 && mt == 0) d.EC[inst] = d.EA[rec.z] + ea + d.EB[ib] + eb;
             }
         }
-    }
-    if (works) {
-        int64_t off[4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) off[x] = dep(m0 + lane + 32 * x, s_pCm, d.mb);
-#pragma unroll
-        for (int y = 0; y < 4; ++y) {
-            const int c = 4 * cg + y;
-            if (c >= ncols) break;  // the same for a warp
-            const float sc = pow2f(-s_e[c]);
-            float2 *C = d.C + s_cbase[c];
-            uint32_t mx = 0u;
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const float2 v = make_float2(acc[x][y].x * sc, acc[x][y].y * sc);
-                C[off[x]] = v;
-                mx = max(mx, absmax_bits(v));
-            }
-            if (d.mxC) {
-                mx = __reduce_max_sync(0xffffffffu, mx);
-                if (lane == 0 && mx) atomicMax(&s_mx[c], mx);
-            }
-        }
-    }
-    if (d.mxC) {
         __syncthreads();
-        if (tid < ncols && s_mx[tid]) record_max(d.mxC + rec.x + ((c0 + tid) >> d.nb), s_mx[tid]);
+        issue_b(0);
+        commit();
+        issue_b(1);
+        commit();
+        const int cg = WC == 4 ? ((tid >> 5) + int(bid)) & 3 : (tid >> 5) % WC;
+        const int r0 = (tid >> 5) / WC * 32 * RX + lane;  // the thread's rows: r0 + 32 x
+        const bool works = 4 * cg < ncols;  // the same for a warp
+        float2 acc[RX][4];
+#pragma unroll
+        for (int x = 0; x < RX; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) acc[x][y] = make_float2(0.f, 0.f);
+        for (int ch = 0; ch < nchunk; ++ch) {
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncthreads();  // chunk ch is in place; every warp is done with chunk ch - 1
+            if (ch + 2 < nchunk) {
+                issue_a(ch + 2);
+                issue_b(ch + 2);
+            }
+            commit();
+            if (works) {
+                const float2 *a_s = sa + ((ch % NST) * NBM + r0) * NLD, *b_s = sb + ((ch % NST) * NBN + 4 * cg) * NLD;
+#pragma unroll
+                for (int kk = 0; kk < NBK; kk += 2) {
+                    float4 a[RX], b[4];
+#pragma unroll
+                    for (int x = 0; x < RX; ++x) a[x] = *reinterpret_cast<const float4 *>(a_s + 32 * x * NLD + kk);
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) b[y] = *reinterpret_cast<const float4 *>(b_s + y * NLD + kk);
+#pragma unroll
+                    for (int x = 0; x < RX; ++x)
+#pragma unroll
+                        for (int y = 0; y < 4; ++y) {
+                            cfma(acc[x][y], make_float2(a[x].x, a[x].y), make_float2(b[y].x, b[y].y));
+                            cfma(acc[x][y], make_float2(a[x].z, a[x].w), make_float2(b[y].z, b[y].w));
+                        }
+                }
+            }
+        }
+        if (works) {
+            int64_t off[RX];
+#pragma unroll
+            for (int x = 0; x < RX; ++x) off[x] = dep(m0 + r0 + 32 * x, s_pCm, d.mb);
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int c = 4 * cg + y;
+                if (c >= ncols) break;  // the same for a warp
+                const float sc = pow2f(-s_e[c]);
+                float2 *C = d.C + s_cbase[c];
+                uint32_t mx = 0u;
+#pragma unroll
+                for (int x = 0; x < RX; ++x) {
+                    const float2 v = make_float2(acc[x][y].x * sc, acc[x][y].y * sc);
+                    C[off[x]] = v;
+                    mx = max(mx, absmax_bits(v));
+                }
+                if (d.mxC) {
+                    mx = __reduce_max_sync(0xffffffffu, mx);
+                    if (lane == 0 && mx) atomicMax(&s_mx[c], mx);
+                }
+            }
+        }
+        if (d.mxC) {
+            __syncthreads();
+            if (tid < ncols && s_mx[tid]) record_max(d.mxC + rec.x + ((c0 + tid) >> d.nb), s_mx[tid]);
+        }
     }
 }
 
@@ -1230,14 +1244,18 @@ static int row_lanes(int kb, int nb) {
 cudaError_t launch_step_row(const StepDesc &d, cudaStream_t s) {
     if (d.kb + d.nb > 8 || d.nb > 4 || d.mb > 40) return cudaErrorInvalidValue;
     if (d.kb >= NARROW_MIN_KB && d.mb >= 7) {
-        const int64_t cols = int64_t(d.max_group) << d.nb;
-        const int subs = cols >= 64 ? 4 : int((cols + NBN - 1) / NBN);
-        const int64_t mtiles = (int64_t(1) << d.mb) / NBM;
-        const int64_t nblk = d.n_ctab * subs * mtiles;
-        if (nblk <= 0) return cudaSuccess;
-        if (nblk > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-        k_step_narrow<<<dim3((unsigned)nblk), 128, NARROW_SMEM, s>>>(d, subs, (int)mtiles);
-        return cudaGetLastError();
+        auto go = [&](auto kernel, int rows, int threads, size_t smem) -> cudaError_t {
+            const int64_t mtiles = (int64_t(1) << d.mb) / rows;
+            const int64_t nblk = d.n_ctab * mtiles;
+            if (nblk <= 0) return cudaSuccess;
+            if (nblk > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+            kernel<<<dim3((unsigned)nblk), threads, smem, s>>>(d, (int)mtiles);
+            return cudaGetLastError();
+        };
+        using W = NarrowTile<1, 4, 4>;
+        using H = NarrowTile<2, 2, 2>;
+        return (d.nInst << d.nb) <= 8 * d.n_groups ? go(k_step_narrow<2, 2, 2, 6>, H::ROWS, H::THREADS, H::SMEM)
+                                                   : go(k_step_narrow<1, 4, 4, 6>, W::ROWS, W::THREADS, W::SMEM);
     }
     const int K = 1 << d.kb;
     const int L = row_lanes(d.kb, d.nb);
@@ -1339,7 +1357,7 @@ cudaError_t launch_step_skinny(const StepDesc &d, cudaStream_t s) {
 
 cudaError_t init_simt_kernels() {
     const cudaError_t e =
-        cudaFuncSetAttribute(k_step_narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, int(NARROW_SMEM));
+        cudaFuncSetAttribute(k_step_narrow<1, 4, 4, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(NarrowTile<1, 4, 4>::SMEM));
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_step_gemm_simt2, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SIMT2_SMEM));
 }
