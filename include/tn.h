@@ -60,7 +60,9 @@ enum {
 /* Arithmetic of the pairwise contractions (accumulation is always FP32;
  * the cross-slice sum and XEB are FP64). */
 enum {
-    TN_FP32 = 0,    /* complex64 operands, FP32 FMA on the CUDA cores */
+    TN_FP32 = 0,    /* complex64 operands, FP32 FMA on the CUDA cores; large steps
+                     * of rescaled plans in FP16x3 (see TN_NCONFIG), whose
+                     * error is no larger */
     TN_TF32 = 1,    /* tensor cores, TF32 operands, FP32 accumulate */
     TN_BF16X3 = 2   /* tensor cores, hi/lo BF16 split, three products */
 };
@@ -309,7 +311,14 @@ int tn_plan_set_kernel(tn_plan_t plan, int32_t step, int32_t kernel);
  *      (SIMT) / the column tiles of one row tile (tensor cores)
  *   3  grouped GEMM, the other walk order
  * The GEMM runs on the tensor cores for TN_TF32 / TN_BF16X3 where the shape
- * allows (K >= 8, 64 <= M < 2^31), on the CUDA cores otherwise. */
+ * allows (K >= 8, 64 <= M < 2^31), on the CUDA cores otherwise.  For TN_FP32
+ * configuration 2 takes the tensor cores as well where a step has K >= 128,
+ * N >= 64, 64 <= M < 2^31, maxima for both operands (tn_options.rescale, no
+ * leaf) and room for its packed B: each operand instance scaled by a power of
+ * two and split into two fp16 halves (22 bits of each value down to 2^-18 of
+ * the instance's largest), three products, units of 64 real k summed in
+ * FP32 registers.  Configuration 3 and tn_plan_set_tc_resident_b(plan, 0)
+ * stay on the FMA kernel. */
 #define TN_NCONFIG 4
 
 /* Set step `step` to configuration `config` (-1: the plan's own choice: 0 or

@@ -360,6 +360,9 @@ int run_step(PlanObj *o, int s, int precision, int64_t sigma, cudaStream_t st) {
         if (!(s < (int)o->config_override.size() && o->config_override[s] >= 0)) d.sched = tnk::tc_rule_schedule(d);
         e = o->amap[s].ok ? tnk::launch_step_gemm_tc(d, &o->amap[s].map, precision, o->err_flag, st)
                           : cudaErrorInvalidValue;  // its TMA descriptor could not be encoded
+    } else if (precision == TN_FP32 && o->amap[s].ok && tnk::tc_fp32_takes(d)) {
+        fam = 2;
+        e = tnk::launch_step_gemm_tc(d, &o->amap[s].map, precision, o->err_flag, st);
     } else {
         fam = 1;
         e = tnk::launch_step_gemm_simt(d, st);

@@ -42,6 +42,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include "kernels.cuh"
 
@@ -265,24 +266,31 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
 //   warp 18    : epilogue metadata (instances, rescale, C offsets, E_C),
 //                a ring of MS tiles ahead of the epilogue.
 // The epilogue warpgroups take registers from the others (setmaxnreg).
-constexpr int NPROD = 256;   // warps 0-7
 // BF16x3: warps 0-3 alone write the split A into TMEM, each thread one row
 // (its warp's lane quadrant), both K steps.  With the two K steps written by
 // warps w and w + 4 at once (same lanes, other columns) the products came
 // out different from run to run; one writer per lane quadrant gives the
 // exact results of the shared-memory form.
 constexpr int NAW = 128;
-constexpr int EPI_WARP0 = 8; // warps 8-15: two per TMEM lane quadrant
-constexpr int NEPI = 256;
+constexpr int NEPI = 256;     // eight epilogue warps: two per TMEM lane quadrant
+constexpr int NPROD = 256;    // warps 0-7
+constexpr int EPI_WARP0 = 8;  // warps 8-15: two per TMEM lane quadrant
 constexpr int MMA_WARP = 16;
 constexpr int TMA_WARP = 17;
-constexpr int META_WARP = 18;  // warp 19 idles
+constexpr int META_WARP = 18; // warp 19 idles
 constexpr int NTHREADS = 640;
 // Register split (setmaxnreg, per warpgroup).  The block is launched with
 // 96 registers a thread (640 x 96 = 61440); after the split: producers
-// 256 x 88 + epilogue 256 x 112 + control warpgroup 128 x 72 = 60416.
-constexpr int LAUNCH_REGS = 96, PROD_REGS = 88, EPI_REGS = 112, CTL_REGS = 72;
-static_assert(NPROD * PROD_REGS + NEPI * EPI_REGS + 128 * CTL_REGS <= NTHREADS * LAUNCH_REGS,
+// 256 x 88 + epilogue 256 x 112 + control warpgroup 128 x 72 = 60416.  FP16x3
+// (packed B only) has no B loaders: warps 4-7 keep 24 (they leave at once) and
+// the epilogue, which also sums a tile's units in registers, takes 144.
+constexpr int LAUNCH_REGS = 96, PROD_REGS = 88, CTL_REGS = 72;
+__host__ __device__ constexpr int epi_regs(int prec) { return prec == 3 ? 144 : 112; }
+__host__ __device__ constexpr int idle_regs(int prec) { return prec == 3 ? 24 : PROD_REGS; }  // warps 4-7
+constexpr int split_regs(int prec) {
+    return NAW * PROD_REGS + (NPROD - NAW) * idle_regs(prec) + NEPI * epi_regs(prec) + 128 * CTL_REGS;
+}
+static_assert(split_regs(2) <= NTHREADS * LAUNCH_REGS && split_regs(3) <= NTHREADS * LAUNCH_REGS,
               "register split above the launch allocation");
 constexpr int MS = 8;         // epilogue metadata ring (tiles ahead of the epilogue)
 constexpr int NACC_MAX = 8;   // accumulators in TMEM (narrow tiles: up to 8 in flight)
@@ -297,7 +305,7 @@ constexpr int TM_A = TMEM_COLS2, TM_ASTAGE = 32;
 constexpr int NTS = 8;
 static_assert(TM_A + NTS * TM_ASTAGE <= 512, "TMEM A stages within the allocation");
 template <int PREC>
-__host__ __device__ constexpr uint32_t tmem_alloc_cols() { return PREC == 2 ? 512u : uint32_t(TMEM_COLS2); }
+__host__ __device__ constexpr uint32_t tmem_alloc_cols() { return PREC >= 2 ? 512u : uint32_t(TMEM_COLS2); }
 
 // Shared-memory layout.  Streaming B (BRES = false): A ring, B MMA stages,
 // raw B pieces, epilogue staging.  Resident B (BRES = true): a pool of
@@ -338,7 +346,8 @@ struct alignas(16) EpiMeta {
     uint32_t mx[TBN];     // max-|component| of a run of an instance's columns, at the run's first column
     int16_t acol[TBN];    // B dictionary: accumulator (complex) column holding tile column c
     int64_t base;         // element offset of tile element (row 0, column 0) in C
-    int32_t ncv, pad;     // valid columns
+    int32_t ncv;          // valid columns
+    int32_t ea;           // exponent of the tile's A instance
 };
 
 // Destination order of one epilogue warp's 32 rows x 16 complex columns.
@@ -505,6 +514,34 @@ struct TileIter {
 // spread over the banks
 __device__ __forceinline__ int stage_swz(int u) { return u ^ (((u >> 3) ^ (u >> 6)) & 7); }
 
+// x = hi + lo in 16-bit halves, rounded to nearest: 16 bits of x in bf16
+// (FP32's range), 22 in fp16 (x scaled into its range)
+__device__ __forceinline__ void split_half(float x, __nv_bfloat16 &h, __nv_bfloat16 &l) {
+    h = __float2bfloat16_rn(x);
+    l = __float2bfloat16_rn(x - __bfloat162float(h));
+}
+__device__ __forceinline__ void split_half(float x, __half &h, __half &l) {
+    h = __float2half_rn(x);
+    l = __float2half_rn(x - __half2float(h));
+}
+__device__ __forceinline__ void split_pair_bf16(float x, float y, uint32_t &hw, uint32_t &lw) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+    const float2 hf = __bfloat1622float2(h);
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(x - hf.x, y - hf.y);
+    hw = *reinterpret_cast<const uint32_t *>(&h);
+    lw = *reinterpret_cast<const uint32_t *>(&lo);
+}
+__device__ __forceinline__ void split_pair_f16(float x, float y, uint32_t &hw, uint32_t &lw) {
+    const __half2 h = __floats2half2_rn(x, y);
+    const float2 hf = __half22float2(h);
+    const __half2 lo = __floats2half2_rn(x - hf.x, y - hf.y);
+    hw = *reinterpret_cast<const uint32_t *>(&h);
+    lw = *reinterpret_cast<const uint32_t *>(&lo);
+}
+// FP16x3 operands are scaled by 2^(14 - e), e the exponent of the
+// instance's largest component: below 2^15, and exact down to 2^-40 of it
+constexpr float HALF_TOP = 16384.f, HALF_UNSCALE = 1.f / (16384.f * 16384.f);
+
 // One producer thread's B piece: column bcol, complex k 4 kqb .. 4 kqb + 3
 // of a chunk (p0, p1 = the four values), expanded into the real 2x2 form
 // (rows 2 bcol: Re, -Im; 2 bcol + 1: Im, Re) in the K-major no-swizzle
@@ -532,13 +569,12 @@ __device__ __forceinline__ void expand_b(uint8_t *base, int bcol, int kqb, const
         *reinterpret_cast<float4 *>(base + off(rb, 8 * kqb, 4)) = sw ? a0 : b0;
         *reinterpret_cast<float4 *>(base + off(rb, 8 * kqb + 4, 4)) = sw ? a1 : b1;
     } else {
-        __align__(16) __nv_bfloat16 h0[8], l0[8], h1[8], l1[8];
+        using H = std::conditional_t<PREC == 3, __half, __nv_bfloat16>;
+        __align__(16) H h0[8], l0[8], h1[8], l1[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            h0[q] = __float2bfloat16_rn(r0[q]);
-            l0[q] = __float2bfloat16_rn(r0[q] - __bfloat162float(h0[q]));
-            h1[q] = __float2bfloat16_rn(r1[q]);
-            l1[q] = __float2bfloat16_rn(r1[q] - __bfloat162float(h1[q]));
+            split_half(r0[q], h0[q], l0[q]);
+            split_half(r1[q], h1[q], l1[q]);
         }
         uint8_t *blo = base + nr * TBKR * 2;
         const uint4 H0 = *reinterpret_cast<uint4 *>(h0), L0 = *reinterpret_cast<uint4 *>(l0);
@@ -563,7 +599,8 @@ __device__ __forceinline__ void expand_b(uint8_t *base, int bcol, int kqb, const
 // stored to hi columns 16 (q / 2) + 4 (q % 2) .. + 3 and the lo columns 8
 // further on, relative to ta (this lane's row of the stage).  tcgen05.st is
 // warp-wide (.sync.aligned).
-__device__ __forceinline__ void split_a_quarter(const uint8_t *slot, int row, int q, uint32_t ta) {
+template <int PREC>
+__device__ __forceinline__ void split_a_quarter(const uint8_t *slot, int row, int q, uint32_t ta, float s) {
     const int sw = row & 7;
     const uint8_t *rowp = slot + row * 128;
     const float4 v0 = *reinterpret_cast<const float4 *>(rowp + (((2 * q) ^ sw) << 4));
@@ -572,11 +609,10 @@ __device__ __forceinline__ void split_a_quarter(const uint8_t *slot, int row, in
     uint32_t hw[4], lw[4];
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(x[2 * p], x[2 * p + 1]);
-        const float2 hf = __bfloat1622float2(h);
-        const __nv_bfloat162 lo = __floats2bfloat162_rn(x[2 * p] - hf.x, x[2 * p + 1] - hf.y);
-        hw[p] = *reinterpret_cast<const uint32_t *>(&h);
-        lw[p] = *reinterpret_cast<const uint32_t *>(&lo);
+        if (PREC == 3)  // s: 2^-e of the instance
+            split_pair_f16(x[2 * p] * s * HALF_TOP, x[2 * p + 1] * s * HALF_TOP, hw[p], lw[p]);
+        else
+            split_pair_bf16(x[2 * p], x[2 * p + 1], hw[p], lw[p]);
     }
     const uint32_t c = ta + uint32_t(16 * (q >> 1) + 4 * (q & 1));
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(c), "r"(hw[0]), "r"(hw[1]),
@@ -737,6 +773,18 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
     // MODE 3: B packed in MMA form in global memory (tc_pack_b, once per
     // launch) and bulk-copied chunk by chunk beside A from L2, B carrying
     // 2^-eb
+    // PREC 3, FP16x3 for FP32 steps (MODE 3 only): operands scaled by powers of
+    // two and split into fp16 halves.  The tensor cores truncate each sum into
+    // the accumulator (relative L2 error 1.0e-6 over 1024 real k of random
+    // signs, the FMA kernel 2.5e-7; 6.5e-8 over 64), so a unit of two chunks
+    // (64 real k) starts from zero, its small products first, and the epilogue
+    // adds the units in FP32 registers, rounded to nearest: the contraction's
+    // error is 3 to 42 % below the FMA kernel's.  Bound by the loads of A and B
+    // from L2 and the tensor cores together.  53-qubit circuit, FP32: 2^12 x
+    // 2^9 x 2^8 with 512 instances 48 -> 7.3 ms, all of it 228 -> 68 ms.
+    constexpr int EPI_REGS = epi_regs(PREC);
+    constexpr bool ASPLIT = PREC >= 2;  // A split into TMEM
+    static_assert(PREC != 3 || MODE == 3, "FP16x3: packed B");
     constexpr bool BRES = MODE == 1 || MODE == 2;
     // MODE 4: packed B with two adjacent column tiles of a row tile (one B
     // instance's 128 columns, or with N = 64 two instances' 64) per MMA of
@@ -797,7 +845,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
             mbar_init(&X.rfull[s], 1);
             // BF16x3 (not packed B): the producers release the A slot once
             // they hold its values; otherwise the MMAs' commit does
-            mbar_init(&X.rempty[s], (PREC == 2 && !BPACK) ? NAW : 1);
+            mbar_init(&X.rempty[s], (ASPLIT && !BPACK) ? NAW : 1);
         }
         for (int s = 0; s < NTS; ++s) {
             mbar_init(&X.afull[s], NAW);
@@ -948,23 +996,26 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                 mbar_wait(&X.rfull[j % nrs], uint32_t(j / nrs) & 1u);
         }
         __syncwarp();
+    } else if (PREC == 3 && warp >= NAW / 32 && warp < NPROD / 32) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(idle_regs(PREC)));
     } else if (warp < NPROD / 32) {
         // ------------------------------------------------------------ B loads, A split
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PROD_REGS));
         const int bcol = tid & 63, kqb = tid >> 6;
         // BF16x3 A (warps 0-3): this thread's row, its warp's TMEM lane
         // quadrant
-        const bool awriter = PREC == 2 && warp < NAW / 32;
+        const bool awriter = ASPLIT && warp < NAW / 32;
         const int arow = 32 * (warp & 3) + lane;
         const uint32_t ta_row = tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(TM_A);
         // one chunk of A from the TMA slot into TMEM stage `stage` (both K
         // steps); the slot is released once read (rel: its barrier, or null)
+        float sa = 1.f;  // FP16x3: the tile's A scale
         auto a_to_tmem = [&](const uint8_t *slot, int stage, uint64_t *rel) {
             const uint32_t ta = ta_row + uint32_t(stage * TM_ASTAGE);
-            split_a_quarter(slot, arow, 0, ta);
-            split_a_quarter(slot, arow, 1, ta);
-            split_a_quarter(slot, arow, 2, ta);
-            split_a_quarter(slot, arow, 3, ta);
+            split_a_quarter<PREC>(slot, arow, 0, ta, sa);
+            split_a_quarter<PREC>(slot, arow, 1, ta, sa);
+            split_a_quarter<PREC>(slot, arow, 2, ta, sa);
+            split_a_quarter<PREC>(slot, arow, 3, ta, sa);
             if (rel) mbar_arrive(rel);
         };
         // loop exits and waits are made warp-uniform: the TMEM stores below
@@ -1012,6 +1063,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
             const int nts = BPACK ? nrs : NTS;
             bool ok = true;
             for (int64_t l = 0; l < my_tiles && ok && !aborted(); l += TSTEP) {
+                if (PREC == 3) {  // the tile's metadata (its slot stays until the tile is stored)
+                    if (!__all_sync(0xffffffffu, mbar_wait(&X.mfull[l % MS], uint32_t(l / MS) & 1u))) {
+                        ok = false;
+                        break;
+                    }
+                    sa = pow2f(-X.epi[l % MS].ea);
+                }
                 for (int c = 0; c < nch; ++c) {
                     // the chunk has landed and the MMAs are done with the
                     // TMEM stage's previous chunk
@@ -1178,6 +1236,59 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                 // chunks of the rings whatever its tile)
                 TileIter it;
                 if (!BPACK && my_tiles > 0) it.start(d, mtiles, n_tiles, tblk, PP);
+                if constexpr (PREC == 3) {
+                    // a unit: two chunks (K >= 32), its own accumulator of two
+                    // in turn
+                    const int64_t units = my_tiles * (nch >> 1);
+                    for (int64_t q = 0; q < units && ok && !*abort_flag; ++q) {
+                        const int acc = int(q & 1);
+                        if (!mbar_wait(&X.tempty[acc], (uint32_t(q >> 1) & 1u) ^ 1u)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint32_t dtm = tmem + uint32_t(acc) * awr, id = idesc(0u, awr);
+                        int st[2];
+                        for (int c = 0; c < 2; ++c) {
+                            st[c] = ts;
+                            if (!mbar_wait(&X.afull[ts], tph)) {
+                                ok = false;
+                                break;
+                            }
+                            if (++ts == nts) {
+                                ts = 0;
+                                tph ^= 1u;
+                            }
+                        }
+                        if (!ok) break;
+                        tc_fence_after();
+                        // hi lo and lo hi of both chunks first, then hi hi
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+#pragma unroll
+                            for (int c = 0; c < 2; ++c) {
+                                const uint32_t a0 = tmem + uint32_t(TM_A + st[c] * TM_ASTAGE);
+                                const uint32_t b0 = smem_u32(sm + C::OFF_RAW + (PACK_ST + st[c]) * C::SLOT_RAW);
+                                const uint32_t bl = b0 + TBNR * TBKR * 2;
+#pragma unroll
+                                for (int j = 0; j < TBKR / 16; ++j) {
+                                    const uint32_t off = uint32_t(2 * j) * LBO;
+                                    const uint32_t ah = a0 + uint32_t(16 * j), al = ah + 8u;
+                                    if (h == 0) {
+                                        mma_f16_ts(dtm, ah, sdesc(bl + off, LBO, SBO), id, (c > 0 || j > 0) ? 1u : 0u);
+                                        mma_f16_ts(dtm, al, sdesc(b0 + off, LBO, SBO), id, 1u);
+                                    } else {
+                                        mma_f16_ts(dtm, ah, sdesc(b0 + off, LBO, SBO), id, 1u);
+                                    }
+                                }
+                            }
+                        for (int c = 0; c < 2; ++c) {
+                            mma_commit(&X.taempty[st[c]]);
+                            mma_commit(&X.rempty[st[c]]);
+                        }
+                        mma_commit(&X.tfull[acc]);
+                    }
+                } else
                 for (int64_t l = 0; l < my_tiles && ok && !*abort_flag; l += TSTEP) {
                     int4 r = make_int4(0, 0, 0, 0);
                     int64_t g = 0;
@@ -1208,7 +1319,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                     const int ctl = (MODE == 2 || d.sched != 0) ? 0 : r.w / TBN;  // the tile's column tile within the resident B
                     const uint32_t bset = smem_u32(sm + C::OFF_RAW + (nrs + ctl * nch) * C::SLOT_RAW);
                     for (int c = 0; c < nch; ++c) {
-                        if (!mbar_wait(PREC == 2 ? &X.afull[ts] : &X.rfull[rs], PREC == 2 ? tph : rph)) {
+                        if (!mbar_wait(ASPLIT ? &X.afull[ts] : &X.rfull[rs], ASPLIT ? tph : rph)) {
                             ok = false;
                             break;
                         }
@@ -1220,7 +1331,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                             issue_pair(dtm, a_of(rs, ts), bch, c == 0);
                         else
                             issue_chunk(dtm, a_of(rs, ts), bch, c == 0);
-                        if (PREC == 2) mma_commit(&X.taempty[ts]);
+                        if (ASPLIT) mma_commit(&X.taempty[ts]);
                         if (PREC == 1 || BPACK) mma_commit(&X.rempty[rs]);
                         if (++rs == nrs) {
                             rs = 0;
@@ -1340,7 +1451,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                 const int inst = inst_c[q];
                 em.inst[c] = inst;
                 em.mx[c] = 0u;
-                em.sc[c] = pow2f(-(ea_c + (MODE >= 2 ? 0 : eb_c[q])));  // dictionary and packed B carry 2^-eb
+                // dictionary and packed B carry 2^-eb, FP16x3 A 2^-ea as well
+                em.sc[c] = PREC == 3 ? HALF_UNSCALE : pow2f(-(ea_c + (MODE >= 2 ? 0 : eb_c[q])));
                 if (MODE == 2) em.acol[c] = int16_t(inst >= 0 ? (ib_c[q] << d.nb) + ((w_c + c) & (N - 1)) : 0);
                 if (inst >= 0 && it.mt == 0 && ((int64_t(w_c) + c) & (N - 1)) == 0)
                     d.EC[inst] = EA_c + ea_c + EB_c[q] + eb_c[q];
@@ -1348,6 +1460,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
             if (lane == 0) {
                 em.base = base_c + dep(it.mt * TBM, d.pCm, d.mb);
                 em.ncv = ncv_c;
+                em.ea = ea_c;
             }
             mbar_arrive(&X.mfull[slot]);  // every lane (count 32): its writes are released
         }
@@ -1413,7 +1526,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
         for (int64_t l = narrow ? sub : 0; l < my_tiles; l += narrow ? 2 : 1) {
             const int acc = int(l & (nacc - 1)), slot = int(l % MS);
             bool w = mbar_wait(&X.mfull[slot], uint32_t(l / MS) & 1u);
-            w = w && mbar_wait(&X.tfull[acc], uint32_t(l >> nacc_sh) & 1u);
+            if (PREC != 3) w = w && mbar_wait(&X.tfull[acc], uint32_t(l >> nacc_sh) & 1u);
             if (!__all_sync(0xffffffffu, w) || __any_sync(0xffffffffu, *abort_flag != 0)) {
                 give_up();
                 break;
@@ -1425,16 +1538,55 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
             // halves of 8 columns this warp reads from the accumulator
             // (non-dictionary tiles of 8 columns: one)
             const int npass = (MODE != 2 && acw < 16) ? 1 : 2;
-            for (int h = 0; h < nh; ++h) {
+            constexpr int HALVES = PREC == 3 ? 2 : 1;
+            uint32_t sum[HALVES][32];  // FP16x3: the tile's sums (float bits)
+            if constexpr (PREC == 3) {
+#pragma unroll
+                for (int i = 0; i < 64; ++i) sum[i >> 5][i & 31] = 0u;
+                const int nu = nch >> 1;
+                for (int u = 0; u < nu; ++u) {
+                    const int64_t q = l * nu + u;
+                    const int ua = int(q & 1);
+                    if (!__all_sync(0xffffffffu, mbar_wait(&X.tfull[ua], uint32_t(q >> 1) & 1u))) {
+                        w = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    if (rows_ok) {
+                        const uint32_t ta = tmem + uint32_t(ua) * awr + uint32_t(sub * 32) + (uint32_t(lanegrp * 32) << 16);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                            for (int c = 0; c < 2; ++c) {
+                                uint32_t v[16];
+                                tmem_ld<16>(ta + uint32_t(64 * h + 16 * c), v);
+                                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                                for (int i = 0; i < 16; ++i)
+                                    sum[h][16 * c + i] =
+                                        __float_as_uint(__uint_as_float(sum[h][16 * c + i]) + __uint_as_float(v[i]));
+                            }
+                        }
+                    }
+                    tc_fence_before();
+                    mbar_arrive(&X.tempty[ua]);
+                }
+                if (!w) {
+                    give_up();
+                    break;
+                }
+            }
+#pragma unroll HALVES
+            for (int h = 0; h < (PREC == 3 ? HALVES : nh); ++h) {
                 const int c0 = narrow ? 0 : h * 32 + sub * 16;  // first column of this warp's block
                 const bool act = rows_ok && c0 < ncv;  // warp-uniform
                 // the block's complex columns (16, or 8 where no tile has
                 // more: NC), every load issued before one wait
-                auto block = [&](auto nc_) {
+                auto block = [&](auto nc_, const uint32_t (&sums)[32]) {
                     constexpr int NC = decltype(nc_)::value;
                     uint32_t r[32];
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) r[q] = 0u;
+                    for (int q = 0; q < 32; ++q) r[q] = PREC == 3 ? sums[q] : 0u;
                     if (act && MODE == 2) {
                         const uint32_t tb = tmem + uint32_t(acc) * awr + (uint32_t(lanegrp * 32) << 16);
                         switch (N < NC ? N : NC) {
@@ -1444,14 +1596,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                             case 8: tmem_gather16<NC, 8>(r, tb, em, c0, ncv); break;
                             default: tmem_gather16<NC, NC>(r, tb, em, c0, ncv); break;
                         }
-                    } else if (act) {
+                    } else if (act && PREC != 3) {
                         const uint32_t ta =
                             tmem + uint32_t(acc) * awr + uint32_t(c0 * 2) + (uint32_t(lanegrp * 32) << 16);
                         if (NC == 16 && npass == 2) tmem_ld<16>(ta + 16u, r + 16);
                         tmem_ld<16>(ta, r);
                         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     }
-                    if (h == nh - 1) {  // the accumulator is free for a later tile
+                    if (PREC != 3 && h == nh - 1) {  // the accumulator is free for a later tile
                         tc_fence_before();
                         mbar_arrive(&X.tempty[acc]);
                     }
@@ -1516,10 +1668,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                         }
                     }
                 };
-                if (ow <= 8)
-                    block(std::integral_constant<int, 8>());
+                if (PREC != 3 && ow <= 8)
+                    block(std::integral_constant<int, 8>(), sum[0]);
                 else
-                    block(std::integral_constant<int, 16>());
+                    block(std::integral_constant<int, 16>(), sum[PREC == 3 ? h : 0]);
                 if (!act || direct || rowst) continue;
                 const int ncw = ncv - c0;  // valid columns of this block
                 __syncwarp();
@@ -1577,6 +1729,7 @@ __global__ void __launch_bounds__(256) k_pack_b(const StepDesc d, int nch) {
     const int K = 1 << d.kb;
     const int k = c * TBK + 4 * kqb;
     const float s = d.mxB ? pow2f(-exp_of(__ldg(d.mxB + ib))) : 1.f;
+    constexpr float t = PREC == 3 ? HALF_TOP : 1.f;
     float4 p0 = make_float4(0.f, 0.f, 0.f, 0.f), p1 = p0;
     if (k + 3 < K) {
         const float4 *src = reinterpret_cast<const float4 *>(d.B + ib * d.sB + (n << d.kb) + k);
@@ -1584,8 +1737,8 @@ __global__ void __launch_bounds__(256) k_pack_b(const StepDesc d, int nch) {
         p1 = __ldg(src + 1);
     }
     expand_b<PREC, RM>(d.bpack + blk * (TBNR * TBKR * 4), bcol, kqb,
-                   make_float4(p0.x * s, p0.y * s, p0.z * s, p0.w * s),
-                   make_float4(p1.x * s, p1.y * s, p1.z * s, p1.w * s));
+                   make_float4(p0.x * s * t, p0.y * s * t, p0.z * s * t, p0.w * s * t),
+                   make_float4(p1.x * s * t, p1.y * s * t, p1.z * s * t, p1.w * s * t));
 }
 
 // Packed B for column-tile pairs (MODE 4): 128 columns x 16 complex k per
@@ -1628,6 +1781,14 @@ int64_t tc_packed_b_bytes(const StepDesc &d) {
 bool gemm_tc_supports(const StepDesc &d) {
     // K >= 8 complex (at least half a chunk), 64 <= M < 2^31 rows
     return d.kb >= 3 && d.mb >= 6 && d.mb <= 30 && d.kb <= 24;
+}
+
+bool tc_fp32_takes(const StepDesc &d) {
+    // K >= 128: below, the FMA kernel's rounding (7.3e-8 at 128 real k) is
+    // less than the split's and a unit's.  A packed tile's 64 columns lie in
+    // one B instance
+    return d.sched == 0 && d.tc_resident_b && d.kb >= 7 && d.nb >= 6 && gemm_tc_supports(d) && d.mxA && d.mxB &&
+           d.bpack && tc_packed_b_bytes(d) <= d.bpack_bytes;
 }
 
 int tc_dictionary_chunks(const StepDesc &d) {
@@ -1683,6 +1844,9 @@ cudaError_t init_kernels() {
     e = cudaFuncSetAttribute(reinterpret_cast<const void *>(k_step_gemm_tc<2, 4>),
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<2, true>());
     if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(reinterpret_cast<const void *>(k_step_gemm_tc<3, 3>),
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<3, true>());
+    if (e != cudaSuccess) return e;
     const void *fns[8] = {reinterpret_cast<const void *>(k_step_gemm_tc<1, 0>),
                           reinterpret_cast<const void *>(k_step_gemm_tc<2, 0>),
                           reinterpret_cast<const void *>(k_step_gemm_tc<1, 1>),
@@ -1729,6 +1893,17 @@ cudaError_t launch_step_gemm_tc(const StepDesc &d, const CUtensorMap *a_map, int
     if (tiles <= 0) return cudaSuccess;
     const int64_t grid = tiles < g_num_sms ? tiles : g_num_sms;
     const dim3 g((unsigned)grid);
+    if (precision == 0) {
+        if (!tc_fp32_takes(d)) return cudaErrorNotSupported;
+        const int nch = 1 << (d.kb - 4);
+        const int64_t blocks = (d.packBn * nch) << (d.nb - 6);
+        const int64_t b = ((int64_t(d.max_group) << d.nb) + TBN - 1) / TBN;  // a row tile's column tiles
+        if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+        k_pack_b<3><<<dim3((unsigned)blocks), 256, 0, s>>>(d, nch);
+        k_step_gemm_tc<3, 3><<<g, NTHREADS, smem_bytes<3, true>(), s>>>(
+            d, mtiles, err, *a_map, PACK_ST, TBN, TBN, b >= 1 && b * grid * 2 <= tiles ? int(b) : 0);
+        return cudaGetLastError();
+    }
     // B as a dictionary (every instance resident for the launch), else
     // resident per group or column tile when it fits the pool, else streamed
     const int ndict = tc_dictionary_chunks(d);

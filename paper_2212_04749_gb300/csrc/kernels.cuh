@@ -118,6 +118,7 @@ int tc_resident_b_chunks(const StepDesc &d);
 // count, else 0.
 int tc_dictionary_chunks(const StepDesc &d);
 // The schedule of a tensor-core step for which none was chosen.
+bool tc_fp32_takes(const StepDesc &d);
 int tc_rule_schedule(const StepDesc &d);
 // Bytes of the packed-B form of a step (every B instance in the MMA layout,
 // 16 KB per 64 columns x 16 complex k), 0 if the step cannot take it.
