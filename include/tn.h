@@ -312,9 +312,9 @@ int tn_plan_set_kernel(tn_plan_t plan, int32_t step, int32_t kernel);
  *   3  grouped GEMM, the other walk order
  * The GEMM runs on the tensor cores for TN_TF32 / TN_BF16X3 where the shape
  * allows (K >= 8, 64 <= M < 2^31), on the CUDA cores otherwise.  For TN_FP32
- * configuration 2 takes the tensor cores as well where a step has K >= 128,
- * N >= 64, 64 <= M < 2^31, maxima for both operands (tn_options.rescale, no
- * leaf) and room for its packed B: each operand instance scaled by a power of
+ * configuration 2 takes the tensor cores as well where a step has K >= 64,
+ * 64 <= M < 2^31, N >= 64 or groups of 32 columns on average, maxima for both
+ * operands (tn_options.rescale, no leaf) and room for its packed B: each operand instance scaled by a power of
  * two and split into two fp16 halves (22 bits of each value down to 2^-18 of
  * the instance's largest), three products, units of 64 real k summed in
  * FP32 registers.  Configuration 3 and tn_plan_set_tc_resident_b(plan, 0)

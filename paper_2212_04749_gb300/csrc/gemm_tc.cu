@@ -45,6 +45,7 @@
 #include <cuda_fp16.h>
 
 #include "kernels.cuh"
+#include "plan.hpp"
 
 namespace tnk {
 
@@ -754,6 +755,9 @@ __device__ __forceinline__ void fold_max16(const uint32_t (&r)[32], EpiMeta &em,
     }
 }
 
+// FP16x3: chunks of a unit
+__host__ __device__ __forceinline__ int unit_chunks(const StepDesc &d) { return d.kb >= 7 ? 2 : 1; }
+
 template <int PREC, int MODE>
 __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 warps on a sub-partition)
     k_step_gemm_tc(const __grid_constant__ StepDesc d, int64_t mtiles, int32_t *err, const __grid_constant__ CUtensorMap tmA, int nrs,
@@ -777,11 +781,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
     // two and split into fp16 halves.  The tensor cores truncate each sum into
     // the accumulator (relative L2 error 1.0e-6 over 1024 real k of random
     // signs, the FMA kernel 2.5e-7; 6.5e-8 over 64), so a unit of two chunks
-    // (64 real k) starts from zero, its small products first, and the epilogue
-    // adds the units in FP32 registers, rounded to nearest: the contraction's
-    // error is 3 to 42 % below the FMA kernel's.  Bound by the loads of A and B
-    // from L2 and the tensor cores together.  53-qubit circuit, FP32: 2^12 x
-    // 2^9 x 2^8 with 512 instances 48 -> 7.3 ms, all of it 228 -> 68 ms.
+    // (64 real k; K = 64: one chunk) starts from zero, its small products
+    // first, and the epilogue adds the units in FP32 registers, rounded to
+    // nearest: the contraction's error is 3 to 43 % below the FMA kernel's.
+    // Bound by the loads of A and B from L2 and the tensor cores together.
+    // 53-qubit circuit, FP32: 2^12 x 2^9 x 2^8 with 512 instances 48 -> 7.5 ms,
+    // all of it 228 -> 49 ms.
     constexpr int EPI_REGS = epi_regs(PREC);
     constexpr bool ASPLIT = PREC >= 2;  // A split into TMEM
     static_assert(PREC != 3 || MODE == 3, "FP16x3: packed B");
@@ -948,7 +953,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                 if (BPACK && (it.f != fprev || it.ct != ctprev)) {
                     const int64_t i0 = int64_t(r.x) + (r.w >> d.nb);
                     const int ib = __ldg(d.instab + i0).y;
-                    if (PP) {
+                    if (PREC == 3 && d.nb < 6) {  // packed per column tile
+                        bsrc = d.bpack + (it.f + it.ct) * nch * int64_t(C::SLOT_B);
+                    } else if (PP) {
                         // N = 64: tile ct is instance ct of the group; the
                         // pad tile (odd groups) repeats the first tile's B
                         const int ib1 = it.ct + 1 < it.nct ? __ldg(d.instab + i0 + 1).y : ib;
@@ -1239,7 +1246,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                 if constexpr (PREC == 3) {
                     // a unit: two chunks (K >= 32), its own accumulator of two
                     // in turn
-                    const int64_t units = my_tiles * (nch >> 1);
+                    const int uc = unit_chunks(d);
+                    const int64_t units = my_tiles * (nch / uc);
                     for (int64_t q = 0; q < units && ok && !*abort_flag; ++q) {
                         const int acc = int(q & 1);
                         if (!mbar_wait(&X.tempty[acc], (uint32_t(q >> 1) & 1u) ^ 1u)) {
@@ -1249,7 +1257,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                         tc_fence_after();
                         const uint32_t dtm = tmem + uint32_t(acc) * awr, id = idesc(0u, awr);
                         int st[2];
-                        for (int c = 0; c < 2; ++c) {
+                        for (int c = 0; c < uc; ++c) {
                             st[c] = ts;
                             if (!mbar_wait(&X.afull[ts], tph)) {
                                 ok = false;
@@ -1267,6 +1275,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                         for (int h = 0; h < 2; ++h)
 #pragma unroll
                             for (int c = 0; c < 2; ++c) {
+                                if (c >= uc) break;
                                 const uint32_t a0 = tmem + uint32_t(TM_A + st[c] * TM_ASTAGE);
                                 const uint32_t b0 = smem_u32(sm + C::OFF_RAW + (PACK_ST + st[c]) * C::SLOT_RAW);
                                 const uint32_t bl = b0 + TBNR * TBKR * 2;
@@ -1282,7 +1291,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                                     }
                                 }
                             }
-                        for (int c = 0; c < 2; ++c) {
+                        for (int c = 0; c < uc; ++c) {
                             mma_commit(&X.taempty[st[c]]);
                             mma_commit(&X.rempty[st[c]]);
                         }
@@ -1543,7 +1552,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
             if constexpr (PREC == 3) {
 #pragma unroll
                 for (int i = 0; i < 64; ++i) sum[i >> 5][i & 31] = 0u;
-                const int nu = nch >> 1;
+                const int nu = nch / unit_chunks(d);
                 for (int u = 0; u < nu; ++u) {
                     const int64_t q = l * nu + u;
                     const int ua = int(q & 1);
@@ -1741,6 +1750,27 @@ __global__ void __launch_bounds__(256) k_pack_b(const StepDesc d, int nch) {
                    make_float4(p1.x * s * t, p1.y * s * t, p1.z * s * t, p1.w * s * t));
 }
 
+// Packed B of steps with N < 64 (FP16x3): the columns of a column tile are
+// those of several instances of its group; block tile * nch + chunk.
+__global__ void __launch_bounds__(256) k_pack_b_tiles(const StepDesc d, int nch) {
+    const int tid = threadIdx.x, bcol = tid & 63, kqb = tid >> 6;
+    const int c = int(blockIdx.x % nch);
+    const int4 r = __ldg(d.trec + blockIdx.x / nch);
+    const int64_t gc = int64_t(r.w) + bcol;
+    float4 p0 = make_float4(0.f, 0.f, 0.f, 0.f), p1 = p0;
+    if (gc < (int64_t(r.y) << d.nb)) {
+        const int ib = __ldg(d.instab + r.x + (gc >> d.nb)).y;
+        const float s = pow2f(-exp_of(__ldg(d.mxB + ib)));
+        const float4 *src = reinterpret_cast<const float4 *>(
+            d.B + ib * d.sB + ((gc & ((1 << d.nb) - 1)) << d.kb) + c * TBK + 4 * kqb);
+        p0 = __ldg(src);
+        p1 = __ldg(src + 1);
+        p0 = make_float4(p0.x * s * HALF_TOP, p0.y * s * HALF_TOP, p0.z * s * HALF_TOP, p0.w * s * HALF_TOP);
+        p1 = make_float4(p1.x * s * HALF_TOP, p1.y * s * HALF_TOP, p1.z * s * HALF_TOP, p1.w * s * HALF_TOP);
+    }
+    expand_b<3>(d.bpack + int64_t(blockIdx.x) * (TBNR * TBKR * 4), bcol, kqb, p0, p1);
+}
+
 // Packed B for column-tile pairs (MODE 4): 128 columns x 16 complex k per
 // 32 KB block (block (ib * N/128 + pair) * nch + chunk) in the layout of a
 // B operand of 256 rows; thread (column, k quad) expands columns c and
@@ -1784,11 +1814,17 @@ bool gemm_tc_supports(const StepDesc &d) {
 }
 
 bool tc_fp32_takes(const StepDesc &d) {
-    // K >= 128: below, the FMA kernel's rounding (7.3e-8 at 128 real k) is
-    // less than the split's and a unit's.  A packed tile's 64 columns lie in
-    // one B instance
-    return d.sched == 0 && d.tc_resident_b && d.kb >= 7 && d.nb >= 6 && gemm_tc_supports(d) && d.mxA && d.mxB &&
-           d.bpack && tc_packed_b_bytes(d) <= d.bpack_bytes;
+    // K >= 64: below, the FMA kernel's rounding (5.1e-8 over 64 real k) is
+    // less than the split's and a unit's.  N < 64: several instances' columns
+    // share a tile, half of it at least on average.  Any number of tiles: one
+    // instance of 2^9 x 64 x 2^7 takes 24.7 us with its B's packing, 26.6 on
+    // the FMA kernel, 2^16 x 64 x 64 36.7 and 81.8
+    if (d.sched != 0 || !d.tc_resident_b || d.kb < tnp::TC_FP32_MIN_KB || !gemm_tc_supports(d) || !d.mxA ||
+        !d.mxB || !d.bpack)
+        return false;
+    if (d.nb >= 6) return tc_packed_b_bytes(d) <= d.bpack_bytes;
+    return (d.nInst << d.nb) >= 32 * d.n_groups &&
+           ((d.n_ctab << (d.kb - 4)) * int64_t(TBNR * TBKR * 4)) <= d.bpack_bytes;
 }
 
 int tc_dictionary_chunks(const StepDesc &d) {
@@ -1896,12 +1932,18 @@ cudaError_t launch_step_gemm_tc(const StepDesc &d, const CUtensorMap *a_map, int
     if (precision == 0) {
         if (!tc_fp32_takes(d)) return cudaErrorNotSupported;
         const int nch = 1 << (d.kb - 4);
-        const int64_t blocks = (d.packBn * nch) << (d.nb - 6);
-        const int64_t b = ((int64_t(d.max_group) << d.nb) + TBN - 1) / TBN;  // a row tile's column tiles
+        const int64_t blocks = d.nb >= 6 ? (d.packBn * nch) << (d.nb - 6) : d.n_ctab * nch;
+        // column tiles dealt in twos: the CTAs that walk one row tile run side
+        // by side, and their A and B at any time fit L2 (a row tile's column
+        // tiles per CTA: 11.2 against 8.3 ms on 2^10 x 2^9 x 64, groups of 32)
+        const int64_t b = ((int64_t(d.max_group) << d.nb) + TBN - 1) / TBN;
         if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-        k_pack_b<3><<<dim3((unsigned)blocks), 256, 0, s>>>(d, nch);
+        if (d.nb >= 6)
+            k_pack_b<3><<<dim3((unsigned)blocks), 256, 0, s>>>(d, nch);
+        else
+            k_pack_b_tiles<<<dim3((unsigned)blocks), 256, 0, s>>>(d, nch);
         k_step_gemm_tc<3, 3><<<g, NTHREADS, smem_bytes<3, true>(), s>>>(
-            d, mtiles, err, *a_map, PACK_ST, TBN, TBN, b >= 1 && b * grid * 2 <= tiles ? int(b) : 0);
+            d, mtiles, err, *a_map, PACK_ST, TBN, TBN, b >= 2 ? 2 : 1);
         return cudaGetLastError();
     }
     // B as a dictionary (every instance resident for the launch), else

@@ -658,6 +658,13 @@ struct Builder {
         }
     }
 
+    // FP32 steps that pack B per column tile (gemm_tc.cu): N < 64, wide groups
+    bool packs_tiles(const Step &st) const {
+        return st.nb < 6 && st.kb >= TC_FP32_MIN_KB && st.kb <= 24 && st.mb >= 6 && st.mb <= 30 &&
+               (P.nodes[st.node].n_inst << st.nb) >= 32 * int64_t(st.n_groups);
+    }
+    bool pack_tiles = false;  // room for them
+
     // Workspace layout; returns total bytes.  own_slots: the outputs of small
     // steps share no memory with other intermediates.
     int64_t layout_workspace(bool emit, bool own_slots = false) {
@@ -892,6 +899,12 @@ struct Builder {
             const int64_t bytes = p.nodes[st.b].n_inst * (int64_t(1) << (st.nb - 6)) * nch * 16384;
             if (bytes <= bpack_cap) p.bpack_bytes = std::max(p.bpack_bytes, bytes);
         }
+        if (pack_tiles)  // N < 64: packed per column tile (FP32 steps)
+            for (const Step &st : p.steps) {
+                if (!packs_tiles(st)) continue;
+                const int64_t bytes = int64_t(st.col_tiles.size()) * (int64_t(1) << (st.kb - 4)) * 16384;
+                if (bytes <= bpack_cap) p.bpack_bytes = std::max(p.bpack_bytes, bytes);
+            }
         p.off_bpack = p.bpack_bytes > 0 ? take(p.bpack_bytes) : -1;
         for (Chain &c : p.chains) {
             const Step &last = p.steps[c.steps.back()];
@@ -1325,6 +1338,14 @@ bool make_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int
     if (!P.chains.empty()) {
         const int64_t with = layout(false, false);
         if (!P.opt.fuse && crosses(plain, with)) B.drop_chains();
+        else plain = with;
+    }
+    // room for B packed per column tile: the same
+    if (P.opt.rescale)
+        for (const Step &st : P.steps) B.pack_tiles = B.pack_tiles || B.packs_tiles(st);
+    if (B.pack_tiles) {
+        const int64_t with = layout(false, false);
+        if (crosses(plain, with)) B.pack_tiles = false;
         else plain = with;
     }
     int64_t slots = 0;

@@ -127,6 +127,9 @@ constexpr int64_t SMALL_DESC_BYTES = 160;
 // one still in use, where these slots add little to the workspace.
 constexpr int64_t SMALL_SLOTS_MAX = int64_t(32) << 20;
 
+// FP32 steps take the tensor cores (FP16x3, gemm_tc.cu) from K = 2^this on.
+constexpr int TC_FP32_MIN_KB = 6;
+
 // A fused chain (SM Sec. V.C): steps s_1..s_L where each step's A operand is
 // the previous step's output, instance counts do not grow, and every side
 // operand B_j is small.  It runs as one kernel at s_L: per output instance
