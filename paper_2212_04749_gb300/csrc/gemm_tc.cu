@@ -2009,9 +2009,11 @@ cudaError_t launch_step_gemm_tc(const StepDesc &d, const CUtensorMap *a_map, int
             k_step_gemm_tc<1, 3><<<g, NTHREADS, smem_bytes<1, true>(), s>>>(d, mtiles, err, *a_map, PACK_ST, acw, ow,
                                                                             block_of());
         } else {
+            // schedule 0: a row tile's column tiles dealt in twos, so that the
+            // CTAs of one row tile run side by side (as for the pairs above)
             k_pack_b<2><<<dim3((unsigned)blocks), 256, 0, s>>>(d, nch);
             k_step_gemm_tc<2, 3><<<g, NTHREADS, smem_bytes<2, true>(), s>>>(d, mtiles, err, *a_map, PACK_ST, acw, ow,
-                                                                            block_of());
+                                                                            d.sched ? block_of() : 2);
         }
         return cudaGetLastError();
     }
