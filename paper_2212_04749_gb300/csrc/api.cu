@@ -358,11 +358,24 @@ int run_step(PlanObj *o, int s, int precision, int64_t sigma, cudaStream_t st) {
     } else if (precision != TN_FP32 && tnk::gemm_tc_supports(d)) {
         fam = 2;
         if (!(s < (int)o->config_override.size() && o->config_override[s] >= 0)) d.sched = tnk::tc_rule_schedule(d);
-        e = o->amap[s].ok ? tnk::launch_step_gemm_tc(d, &o->amap[s].map, precision, o->err_flag, st)
-                          : cudaErrorInvalidValue;  // its TMA descriptor could not be encoded
+        if (d.tc_resident_b && tnk::tc_dictionary_chunks(d) == 0 && tnk::tc_resident_b_chunks(d) == 0 &&
+            tnk::step_narrow_takes(d, false)) {
+            fam = 1;
+            e = tnk::launch_step_narrow(d, st);
+        } else if (o->amap[s].ok) {
+            e = tnk::launch_step_gemm_tc(d, &o->amap[s].map, precision, o->err_flag, st);
+        } else {
+            e = cudaErrorInvalidValue;  // its TMA descriptor could not be encoded
+        }
     } else if (precision == TN_FP32 && o->amap[s].ok && tnk::tc_fp32_takes(d)) {
         fam = 2;
         e = tnk::launch_step_gemm_tc(d, &o->amap[s].map, precision, o->err_flag, st);
+    } else if (tnk::step_outer_takes(d)) {
+        fam = 1;
+        e = tnk::launch_step_outer(d, st);
+    } else if (tnk::step_narrow_takes(d, true)) {
+        fam = 1;
+        e = tnk::launch_step_narrow(d, st);
     } else {
         fam = 1;
         e = tnk::launch_step_gemm_simt(d, st);

@@ -675,6 +675,107 @@ __global__ void __launch_bounds__(128) k_step_gemm_simt2(const StepDesc d, int c
     }
 }
 
+// Steps with a short row and many columns (K <= 32, N >= 32, M >= 32; reached
+// by FP32 steps and, K <= 4, by those that the tensor cores do not take):
+// nearly all of their bytes are C's.  A block takes a column tile (64 columns, B in
+// shared memory) and 256 RX `passes` rows; a thread holds RX rows of A in
+// registers and walks the columns, B's entries as broadcasts, so that a
+// warp's 32 rows, neighbours in C where the layout allows, are stored by one
+// instruction.  Bound by HBM (C), from K = 16 on by the FMA rate.  The GEMM
+// kernel stages 16 k a chunk, stores 16 rows an instruction and pads 32
+// columns to 64: 7.36 ms for 2^15 x 4 x 32 with 1024 instances (9.7 GB, 1.43
+// ms), 1.69 here; 2^10 x 32 x 32 with 8192 (1.1 ms of FMA) and 2^14 x 16 x 32
+// with 256 together 5.7, 2.2 here.
+// (rlog: log2 of the rows side by side, min(M, 256); the block's other
+// threads take other columns.)
+template <int KB, int RX>
+__global__ void __launch_bounds__(256) k_step_outer(const StepDesc d, int rlog, int passes, int mtiles) {
+    constexpr int K = 1 << KB;
+    __shared__ __align__(16) float2 s_b[64 * K];
+    __shared__ int64_t s_cbase[64];
+    __shared__ float s_sc[64];
+    __shared__ uint32_t s_mx[64];
+    __shared__ int8_t s_pCm[40];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int mt = int(blockIdx.x % mtiles);
+    // {first instance, count, A instance, first column} of 64 columns
+    const int4 rec = __ldg(d.trec + blockIdx.x / mtiles);
+    const int N = 1 << d.nb;
+    const int ncols = int(min((int64_t(rec.y) << d.nb) - rec.w, int64_t(64)));
+    if (tid < 40) s_pCm[tid] = d.pCm[tid];
+    if (tid < 64) {
+        s_mx[tid] = 0u;
+        if (tid < ncols) {
+            const int64_t inst = rec.x + ((int64_t(rec.w) + tid) >> d.nb);
+            const int n = (rec.w + tid) & (N - 1);
+            const int ib = d.instab[inst].y;
+            const int ea = d.mxA ? exp_of(d.mxA[rec.z]) : 0, eb = d.mxB ? exp_of(d.mxB[ib]) : 0;
+            s_cbase[tid] = inst * d.sC + dep(n, d.pCn, d.nb);
+            s_sc[tid] = pow2f(-(ea + eb));
+            if (n == 0 && mt == 0) d.EC[inst] = d.EA[rec.z] + ea + d.EB[ib] + eb;
+        }
+    }
+    for (int e = tid; e < ncols * K; e += 256) {
+        const int64_t gc = int64_t(rec.w) + (e >> KB);
+        const int ib = d.instab[rec.x + (gc >> d.nb)].y;
+        s_b[e] = __ldg(d.B + int64_t(ib) * d.sB + ((gc & (N - 1)) << KB) + (e & (K - 1)));
+    }
+    __syncthreads();
+    const int R = 1 << rlog, cw = 64 >> (8 - rlog);
+    const int c0 = (tid >> rlog) * cw, c1 = min(c0 + cw, ncols);  // the same for a warp
+    const int run = N < 64 ? N - 1 : 63;                          // columns of an instance in the tile, less one
+    const float2 *A = d.A + int64_t(rec.z) * d.sA;
+    const int64_t m0 = int64_t(mt) * passes * (RX << rlog) + (tid & (R - 1));
+    for (int p = 0; p < passes; ++p) {
+        float2 a[RX][K];
+        float2 *C[RX];
+#pragma unroll
+        for (int x = 0; x < RX; ++x) {
+            const int64_t m = m0 + (int64_t(p * RX + x) << rlog);
+            if (KB == 0) {
+                a[x][0] = __ldg(A + m);
+            } else {
+#pragma unroll
+                for (int k = 0; k < K; k += 2) {
+                    const float4 v = __ldg(reinterpret_cast<const float4 *>(A + (m << KB) + k));
+                    a[x][k] = make_float2(v.x, v.y);
+                    a[x][k + (KB > 0)] = make_float2(v.z, v.w);
+                }
+            }
+            C[x] = d.C + dep(m, s_pCm, d.mb);
+        }
+        uint32_t mx = 0u;
+        for (int c = c0; c < c1; ++c) {
+            float2 acc[RX];
+#pragma unroll
+            for (int x = 0; x < RX; ++x) acc[x] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const float2 b = s_b[(c << KB) + k];
+#pragma unroll
+                for (int x = 0; x < RX; ++x) cfma(acc[x], a[x][k], b);
+            }
+            const float sc = s_sc[c];
+            const int64_t off = s_cbase[c];
+#pragma unroll
+            for (int x = 0; x < RX; ++x) {
+                const float2 v = make_float2(acc[x].x * sc, acc[x].y * sc);
+                C[x][off] = v;
+                mx = max(mx, absmax_bits(v));
+            }
+            if (d.mxC && (((c & run) == run) || c + 1 == c1)) {  // the instance's last column here
+                mx = __reduce_max_sync(0xffffffffu, mx);
+                if (lane == 0 && mx) atomicMax(&s_mx[c & ~run], mx);
+                mx = 0u;
+            }
+        }
+    }
+    if (d.mxC) {
+        __syncthreads();
+        if (tid < ncols && s_mx[tid]) record_max(d.mxC + rec.x + ((int64_t(rec.w) + tid) >> d.nb), s_mx[tid]);
+    }
+}
+
 // Steps with a long row and few columns per A instance (K >= 32, K N <= 256,
 // M >= 128), grouped: a block takes 128 rows of a group's A instance and all
 // of the group's concatenated columns (the instances that share it), 8 or 16
@@ -1241,22 +1342,34 @@ static int row_lanes(int kb, int nb) {
     return L;
 }
 
+cudaError_t launch_step_narrow(const StepDesc &d, cudaStream_t s) {
+    auto go = [&](auto kernel, int rows, int threads, size_t smem) -> cudaError_t {
+        const int64_t mtiles = (int64_t(1) << d.mb) / rows;
+        const int64_t nblk = d.n_ctab * mtiles;
+        if (nblk <= 0) return cudaSuccess;
+        if (nblk > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+        kernel<<<dim3((unsigned)nblk), threads, smem, s>>>(d, (int)mtiles);
+        return cudaGetLastError();
+    };
+    using W = NarrowTile<1, 4, 4>;
+    using H = NarrowTile<2, 2, 2>;
+    return (d.nInst << d.nb) <= 8 * d.n_groups ? go(k_step_narrow<2, 2, 2, 6>, H::ROWS, H::THREADS, H::SMEM)
+                                               : go(k_step_narrow<1, 4, 4, 6>, W::ROWS, W::THREADS, W::SMEM);
+}
+
+bool step_narrow_takes(const StepDesc &d, bool fp32) {
+    // grouped GEMMs with few columns per A instance: a tile of 64 columns is
+    // mostly padding on the FMA kernel, and on the tensor cores, where B does
+    // not stay resident, the loads of A and B chunk by chunk set the pace
+    // (2^12 x 2^9 x 4 with 1024 A instances, 17 GB: 7.40 ms; 3.37 here).  With
+    // fewer than two blocks an SM a long K would run on a few SMs
+    return d.kb >= NARROW_MIN_KB && d.mb >= 7 && d.mb <= 40 && (d.nInst << d.nb) <= (fp32 ? 16 : 8) * d.n_groups &&
+           (d.n_ctab << (d.mb - 7)) >= 304;
+}
+
 cudaError_t launch_step_row(const StepDesc &d, cudaStream_t s) {
     if (d.kb + d.nb > 8 || d.nb > 4 || d.mb > 40) return cudaErrorInvalidValue;
-    if (d.kb >= NARROW_MIN_KB && d.mb >= 7) {
-        auto go = [&](auto kernel, int rows, int threads, size_t smem) -> cudaError_t {
-            const int64_t mtiles = (int64_t(1) << d.mb) / rows;
-            const int64_t nblk = d.n_ctab * mtiles;
-            if (nblk <= 0) return cudaSuccess;
-            if (nblk > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-            kernel<<<dim3((unsigned)nblk), threads, smem, s>>>(d, (int)mtiles);
-            return cudaGetLastError();
-        };
-        using W = NarrowTile<1, 4, 4>;
-        using H = NarrowTile<2, 2, 2>;
-        return (d.nInst << d.nb) <= 8 * d.n_groups ? go(k_step_narrow<2, 2, 2, 6>, H::ROWS, H::THREADS, H::SMEM)
-                                                   : go(k_step_narrow<1, 4, 4, 6>, W::ROWS, W::THREADS, W::SMEM);
-    }
+    if (d.kb >= NARROW_MIN_KB && d.mb >= 7) return launch_step_narrow(d, s);
     const int K = 1 << d.kb;
     const int L = row_lanes(d.kb, d.nb);
     const int R = 32 / L;
@@ -1318,6 +1431,36 @@ cudaError_t launch_step_gemm_simt(const StepDesc &d, cudaStream_t s) {
     } else {
         k_step_gemm_simt<<<dim3((unsigned)blocks), 256, 0, s>>>(d, (int)ctiles, (int)mtiles);
     }
+    return cudaGetLastError();
+}
+
+bool step_outer_takes(const StepDesc &d) { return d.kb <= 5 && d.nb >= 5 && d.mb >= 5 && d.mb <= 40; }
+
+cudaError_t launch_step_outer(const StepDesc &d, cudaStream_t s) {
+    if (!step_outer_takes(d)) return cudaErrorInvalidValue;
+    const int rlog = d.mb < 8 ? d.mb : 8, rx = d.mb >= 9 && d.kb <= 4 ? 2 : 1;
+    // up to four passes of rows for one B tile, while that leaves eight blocks an SM
+    int passes = 1;
+    const int64_t tiles = (int64_t(1) << d.mb) / (rx << rlog);
+    while (passes < 4 && passes < tiles && d.n_ctab * (tiles / (2 * passes)) >= 1216) passes *= 2;
+    const int64_t mtiles = tiles / passes, blocks = d.n_ctab * mtiles;
+    if (blocks <= 0) return cudaSuccess;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    const dim3 g((unsigned)blocks);
+#define TN_OUTER(KB_)                                                                   \
+    do {                                                                                \
+        if (rx == 2) k_step_outer<KB_, 2><<<g, 256, 0, s>>>(d, rlog, passes, (int)mtiles); \
+        else k_step_outer<KB_, 1><<<g, 256, 0, s>>>(d, rlog, passes, (int)mtiles);      \
+    } while (0)
+    switch (d.kb) {
+        case 0: TN_OUTER(0); break;
+        case 1: TN_OUTER(1); break;
+        case 2: TN_OUTER(2); break;
+        case 3: TN_OUTER(3); break;
+        case 4: TN_OUTER(4); break;
+        default: k_step_outer<5, 1><<<g, 256, 0, s>>>(d, rlog, passes, (int)mtiles); break;
+    }
+#undef TN_OUTER
     return cudaGetLastError();
 }
 

@@ -76,6 +76,15 @@ cudaError_t launch_fill(const FillJobD *jobs, int64_t njobs, const LeafHighD *hi
                         float2 *ws, cudaStream_t s);
 cudaError_t launch_step_row(const StepDesc &d, cudaStream_t s);
 cudaError_t launch_step_gemm_simt(const StepDesc &d, cudaStream_t s);
+// Steps with K <= 32, N >= 32 and M >= 32 on the grouped GEMM's configurations
+// (FP32): a thread's rows in registers against a column tile.
+bool step_outer_takes(const StepDesc &d);
+cudaError_t launch_step_outer(const StepDesc &d, cudaStream_t s);
+// Grouped GEMMs with few columns per A instance and enough blocks, on the row
+// kernel's tiles (fp32: against the FMA kernel, else against tensor-core
+// tiles that stream B).
+bool step_narrow_takes(const StepDesc &d, bool fp32);
+cudaError_t launch_step_narrow(const StepDesc &d, cudaStream_t s);
 // Steps with M N <= 32 outputs per instance, N <= 8, and K >= 64: dot
 // products of K-contiguous runs, several rows and columns per unit (FP32).
 bool step_skinny_takes(const StepDesc &d);
