@@ -1530,12 +1530,13 @@ cudaError_t launch_extract(const float2 *root, const int32_t *E, const int32_t *
 // one cluster as the whole grid, no more blocks than have work (a power of
 // two; a few thousand amplitudes stay on one SM)
 template <class... P, class... A>
-static cudaError_t launch_cluster(void (*fn)(P...), int64_t k, cudaStream_t s, A... args) {
-    cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn),
-                                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
+static cudaError_t launch_cluster(void (*fn)(P...), int64_t k, int64_t per_block, cudaStream_t s, A... args) {
     unsigned blocks = 1;
-    while (blocks < unsigned(RED_CLUSTER) && int64_t(blocks) * RED_THREADS < k) blocks <<= 1;
+    while (blocks < unsigned(RED_CLUSTER) && blocks * per_block < k) blocks <<= 1;
+    cudaError_t e = cudaSuccess;
+    if (blocks > 8)
+        e = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(RED_THREADS);
@@ -1545,18 +1546,70 @@ static cudaError_t launch_cluster(void (*fn)(P...), int64_t k, cudaStream_t s, A
     at[0].val.clusterDim.x = blocks;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = blocks > 1 ? 1 : 0;
     e = cudaLaunchKernelEx(&cfg, fn, args...);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_xeb(const double *amps, int64_t k, double scale, double *out, cudaStream_t s) {
-    return launch_cluster(k_xeb, k, s, reinterpret_cast<const double2 *>(amps), k, scale, out);
+    return launch_cluster(k_xeb, k, RED_THREADS, s, reinterpret_cast<const double2 *>(amps), k, scale, out);
+}
+
+// Batches of at most 32 completions: a row per thread, its |a|^2 in registers,
+// so neither a tile nor a second read (8 completions: 256 rows 8.2 us in tiles,
+// 4.1 here; 65536 rows of 16: 39 and 16.5, of 32: 49 and 28.9).
+template <int R>
+__global__ void __launch_bounds__(128) k_sample_rows(const double2 *__restrict__ amps, int64_t k,
+                                                     const double *__restrict__ uniform, int64_t *__restrict__ picks) {
+    constexpr int N = 1 << R, H = N < 16 ? N : 16;  // loads in flight
+    const int64_t p = int64_t(blockIdx.x) * 128 + threadIdx.x;
+    if (p >= k) return;
+    const double u = uniform[p];
+    double w[N], tot = 0.0;
+#pragma unroll
+    for (int h = 0; h < N; h += H) {
+        double2 v[H];
+#pragma unroll
+        for (int x = 0; x < H; ++x) v[x] = amps[(p << R) + h + x];
+#pragma unroll
+        for (int x = 0; x < H; ++x) {
+            w[h + x] = __dadd_rn(__dmul_rn(v[x].x, v[x].x), __dmul_rn(v[x].y, v[x].y));
+            tot = __dadd_rn(tot, w[h + x]);
+        }
+    }
+    const double thr = __dmul_rn(u, tot);
+    double c = 0.0;
+    int pick = N - 1;
+    bool open = true;
+#pragma unroll
+    for (int x = 0; x < N; ++x) {
+        c = __dadd_rn(c, w[x]);
+        if (open && c > thr) {
+            pick = x;
+            open = false;
+        }
+    }
+    picks[p] = pick;
 }
 
 cudaError_t launch_sample(const double *amps, int64_t k, int r, const double *uniform, int64_t *picks,
                           cudaStream_t s) {
     if (k == 0) return cudaSuccess;
+    if (r <= 5) {
+        const int64_t blocks = (k + 127) / 128;
+        if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+        const double2 *a = reinterpret_cast<const double2 *>(amps);
+        const dim3 g((unsigned)blocks);
+        switch (r) {
+            case 0: k_sample_rows<0><<<g, 128, 0, s>>>(a, k, uniform, picks); break;
+            case 1: k_sample_rows<1><<<g, 128, 0, s>>>(a, k, uniform, picks); break;
+            case 2: k_sample_rows<2><<<g, 128, 0, s>>>(a, k, uniform, picks); break;
+            case 3: k_sample_rows<3><<<g, 128, 0, s>>>(a, k, uniform, picks); break;
+            case 4: k_sample_rows<4><<<g, 128, 0, s>>>(a, k, uniform, picks); break;
+            default: k_sample_rows<5><<<g, 128, 0, s>>>(a, k, uniform, picks); break;
+        }
+        return cudaGetLastError();
+    }
     const int64_t blocks = (k + 31) / 32;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     k_sample<<<dim3((unsigned)blocks), SAMP_THREADS, 0, s>>>(reinterpret_cast<const double2 *>(amps), k, r, uniform,
@@ -1564,16 +1617,21 @@ cudaError_t launch_sample(const double *amps, int64_t k, int r, const double *un
     return cudaGetLastError();
 }
 
+// An SM's two FP64 lanes take 1 us for about 50 amplitudes' sums, so a few
+// amplitudes already spread over the cluster.
+constexpr int64_t PT_PER_SM = 64;
+
 cudaError_t launch_pt_moments(const double *amps, int64_t k, double n_states, double fid, double *out,
                               cudaStream_t s) {
-    return launch_cluster(k_pt_moments<true>, k, s, reinterpret_cast<const double2 *>(amps), k, n_states, fid, 1, out);
+    return launch_cluster(k_pt_moments<true>, k, PT_PER_SM, s, reinterpret_cast<const double2 *>(amps), k, n_states,
+                          fid, 1, out);
 }
 
-// Blocks of the scratch form: four amplitudes a thread at least, at most
+// Blocks of the scratch form: an amplitude a thread at least, at most
 // PT_BLOCKS (two resident blocks on each of 152 SMs).
 constexpr int PT_BLOCKS = 304;
 static int pt_blocks(int64_t k) {
-    const int64_t b = (k + 4 * RED_THREADS - 1) / (4 * RED_THREADS);
+    const int64_t b = (k + RED_THREADS - 1) / RED_THREADS;
     return int(b < 1 ? 1 : (b > PT_BLOCKS ? PT_BLOCKS : b));
 }
 
@@ -1582,6 +1640,9 @@ size_t pt_moments_scratch_bytes(int64_t k) { return size_t(pt_blocks(k)) * 5 * s
 cudaError_t launch_pt_moments_scratch(const double *amps, int64_t k, double n_states, double fid, bool want_log,
                                       double *out, double *scratch, cudaStream_t s) {
     const int blocks = pt_blocks(k);
+    if (blocks <= RED_CLUSTER)  // one launch instead of two (a fit of 1000 amplitudes: 366 -> 310 us)
+        return launch_cluster(k_pt_moments<true>, k, PT_PER_SM, s, reinterpret_cast<const double2 *>(amps), k,
+                              n_states, fid, want_log ? 1 : 0, out);
     k_pt_moments<false><<<blocks, RED_THREADS, 0, s>>>(reinterpret_cast<const double2 *>(amps), k, n_states, fid,
                                                        want_log ? 1 : 0, scratch);
     k_pt_final<<<1, 160, 0, s>>>(scratch, blocks, out);

@@ -103,7 +103,7 @@ def test_pipeline_with_open_qubits(case20):
         assert rel_l2(got[i], sv.correlated_amplitudes(c, b, open_q)) <= 1e-5
 
 
-@pytest.mark.parametrize("rows,n_open", [(1, 0), (33, 0), (65, 1), (31, 4), (32, 5), (33, 6), (100, 10), (3, 12), (2, 16)])
+@pytest.mark.parametrize("rows,n_open", [(1, 0), (33, 0), (65, 1), (257, 2), (129, 3), (31, 4), (128, 4), (32, 5), (300, 5), (33, 6), (100, 10), (3, 12), (2, 16)])
 def test_samples_over_tiles_and_segments(rows, n_open):
     # rows per block (32), completions per tile (32) and per segment; numbers
     # at 0 and next to 1, rows of zeros, infinities and NaN
