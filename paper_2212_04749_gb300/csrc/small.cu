@@ -7,16 +7,17 @@
 // cluster of up to 16 blocks runs a list of them: the steps are sorted into
 // phases on the host, a phase's steps depend on earlier phases only and run
 // side by side, and a cluster barrier between phases takes the place of the
-// launch.  A phase costs its barrier and two round trips to L2 (the instance
-// pair, then maxima, A and B together).
+// launch.  A phase costs its barrier and one round trip to L2 (maxima,
+// exponents, A and B together); a warp looks up its part of the next phase and
+// the instances there between its arrival at the barrier and the wait.
+// 64 amplitudes of 3x4 with 8 cycles: 34.9 us with the look-up and the
+// exponents' loads behind the barrier, 32.6 so; as separate launches 177.
 //
 // An output C[i](m, n) is one sum over k, split over 2^lanes_log2
 // neighbouring lanes where a step has fewer outputs than the cluster has
 // threads, in FP32 FMA; rescale and exponents as in the other step kernels.
 // Operands written by an earlier phase of the same launch come from other
 // SMs, so they are read past L1 (ld.global.cg).
-#include <cooperative_groups.h>
-
 #include "kernels.cuh"
 
 namespace tnk {
@@ -43,10 +44,18 @@ __device__ __forceinline__ void sm_cfma(float2 &acc, float2 a, float2 b) {
     acc.y = fmaf(a.y, b.x, acc.y);
 }
 
+// The instances of output `first + lane` of a step (the last one's where
+// there is none): nothing that an earlier phase writes.
+__device__ __forceinline__ int2 small_instances(const SmallDesc &d, int lg, int first, int lane) {
+    const int o = (first + lane) >> lg;
+    return __ldg(d.instab + ((o < d.outputs ? o : 0) >> d.mnb));
+}
+
 // U x 32 lanes of one step (lane groups of 2^lg lanes, one output each), U
-// outputs a lane at once so that their loads are in flight together.
+// outputs a lane at once so that their loads are in flight together; ab0: the
+// first ones' instances (small_instances).
 template <int U>
-__device__ __forceinline__ void small_outputs(const SmallDesc &d, int lg, int first, int lane) {
+__device__ __forceinline__ void small_outputs(const SmallDesc &d, int lg, int first, int lane, int2 ab0) {
     const int sub = lane & ((1 << lg) - 1);
     bool valid[U];
     int i[U], mn[U];
@@ -58,15 +67,19 @@ __device__ __forceinline__ void small_outputs(const SmallDesc &d, int lg, int fi
         const int oc = valid[u] ? o : 0;
         i[u] = oc >> d.mnb;
         mn[u] = oc & ((1 << d.mnb) - 1);
-        ab[u] = __ldg(d.instab + i[u]);
+        ab[u] = u == 0 ? ab0 : __ldg(d.instab + i[u]);
     }
     uint32_t ma[U], mb[U];
+    int32_t Ea[U], Eb[U];  // loaded with the operands: at the end they would be one more round trip
     const float2 *a[U], *b[U];
     float2 acc[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         ma[u] = d.mxA ? __ldcg(d.mxA + ab[u].x) : 0u;
         mb[u] = d.mxB ? __ldcg(d.mxB + ab[u].y) : 0u;
+        const bool first_of = mn[u] == 0 && sub == 0;
+        Ea[u] = first_of ? __ldcg(d.EA + ab[u].x) : 0;
+        Eb[u] = first_of ? __ldcg(d.EB + ab[u].y) : 0;
         a[u] = d.A + int64_t(ab[u].x) * d.sA + (int64_t(mn[u] >> d.nb) << d.kb);
         b[u] = d.B + int64_t(ab[u].y) * d.sB + (int64_t(mn[u] & ((1 << d.nb) - 1)) << d.kb);
         acc[u] = make_float2(0.f, 0.f);
@@ -118,7 +131,7 @@ __device__ __forceinline__ void small_outputs(const SmallDesc &d, int lg, int fi
             int64_t c = int64_t(i[u]) * d.sC;
             for (int j = 0; j < d.mnb; ++j) c += int64_t((mn[u] >> j) & 1) << d.pC[j];
             d.C[c] = v;
-            if (mn[u] == 0) d.EC[i[u]] = __ldcg(d.EA + ab[u].x) + ea + __ldcg(d.EB + ab[u].y) + eb;
+            if (mn[u] == 0) d.EC[i[u]] = Ea[u] + ea + Eb[u] + eb;
             mx = __float_as_uint(fmaxf(fabsf(v.x), fabsf(v.y)));
         }
         if (d.mxC) {
@@ -142,21 +155,45 @@ __global__ void __launch_bounds__(SM_THREADS) k_small_steps(const __grid_constan
         reinterpret_cast<uint4 *>(sd + s)[q] = __ldg(reinterpret_cast<const uint4 *>(p.descs + p.step[s]) + q);
     }
     __syncthreads();
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
     const int nw = int(gridDim.x) * SM_WARPS, gw = int(blockIdx.x) + warp * int(gridDim.x);
-    int s0 = 0;
-    for (int ph = 0; ph < p.n_phases; ++ph) {
-        const int s1 = p.phase_end[ph];
-        if (ph > 0) cl.sync();  // release / acquire: the last phase's outputs, maxima and exponents are visible
-        int s = s0;
-        for (int w = gw; w < p.wend[s1 - 1]; w += nw) {
-            while (w >= p.wend[s]) ++s;
-            const int local = w - (s > s0 ? p.wend[s - 1] : 0);
-            if (p.four[s]) small_outputs<4>(sd[s], p.lanes_log2[s], local * 128, lane);
-            else small_outputs<1>(sd[s], p.lanes_log2[s], local * 32, lane);
+    int s0 = 0, s1 = p.phase_end[0], s = 0, local = 0;
+    // the step and place of the phase's warp w (s: from the phase's first step on)
+    auto locate = [&](int w) {
+        while (w >= p.wend[s]) ++s;
+        local = w - (s > s0 ? p.wend[s - 1] : 0);
+    };
+    auto instances = [&] {
+        return small_instances(sd[s], p.lanes_log2[s], local * (p.four[s] ? 128 : 32), lane);
+    };
+    int2 ab = make_int2(0, 0);
+    bool mine = gw < p.wend[s1 - 1];
+    if (mine) {
+        locate(gw);
+        ab = instances();
+    }
+    for (int ph = 0;;) {
+        for (int w = gw; mine;) {
+            if (p.four[s]) small_outputs<4>(sd[s], p.lanes_log2[s], local * 128, lane, ab);
+            else small_outputs<1>(sd[s], p.lanes_log2[s], local * 32, lane, ab);
+            w += nw;
+            mine = w < p.wend[s1 - 1];
+            if (mine) {
+                locate(w);
+                ab = instances();
+            }
         }
-        s0 = s1;
+        if (++ph == p.n_phases) break;
+        // release: this phase's outputs, maxima and exponents; meanwhile the
+        // next phase's place and instances, which depend on none of them
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        s = s0 = s1;
+        s1 = p.phase_end[ph];
+        mine = gw < p.wend[s1 - 1];
+        if (mine) {
+            locate(gw);
+            ab = instances();
+        }
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     }
 }
 
