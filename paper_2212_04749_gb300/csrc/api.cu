@@ -348,7 +348,12 @@ int run_step(PlanObj *o, int s, int precision, int64_t sigma, cudaStream_t st) {
     d.tc_pair = o->tc_pair ? 1 : 0;
     cudaError_t e;
     int fam;
-    if (cfg < 2) {
+    const bool chosen = s < (int)o->pinned.size() && o->pinned[s];  // by the caller: runs as it is
+    const bool on_tc = cfg >= 2 && precision != TN_FP32 && tnk::gemm_tc_supports(d) && !tnk::step_skinny_takes(d);
+    if (sigma < 0 && !chosen && tnk::step_few_takes(d, on_tc)) {
+        fam = 1;
+        e = tnk::launch_step_few(d, st);
+    } else if (cfg < 2) {
         fam = 0;
         e = tnk::launch_step_row(d, st);
     } else if (tnk::step_skinny_takes(d)) {
@@ -1312,8 +1317,16 @@ int tn_plan_select(tn_plan_t plan, int precision, const uint16_t *params16, floa
             }
         }
         o->config_override[s] = b1;
-        // (a small step that shares a launch runs the same whatever is chosen)
-        if (uncertain) uncertain[s] = (have2 && y2 - y1 < margin && !merges(o, s)) ? 1 : 0;
+        // (a small step that shares a launch, and one of few multiply-adds, run
+        // the same whatever is chosen)
+        tnk::StepDesc t;
+        std::memset(&t, 0, sizeof(t));
+        t.mb = P.steps[s].mb;
+        t.kb = P.steps[s].kb;
+        t.nb = P.steps[s].nb;
+        t.nInst = P.nodes[P.steps[s].node].n_inst;
+        const bool same = merges(o, s) || tnk::step_few_takes(t, precision != TN_FP32);
+        if (uncertain) uncertain[s] = (have2 && y2 - y1 < margin && !same) ? 1 : 0;
     }
     o->drop_graphs();
     g_err.clear();

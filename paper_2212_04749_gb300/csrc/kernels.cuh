@@ -210,6 +210,10 @@ struct SmallArgs {
 };
 static_assert(sizeof(SmallArgs) <= 4096, "kernel parameters");
 cudaError_t init_small_kernel();
+// A single step of few multiply-adds, a thread or a few lanes per output
+// (FP32; tc: it would run on the tensor cores otherwise).
+bool step_few_takes(const StepDesc &d, bool tc);
+cudaError_t launch_step_few(const StepDesc &d, cudaStream_t s);
 cudaError_t launch_small(const SmallArgs &a, cudaStream_t s);
 
 // Cost-model MLP (mlp.cu); sizes and parameter layout in include/tn.h.

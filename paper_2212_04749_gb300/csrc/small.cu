@@ -18,6 +18,8 @@
 // threads, in FP32 FMA; rescale and exponents as in the other step kernels.
 // Operands written by an earlier phase of the same launch come from other
 // SMs, so they are read past L1 (ld.global.cg).
+#include <cstring>
+
 #include "kernels.cuh"
 
 namespace tnk {
@@ -197,7 +199,111 @@ __global__ void __launch_bounds__(SM_THREADS) k_small_steps(const __grid_constan
     }
 }
 
+// One step of few multiply-adds, too many for the cluster: an output per group
+// of 2^lg lanes over the whole chip, rows of A in neighbouring lanes (they are
+// neighbours in C where the layout allows).  Operands come through L1: 16
+// bytes a multiply-add.  Latency-bound: the tiled kernels put such a step on
+// a few SMs and walk K serially there (2^11 x 32 x 32 in FP32 16.3 us, 8.2
+// here; 2^15 x 8 x 8 24.8 and 10.0 on the row kernel; 33 instances of 2^4 x 64
+// x 8 26.1 and 6.0).  (d.nb: the row bits, which come first in pC.)
+constexpr int FEW_THREADS = 256;
+
+__global__ void __launch_bounds__(FEW_THREADS) k_step_few(const __grid_constant__ SmallDesc d, int lg) {
+    __shared__ uint32_t s_mx;
+    const int t = int(blockIdx.x) * FEW_THREADS + int(threadIdx.x), sub = t & ((1 << lg) - 1), o = t >> lg;
+    const bool valid = o < d.outputs, one = d.mnb + lg >= 8;  // one: a block's outputs belong to one instance
+    const int oc = valid ? o : 0, i = oc >> d.mnb, mn = oc & ((1 << d.mnb) - 1);
+    if (threadIdx.x == 0) s_mx = 0u;
+    if (d.mxC && one) __syncthreads();
+    const int2 ab = __ldg(d.instab + i);
+    const uint32_t ma = d.mxA ? __ldg(d.mxA + ab.x) : 0u, mb = d.mxB ? __ldg(d.mxB + ab.y) : 0u;
+    const float2 *a = d.A + int64_t(ab.x) * d.sA + (int64_t(mn & ((1 << d.nb) - 1)) << d.kb);
+    const float2 *b = d.B + int64_t(ab.y) * d.sB + (int64_t(mn >> d.nb) << d.kb);
+    int64_t c = int64_t(i) * d.sC;
+    for (int j = 0; j < d.mnb; ++j) c += int64_t((mn >> j) & 1) << d.pC[j];
+    float2 acc = make_float2(0.f, 0.f);
+    if (d.kb == 0) {
+        sm_cfma(acc, __ldg(a), __ldg(b));
+    } else {
+        const int pieces = 1 << (d.kb - 1);
+#pragma unroll 4
+        for (int q = sub; q < pieces; q += 1 << lg) {
+            const float4 x = __ldg(reinterpret_cast<const float4 *>(a) + q);
+            const float4 y = __ldg(reinterpret_cast<const float4 *>(b) + q);
+            sm_cfma(acc, make_float2(x.x, x.y), make_float2(y.x, y.y));
+            sm_cfma(acc, make_float2(x.z, x.w), make_float2(y.z, y.w));
+        }
+    }
+    for (int s = 1; s < (1 << lg); s <<= 1) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, s);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, s);
+    }
+    const int ea = sm_exp(ma), eb = sm_exp(mb);
+    const int e1 = max(-126, min(126, ea + eb)), e2 = ea + eb - e1;
+    const float sc = __int_as_float((127 - e1) << 23), s2 = __int_as_float((127 - e2) << 23);
+    const float2 v = make_float2(acc.x * sc * s2, acc.y * sc * s2);
+    uint32_t mx = 0u;
+    if (valid && sub == 0) {
+        d.C[c] = v;
+        if (mn == 0) d.EC[i] = __ldg(d.EA + ab.x) + ea + __ldg(d.EB + ab.y) + eb;
+        mx = __float_as_uint(fmaxf(fabsf(v.x), fabsf(v.y)));
+    }
+    if (!d.mxC) return;
+    if (one) {
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if ((threadIdx.x & 31) == 0 && mx) atomicMax(&s_mx, mx);
+        __syncthreads();
+        if (threadIdx.x == 0 && s_mx) atomicMax(d.mxC + i, s_mx);
+    } else if (d.mnb + lg >= 5) {
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if ((threadIdx.x & 31) == 0 && mx) atomicMax(d.mxC + i, mx);
+    } else if (mx) {
+        atomicMax(d.mxC + i, mx);
+    }
+}
+
 }  // namespace
+
+bool step_few_takes(const StepDesc &d, bool tc) {
+    // 2^23 multiply-adds (128 MB through L1, 4 us); against the tensor cores,
+    // whose persistent kernel takes 14 us for any small step, 2^21: 2^14 x 16 x
+    // 16 takes 16.3 us here and 14.2 there, 2^11 x 32 x 32 8.2 and 16.3
+    if (d.kb > 10 || d.mb + d.nb > 18) return false;
+    return (d.nInst << (d.mb + d.nb)) <= (int64_t(1) << 18) &&
+           (d.nInst << (d.mb + d.nb + d.kb)) <= (int64_t(1) << (tc ? 21 : 23));
+}
+
+cudaError_t launch_step_few(const StepDesc &d, cudaStream_t s) {
+    if (!step_few_takes(d, false) || d.inst0 != 0) return cudaErrorInvalidValue;
+    SmallDesc r;
+    std::memset(&r, 0, sizeof(r));
+    r.A = d.A;
+    r.B = d.B;
+    r.C = d.C;
+    r.instab = d.instab;
+    r.EA = d.EA;
+    r.EB = d.EB;
+    r.EC = d.EC;
+    r.mxA = d.mxA;
+    r.mxB = d.mxB;
+    r.mxC = d.mxC;
+    r.sA = d.sA;
+    r.sB = d.sB;
+    r.sC = d.sC;
+    r.kb = (int8_t)d.kb;
+    r.nb = (int8_t)d.mb;
+    r.mnb = (int8_t)(d.mb + d.nb);
+    r.outputs = (int32_t)(d.nInst << (d.mb + d.nb));
+    for (int j = 0; j < d.mb; ++j) r.pC[j] = d.pCm[j];
+    for (int j = 0; j < d.nb; ++j) r.pC[d.mb + j] = d.pCn[j];
+    if (r.outputs <= 0) return cudaSuccess;
+    // lanes per output: while the chip has threads to spare and a lane two entries
+    int lg = 0;
+    while (lg < 5 && lg < d.kb - 1 && (int64_t(r.outputs) << (lg + 1)) <= 131072) ++lg;
+    const int64_t blocks = ((int64_t(r.outputs) << lg) + FEW_THREADS - 1) / FEW_THREADS;
+    k_step_few<<<dim3((unsigned)blocks), FEW_THREADS, 0, s>>>(r, lg);
+    return cudaGetLastError();
+}
 
 cudaError_t init_small_kernel() {
     cudaError_t e = cudaFuncSetAttribute(k_small_steps, cudaFuncAttributeMaxDynamicSharedMemorySize,
