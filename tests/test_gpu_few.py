@@ -19,7 +19,7 @@ pytestmark = pytest.mark.gpu
 
 def _takes(st, log2_macs):
     out = st["n_inst"] << (st["mb"] + st["nb"])
-    return (st["kb"] <= 10 and out <= 1 << 18 and out << st["kb"] <= 1 << log2_macs and
+    return (st["kb"] <= 10 and out <= 1 << 20 and out << st["kb"] <= 1 << log2_macs and
             (out > 1 << 14 or out << st["kb"] > 1 << 18))
 
 
