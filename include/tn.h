@@ -314,18 +314,25 @@ int tn_plan_set_kernel(tn_plan_t plan, int32_t step, int32_t kernel);
  * allows (K >= 8, 64 <= M < 2^31), on the CUDA cores otherwise.  For TN_FP32
  * configuration 2 takes the tensor cores as well where a step has K >= 64,
  * 64 <= M < 2^31, N >= 64 or groups of 32 columns on average, maxima for both
- * operands (tn_options.rescale, no leaf) and room for its packed B: each operand instance scaled by a power of
- * two and split into two fp16 halves (22 bits of each value down to 2^-18 of
- * the instance's largest), three products, units of 64 real k summed in
- * FP32 registers.  Configuration 3 and tn_plan_set_tc_resident_b(plan, 0)
- * stay on the FMA kernel. */
+ * operands (tn_options.rescale, no leaf) and room for its packed B: each
+ * operand instance scaled by a power of two and split into two fp16 halves
+ * (22 bits of each value down to 2^-18 of the instance's largest), three
+ * products, units of 64 real k summed in FP32 registers.  Configuration 3 and
+ * tn_plan_set_tc_resident_b(plan, 0) stay on the FMA kernel.  Steps whose
+ * shape leaves the GEMM's tiles empty (few outputs or few columns per
+ * instance, K <= 4 or, in TN_FP32, <= 32) take kernels of their own under
+ * configurations 2 and 3, in FP32 (family 1 of tn_plan_step_times).  A step of
+ * at most 2^20 outputs and 2^23 complex multiply-adds (2^21 where it would run
+ * on the tensor cores) runs an output per thread in FP32 under every
+ * configuration that the caller did not set for it; the autotuner then times
+ * that under each. */
 #define TN_NCONFIG 4
 
 /* Set step `step` to configuration `config` (-1: the plan's own choice: 0 or
  * 2, on the tensor cores 3 where a group's resident B would leave the stream
  * of A too little of the shared memory).
- * A step given a configuration (>= 0) then runs by itself even if it is small
- * (see tn_plan_step_times, family 4); config + TN_CONFIG_TUNED, with config as
+ * A step given a configuration (>= 0) then runs by itself, and as that says,
+ * even if it is small (see tn_plan_step_times, family 4, and above); config + TN_CONFIG_TUNED, with config as
  * tn_plan_get_configs returned it for a tuned plan of the same shape, leaves
  * small steps together, as tn_plan_autotune and tn_plan_select do.
  * TN_EINVAL for a configuration the step's shape does not allow. */
@@ -446,7 +453,7 @@ int tn_plan_check(tn_plan_t plan, void *stream);
  * events around every launch, read back by tn_plan_step_times, which
  * synchronises the events); ms has n_steps entries.  kernel (may be NULL)
  * receives the kernel family each step last ran: 0 per-row SIMT, 1 tiled
- * SIMT GEMM, 2 tensor-core GEMM, 3 fused chain (the chain's time is booked
+ * SIMT GEMM (and the forms for other shapes), 2 tensor-core GEMM, 3 fused chain (the chain's time is booked
  * on its last step), 4 small steps (at most 2^18 complex multiply-adds and
  * 2^14 outputs each, no kernel set for them by tn_plan_set_config) that share one launch (its
  * time is booked on the last of them). */
