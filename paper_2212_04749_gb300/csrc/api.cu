@@ -1186,7 +1186,15 @@ int tn_plan_autotune(tn_plan_t plan, int precision, int32_t reps, const uint8_t 
     o->config_override.assign(ns, -1);
     const int nchains = (int)P.chains.size();
     const std::vector<int8_t> prev_chain = o->chain_on;
-    o->chain_on.assign(nchains, 0);  // configurations are timed on the separate steps
+    // configurations are timed on the separate steps; chains that hold no
+    // selected step run as they would
+    if (step_mask) {
+        o->chain_on.resize(nchains, -1);
+        for (int s = 0; s < ns; ++s)
+            if (step_mask[s] && P.steps[s].chain >= 0) o->chain_on[P.steps[s].chain] = 0;
+    } else {
+        o->chain_on.assign(nchains, 0);
+    }
     o->drop_graphs();
     int rc = TN_OK;
     for (int c = 0; c < TN_NCONFIG && rc == TN_OK; ++c) {
@@ -1317,15 +1325,16 @@ int tn_plan_select(tn_plan_t plan, int precision, const uint16_t *params16, floa
             }
         }
         o->config_override[s] = b1;
-        // (a small step that shares a launch, and one of few multiply-adds, run
-        // the same whatever is chosen)
+        // (a small step that shares a launch, one of a fused chain and one of few
+        // multiply-adds run the same whatever is chosen)
         tnk::StepDesc t;
         std::memset(&t, 0, sizeof(t));
         t.mb = P.steps[s].mb;
         t.kb = P.steps[s].kb;
         t.nb = P.steps[s].nb;
         t.nInst = P.nodes[P.steps[s].node].n_inst;
-        const bool same = merges(o, s) || tnk::step_few_takes(t, precision != TN_FP32);
+        const bool same = merges(o, s) || o->chain_fused(P.steps[s].chain) ||
+                          tnk::step_few_takes(t, precision != TN_FP32);
         if (uncertain) uncertain[s] = (have2 && y2 - y1 < margin && !same) ? 1 : 0;
     }
     o->drop_graphs();
