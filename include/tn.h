@@ -317,7 +317,7 @@ int tn_plan_set_kernel(tn_plan_t plan, int32_t step, int32_t kernel);
  * operands (tn_options.rescale, no leaf) and room for its packed B: each
  * operand instance scaled by a power of two and split into two fp16 halves
  * (22 bits of each value down to 2^-18 of the instance's largest), three
- * products, units of 64 real k summed in FP32 registers.  Configuration 3 and
+ * products, units of 32 or 64 real k summed in FP32 registers.  Configuration 3 and
  * tn_plan_set_tc_resident_b(plan, 0) stay on the FMA kernel.  Steps whose
  * shape leaves the GEMM's tiles empty (few outputs or few columns per
  * instance, K <= 4 or, in TN_FP32, <= 32) take kernels of their own under

@@ -755,10 +755,7 @@ __device__ __forceinline__ void fold_max16(const uint32_t (&r)[32], EpiMeta &em,
     }
 }
 
-// FP16x3: chunks of a unit
-__host__ __device__ __forceinline__ int unit_chunks(const StepDesc &d) { return d.kb >= 7 ? 2 : 1; }
-
-template <int PREC, int MODE>
+template <int PREC, int MODE, int UC = 1>  // UC: FP16x3, chunks of a unit
 __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 warps on a sub-partition)
     k_step_gemm_tc(const __grid_constant__ StepDesc d, int64_t mtiles, int32_t *err, const __grid_constant__ CUtensorMap tmA, int nrs,
                    int acw, int ow, int tblk) {
@@ -780,13 +777,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
     // PREC 3, FP16x3 for FP32 steps (MODE 3 only): operands scaled by powers of
     // two and split into fp16 halves.  The tensor cores truncate each sum into
     // the accumulator (relative L2 error 1.0e-6 over 1024 real k of random
-    // signs, the FMA kernel 2.5e-7; 6.5e-8 over 64), so a unit of two chunks
-    // (64 real k; K = 64: one chunk) starts from zero, its small products
-    // first, and the epilogue adds the units in FP32 registers, rounded to
-    // nearest: the contraction's error is 3 to 43 % below the FMA kernel's.
+    // signs, the FMA kernel 2.5e-7; 6.5e-8 over 64), so a unit of one chunk
+    // (32 real k; K >= 512: two) starts from zero, its small products first,
+    // and the epilogue adds the units in FP32 registers, rounded to nearest:
+    // the contraction's error is below the FMA kernel's.
     // Bound by the loads of A and B from L2 and the tensor cores together.
-    // 53-qubit circuit, FP32: 2^12 x 2^9 x 2^8 with 512 instances 48 -> 7.5 ms,
-    // all of it 228 -> 49 ms.
+    // 53-qubit circuit, FP32: 2^12 x 2^9 x 2^8 with 512 instances 48 -> 7.4 ms,
+    // all of it 228 -> 48.4 ms.
     constexpr int EPI_REGS = epi_regs(PREC);
     constexpr bool ASPLIT = PREC >= 2;  // A split into TMEM
     static_assert(PREC != 3 || MODE == 3, "FP16x3: packed B");
@@ -1244,10 +1241,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                 TileIter it;
                 if (!BPACK && my_tiles > 0) it.start(d, mtiles, n_tiles, tblk, PP);
                 if constexpr (PREC == 3) {
-                    // a unit: two chunks (K >= 32), its own accumulator of two
-                    // in turn
-                    const int uc = unit_chunks(d);
-                    const int64_t units = my_tiles * (nch / uc);
+                    // a unit: UC chunks, its own accumulator of two in turn
+                    const int64_t units = my_tiles * (nch / UC);
                     for (int64_t q = 0; q < units && ok && !*abort_flag; ++q) {
                         const int acc = int(q & 1);
                         if (!mbar_wait(&X.tempty[acc], (uint32_t(q >> 1) & 1u) ^ 1u)) {
@@ -1256,8 +1251,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                         }
                         tc_fence_after();
                         const uint32_t dtm = tmem + uint32_t(acc) * awr, id = idesc(0u, awr);
-                        int st[2];
-                        for (int c = 0; c < uc; ++c) {
+                        int st[UC];
+                        for (int c = 0; c < UC; ++c) {
                             st[c] = ts;
                             if (!mbar_wait(&X.afull[ts], tph)) {
                                 ok = false;
@@ -1274,8 +1269,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
 #pragma unroll
                         for (int h = 0; h < 2; ++h)
 #pragma unroll
-                            for (int c = 0; c < 2; ++c) {
-                                if (c >= uc) break;
+                            for (int c = 0; c < UC; ++c) {
                                 const uint32_t a0 = tmem + uint32_t(TM_A + st[c] * TM_ASTAGE);
                                 const uint32_t b0 = smem_u32(sm + C::OFF_RAW + (PACK_ST + st[c]) * C::SLOT_RAW);
                                 const uint32_t bl = b0 + TBNR * TBKR * 2;
@@ -1291,7 +1285,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                                     }
                                 }
                             }
-                        for (int c = 0; c < uc; ++c) {
+                        for (int c = 0; c < UC; ++c) {
                             mma_commit(&X.taempty[st[c]]);
                             mma_commit(&X.rempty[st[c]]);
                         }
@@ -1552,7 +1546,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
             if constexpr (PREC == 3) {
 #pragma unroll
                 for (int i = 0; i < 64; ++i) sum[i >> 5][i & 31] = 0u;
-                const int nu = nch / unit_chunks(d);
+                const int nu = nch / UC;
                 for (int u = 0; u < nu; ++u) {
                     const int64_t q = l * nu + u;
                     const int ua = int(q & 1);
@@ -1880,9 +1874,11 @@ cudaError_t init_kernels() {
     e = cudaFuncSetAttribute(reinterpret_cast<const void *>(k_step_gemm_tc<2, 4>),
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<2, true>());
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(reinterpret_cast<const void *>(k_step_gemm_tc<3, 3>),
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<3, true>());
-    if (e != cudaSuccess) return e;
+    for (const void *fn : {reinterpret_cast<const void *>(k_step_gemm_tc<3, 3, 1>),
+                           reinterpret_cast<const void *>(k_step_gemm_tc<3, 3, 2>)}) {
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<3, true>());
+        if (e != cudaSuccess) return e;
+    }
     const void *fns[8] = {reinterpret_cast<const void *>(k_step_gemm_tc<1, 0>),
                           reinterpret_cast<const void *>(k_step_gemm_tc<2, 0>),
                           reinterpret_cast<const void *>(k_step_gemm_tc<1, 1>),
@@ -1942,8 +1938,17 @@ cudaError_t launch_step_gemm_tc(const StepDesc &d, const CUtensorMap *a_map, int
             k_pack_b<3><<<dim3((unsigned)blocks), 256, 0, s>>>(d, nch);
         else
             k_pack_b_tiles<<<dim3((unsigned)blocks), 256, 0, s>>>(d, nch);
-        k_step_gemm_tc<3, 3><<<g, NTHREADS, smem_bytes<3, true>(), s>>>(
-            d, mtiles, err, *a_map, PACK_ST, TBN, TBN, b >= 2 ? 2 : 1);
+        // Chunks of a unit: two where the FMA kernel's own rounding is largest
+        // (53-qubit circuit, relative L2 error over 320 oracle amplitudes and
+        // time: FMA 1.71e-6, 228 ms; two from K = 128 on 1.76e-6, 45.9; from
+        // K = 512 on 1.57e-6, 48.4; one always 1.51e-6, about 52)
+        const int step = b >= 2 ? 2 : 1;
+        if (d.kb >= 9)
+            k_step_gemm_tc<3, 3, 2><<<g, NTHREADS, smem_bytes<3, true>(), s>>>(d, mtiles, err, *a_map, PACK_ST, TBN,
+                                                                               TBN, step);
+        else
+            k_step_gemm_tc<3, 3, 1><<<g, NTHREADS, smem_bytes<3, true>(), s>>>(d, mtiles, err, *a_map, PACK_ST, TBN,
+                                                                               TBN, step);
         return cudaGetLastError();
     }
     // B as a dictionary (every instance resident for the launch), else
