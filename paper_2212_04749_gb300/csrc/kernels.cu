@@ -10,6 +10,9 @@
 //                    contraction of SM Sec. V.A
 //   k_step_gemm_simt tiled complex GEMM with gathered (bit-permuted) operand
 //                    loads, FP32 FMA; the plain FP32 form of big x big steps
+//   k_step_narrow    long rows, few columns per A instance
+//   k_step_outer     short rows, many columns
+//   k_step_skinny    few outputs per instance, long K
 //   k_accumulate     amp[p] += sum over the batch's slices of the root
 //                    partials times 2^E, complex128, fixed slice order
 //                    (first-level slicing, SM Sec. IV.B)
@@ -19,14 +22,15 @@
 //   k_pt_hist        histogram of x = N |amp|^2 (integer counts)
 //   k_sample         one completion per correlated batch, drawn with
 //                    probability |amp|^2 / sum over the batch (perfect
-//                    sample from a batch, main text on Fig. 3(b), SM Sec. II)
+//                    sample from a batch, main text on Fig. 3(b), SM Sec. II);
+//                    k_sample_rows: batches of at most 32 completions
 //
 // Power-of-two rescaling: every produced instance records the largest
 // |component| of its entries (as float bits, atomicMax of non-negative
 // floats); its consumer multiplies the loaded values by 2^-e, e the
 // exponent of that maximum, and adds e to the output's exponent E.  Scaling
-// by a power of two is exact, so with and without it the FP32 results are
-// bitwise the same (barring subnormals).
+// by a power of two is exact, so with and without it the FP32 results of
+// these kernels are bitwise the same (barring subnormals).
 #include <cooperative_groups.h>
 
 #include "kernels.cuh"
