@@ -18,22 +18,35 @@ import numpy as np
 from . import tn
 
 
+def _torch_stream(torch, stream, device):
+    """`stream` (a torch stream, a raw handle, None: the current stream) as a
+    torch stream.  Torch's streams do not order themselves against one
+    another, so buffers are made, kernels launched and results read with it
+    as the current stream."""
+    if stream is None:
+        return torch.cuda.current_stream(device)
+    if isinstance(stream, int):
+        return torch.cuda.ExternalStream(stream, device=device) if stream else torch.cuda.default_stream(device)
+    return stream
+
+
 def porter_thomas_fit(amps, k, n_qubits, stream=None, iters=60, tol=1e-13):
-    """amps: device complex128 amplitudes (2k doubles, a torch CUDA tensor).
+    """amps: device complex128 amplitudes (2k doubles, a torch CUDA tensor),
+    complete on `stream` (default: the current stream).
     Returns a dict: fidelity (maximum likelihood, kept in [0, 1 - 1e-12]),
     stderr, loglik (up to the constant), linear (N <p> - 1), linear_stderr,
     iterations."""
     import torch
 
-    out = torch.empty(5, dtype=torch.float64, device=amps.device)
-    scratch = torch.empty(tn.tn_pt_moments_scratch_bytes(k), dtype=torch.uint8, device=amps.device)
-    if isinstance(stream, torch.cuda.Stream):  # the kernels run there, not on the stream these were made on
-        out.record_stream(stream)
-        scratch.record_stream(stream)
+    st = _torch_stream(torch, stream, amps.device)
+    with torch.cuda.stream(st):
+        out = torch.empty(5, dtype=torch.float64, device=amps.device)
+        scratch = torch.empty(tn.tn_pt_moments_scratch_bytes(k), dtype=torch.uint8, device=amps.device)
 
     def moments(f, log=False):
-        tn.tn_pt_moments_scratch(amps, k, n_qubits, f, out, scratch, want_log=log, stream=stream)
-        return out.cpu().numpy()  # synchronises with the launch
+        with torch.cuda.stream(st):
+            tn.tn_pt_moments_scratch(amps, k, n_qubits, f, out, scratch, want_log=log, stream=st)
+            return out.cpu().numpy()  # copied on st, after the launch
 
     top = 1.0 - 1e-12
     s = moments(0.0)
@@ -55,12 +68,15 @@ def porter_thomas_fit(amps, k, n_qubits, stream=None, iters=60, tol=1e-13):
 
 def porter_thomas_histogram(amps, k, n_qubits, x_max=8.0, nbins=64, stream=None):
     """Counts of x = 2^n |amp|^2 in nbins equal bins over [0, x_max), then
-    the count at or above x_max (numpy int64, nbins + 1 entries)."""
+    the count at or above x_max (numpy int64, nbins + 1 entries).  amps and
+    stream as for porter_thomas_fit."""
     import torch
 
-    counts = torch.zeros(nbins + 1, dtype=torch.int64, device=amps.device)
-    tn.tn_pt_histogram(amps, k, n_qubits, x_max, nbins, counts, stream=stream)
-    return counts.cpu().numpy()
+    st = _torch_stream(torch, stream, amps.device)
+    with torch.cuda.stream(st):
+        counts = torch.zeros(nbins + 1, dtype=torch.int64, device=amps.device)
+        tn.tn_pt_histogram(amps, k, n_qubits, x_max, nbins, counts, stream=st)
+        return counts.cpu().numpy()
 
 
 def porter_thomas_expected(nbins, x_max, k, fidelity):

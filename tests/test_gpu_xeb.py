@@ -121,3 +121,25 @@ def test_moments_scratch_form_and_xeb_at_block_edges(k, f):
     assert abs(out[0].item() - want) <= 1e-12 * max(abs(want), 1.0)
     with pytest.raises(tn.TnError):
         tn.tn_pt_moments_scratch(d, k, n, f, out, scratch[:-1])
+
+
+@pytest.mark.parametrize("kind", ["stream", "handle", "current"])
+def test_analysis_on_a_stream_that_is_still_busy(kind):
+    # the amplitudes arrive 50 ms late on a stream of their own: the sums and
+    # counts read are those of the late amplitudes, from the first pass on
+    torch, tn = require_cuda()
+    from paper_2212_04749_gb300 import xeb
+    n, k = 24, 50001
+    d = _dev(torch, _amps(k, n, 6))
+    fit, hist = xeb.porter_thomas_fit(d, k, n), xeb.porter_thomas_histogram(d, k, n)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    arg = {"stream": side, "handle": side.cuda_stream, "current": None}[kind]
+    for f, want in ((xeb.porter_thomas_fit, fit), (xeb.porter_thomas_histogram, hist)):
+        with torch.cuda.stream(side):
+            late = torch.zeros_like(d)
+            torch.cuda._sleep(100_000_000)
+            late.copy_(d)
+        with torch.cuda.stream(side if kind == "current" else torch.cuda.default_stream()):
+            got = f(late, k, n, stream=arg)
+        assert np.array_equal(got, want) if isinstance(want, np.ndarray) else got == want
