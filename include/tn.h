@@ -61,8 +61,9 @@ enum {
  * the cross-slice sum and XEB are FP64). */
 enum {
     TN_FP32 = 0,    /* complex64 operands, FP32 FMA on the CUDA cores; large steps
-                     * of rescaled plans in FP16x3 (see TN_NCONFIG), whose
-                     * error is no larger */
+                     * of rescaled plans in BF16x6 on the tensor cores, which
+                     * keeps every bit of them (see TN_NCONFIG,
+                     * tn_plan_set_tc_fp32) */
     TN_TF32 = 1,    /* tensor cores, TF32 operands, FP32 accumulate */
     TN_BF16X3 = 2   /* tensor cores, hi/lo BF16 split, three products */
 };
@@ -314,10 +315,12 @@ int tn_plan_set_kernel(tn_plan_t plan, int32_t step, int32_t kernel);
  * allows (K >= 8, 64 <= M < 2^31), on the CUDA cores otherwise.  For TN_FP32
  * configuration 2 takes the tensor cores as well where a step has K >= 64,
  * 64 <= M < 2^31, N >= 64 or groups of 32 columns on average, maxima for both
- * operands (tn_options.rescale, no leaf) and room for its packed B: each
- * operand instance scaled by a power of two and split into two fp16 halves
- * (22 bits of each value down to 2^-18 of the instance's largest), three
- * products, units of 32 or 64 real k summed in FP32 registers.  Configuration 3 and
+ * operands (tn_options.rescale, no leaf) and room for its packed B (BF16x6):
+ * each operand value split into three bf16 parts, which hold all of its 24
+ * bits, and the six products of parts down to 2^-16 of the whole, in units of
+ * 32 or 64 real k whose sums are added in FP32 registers.  (An infinity in
+ * an operand gives NaN there, infinity or NaN on the FMA kernel.)
+ * Configuration 3, tn_plan_set_tc_fp32(plan, 0) and
  * tn_plan_set_tc_resident_b(plan, 0) stay on the FMA kernel.  Steps whose
  * shape leaves the GEMM's tiles empty (few outputs or few columns per
  * instance, K <= 4 or, in TN_FP32, <= 32) take kernels of their own under
@@ -347,6 +350,11 @@ int tn_plan_set_config(tn_plan_t plan, int32_t step, int32_t config);
  * chunk next to A.  Both forms compute the same values; the switch exists
  * to measure and test the streaming form.  TN_EINVAL for a null plan. */
 int tn_plan_set_tc_resident_b(tn_plan_t plan, int32_t enable);
+
+/* FP32 steps on the tensor cores (BF16x6, see TN_NCONFIG): enable = 1 (the
+ * default) where a step's shape allows, 0 every FP32 step by FMA.  TF32 and
+ * BF16x3 are unaffected.  TN_EINVAL for a null plan. */
+int tn_plan_set_tc_fp32(tn_plan_t plan, int32_t enable);
 
 /* Column-tile pairs in the tensor-core BF16x3 form with packed B
  * (configuration 2, N >= 64 per instance, K >= 256): enable = 1 (the default) walks

@@ -43,6 +43,7 @@ struct PlanObj {
     std::vector<AMap> amap;           // per step: TMA descriptor of A (tensor-core steps)
     std::vector<tnk::ChainDesc> chain_desc;  // per fused chain
     int32_t *err_flag = nullptr;      // device word for bounded waits
+    bool tc_fp32 = true;              // FP32 steps take the tensor cores where they may
     bool tc_resident_b = true;        // tensor-core GEMM keeps B in shared memory where it fits
     bool tc_pair = true;              // tensor-core GEMM: column-tile pairs (N = 256 MMAs) where packed B allows
     bool profile = false;
@@ -154,8 +155,9 @@ void build_descs(PlanObj *o) {
         d.ptab = st.n_pair_tiles > 0 ? at<const int2>(o, st.off_pair_tab) : nullptr;
         d.n_ptab = st.n_pair_tiles;
         d.instab = at<const int2>(o, st.off_inst_ab);
-        d.bpack = P.bpack_bytes > 0 ? at<uint8_t>(o, P.off_bpack) : nullptr;
+        d.bpack = P.bpack32_bytes > 0 ? at<uint8_t>(o, P.off_bpack) : nullptr;
         d.bpack_bytes = P.bpack_bytes;
+        d.bpack32_bytes = P.bpack32_bytes;
 
         int64_t mg = 0;
         for (int64_t g = 0; g < st.n_groups; ++g) mg = std::max(mg, st.group_first[g + 1] - st.group_first[g]);
@@ -344,6 +346,7 @@ int run_step(PlanObj *o, int s, int precision, int64_t sigma, cudaStream_t st) {
     tnk::StepDesc d = o->desc[s];
     if (sigma >= 0) apply_window(o, S, sigma, d);
     d.sched = cfg & 1;
+    d.tc_fp32 = o->tc_fp32 ? 1 : 0;
     d.tc_resident_b = o->tc_resident_b ? 1 : 0;
     d.tc_pair = o->tc_pair ? 1 : 0;
     cudaError_t e;
@@ -1128,6 +1131,14 @@ int tn_plan_set_tc_resident_b(tn_plan_t plan, int32_t enable) {
     if (!plan) return set_err(TN_EINVAL, "tn_plan_set_tc_resident_b: null plan");
     PlanObj *o = reinterpret_cast<PlanObj *>(plan);
     o->tc_resident_b = enable != 0;
+    o->drop_graphs();
+    return TN_OK;
+}
+
+int tn_plan_set_tc_fp32(tn_plan_t plan, int32_t enable) {
+    if (!plan) return set_err(TN_EINVAL, "tn_plan_set_tc_fp32: null plan");
+    PlanObj *o = reinterpret_cast<PlanObj *>(plan);
+    o->tc_fp32 = enable != 0;
     o->drop_graphs();
     return TN_OK;
 }

@@ -15,6 +15,9 @@
 //   BF16x3 : x = hi + lo with hi = bf16(x), lo = bf16(x - hi); three
 //            kind::f16 products hi*hi + hi*lo + lo*hi into the same FP32
 //            accumulator.
+//   BF16x6 : FP32 operands, x = h + m + l in three bf16 parts, which hold all
+//            24 bits; six products (h h, h m, m h, m m, h l, l h), a tile's
+//            sum cut into units that are added in FP32 registers.
 //
 // Tile: 128 rows x 64 complex columns (MMA M = 128, N = 128), K in chunks
 // of 16 complex (32 real).  A arrives by TMA as 128 rows of 128 bytes in
@@ -38,11 +41,9 @@
 // Every mbarrier wait is bounded; on timeout the kernel records an error
 // code in *err, skips the remaining work, frees its TMEM and returns.
 #include <algorithm>
-#include <type_traits>
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
-#include <cuda_fp16.h>
 
 #include "kernels.cuh"
 #include "plan.hpp"
@@ -282,7 +283,7 @@ constexpr int META_WARP = 18; // warp 19 idles
 constexpr int NTHREADS = 640;
 // Register split (setmaxnreg, per warpgroup).  The block is launched with
 // 96 registers a thread (640 x 96 = 61440); after the split: producers
-// 256 x 88 + epilogue 256 x 112 + control warpgroup 128 x 72 = 60416.  FP16x3
+// 256 x 88 + epilogue 256 x 112 + control warpgroup 128 x 72 = 60416.  BF16x6
 // (packed B only) has no B loaders: warps 4-7 keep 24 (they leave at once) and
 // the epilogue, which also sums a tile's units in registers, takes 144.
 constexpr int LAUNCH_REGS = 96, PROD_REGS = 88, CTL_REGS = 72;
@@ -298,13 +299,15 @@ constexpr int NACC_MAX = 8;   // accumulators in TMEM (narrow tiles: up to 8 in 
 constexpr int TMEM_COLS2 = 256;  // accumulators
 // BF16x3 also keeps the split A chunks in TMEM, 32 columns a stage after
 // the accumulators (at most 8 stages), so it allocates all 512 columns
-constexpr int TM_A = TMEM_COLS2, TM_ASTAGE = 32;
+constexpr int TM_A = TMEM_COLS2;
+// a stage: two K steps (16 real k) of 8 columns per part
+__host__ __device__ constexpr int tm_astage(int prec) { return prec == 3 ? 48 : 32; }
 // resident B: the TMEM A stages (8) run apart from the TMA ring (the ring
 // slot is free once the producers have read it), so the A stream runs up
 // to nrs + 8 chunks ahead of the MMAs; packed B ties a stage to its ring
 // slot (the slot also holds the chunk's B)
 constexpr int NTS = 8;
-static_assert(TM_A + NTS * TM_ASTAGE <= 512, "TMEM A stages within the allocation");
+static_assert(TM_A + NTS * tm_astage(2) <= 512, "TMEM A stages within the allocation");
 template <int PREC>
 __host__ __device__ constexpr uint32_t tmem_alloc_cols() { return PREC >= 2 ? 512u : uint32_t(TMEM_COLS2); }
 
@@ -321,6 +324,7 @@ struct Cfg {
     static constexpr int SLOT_RAW = TBM * TBK * 8;    // FP32 A chunk: 128 rows x 128 bytes, 128-byte swizzle
     static constexpr int SLOT_B = TBNR * TBKR * 4;    // one B chunk in MMA form (TF32, or BF16 hi + lo)
     static constexpr int SLOT_BRAW = TBN * TBK * 8;   // raw complex64 B chunk
+    static constexpr int PACK_B = PREC == 3 ? TBNR * TBKR * 6 : SLOT_B;  // packed B chunk (BF16x6: three planes)
     static constexpr int STAGE = 8 * 32 * 16 * 8;     // 4 KB per epilogue warp, in destination order
     static constexpr int NSLOT = 11;                  // resident-B pool
     static constexpr int OFF_RAW = 0;
@@ -333,11 +337,16 @@ struct Cfg {
 };
 constexpr int BRES_MAX_B = 8;  // resident B: at most 8 chunks (nct x nch), so at least 3 A stages
 constexpr int PACK_ST = 5;     // packed B: 5 stages of (A chunk, B chunk) in the pool
+constexpr int PACK_ST6 = 4;    // BF16x6: 4 of (16 KB, 24 KB)
+__host__ __device__ constexpr int pack_stages(int prec) { return prec == 3 ? PACK_ST6 : PACK_ST; }
 // packed B, column-tile pairs (MODE 4): 3 stages of (A chunk, B chunk of
 // 256 real columns = 2 slots): slots 0-2 A, 3-8 B
 constexpr int PAIR_ST = 3;
 static_assert(2 * PACK_ST <= Cfg<2, true>::NSLOT && PACK_ST <= Cfg<2, true>::RST, "packed-B stages fit the pool");
 static_assert(3 * PAIR_ST <= Cfg<2, true>::NSLOT, "paired packed-B stages fit the pool");
+static_assert(PACK_ST6 * (Cfg<3, true>::SLOT_RAW + Cfg<3, true>::PACK_B) <= Cfg<3, true>::NSLOT * Cfg<3, true>::SLOT_RAW &&
+                  TM_A + PACK_ST6 * tm_astage(3) <= 512,
+              "BF16x6 stages fit the pool and TMEM");
 
 // Per-tile epilogue metadata, written by the metadata warp into a ring of
 // MS slots ahead of the epilogue.
@@ -515,39 +524,40 @@ struct TileIter {
 // spread over the banks
 __device__ __forceinline__ int stage_swz(int u) { return u ^ (((u >> 3) ^ (u >> 6)) & 7); }
 
-// x = hi + lo in 16-bit halves, rounded to nearest: 16 bits of x in bf16
-// (FP32's range), 22 in fp16 (x scaled into its range)
-__device__ __forceinline__ void split_half(float x, __nv_bfloat16 &h, __nv_bfloat16 &l) {
-    h = __float2bfloat16_rn(x);
-    l = __float2bfloat16_rn(x - __bfloat162float(h));
+// x = h + l (BF16x3: 16 bits of x) or h + m + l (BF16x6: all 24, exact) in
+// bf16 parts, each the rest so far rounded to nearest
+template <int P>
+__device__ __forceinline__ void split_bf16(float x, __nv_bfloat16 (&part)[P]) {
+#pragma unroll
+    for (int q = 0; q < P; ++q) {
+        part[q] = __float2bfloat16_rn(x);
+        x -= __bfloat162float(part[q]);  // exact
+    }
 }
-__device__ __forceinline__ void split_half(float x, __half &h, __half &l) {
-    h = __float2half_rn(x);
-    l = __float2half_rn(x - __half2float(h));
+template <int P>
+__device__ __forceinline__ void split_pair_bf16(float x, float y, uint32_t (&word)[P]) {
+#pragma unroll
+    for (int q = 0; q < P; ++q) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+        const float2 f = __bfloat1622float2(h);
+        x -= f.x;
+        y -= f.y;
+        word[q] = *reinterpret_cast<const uint32_t *>(&h);
+    }
 }
-__device__ __forceinline__ void split_pair_bf16(float x, float y, uint32_t &hw, uint32_t &lw) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
-    const float2 hf = __bfloat1622float2(h);
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(x - hf.x, y - hf.y);
-    hw = *reinterpret_cast<const uint32_t *>(&h);
-    lw = *reinterpret_cast<const uint32_t *>(&lo);
-}
-__device__ __forceinline__ void split_pair_f16(float x, float y, uint32_t &hw, uint32_t &lw) {
-    const __half2 h = __floats2half2_rn(x, y);
-    const float2 hf = __half22float2(h);
-    const __half2 lo = __floats2half2_rn(x - hf.x, y - hf.y);
-    hw = *reinterpret_cast<const uint32_t *>(&h);
-    lw = *reinterpret_cast<const uint32_t *>(&lo);
-}
-// FP16x3 operands are scaled by 2^(14 - e), e the exponent of the
-// instance's largest component: below 2^15, and exact down to 2^-40 of it
-constexpr float HALF_TOP = 16384.f, HALF_UNSCALE = 1.f / (16384.f * 16384.f);
+__host__ __device__ constexpr int n_parts(int prec) { return prec == 3 ? 3 : 2; }
+// BF16x6 operands are scaled by 2^(40 - e), e the exponent of the instance's
+// largest component: products and their sums stay far from overflow, and an
+// entry down to 2^-143 of the largest keeps its last part above the
+// subnormals, so that every entry that FP32 holds is split exactly.
+constexpr float SPLIT_TOP = 0x1p40f, SPLIT_UNSCALE = 0x1p-80f;
 
 // One producer thread's B piece: column bcol, complex k 4 kqb .. 4 kqb + 3
 // of a chunk (p0, p1 = the four values), expanded into the real 2x2 form
 // (rows 2 bcol: Re, -Im; 2 bcol + 1: Im, Re) in the K-major no-swizzle
 // layout of a B chunk of nr rows (MMA N: 128, or 256 for a column-tile
-// pair); BF16x3 stores the hi plane, then the lo plane nr x 64 bytes on.
+// pair); BF16x3 stores the hi plane, then the lo plane nr x 64 bytes on,
+// BF16x6 its three planes likewise.
 template <int PREC, bool RM = false>
 __device__ __forceinline__ void expand_b(uint8_t *base, int bcol, int kqb, const float4 p0, const float4 p1,
                                          int nr = TBNR) {
@@ -570,34 +580,40 @@ __device__ __forceinline__ void expand_b(uint8_t *base, int bcol, int kqb, const
         *reinterpret_cast<float4 *>(base + off(rb, 8 * kqb, 4)) = sw ? a0 : b0;
         *reinterpret_cast<float4 *>(base + off(rb, 8 * kqb + 4, 4)) = sw ? a1 : b1;
     } else {
-        using H = std::conditional_t<PREC == 3, __half, __nv_bfloat16>;
-        __align__(16) H h0[8], l0[8], h1[8], l1[8];
+        constexpr int P = n_parts(PREC);
+        __align__(16) __nv_bfloat16 e0[P][8], e1[P][8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            split_half(r0[q], h0[q], l0[q]);
-            split_half(r1[q], h1[q], l1[q]);
+            __nv_bfloat16 s0[P], s1[P];
+            split_bf16<P>(r0[q], s0);
+            split_bf16<P>(r1[q], s1);
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                e0[p][q] = s0[p];
+                e1[p][q] = s1[p];
+            }
         }
-        uint8_t *blo = base + nr * TBKR * 2;
-        const uint4 H0 = *reinterpret_cast<uint4 *>(h0), L0 = *reinterpret_cast<uint4 *>(l0);
-        const uint4 H1 = *reinterpret_cast<uint4 *>(h1), L1 = *reinterpret_cast<uint4 *>(l1);
         const uint32_t oa = off(ra, 8 * kqb, 2), ob = off(rb, 8 * kqb, 2);
-        *reinterpret_cast<uint4 *>(base + oa) = sw ? H1 : H0;
-        *reinterpret_cast<uint4 *>(blo + oa) = sw ? L1 : L0;
-        *reinterpret_cast<uint4 *>(base + ob) = sw ? H0 : H1;
-        *reinterpret_cast<uint4 *>(blo + ob) = sw ? L0 : L1;
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            uint8_t *plane = base + p * nr * TBKR * 2;
+            const uint4 E0 = *reinterpret_cast<uint4 *>(e0[p]), E1 = *reinterpret_cast<uint4 *>(e1[p]);
+            *reinterpret_cast<uint4 *>(plane + oa) = sw ? E1 : E0;
+            *reinterpret_cast<uint4 *>(plane + ob) = sw ? E0 : E1;
+        }
     }
 }
 
-// BF16x3: the A operand goes to tensor memory.  A chunk arrives by TMA as
+// BF16x3 and BF16x6: the A operand goes to tensor memory.  A chunk arrives by TMA as
 // 128 rows of 32 real k (128 bytes, 128-byte swizzle).  The A stage in TMEM
-// is 32 columns (128 lanes = rows): K step h (16 real k, 8 columns of
-// packed bf16 pairs, lower k in the low half) holds hi in columns
-// 16 h .. 16 h + 7 and lo in the next 8.  The MMAs then read only B from
-// shared memory.
+// is 32 columns (BF16x6: 48; 128 lanes = rows): K step h (16 real k, 8
+// columns of packed bf16 pairs a part, lower k in the low half) holds its
+// first part in columns 8 P h .. 8 P h + 7, P parts, and each other in the
+// next 8.  The MMAs then read only B from shared memory.
 //
 // Quarter q (real k 8 q .. 8 q + 7, logical 16-byte units 2 q, 2 q + 1) of
-// this thread's row: read from the swizzled slot, split into hi and lo,
-// stored to hi columns 16 (q / 2) + 4 (q % 2) .. + 3 and the lo columns 8
+// this thread's row: read from the swizzled slot, split into its parts, the
+// first stored to columns 8 P (q / 2) + 4 (q % 2) .. + 3 and each other 8
 // further on, relative to ta (this lane's row of the stage).  tcgen05.st is
 // warp-wide (.sync.aligned).
 template <int PREC>
@@ -607,21 +623,21 @@ __device__ __forceinline__ void split_a_quarter(const uint8_t *slot, int row, in
     const float4 v0 = *reinterpret_cast<const float4 *>(rowp + (((2 * q) ^ sw) << 4));
     const float4 v1 = *reinterpret_cast<const float4 *>(rowp + (((2 * q + 1) ^ sw) << 4));
     const float x[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-    uint32_t hw[4], lw[4];
+    constexpr int P = n_parts(PREC);
+    uint32_t w[4][P];
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
         if (PREC == 3)  // s: 2^-e of the instance
-            split_pair_f16(x[2 * p] * s * HALF_TOP, x[2 * p + 1] * s * HALF_TOP, hw[p], lw[p]);
+            split_pair_bf16<P>(x[2 * p] * s * SPLIT_TOP, x[2 * p + 1] * s * SPLIT_TOP, w[p]);
         else
-            split_pair_bf16(x[2 * p], x[2 * p + 1], hw[p], lw[p]);
+            split_pair_bf16<P>(x[2 * p], x[2 * p + 1], w[p]);
     }
-    const uint32_t c = ta + uint32_t(16 * (q >> 1) + 4 * (q & 1));
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(c), "r"(hw[0]), "r"(hw[1]),
-                 "r"(hw[2]), "r"(hw[3])
-                 : "memory");
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(c + 8u), "r"(lw[0]), "r"(lw[1]),
-                 "r"(lw[2]), "r"(lw[3])
-                 : "memory");
+    const uint32_t c = ta + uint32_t(8 * P * (q >> 1) + 4 * (q & 1));
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(c + uint32_t(8 * p)),
+                     "r"(w[0][p]), "r"(w[1][p]), "r"(w[2][p]), "r"(w[3][p])
+                     : "memory");
 }
 
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -755,7 +771,7 @@ __device__ __forceinline__ void fold_max16(const uint32_t (&r)[32], EpiMeta &em,
     }
 }
 
-template <int PREC, int MODE, int UC = 1>  // UC: FP16x3, chunks of a unit
+template <int PREC, int MODE, int UC = 1>  // UC: BF16x6, chunks of a unit
 __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 warps on a sub-partition)
     k_step_gemm_tc(const __grid_constant__ StepDesc d, int64_t mtiles, int32_t *err, const __grid_constant__ CUtensorMap tmA, int nrs,
                    int acw, int ow, int tblk) {
@@ -774,20 +790,20 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
     // MODE 3: B packed in MMA form in global memory (tc_pack_b, once per
     // launch) and bulk-copied chunk by chunk beside A from L2, B carrying
     // 2^-eb
-    // PREC 3, FP16x3 for FP32 steps (MODE 3 only): operands scaled by powers of
-    // two and split into fp16 halves.  The tensor cores truncate each sum into
-    // the accumulator (relative L2 error 1.0e-6 over 1024 real k of random
-    // signs, the FMA kernel 2.5e-7; 6.5e-8 over 64), so a unit of one chunk
-    // (32 real k; K >= 512: two) starts from zero, its small products first,
-    // and the epilogue adds the units in FP32 registers, rounded to nearest:
-    // the contraction's error is below the FMA kernel's.
-    // Bound by a unit's chain of load, split, MMAs and drain over two
-    // accumulators (tensor pipe 26 %, L2 21 %, shared memory 18 %).
-    // 53-qubit circuit, FP32: 2^12 x 2^9 x 2^8 with 512 instances 48 -> 7.4 ms,
-    // all of it 228 -> 48.4 ms.
+    // PREC 3, BF16x6 for FP32 steps (MODE 3 only): operands scaled by powers of
+    // two and split into three bf16 parts, which hold every bit of them; of
+    // the nine products the three below 2^-24 of the whole are left out.  The
+    // tensor cores truncate each sum into the accumulator (relative L2 error
+    // 1.0e-6 over 1024 real k of random signs, the FMA kernel 2.5e-7; 6.5e-8
+    // over 64), so a unit of one chunk (32 real k; K >= 128: two) starts from
+    // zero, its small products first, and the epilogue adds the units in FP32
+    // registers, rounded to nearest: the error is below the FMA kernel's (0.8
+    // of it over 45 random plans of 16 to 20 qubits, also where entries 2^-80
+    // of an instance's largest decide; 1.53e-6 and 1.68e-6 on 53 qubits).
+    // 53-qubit circuit, FP32, all of it: 230 ms on the FMA kernel, 64.5 here.
     constexpr int EPI_REGS = epi_regs(PREC);
     constexpr bool ASPLIT = PREC >= 2;  // A split into TMEM
-    static_assert(PREC != 3 || MODE == 3, "FP16x3: packed B");
+    static_assert(PREC != 3 || MODE == 3, "BF16x6: packed B");
     constexpr bool BRES = MODE == 1 || MODE == 2;
     // MODE 4: packed B with two adjacent column tiles of a row tile (one B
     // instance's 128 columns, or with N = 64 two instances' 64) per MMA of
@@ -803,6 +819,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment: the swizzled A slots are whole 8-row atoms
     uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    // packed B: stage st's chunk, behind the A slots
+    auto packed_b = [sm](int st) {
+        return sm + C::OFF_RAW + (PAIR ? (PAIR_ST + 2 * st) * C::SLOT_RAW : pack_stages(PREC) * C::SLOT_RAW + st * C::PACK_B);
+    };
     Ctrl &X = *reinterpret_cast<Ctrl *>(sm + C::OFF_CTRL);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t n_tiles = (PP ? d.n_ptab : d.n_ctab) * mtiles;
@@ -952,7 +972,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                     const int64_t i0 = int64_t(r.x) + (r.w >> d.nb);
                     const int ib = __ldg(d.instab + i0).y;
                     if (PREC == 3 && d.nb < 6) {  // packed per column tile
-                        bsrc = d.bpack + (it.f + it.ct) * nch * int64_t(C::SLOT_B);
+                        bsrc = d.bpack + (it.f + it.ct) * nch * int64_t(C::PACK_B);
                     } else if (PP) {
                         // N = 64: tile ct is instance ct of the group; the
                         // pad tile (odd groups) repeats the first tile's B
@@ -965,7 +985,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                         // this column tile (pair) are consecutive
                         const int pb = PAIR ? 7 : 6;
                         const int64_t blk = (int64_t(ib) << (d.nb - pb)) + ((r.w & (N - 1)) >> pb);
-                        bsrc = d.bpack + blk * nch * int64_t(TSTEP * C::SLOT_B);
+                        bsrc = d.bpack + blk * nch * int64_t(TSTEP * C::PACK_B);
                     }
                     fprev = it.f;
                     ctprev = it.ct;
@@ -975,9 +995,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                         ok = false;
                         break;
                     }
-                    mbar_expect_tx(&X.rfull[rs], BPACK ? C::SLOT_RAW + TSTEP * C::SLOT_B : C::SLOT_RAW);
+                    mbar_expect_tx(&X.rfull[rs], BPACK ? C::SLOT_RAW + TSTEP * C::PACK_B : C::SLOT_RAW);
                     tma_load_3d(smem_u32(sm + C::OFF_RAW + rs * C::SLOT_RAW), &tmA, TBKR * c, m0, r.z, &X.rfull[rs]);
-                    const uint32_t bdst = smem_u32(sm + C::OFF_RAW + (PAIR ? PAIR_ST + 2 * rs : PACK_ST + rs) * C::SLOT_RAW);
+                    const uint32_t bdst = smem_u32(packed_b(rs));
                     if (PP) {  // hi planes of both tiles, then both lo planes
                         constexpr int PL = C::SLOT_B / 2;
                         const uint8_t *s0 = bsrc + int64_t(c) * C::SLOT_B, *s1 = bsrc1 + int64_t(c) * C::SLOT_B;
@@ -986,7 +1006,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                         bulk_load(bdst + 2 * PL, s0 + PL, PL, &X.rfull[rs]);
                         bulk_load(bdst + 3 * PL, s1 + PL, PL, &X.rfull[rs]);
                     } else if (BPACK) {
-                        bulk_load(bdst, bsrc + c * TSTEP * C::SLOT_B, TSTEP * C::SLOT_B, &X.rfull[rs]);
+                        bulk_load(bdst, bsrc + c * TSTEP * C::PACK_B, TSTEP * C::PACK_B, &X.rfull[rs]);
                     }
                     if (++rs == nrs) {
                         rs = 0;
@@ -1014,9 +1034,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
         const uint32_t ta_row = tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(TM_A);
         // one chunk of A from the TMA slot into TMEM stage `stage` (both K
         // steps); the slot is released once read (rel: its barrier, or null)
-        float sa = 1.f;  // FP16x3: the tile's A scale
+        float sa = 1.f;  // BF16x6: the tile's A scale
         auto a_to_tmem = [&](const uint8_t *slot, int stage, uint64_t *rel) {
-            const uint32_t ta = ta_row + uint32_t(stage * TM_ASTAGE);
+            const uint32_t ta = ta_row + uint32_t(stage * tm_astage(PREC));
             split_a_quarter<PREC>(slot, arow, 0, ta, sa);
             split_a_quarter<PREC>(slot, arow, 1, ta, sa);
             split_a_quarter<PREC>(slot, arow, 2, ta, sa);
@@ -1229,7 +1249,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
             // the A operand of a chunk: TF32, the TMA slot; BF16x3, the TMEM stage
             auto a_of = [&](int rs, int tstage) {
                 return PREC == 1 ? smem_u32(sm + C::OFF_RAW + rs * C::SLOT_RAW)
-                                 : tmem + uint32_t(TM_A + tstage * TM_ASTAGE);
+                                 : tmem + uint32_t(TM_A + tstage * tm_astage(PREC));
             };
             bool ok = true;
             if constexpr (BRES || BPACK) {
@@ -1251,7 +1271,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                             break;
                         }
                         tc_fence_after();
-                        const uint32_t dtm = tmem + uint32_t(acc) * awr, id = idesc(0u, awr);
+                        const uint32_t dtm = tmem + uint32_t(acc) * awr, id = idesc(1u, awr);
                         int st[UC];
                         for (int c = 0; c < UC; ++c) {
                             st[c] = ts;
@@ -1266,25 +1286,22 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                         }
                         if (!ok) break;
                         tc_fence_after();
-                        // hi lo and lo hi of both chunks first, then hi hi
+                        // parts i of A and j of B: those with i + j = 2
+                        // of every chunk first, then 1, then 0
 #pragma unroll
-                        for (int h = 0; h < 2; ++h)
+                        for (int ij = 2; ij >= 0; --ij)
 #pragma unroll
                             for (int c = 0; c < UC; ++c) {
-                                const uint32_t a0 = tmem + uint32_t(TM_A + st[c] * TM_ASTAGE);
-                                const uint32_t b0 = smem_u32(sm + C::OFF_RAW + (PACK_ST + st[c]) * C::SLOT_RAW);
-                                const uint32_t bl = b0 + TBNR * TBKR * 2;
+                                const uint32_t a0 = tmem + uint32_t(TM_A + st[c] * tm_astage(PREC));
+                                const uint32_t b0 = smem_u32(packed_b(st[c]));
 #pragma unroll
-                                for (int j = 0; j < TBKR / 16; ++j) {
-                                    const uint32_t off = uint32_t(2 * j) * LBO;
-                                    const uint32_t ah = a0 + uint32_t(16 * j), al = ah + 8u;
-                                    if (h == 0) {
-                                        mma_f16_ts(dtm, ah, sdesc(bl + off, LBO, SBO), id, (c > 0 || j > 0) ? 1u : 0u);
-                                        mma_f16_ts(dtm, al, sdesc(b0 + off, LBO, SBO), id, 1u);
-                                    } else {
-                                        mma_f16_ts(dtm, ah, sdesc(b0 + off, LBO, SBO), id, 1u);
-                                    }
-                                }
+                                for (int k = 0; k < TBKR / 16; ++k)
+#pragma unroll
+                                    for (int i = 0; i <= ij; ++i)
+                                        mma_f16_ts(dtm, a0 + uint32_t(8 * (3 * k + i)),
+                                                   sdesc(b0 + uint32_t((ij - i) * TBNR * TBKR * 2) +
+                                                             uint32_t(2 * k) * LBO, LBO, SBO),
+                                                   id, (ij < 2 || c > 0 || k > 0 || i > 0) ? 1u : 0u);
                             }
                         for (int c = 0; c < UC; ++c) {
                             mma_commit(&X.taempty[st[c]]);
@@ -1329,7 +1346,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                         }
                         tc_fence_after();
                         const uint32_t bch =
-                            BPACK ? smem_u32(sm + C::OFF_RAW + (PAIR ? PAIR_ST + 2 * rs : PACK_ST + rs) * C::SLOT_RAW)
+                            BPACK ? smem_u32(packed_b(rs))
                                   : bset + c * C::SLOT_RAW;
                         if (PAIR)
                             issue_pair(dtm, a_of(rs, ts), bch, c == 0);
@@ -1455,8 +1472,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
                 const int inst = inst_c[q];
                 em.inst[c] = inst;
                 em.mx[c] = 0u;
-                // dictionary and packed B carry 2^-eb, FP16x3 A 2^-ea as well
-                em.sc[c] = PREC == 3 ? HALF_UNSCALE : pow2f(-(ea_c + (MODE >= 2 ? 0 : eb_c[q])));
+                // dictionary and packed B carry 2^-eb, BF16x6 A 2^-ea as well
+                em.sc[c] = PREC == 3 ? SPLIT_UNSCALE : pow2f(-(ea_c + (MODE >= 2 ? 0 : eb_c[q])));
                 if (MODE == 2) em.acol[c] = int16_t(inst >= 0 ? (ib_c[q] << d.nb) + ((w_c + c) & (N - 1)) : 0);
                 if (inst >= 0 && it.mt == 0 && ((int64_t(w_c) + c) & (N - 1)) == 0)
                     d.EC[inst] = EA_c + ea_c + EB_c[q] + eb_c[q];
@@ -1543,7 +1560,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
             // (non-dictionary tiles of 8 columns: one)
             const int npass = (MODE != 2 && acw < 16) ? 1 : 2;
             constexpr int HALVES = PREC == 3 ? 2 : 1;
-            uint32_t sum[HALVES][32];  // FP16x3: the tile's sums (float bits)
+            uint32_t sum[HALVES][32];  // BF16x6: the tile's sums (float bits)
             if constexpr (PREC == 3) {
 #pragma unroll
                 for (int i = 0; i < 64; ++i) sum[i >> 5][i & 31] = 0u;
@@ -1733,19 +1750,19 @@ __global__ void __launch_bounds__(256) k_pack_b(const StepDesc d, int nch) {
     const int K = 1 << d.kb;
     const int k = c * TBK + 4 * kqb;
     const float s = d.mxB ? pow2f(-exp_of(__ldg(d.mxB + ib))) : 1.f;
-    constexpr float t = PREC == 3 ? HALF_TOP : 1.f;
+    constexpr float t = PREC == 3 ? SPLIT_TOP : 1.f;
     float4 p0 = make_float4(0.f, 0.f, 0.f, 0.f), p1 = p0;
     if (k + 3 < K) {
         const float4 *src = reinterpret_cast<const float4 *>(d.B + ib * d.sB + (n << d.kb) + k);
         p0 = __ldg(src);
         p1 = __ldg(src + 1);
     }
-    expand_b<PREC, RM>(d.bpack + blk * (TBNR * TBKR * 4), bcol, kqb,
+    expand_b<PREC, RM>(d.bpack + blk * Cfg<PREC, true>::PACK_B, bcol, kqb,
                    make_float4(p0.x * s * t, p0.y * s * t, p0.z * s * t, p0.w * s * t),
                    make_float4(p1.x * s * t, p1.y * s * t, p1.z * s * t, p1.w * s * t));
 }
 
-// Packed B of steps with N < 64 (FP16x3): the columns of a column tile are
+// Packed B of steps with N < 64 (BF16x6): the columns of a column tile are
 // those of several instances of its group; block tile * nch + chunk.
 __global__ void __launch_bounds__(256) k_pack_b_tiles(const StepDesc d, int nch) {
     const int tid = threadIdx.x, bcol = tid & 63, kqb = tid >> 6;
@@ -1760,10 +1777,10 @@ __global__ void __launch_bounds__(256) k_pack_b_tiles(const StepDesc d, int nch)
             d.B + ib * d.sB + ((gc & ((1 << d.nb) - 1)) << d.kb) + c * TBK + 4 * kqb);
         p0 = __ldg(src);
         p1 = __ldg(src + 1);
-        p0 = make_float4(p0.x * s * HALF_TOP, p0.y * s * HALF_TOP, p0.z * s * HALF_TOP, p0.w * s * HALF_TOP);
-        p1 = make_float4(p1.x * s * HALF_TOP, p1.y * s * HALF_TOP, p1.z * s * HALF_TOP, p1.w * s * HALF_TOP);
+        p0 = make_float4(p0.x * s * SPLIT_TOP, p0.y * s * SPLIT_TOP, p0.z * s * SPLIT_TOP, p0.w * s * SPLIT_TOP);
+        p1 = make_float4(p1.x * s * SPLIT_TOP, p1.y * s * SPLIT_TOP, p1.z * s * SPLIT_TOP, p1.w * s * SPLIT_TOP);
     }
-    expand_b<3>(d.bpack + int64_t(blockIdx.x) * (TBNR * TBKR * 4), bcol, kqb, p0, p1);
+    expand_b<3>(d.bpack + int64_t(blockIdx.x) * Cfg<3, true>::PACK_B, bcol, kqb, p0, p1);
 }
 
 // Packed B for column-tile pairs (MODE 4): 128 columns x 16 complex k per
@@ -1810,16 +1827,16 @@ bool gemm_tc_supports(const StepDesc &d) {
 
 bool tc_fp32_takes(const StepDesc &d) {
     // K >= 64: below, the FMA kernel's rounding (5.1e-8 over 64 real k) is
-    // less than the split's and a unit's.  N < 64: several instances' columns
+    // less than a unit's.  N < 64: several instances' columns
     // share a tile, half of it at least on average.  Any number of tiles: one
     // instance of 2^9 x 64 x 2^7 takes 24.7 us with its B's packing, 26.6 on
     // the FMA kernel, 2^16 x 64 x 64 36.7 and 81.8
-    if (d.sched != 0 || !d.tc_resident_b || d.kb < tnp::TC_FP32_MIN_KB || !gemm_tc_supports(d) || !d.mxA ||
+    if (d.sched != 0 || !d.tc_resident_b || !d.tc_fp32 || d.kb < tnp::TC_FP32_MIN_KB || !gemm_tc_supports(d) || !d.mxA ||
         !d.mxB || !d.bpack)
         return false;
-    if (d.nb >= 6) return tc_packed_b_bytes(d) <= d.bpack_bytes;
+    if (d.nb >= 6) return tc_packed_b_bytes(d) / 4 * 6 <= d.bpack32_bytes;
     return (d.nInst << d.nb) >= 32 * d.n_groups &&
-           ((d.n_ctab << (d.kb - 4)) * int64_t(TBNR * TBKR * 4)) <= d.bpack_bytes;
+           ((d.n_ctab << (d.kb - 4)) * int64_t(Cfg<3, true>::PACK_B)) <= d.bpack32_bytes;
 }
 
 int tc_dictionary_chunks(const StepDesc &d) {
@@ -1939,16 +1956,16 @@ cudaError_t launch_step_gemm_tc(const StepDesc &d, const CUtensorMap *a_map, int
             k_pack_b<3><<<dim3((unsigned)blocks), 256, 0, s>>>(d, nch);
         else
             k_pack_b_tiles<<<dim3((unsigned)blocks), 256, 0, s>>>(d, nch);
-        // Chunks of a unit: two where the FMA kernel's own rounding is largest
+        // Chunks of a unit: two where the FMA kernel's own rounding is larger
         // (53-qubit circuit, relative L2 error over 320 oracle amplitudes and
-        // time: FMA 1.71e-6, 228 ms; two from K = 128 on 1.76e-6, 45.9; from
-        // K = 512 on 1.57e-6, 48.4; one always 1.51e-6, about 52)
+        // time: FMA 1.68e-6, 230 ms; two from K = 128 on 1.53e-6, 64.5; from
+        // K = 256 on 1.45e-6, 67.2; one always 1.34e-6, 72.3)
         const int step = b >= 2 ? 2 : 1;
-        if (d.kb >= 9)
-            k_step_gemm_tc<3, 3, 2><<<g, NTHREADS, smem_bytes<3, true>(), s>>>(d, mtiles, err, *a_map, PACK_ST, TBN,
+        if (d.kb >= 7)
+            k_step_gemm_tc<3, 3, 2><<<g, NTHREADS, smem_bytes<3, true>(), s>>>(d, mtiles, err, *a_map, PACK_ST6, TBN,
                                                                                TBN, step);
         else
-            k_step_gemm_tc<3, 3, 1><<<g, NTHREADS, smem_bytes<3, true>(), s>>>(d, mtiles, err, *a_map, PACK_ST, TBN,
+            k_step_gemm_tc<3, 3, 1><<<g, NTHREADS, smem_bytes<3, true>(), s>>>(d, mtiles, err, *a_map, PACK_ST6, TBN,
                                                                                TBN, step);
         return cudaGetLastError();
     }

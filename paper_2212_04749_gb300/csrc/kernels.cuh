@@ -26,6 +26,7 @@ struct StepDesc {
     const int32_t *outA, *outB;   // [nOut]
     int32_t nOutA, nOutB, nOut;
     int32_t sched;                // schedule variant of the step's kernel (0 or 1; the autotuner's choice)
+    int32_t tc_fp32;              // FP32 steps may take the tensor cores (BF16x6)
     int32_t tc_resident_b;        // tensor cores: keep B resident in shared memory where it fits
     int32_t tc_pair;              // tensor cores: BF16x3 packed B, schedule 0, N >= 64, K >= 256: column tiles in pairs (N = 256 MMAs)
     int32_t pad_;
@@ -53,7 +54,7 @@ struct StepDesc {
     int64_t inst0, tile0, ptile0;
     int64_t packB0, packBn;       // B instances that a packed B has to hold
     uint8_t *bpack;               // tensor cores: scratch for B packed in MMA form (null: none)
-    int64_t bpack_bytes;
+    int64_t bpack_bytes, bpack32_bytes;  // of it for TF32 and BF16x3, for FP32
     int8_t pAm[40];
     int8_t pBn[24];
     int8_t pCm[40];

@@ -658,12 +658,17 @@ struct Builder {
         }
     }
 
-    // FP32 steps that pack B per column tile (gemm_tc.cu): N < 64, wide groups
-    bool packs_tiles(const Step &st) const {
-        return st.nb < 6 && st.kb >= TC_FP32_MIN_KB && st.kb <= 24 && st.mb >= 6 && st.mb <= 30 &&
-               (P.nodes[st.node].n_inst << st.nb) >= 32 * int64_t(st.n_groups);
+    // Bytes of a step's B packed for FP32 on the tensor cores (gemm_tc.cu: 24
+    // KB a chunk; per column tile where N < 64 and groups are wide), 0 if it
+    // does not go there.
+    int64_t pack32_bytes(const Step &st) const {
+        if (st.kb < TC_FP32_MIN_KB || st.kb > 24 || st.mb < 6 || st.mb > 30) return 0;
+        const int64_t chunks = (int64_t(1) << (st.kb - 4)) * 24576;
+        if (st.nb >= 6) return P.nodes[st.b].n_inst * (int64_t(1) << (st.nb - 6)) * chunks;
+        if ((P.nodes[st.node].n_inst << st.nb) < 32 * int64_t(st.n_groups)) return 0;
+        return int64_t(st.col_tiles.size()) * chunks;
     }
-    bool pack_tiles = false;  // room for them
+    bool pack32 = false;  // room for them
 
     // Workspace layout; returns total bytes.  own_slots: the outputs of small
     // steps share no memory with other intermediates.
@@ -899,13 +904,13 @@ struct Builder {
             const int64_t bytes = p.nodes[st.b].n_inst * (int64_t(1) << (st.nb - 6)) * nch * 16384;
             if (bytes <= bpack_cap) p.bpack_bytes = std::max(p.bpack_bytes, bytes);
         }
-        if (pack_tiles)  // N < 64: packed per column tile (FP32 steps)
+        p.bpack32_bytes = p.bpack_bytes;
+        if (pack32)  // half as much again as the 16 KB a chunk above
             for (const Step &st : p.steps) {
-                if (!packs_tiles(st)) continue;
-                const int64_t bytes = int64_t(st.col_tiles.size()) * (int64_t(1) << (st.kb - 4)) * 16384;
-                if (bytes <= bpack_cap) p.bpack_bytes = std::max(p.bpack_bytes, bytes);
+                const int64_t bytes = pack32_bytes(st);
+                if (bytes <= bpack_cap / 2 * 3) p.bpack32_bytes = std::max(p.bpack32_bytes, bytes);
             }
-        p.off_bpack = p.bpack_bytes > 0 ? take(p.bpack_bytes) : -1;
+        p.off_bpack = p.bpack32_bytes > 0 ? take(p.bpack32_bytes) : -1;
         for (Chain &c : p.chains) {
             const Step &last = p.steps[c.steps.back()];
             const int64_t ni = p.nodes[last.node].n_inst;
@@ -1340,12 +1345,12 @@ bool make_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int
         if (!P.opt.fuse && crosses(plain, with)) B.drop_chains();
         else plain = with;
     }
-    // room for B packed per column tile: the same
+    // room for B packed for FP32: the same
     if (P.opt.rescale)
-        for (const Step &st : P.steps) B.pack_tiles = B.pack_tiles || B.packs_tiles(st);
-    if (B.pack_tiles) {
+        for (const Step &st : P.steps) B.pack32 = B.pack32 || B.pack32_bytes(st) > 0;
+    if (B.pack32) {
         const int64_t with = layout(false, false);
-        if (crosses(plain, with)) B.pack_tiles = false;
+        if (crosses(plain, with)) B.pack32 = false;
         else plain = with;
     }
     int64_t slots = 0;

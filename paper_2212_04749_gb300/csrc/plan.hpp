@@ -127,7 +127,7 @@ constexpr int64_t SMALL_DESC_BYTES = 160;
 // one still in use, where these slots add little to the workspace.
 constexpr int64_t SMALL_SLOTS_MAX = int64_t(32) << 20;
 
-// FP32 steps take the tensor cores (FP16x3, gemm_tc.cu) from K = 2^this on.
+// FP32 steps take the tensor cores (BF16x6, gemm_tc.cu) from K = 2^this on.
 constexpr int TC_FP32_MIN_KB = 6;
 
 // A fused chain (SM Sec. V.C): steps s_1..s_L where each step's A operand is
@@ -205,7 +205,9 @@ struct Plan {
     std::vector<int64_t> emax_prefix;       // [lv]: bytes covering the nodes of level <= lv
     int64_t off_scratch = -1;               // 256 bytes of device scratch (error word)
     int64_t off_small = -1;                 // per step: descriptor for small.cu, written at bind time
-    int64_t off_bpack = -1, bpack_bytes = 0; // tensor cores: room for one step's B packed in MMA form
+    // tensor cores: room for one step's B packed in MMA form, bpack_bytes of
+    // it for TF32 and BF16x3, bpack32_bytes (the region) for FP32
+    int64_t off_bpack = -1, bpack_bytes = 0, bpack32_bytes = 0;
     // host images uploaded at bind time: (offset, bytes)
     std::vector<std::pair<int64_t, std::vector<uint8_t>>> uploads;
 };

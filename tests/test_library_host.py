@@ -264,7 +264,7 @@ def test_tensor_core_switches(tn):
     # null plan is an argument error, and either setting leaves the plan's
     # configuration choices as they were
     lib = tn.load()
-    for fn in ("tn_plan_set_tc_resident_b", "tn_plan_set_tc_pairs"):
+    for fn in ("tn_plan_set_tc_resident_b", "tn_plan_set_tc_fp32", "tn_plan_set_tc_pairs"):
         assert getattr(lib, fn)(None, 1) == tn.TN_EINVAL
     w = make_workload("grid5x6_m14")
     p = tn.Plan(w.circuit, w.bits, w.tree.ssa, w.tree.sliced)
@@ -272,6 +272,7 @@ def test_tensor_core_switches(tn):
     for on in (False, True):
         p.tn_plan_set_tc_pairs(on)
         p.tn_plan_set_tc_resident_b(on)
+        p.tn_plan_set_tc_fp32(on)
         assert np.array_equal(p.tn_plan_get_configs(), base)
 
 
