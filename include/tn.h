@@ -468,6 +468,23 @@ int tn_plan_check(tn_plan_t plan, void *stream);
 int tn_plan_profile(tn_plan_t plan, int enable);
 int tn_plan_step_times(tn_plan_t plan, double *ms, int32_t *kernel, int32_t n);
 
+/* The kernel that each step last ran (n entries, -1: none yet).  Families of
+ * tn_plan_step_times: 0 is ROW and, under configurations 0 and 1, NARROW; 1
+ * SIMT, SKINNY, OUTER, FEW and the other NARROW; 2 TC and TC_FP32. */
+enum {
+    TN_FORM_ROW = 0,     /* k_step_row: rows in a few lanes' registers */
+    TN_FORM_SIMT = 1,    /* k_step_gemm_simt, k_step_gemm_simt2: FP32 FMA GEMM */
+    TN_FORM_TC = 2,      /* k_step_gemm_tc: TF32, BF16x3 */
+    TN_FORM_CHAIN = 3,   /* k_chain: fused chain */
+    TN_FORM_SMALL = 4,   /* k_small_steps: merged small steps */
+    TN_FORM_NARROW = 5,  /* k_step_narrow: long rows, few columns per A instance */
+    TN_FORM_OUTER = 6,   /* k_step_outer: short rows, many columns */
+    TN_FORM_SKINNY = 7,  /* k_step_skinny: few outputs per instance, long K */
+    TN_FORM_FEW = 8,     /* k_step_few: few multiply-adds, an output per thread */
+    TN_FORM_TC_FP32 = 9  /* k_step_gemm_tc: FP32 as BF16x6 */
+};
+int tn_plan_step_forms(tn_plan_t plan, int32_t *form, int32_t n);
+
 /* FP32 fused multiply-add throughput probe (no counterpart in the paper: it
  * measures the denominator of the FP32 form's roofline, the rate of the
  * CUDA cores' FP32 FMA pipes on this device).  Launches `blocks` blocks of

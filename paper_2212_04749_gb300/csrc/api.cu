@@ -50,7 +50,8 @@ struct PlanObj {
     std::vector<cudaEvent_t> ev;          // pool, two per profiled launch
     std::vector<int> ev_step;             // step of each recorded pair
     size_t ev_used = 0;
-    std::vector<int32_t> step_kernel;     // kernel family each step ran last (0 row, 1 SIMT GEMM, 2 TC GEMM)
+    std::vector<int32_t> step_kernel;     // kernel family each step ran last (tn_plan_step_times)
+    std::vector<int32_t> step_form;       // TN_FORM_* each step ran last
     std::vector<int32_t> config_override; // per step: -1 plan choice, else a configuration (tn.h)
     // per fused chain: run as one kernel (1), as its steps (0), or not chosen
     // (-1: one kernel, unless all its steps are small: those share the merged
@@ -327,6 +328,42 @@ void apply_window(const PlanObj *o, const tnp::Step &S, int64_t sigma, tnk::Step
     d.packBn = B.n_out;
 }
 
+// The kernel (TN_FORM_*) of a step under configuration cfg, and its schedule
+// (d.sched).  ruled: nobody chose the configuration; few: an output per
+// thread is allowed; map_ok: A has a TMA descriptor (FP32; the other
+// precisions fail without one).
+int step_form(tnk::StepDesc &d, int cfg, bool ruled, int precision, bool few, bool map_ok) {
+    d.sched = cfg & 1;
+    const bool skinny = tnk::step_skinny_takes(d);
+    const bool on_tc = cfg >= 2 && precision != TN_FP32 && tnk::gemm_tc_supports(d) && !skinny;
+    if (few && tnk::step_few_takes(d, on_tc)) return TN_FORM_FEW;
+    if (cfg < 2) return tnk::step_row_narrow(d) ? TN_FORM_NARROW : TN_FORM_ROW;
+    if (skinny) return TN_FORM_SKINNY;  // few outputs per instance and a long K (e.g. the root)
+    if (on_tc) {
+        if (ruled) d.sched = tnk::tc_rule_schedule(d);
+        return d.tc_resident_b && tnk::tc_dictionary_chunks(d) == 0 && tnk::tc_resident_b_chunks(d) == 0 &&
+                       tnk::step_narrow_takes(d, false)
+                   ? TN_FORM_NARROW
+                   : TN_FORM_TC;
+    }
+    if (precision == TN_FP32 && map_ok && tnk::tc_fp32_takes(d)) return TN_FORM_TC_FP32;
+    if (tnk::step_outer_takes(d)) return TN_FORM_OUTER;
+    return tnk::step_narrow_takes(d, true) ? TN_FORM_NARROW : TN_FORM_SIMT;
+}
+
+// The family (tn_plan_step_times) of a TN_FORM_* under a configuration.
+int family_of(int form, int cfg) {
+    switch (form) {
+        case TN_FORM_ROW: return 0;
+        case TN_FORM_NARROW: return cfg < 2 ? 0 : 1;
+        case TN_FORM_TC:
+        case TN_FORM_TC_FP32: return 2;
+        case TN_FORM_CHAIN: return 3;
+        case TN_FORM_SMALL: return 4;
+        default: return 1;
+    }
+}
+
 // sigma >= 0: only the output instances of that slice of the pass
 int run_step(PlanObj *o, int s, int precision, int64_t sigma, cudaStream_t st) {
     const tnp::Step &S = o->P.steps[s];
@@ -345,50 +382,26 @@ int run_step(PlanObj *o, int s, int precision, int64_t sigma, cudaStream_t st) {
     const int cfg = effective_config(o, s);
     tnk::StepDesc d = o->desc[s];
     if (sigma >= 0) apply_window(o, S, sigma, d);
-    d.sched = cfg & 1;
     d.tc_fp32 = o->tc_fp32 ? 1 : 0;
     d.tc_resident_b = o->tc_resident_b ? 1 : 0;
     d.tc_pair = o->tc_pair ? 1 : 0;
-    cudaError_t e;
-    int fam;
     const bool chosen = s < (int)o->pinned.size() && o->pinned[s];  // by the caller: runs as it is
-    const bool on_tc = cfg >= 2 && precision != TN_FP32 && tnk::gemm_tc_supports(d) && !tnk::step_skinny_takes(d);
-    if (sigma < 0 && !chosen && tnk::step_few_takes(d, on_tc)) {
-        fam = 1;
-        e = tnk::launch_step_few(d, st);
-    } else if (cfg < 2) {
-        fam = 0;
-        e = tnk::launch_step_row(d, st);
-    } else if (tnk::step_skinny_takes(d)) {
-        // few outputs per instance and a long K (e.g. the root)
-        fam = 1;
-        e = tnk::launch_step_skinny(d, st);
-    } else if (precision != TN_FP32 && tnk::gemm_tc_supports(d)) {
-        fam = 2;
-        if (!(s < (int)o->config_override.size() && o->config_override[s] >= 0)) d.sched = tnk::tc_rule_schedule(d);
-        if (d.tc_resident_b && tnk::tc_dictionary_chunks(d) == 0 && tnk::tc_resident_b_chunks(d) == 0 &&
-            tnk::step_narrow_takes(d, false)) {
-            fam = 1;
-            e = tnk::launch_step_narrow(d, st);
-        } else if (o->amap[s].ok) {
-            e = tnk::launch_step_gemm_tc(d, &o->amap[s].map, precision, o->err_flag, st);
-        } else {
-            e = cudaErrorInvalidValue;  // its TMA descriptor could not be encoded
-        }
-    } else if (precision == TN_FP32 && o->amap[s].ok && tnk::tc_fp32_takes(d)) {
-        fam = 2;
-        e = tnk::launch_step_gemm_tc(d, &o->amap[s].map, precision, o->err_flag, st);
-    } else if (tnk::step_outer_takes(d)) {
-        fam = 1;
-        e = tnk::launch_step_outer(d, st);
-    } else if (tnk::step_narrow_takes(d, true)) {
-        fam = 1;
-        e = tnk::launch_step_narrow(d, st);
-    } else {
-        fam = 1;
-        e = tnk::launch_step_gemm_simt(d, st);
+    const bool ruled = !(s < (int)o->config_override.size() && o->config_override[s] >= 0);
+    const int form = step_form(d, cfg, ruled, precision, sigma < 0 && !chosen, o->amap[s].ok);
+    cudaError_t e;
+    switch (form) {
+        case TN_FORM_FEW: e = tnk::launch_step_few(d, st); break;
+        case TN_FORM_ROW: e = tnk::launch_step_row(d, st); break;
+        case TN_FORM_NARROW: e = cfg < 2 ? tnk::launch_step_row(d, st) : tnk::launch_step_narrow(d, st); break;
+        case TN_FORM_SKINNY: e = tnk::launch_step_skinny(d, st); break;
+        case TN_FORM_OUTER: e = tnk::launch_step_outer(d, st); break;
+        case TN_FORM_SIMT: e = tnk::launch_step_gemm_simt(d, st); break;
+        default:
+            e = o->amap[s].ok ? tnk::launch_step_gemm_tc(d, &o->amap[s].map, precision, o->err_flag, st)
+                              : cudaErrorInvalidValue;  // its TMA descriptor could not be encoded
     }
-    o->step_kernel[s] = fam;
+    o->step_form[s] = form;
+    o->step_kernel[s] = family_of(form, cfg);
     if (e != cudaSuccess)
         return set_err(TN_ECUDA, "step " + std::to_string(s) + ": " + cudaGetErrorString(e));
     return TN_OK;
@@ -396,7 +409,10 @@ int run_step(PlanObj *o, int s, int precision, int64_t sigma, cudaStream_t st) {
 
 int run_group(PlanObj *o, tnk::SmallArgs g, cudaStream_t st) {
     g.descs = at<const tnk::SmallDesc>(o, o->P.off_small);
-    for (int j = 0; j < g.n_steps; ++j) o->step_kernel[g.step[j]] = 4;
+    for (int j = 0; j < g.n_steps; ++j) {
+        o->step_form[g.step[j]] = TN_FORM_SMALL;
+        o->step_kernel[g.step[j]] = 4;
+    }
     const cudaError_t e = tnk::launch_small(g, st);
     if (e != cudaSuccess) return set_err(TN_ECUDA, std::string("small steps: ") + cudaGetErrorString(e));
     return TN_OK;
@@ -573,8 +589,12 @@ void step_features(const tnp::Plan &P, int s, int precision, int c, float *f) {
 void start_launches(PlanObj *o) {
     const tnp::Plan &P = o->P;
     o->step_kernel.resize(P.steps.size(), -1);
+    o->step_form.resize(P.steps.size(), -1);
     for (size_t s = 0; s < P.steps.size(); ++s)
-        if (o->chain_fused(P.steps[s].chain)) o->step_kernel[s] = 3;
+        if (o->chain_fused(P.steps[s].chain)) {
+            o->step_form[s] = TN_FORM_CHAIN;
+            o->step_kernel[s] = 3;
+        }
     o->ev_used = 0;
     o->ev_step.clear();
 }
@@ -1036,6 +1056,13 @@ int tn_pt_histogram(const double *amps, int64_t k, int32_t n_qubits, double x_ma
                                         reinterpret_cast<unsigned long long *>(counts_dev), st);
     if (e != cudaSuccess) return set_err(TN_ECUDA, std::string("pt_histogram: ") + cudaGetErrorString(e));
     g_err.clear();
+    return TN_OK;
+}
+
+int tn_plan_step_forms(tn_plan_t plan, int32_t *form, int32_t n) {
+    if (!plan || (n > 0 && !form)) return set_err(TN_EINVAL, "tn_plan_step_forms: null argument");
+    const PlanObj *o = reinterpret_cast<const PlanObj *>(plan);
+    for (int32_t i = 0; i < n; ++i) form[i] = i < (int32_t)o->step_form.size() ? o->step_form[i] : -1;
     return TN_OK;
 }
 

@@ -1371,9 +1371,11 @@ bool step_narrow_takes(const StepDesc &d, bool fp32) {
            (d.n_ctab << (d.mb - 7)) >= 304;
 }
 
+bool step_row_narrow(const StepDesc &d) { return d.kb >= NARROW_MIN_KB && d.mb >= 7; }
+
 cudaError_t launch_step_row(const StepDesc &d, cudaStream_t s) {
     if (d.kb + d.nb > 8 || d.nb > 4 || d.mb > 40) return cudaErrorInvalidValue;
-    if (d.kb >= NARROW_MIN_KB && d.mb >= 7) return launch_step_narrow(d, s);
+    if (step_row_narrow(d)) return launch_step_narrow(d, s);
     const int K = 1 << d.kb;
     const int L = row_lanes(d.kb, d.nb);
     const int R = 32 / L;

@@ -76,6 +76,8 @@ struct LeafHighD {
 cudaError_t launch_fill(const FillJobD *jobs, int64_t njobs, const LeafHighD *highs, int64_t batch,
                         float2 *ws, cudaStream_t s);
 cudaError_t launch_step_row(const StepDesc &d, cudaStream_t s);
+// Whether launch_step_row takes the narrow tiles.
+bool step_row_narrow(const StepDesc &d);
 cudaError_t launch_step_gemm_simt(const StepDesc &d, cudaStream_t s);
 // Steps with K <= 32, N >= 32 and M >= 32 on the grouped GEMM's configurations
 // (FP32): a thread's rows in registers against a column tile.

@@ -10,17 +10,12 @@ import pytest
 
 from gpu_helpers import rel_l2, run_plan
 from oracle import sv
+from paper_2212_04749_gb300 import tn
 from rqc import grid_layout, network_structure, random_circuit
 from rqc.bitstrings import uniform_bitstrings
 from rqc.tree import candidate_trees
 
 pytestmark = pytest.mark.gpu
-
-
-def _takes(st, log2_macs):
-    out = st["n_inst"] << (st["mb"] + st["nb"])
-    return (st["kb"] <= 10 and out <= 1 << 20 and out << st["kb"] <= 1 << log2_macs and
-            (out > 1 << 14 or out << st["kb"] > 1 << 18))
 
 
 @pytest.mark.parametrize("prec,rescale,tol", [("fp32", 0, 1e-5), ("fp32", 1, 1e-5), ("bf16x3", 1, 1e-4)])
@@ -33,5 +28,5 @@ def test_steps_of_few_multiply_adds(layout, cycles, rows, seed, tree, prec, resc
     bits = uniform_bitstrings(c.n_qubits, rows, seed=5)
     ssa = candidate_trees(network_structure(c), rows, seed=seed, trials=3)[tree]
     got, p = run_plan(c, bits, ssa, precision=prec, rescale=rescale)
-    assert any(_takes(st, 23 if prec == "fp32" else 21) for st in p.tn_plan_steps())
+    assert tn.TN_FORM_FEW in p.tn_plan_step_forms()
     assert rel_l2(got, sv.amplitudes(c, bits)) <= tol

@@ -17,6 +17,7 @@ import pytest
 
 from gpu_helpers import rel_l2, run_plan
 from oracle import sv
+from paper_2212_04749_gb300 import tn
 from rqc import grid_layout, network_structure, random_circuit
 from rqc.bitstrings import uniform_bitstrings
 from rqc.tree import candidate_trees
@@ -24,8 +25,16 @@ from rqc.tree import candidate_trees
 pytestmark = pytest.mark.gpu
 
 
-def _takes(st):
-    return st["mb"] >= 6 and st["kb"] >= 6 and (st["nb"] >= 6 or (st["n_inst"] << st["nb"]) >= 32 * st["n_groups"])
+def _both(c, bits, ssa):
+    """Amplitudes with the plan's own FP32 kernels and with the steps that
+    went to the tensor cores on FMAs (configuration 3)."""
+    got, p = run_plan(c, bits, ssa, precision="fp32")
+    on_tc = p.tn_plan_step_forms() == tn.TN_FORM_TC_FP32
+    assert np.any(on_tc)
+    own = iter(on_tc)
+    fma, q = run_plan(c, bits, ssa, precision="fp32", force_config=lambda st: 3 if next(own) else None)
+    assert not np.any(np.isin(q.tn_plan_step_forms(), (tn.TN_FORM_TC_FP32, tn.TN_FORM_TC)))
+    return got, fma
 
 
 @pytest.mark.parametrize("layout,cycles,rows,seed,tree", [
@@ -37,12 +46,11 @@ def test_error_is_that_of_fp32(layout, cycles, rows, seed, tree):
     bits = uniform_bitstrings(c.n_qubits, rows, seed=5)
     ssa = candidate_trees(network_structure(c), rows, seed=seed, trials=3)[tree]
     ref = sv.amplitudes(c, bits)
-    got, p = run_plan(c, bits, ssa, precision="fp32")
-    assert any(_takes(st) for st in p.tn_plan_steps())
-    fma, _ = run_plan(c, bits, ssa, precision="fp32", force_config=lambda st: 3 if _takes(st) else None)
+    got, fma = _both(c, bits, ssa)
     err, own = rel_l2(got, ref), rel_l2(fma, ref)
     assert own <= 1e-5 and err <= 1.1 * own
-    plain, _ = run_plan(c, bits, ssa, precision="fp32", rescale=0)  # no maxima, no scales: the FMA kernel
+    plain, p = run_plan(c, bits, ssa, precision="fp32", rescale=0)  # no maxima, no scales: the FMA kernel
+    assert not np.any(p.tn_plan_step_forms() == tn.TN_FORM_TC_FP32)
     assert rel_l2(plain, ref) <= 1e-5
 
 
@@ -81,9 +89,6 @@ def test_small_entries_beside_large_ones_keep_their_bits(layout, cycles, rows, s
     bits = uniform_bitstrings(c.n_qubits, rows, seed=5)
     ssa = candidate_trees(network_structure(c), rows, seed=seed, trials=3)[tree]
     ref = sv.amplitudes(c, bits)
-    got, p = run_plan(c, bits, ssa, precision="fp32")
-    assert any(_takes(st) for st in p.tn_plan_steps())
-    fma, _ = run_plan(c, bits, ssa, precision="fp32", force_config=lambda st: 3 if _takes(st) else None)
+    got, fma = _both(c, bits, ssa)
     err, own = rel_l2(got, ref), rel_l2(fma, ref)
-    print(f"split {err:.2e}, FMA {own:.2e}")
     assert own <= 1e-5 and err <= 1.1 * own

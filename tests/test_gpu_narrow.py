@@ -9,6 +9,7 @@ import pytest
 
 from gpu_helpers import rel_l2, run_plan
 from oracle import sv
+from paper_2212_04749_gb300 import tn
 from rqc import grid_layout, network_structure, random_circuit
 from rqc.bitstrings import uniform_bitstrings
 from rqc.tree import candidate_trees
@@ -36,6 +37,6 @@ def test_tiles_of_columns(layout, cycles, rows, seed, tree, step, wide, many, re
     got, p = run_plan(c, bits, ssa, precision="fp32", rescale=rescale,
                       force_kernel=lambda st: 0 if _takes(st) else None)
     st = p.tn_plan_steps()[step]
-    assert _takes(st)
+    assert p.tn_plan_step_forms()[step] == tn.TN_FORM_NARROW
     assert ((st["n_inst"] << st["nb"]) > 8 * st["n_groups"], (st["max_group"] << st["nb"]) > 16) == (wide, many)
     assert rel_l2(got, sv.amplitudes(c, bits)) <= 1e-5

@@ -9,6 +9,7 @@ import pytest
 
 from gpu_helpers import rel_l2, run_plan
 from oracle import sv
+from paper_2212_04749_gb300 import tn
 from rqc import grid_layout, network_structure, random_circuit
 from rqc.bitstrings import uniform_bitstrings
 from rqc.tree import candidate_trees
@@ -43,5 +44,11 @@ def test_steps_off_the_gemm_tiles(layout, cycles, rows, seed, tree, step, kind, 
     ssa = candidate_trees(network_structure(c), rows, seed=seed, trials=3)[tree]
     got, p = run_plan(c, bits, ssa, precision=prec, rescale=rescale,
                       force_config=lambda st: 2 if _outer(st) or _narrow(st) else None)
-    assert kind(p.tn_plan_steps()[step])
+    st = p.tn_plan_steps()[step]
+    form = p.tn_plan_step_forms()[step]
+    want = tn.TN_FORM_OUTER if kind is _outer else tn.TN_FORM_NARROW
+    if prec == "bf16x3" and st["kb"] >= 3 and st["mb"] >= 6:  # tensor cores, unless B is streamed for few columns
+        streams_few = st["kb"] >= 8 and (st["n_inst"] << st["nb"]) <= 8 * st["n_groups"]
+        want = tn.TN_FORM_NARROW if kind is _narrow and streams_few else tn.TN_FORM_TC
+    assert form == want
     assert rel_l2(got, sv.amplitudes(c, bits)) <= {"fp32": 1e-5, "bf16x3": 1e-4}[prec]

@@ -10,6 +10,7 @@ import pytest
 
 from gpu_helpers import rel_l2, run_plan
 from oracle import sv
+from paper_2212_04749_gb300 import tn
 from rqc import grid_layout, network_structure, random_circuit
 from rqc.bitstrings import uniform_bitstrings
 from rqc.tree import candidate_trees
@@ -34,7 +35,8 @@ def test_few_outputs_long_k(layout, open_q, tree, rescale):
     ssa = candidate_trees(network_structure(c), 37, seed=2, trials=2)[tree]
     got, p = run_plan(c, bits, ssa, precision="fp32", open_qubits=open_q, rescale=rescale,
                       force_kernel=lambda st: 1 if _takes(st) else None)
-    assert any(_takes(st) for st in p.tn_plan_steps())
+    takes = np.array([_takes(st) for st in p.tn_plan_steps()])
+    assert np.any(takes) and np.all(p.tn_plan_step_forms()[takes] == tn.TN_FORM_SKINNY)
     r = len(open_q)
     ref = np.zeros((len(bits), 1 << r), np.complex128)
     for x in range(1 << r):

@@ -259,6 +259,13 @@ def test_config_override_rules(tn):
     assert p.tn_plan_get_configs()[big] == base[big]
 
 
+def test_step_forms_before_a_contraction(tn):
+    assert tn.load().tn_plan_step_forms(None, None, 1) == tn.TN_EINVAL
+    w = make_workload("grid3x4_m8")
+    p = tn.Plan(w.circuit, w.bits, w.tree.ssa, w.tree.sliced)
+    assert np.all(p.tn_plan_step_forms() == -1)
+
+
 def test_tensor_core_switches(tn):
     # the resident-B and column-tile-pair switches act at launch time: a
     # null plan is an argument error, and either setting leaves the plan's
