@@ -715,7 +715,7 @@ def run_ours(args, world, rank, local):
         # amplitudes read back to pinned host memory; steady-state time per
         # batch between the first and the last result
         from paper_2212_04749_gb300.pipeline import contract_batches
-        cfg_now = plan.tn_plan_get_configs()
+        cfg_now = plan.tn_plan_get_choices()
         chains_now = plan.tn_plan_get_chains()
         marks = []
         # further workspaces: the next batches are planned (two host threads)

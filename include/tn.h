@@ -335,11 +335,15 @@ int tn_plan_set_kernel(tn_plan_t plan, int32_t step, int32_t kernel);
  * 2, on the tensor cores 3 where a group's resident B would leave the stream
  * of A too little of the shared memory).
  * A step given a configuration (>= 0) then runs by itself, and as that says,
- * even if it is small (see tn_plan_step_times, family 4, and above); config + TN_CONFIG_TUNED, with config as
- * tn_plan_get_configs returned it for a tuned plan of the same shape, leaves
- * small steps together, as tn_plan_autotune and tn_plan_select do.
+ * even if it is small (see tn_plan_step_times, family 4, and above); with
+ * TN_CONFIG_TUNED added it leaves small steps together, as tn_plan_autotune
+ * and tn_plan_select do.  Chains that the plan fuses without
+ * tn_options.fuse: a configuration without TN_CONFIG_TUNED for one of their
+ * steps, or TN_CONFIG_TUNED + TN_CONFIG_UNFUSED added to it, runs the chain
+ * as its steps; -1 as the plan would.
  * TN_EINVAL for a configuration the step's shape does not allow. */
 #define TN_CONFIG_TUNED 16
+#define TN_CONFIG_UNFUSED 32
 int tn_plan_set_config(tn_plan_t plan, int32_t step, int32_t config);
 
 /* Tensor-core form of the grouped GEMM.  enable = 1 (the default): where B
@@ -381,6 +385,12 @@ int tn_plan_get_chains(tn_plan_t plan, int32_t *enabled, int32_t n);
 /* Configuration each step will run with (the plan's choice where none was
  * set); n entries. */
 int tn_plan_get_configs(tn_plan_t plan, int32_t *config, int32_t n);
+
+/* What was chosen for each step (n entries), as tn_plan_set_config takes it:
+ * handed step by step to another plan of the same shape, that plan runs as
+ * this one does (reported chains: tn_plan_get_chains, tn_plan_set_chain).
+ * -1 where nothing was chosen, else a configuration with its flags. */
+int tn_plan_get_choices(tn_plan_t plan, int32_t *choice, int32_t n);
 
 /* Cost-model features: TN_NFEAT floats per step for configuration `config`
  * at `precision` (row-major n_steps x TN_NFEAT, host memory), and whether

@@ -1123,6 +1123,8 @@ int tn_plan_set_config(tn_plan_t plan, int32_t step, int32_t config) {
     PlanObj *o = reinterpret_cast<PlanObj *>(plan);
     const tnp::Plan &P = o->P;
     if (step < 0 || step >= (int32_t)P.steps.size()) return set_err(TN_EINVAL, "tn_plan_set_config: bad step");
+    const bool unfused = config >= TN_CONFIG_TUNED + TN_CONFIG_UNFUSED;
+    if (unfused) config -= TN_CONFIG_UNFUSED;
     const bool tuned = config >= TN_CONFIG_TUNED;
     if (tuned) config -= TN_CONFIG_TUNED;
     if (config < -1 || config >= TN_NCONFIG) return set_err(TN_EINVAL, "tn_plan_set_config: bad configuration");
@@ -1133,6 +1135,12 @@ int tn_plan_set_config(tn_plan_t plan, int32_t step, int32_t config) {
     // a step whose kernel was chosen runs by itself even if it is small
     o->pinned.resize(P.steps.size(), 0);
     o->pinned[step] = !tuned && config >= 0;
+    // a chain that the plan formed by itself: run as its steps, or as the plan would
+    const int c = P.steps[step].chain;
+    if (!P.opt.fuse && c >= 0 && (unfused || config < 0)) {
+        o->chain_on.resize(P.chains.size(), -1);
+        o->chain_on[c] = unfused ? 0 : -1;
+    }
     o->drop_graphs();
     return TN_OK;
 }
@@ -1182,6 +1190,20 @@ int tn_plan_get_configs(tn_plan_t plan, int32_t *config, int32_t n) {
     if (!plan || (n > 0 && !config)) return set_err(TN_EINVAL, "tn_plan_get_configs: null argument");
     PlanObj *o = reinterpret_cast<PlanObj *>(plan);
     for (int32_t s = 0; s < n && s < (int32_t)o->P.steps.size(); ++s) config[s] = effective_config(o, s);
+    return TN_OK;
+}
+
+int tn_plan_get_choices(tn_plan_t plan, int32_t *choice, int32_t n) {
+    if (!plan || (n > 0 && !choice)) return set_err(TN_EINVAL, "tn_plan_get_choices: null argument");
+    const PlanObj *o = reinterpret_cast<const PlanObj *>(plan);
+    for (int32_t s = 0; s < n && s < (int32_t)o->P.steps.size(); ++s) {
+        const int32_t c = s < (int32_t)o->config_override.size() ? o->config_override[s] : -1;
+        const bool pin = s < (int32_t)o->pinned.size() && o->pinned[s];
+        const int ch = o->P.steps[s].chain;
+        choice[s] = c;
+        if (c >= 0 && !pin)
+            choice[s] += TN_CONFIG_TUNED + (!o->P.opt.fuse && ch >= 0 && o->chain_state(ch) == 0 ? TN_CONFIG_UNFUSED : 0);
+    }
     return TN_OK;
 }
 

@@ -36,8 +36,10 @@ def contract_batches(circ, batches, tree_ssa, sliced, precision, workspace, stre
     later batches are then planned and their tables uploaded while the
     current batch runs).  stream: the torch CUDA stream the
     contractions run on (default: the current stream).  configs: optional
-    per-step configurations applied to every plan (all batches must then
-    yield plans with the same step count); chains: optional per-chain fused
+    per-step choices applied to every plan (all batches must then yield
+    plans with the same step count), as tn_plan_get_choices gives them (or
+    bare configurations, as tn_plan_get_configs gives them, which leave out
+    what was chosen for the plan's own chains); chains: optional per-chain fused
     flags (tn_plan_set_chain) applied likewise.  The amplitudes are complex128
     numpy arrays in input order (rows x 2^|open qubits| with
     opts open_qubits / open_mask), read from pinned host memory after the
@@ -95,7 +97,7 @@ def contract_batches(circ, batches, tree_ssa, sliced, precision, workspace, stre
                 futs[j] = ex.submit(plan_of, j, done.get(j % nws))
             if configs is not None:
                 for s, c in enumerate(configs):
-                    p.tn_plan_set_config(s, int(c) + (TN_CONFIG_TUNED if c >= 0 else 0))
+                    p.tn_plan_set_config(s, int(c) + (TN_CONFIG_TUNED if 0 <= c < TN_CONFIG_TUNED else 0))
             if chains is not None:
                 for c, on in enumerate(chains):
                     p.tn_plan_set_chain(c, int(on))

@@ -22,7 +22,7 @@ PRECISIONS = {"fp32": TN_FP32, "tf32": TN_TF32, "bf16x3": TN_BF16X3}
 EXPORTS = ("tn_options_default", "tn_network", "tn_plan", "tn_plan_query", "tn_plan_launches",
            "tn_plan_widths", "tn_plan_steps",
            "tn_plan_bind", "tn_contract", "tn_contract_slices", "tn_xeb", "tn_plan_profile",
-           "tn_plan_step_times", "tn_plan_step_forms", "tn_plan_set_kernel", "tn_plan_set_config", "tn_plan_set_tc_resident_b", "tn_plan_set_tc_fp32", "tn_plan_set_tc_pairs", "tn_plan_get_configs", "tn_pt_moments",
+           "tn_plan_step_times", "tn_plan_step_forms", "tn_plan_set_kernel", "tn_plan_set_config", "tn_plan_set_tc_resident_b", "tn_plan_set_tc_fp32", "tn_plan_set_tc_pairs", "tn_plan_get_configs", "tn_plan_get_choices", "tn_pt_moments",
            "tn_pt_moments_scratch_bytes", "tn_pt_moments_scratch", "tn_pt_histogram", "tn_sample_completions",
            "tn_plan_features", "tn_plan_autotune", "tn_plan_select", "tn_mlp_grad_scratch_bytes",
            "tn_mlp_forward", "tn_mlp_grad", "tn_mlp_adam", "tn_mlp_to_half", "tn_mlp_forward_f16",
@@ -32,7 +32,7 @@ TN_STATIC_SCRATCH_BYTES = 64 << 20
 TN_PT_MAX_BINS = 8192
 TN_MAX_OPEN = 16
 TN_NCONFIG = 4
-TN_CONFIG_TUNED = 16
+TN_CONFIG_TUNED, TN_CONFIG_UNFUSED = 16, 32
 (TN_FORM_ROW, TN_FORM_SIMT, TN_FORM_TC, TN_FORM_CHAIN, TN_FORM_SMALL, TN_FORM_NARROW, TN_FORM_OUTER, TN_FORM_SKINNY,
  TN_FORM_FEW, TN_FORM_TC_FP32) = range(10)
 TN_NFEAT = TN_MLP_IN = 24
@@ -132,6 +132,7 @@ def load(build_if_missing: bool = False):
         "tn_plan_set_tc_fp32": (ctypes.c_int, [vp, i32]),
         "tn_plan_set_tc_pairs": (ctypes.c_int, [vp, i32]),
         "tn_plan_get_configs": (ctypes.c_int, [vp, vp, i32]),
+        "tn_plan_get_choices": (ctypes.c_int, [vp, vp, i32]),
         "tn_plan_features": (ctypes.c_int, [vp, ctypes.c_int, i32, vp, vp, i32]),
         "tn_plan_autotune": (ctypes.c_int, [vp, ctypes.c_int, i32, vp, vp, vp, vp]),
         "tn_plan_select": (ctypes.c_int, [vp, ctypes.c_int, vp, ctypes.c_float, vp, ctypes.c_size_t, vp, vp]),
@@ -360,6 +361,12 @@ class Plan:
         n = self.info["n_steps"]
         c = np.zeros(max(n, 1), np.int32)
         _check(self._lib.tn_plan_get_configs(self.h, c.ctypes.data, n))
+        return c[:n]
+
+    def tn_plan_get_choices(self):
+        n = self.info["n_steps"]
+        c = np.zeros(max(n, 1), np.int32)
+        _check(self._lib.tn_plan_get_choices(self.h, c.ctypes.data, n))
         return c[:n]
 
     def tn_plan_features(self, precision, config):

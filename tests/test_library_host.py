@@ -259,6 +259,41 @@ def test_config_override_rules(tn):
     assert p.tn_plan_get_configs()[big] == base[big]
 
 
+def test_choices_carry_to_another_plan(tn):
+    # configurations set by hand, tuned ones, and chains that the plan formed
+    # by itself and that were measured to be slower than their steps
+    assert tn.load().tn_plan_get_choices(None, None, 1) == tn.TN_EINVAL
+    c = random_circuit(grid_layout(4, 5), 12, seed=41)
+    bits = uniform_bitstrings(c.n_qubits, 700, seed=6)
+    ssa = candidate_trees(network_structure(c), 700, seed=4, trials=3)[0]
+    p, q = (tn.Plan(c, bits, ssa) for _ in range(2))
+    n = p.info["n_steps"]
+    assert np.all(p.tn_plan_get_choices() == -1)
+    base = p.tn_plan_launches()
+    row = [st["nb"] <= 4 and st["kb"] + st["nb"] <= 8 for st in p.tn_plan_steps()]
+    for s in range(n):
+        p.tn_plan_set_config(s, (0 if row[s] else 2) + tn.TN_CONFIG_TUNED)
+    assert np.all(p.tn_plan_get_choices() == np.where(row, 16, 18)) and p.tn_plan_launches() == base
+    for s in range(n):
+        p.tn_plan_set_config(s, (0 if row[s] else 2) + tn.TN_CONFIG_TUNED + tn.TN_CONFIG_UNFUSED)
+    own = p.tn_plan_get_choices()
+    fused = own >= 48  # steps of the plan's own chains
+    assert np.all(own == np.where(row, 16, 18) + 32 * fused) and fused.sum() >= 2
+    apart = p.tn_plan_launches()
+    assert apart > base
+    for s in range(n):
+        q.tn_plan_set_config(s, own[s])
+    assert q.tn_plan_launches() == apart and np.array_equal(q.tn_plan_get_choices(), own)
+    p.tn_plan_set_config(n - 1, 3)
+    assert p.tn_plan_get_choices()[n - 1] == 3
+    for s in range(n):
+        p.tn_plan_set_config(s, -1)
+    assert p.tn_plan_launches() == base and np.all(p.tn_plan_get_choices() == -1)
+    for bad in (4, 20, 34, 52, 64):
+        with pytest.raises(tn.TnError):
+            p.tn_plan_set_config(0, bad)
+
+
 def test_step_forms_before_a_contraction(tn):
     assert tn.load().tn_plan_step_forms(None, None, 1) == tn.TN_EINVAL
     w = make_workload("grid3x4_m8")
