@@ -1229,8 +1229,10 @@ int tn_plan_autotune(tn_plan_t plan, int precision, int32_t reps, const uint8_t 
     const tnp::Plan &P = o->P;
     const int ns = (int)P.steps.size();
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    std::vector<int32_t> cur(ns);
-    for (int s = 0; s < ns; ++s) cur[s] = effective_config(o, s);
+    // the steps' choices as they are (-1: the plan's own, which its rules may
+    // take further than a configuration says)
+    o->config_override.resize(ns, -1);
+    const std::vector<int32_t> cur = o->config_override;
     std::vector<double> best(size_t(ns) * TN_NCONFIG, NAN), ms(ns);
     const bool prof = o->profile;
     o->profile = true;  // CUDA events around every step launch

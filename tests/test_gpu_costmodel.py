@@ -195,6 +195,26 @@ def test_autotuner_picks_fastest_measured_and_keeps_parity(case20, prec):
     assert err <= (1e-5 if prec == "fp32" else 1e-3)
 
 
+def test_masked_autotuning_leaves_the_other_steps_choices(case20):
+    # steps without a choice keep the plan's own rules, a step set by hand
+    # stays set
+    torch, tn = require_cuda()
+    c, bits, ssa, sl, _ = case20
+    p = tn.Plan(c, bits, ssa, sl)
+    ws = torch.empty(p.info["workspace_bytes"], dtype=torch.uint8, device="cuda")
+    st = torch.cuda.current_stream()
+    p.tn_plan_bind(ws, stream=st)
+    amps = torch.zeros(2 * len(bits), dtype=torch.float64, device="cuda")
+    n = p.info["n_steps"]
+    mask = np.zeros(n, np.uint8)
+    mask[n // 2] = 1
+    p.tn_plan_set_config(n - 1, 3)
+    p.tn_plan_autotune("bf16x3", amps, reps=1, step_mask=mask, stream=st)
+    own = p.tn_plan_get_choices()
+    assert own[n // 2] >= tn.TN_CONFIG_TUNED and own[n - 1] == 3
+    assert np.all(np.delete(own, [n // 2, n - 1]) == -1)
+
+
 def test_cost_model_gain_over_the_rule_and_regret():
     # Train on the autotuner's timings of seeded random plans, then configure
     # held-out plans with the network alone (no measurement) and compare the
