@@ -89,6 +89,7 @@ struct PlanObj {
     std::map<int, Sched> scheds;  // by level; dropped with the graphs
     bool merge_small = true;                      // small steps run together (off while the autotuner times them singly)
     std::vector<uint8_t> pinned;                  // per step: the caller chose its kernel (tn_plan_set_config)
+    std::vector<uint8_t> apart;                   // per step: the autotuner times it (with a mask), so it merges with none
     std::map<GraphKey, cudaGraphExec_t> graphs;  // captured tn_contract launch sequences
     cudaStream_t cap_stream = nullptr;           // private stream the sequences are captured on
     void drop_graphs() {
@@ -420,7 +421,8 @@ int run_group(PlanObj *o, tnk::SmallArgs g, cudaStream_t st) {
 
 // Whether step s may share a launch with other small steps.
 bool merges(const PlanObj *o, int s) {
-    return o->merge_small && o->P.steps[s].small && !(s < (int)o->pinned.size() && o->pinned[s]);
+    return o->merge_small && o->P.steps[s].small && !(s < (int)o->pinned.size() && o->pinned[s]) &&
+           !(s < (int)o->apart.size() && o->apart[s]);
 }
 
 // Launch order for a slice batch of recompute level lv (64: every step).
@@ -1238,13 +1240,9 @@ int tn_plan_autotune(tn_plan_t plan, int precision, int32_t reps, const uint8_t 
     o->profile = true;  // CUDA events around every step launch
     // Every step in a launch of its own; with a mask, the steps that are not
     // timed share launches as ever.
-    const std::vector<uint8_t> prev_pinned = o->pinned;
-    if (step_mask) {
-        o->pinned.resize(ns, 0);
-        for (int s = 0; s < ns; ++s) o->pinned[s] |= step_mask[s] != 0;
-    } else {
-        o->merge_small = false;
-    }
+    // (A timed step runs the kernel that it will run by itself later.)
+    if (step_mask) o->apart.assign(step_mask, step_mask + ns);
+    else o->merge_small = false;
     o->config_override.assign(ns, -1);
     const int nchains = (int)P.chains.size();
     const std::vector<int8_t> prev_chain = o->chain_on;
@@ -1298,7 +1296,7 @@ int tn_plan_autotune(tn_plan_t plan, int precision, int32_t reps, const uint8_t 
         o->config_override[s] = pick;
     }
     o->merge_small = true;
-    o->pinned = prev_pinned;
+    o->apart.clear();
     // fused chains: each kept fused only where its kernel beats the sum of
     // its steps' best times (the chain's time is booked on its last step)
     // (with a step mask only some steps were timed: the chains keep their

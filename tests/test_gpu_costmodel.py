@@ -215,6 +215,27 @@ def test_masked_autotuning_leaves_the_other_steps_choices(case20):
     assert np.all(np.delete(own, [n // 2, n - 1]) == -1)
 
 
+def test_masked_autotuning_times_the_kernel_that_runs_afterwards():
+    # a step of few multiply-adds takes k_step_few whatever is chosen, in the
+    # timed runs too
+    torch, tn = require_cuda()
+    c = random_circuit(grid_layout(4, 5), 10, seed=21)
+    bits = uniform_bitstrings(20, 37, seed=5)
+    ssa = candidate_trees(network_structure(c), 37, seed=2, trials=3)[5]
+    p = tn.Plan(c, bits, ssa)
+    ws = torch.empty(p.info["workspace_bytes"], dtype=torch.uint8, device="cuda")
+    st = torch.cuda.current_stream()
+    p.tn_plan_bind(ws, stream=st)
+    amps = torch.zeros(2 * len(bits), dtype=torch.float64, device="cuda")
+    p.tn_contract(amps, "fp32", stream=st)
+    few = p.tn_plan_step_forms() == tn.TN_FORM_FEW
+    assert np.any(few)
+    p.tn_plan_autotune("fp32", amps, reps=1, step_mask=few, stream=st)
+    assert np.all(p.tn_plan_step_forms()[few] == tn.TN_FORM_FEW)
+    p.tn_contract(amps, "fp32", stream=st)
+    assert np.all(p.tn_plan_step_forms()[few] == tn.TN_FORM_FEW)
+
+
 def test_cost_model_gain_over_the_rule_and_regret():
     # Train on the autotuner's timings of seeded random plans, then configure
     # held-out plans with the network alone (no measurement) and compare the
