@@ -219,6 +219,9 @@ def test_masked_autotuning_times_the_kernel_that_runs_afterwards():
     # a step of few multiply-adds takes k_step_few whatever is chosen, in the
     # timed runs too
     torch, tn = require_cuda()
+    from rqc import grid_layout, network_structure, random_circuit
+    from rqc.bitstrings import uniform_bitstrings
+    from rqc.tree import candidate_trees
     c = random_circuit(grid_layout(4, 5), 10, seed=21)
     bits = uniform_bitstrings(20, 37, seed=5)
     ssa = candidate_trees(network_structure(c), 37, seed=2, trials=3)[5]
