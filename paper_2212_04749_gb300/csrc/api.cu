@@ -388,7 +388,7 @@ int run_step(PlanObj *o, int s, int precision, int64_t sigma, cudaStream_t st) {
     d.tc_pair = o->tc_pair ? 1 : 0;
     const bool chosen = s < (int)o->pinned.size() && o->pinned[s];  // by the caller: runs as it is
     const bool ruled = !(s < (int)o->config_override.size() && o->config_override[s] >= 0);
-    const int form = step_form(d, cfg, ruled, precision, sigma < 0 && !chosen, o->amap[s].ok);
+    const int form = step_form(d, cfg, ruled, precision, !chosen, o->amap[s].ok);
     cudaError_t e;
     switch (form) {
         case TN_FORM_FEW: e = tnk::launch_step_few(d, st); break;
@@ -599,6 +599,38 @@ void start_launches(PlanObj *o) {
         }
     o->ev_used = 0;
     o->ev_step.clear();
+}
+
+// Estimated time (us) of a pass over the steps of level <= lv (-1: none),
+// of whole steps or of those that hold one slice's instances: a launch costs
+// about 5 us whatever it computes, a merged one 5 and 2 a phase, and the
+// other steps their bytes or flops at about the rates that they reach.
+double pass_us(PlanObj *o, int precision, int lv, bool narrow) {
+    if (lv < 0) return 0.0;
+    const tnp::Plan &P = o->P;
+    const PlanObj::Sched &order = schedule(o, lv);
+    double t = 10.0;  // maxima cleared, leaves filled
+    for (const PlanObj::Sched::Item &it : order.items) {
+        if (it.group >= 0) {
+            t += 5.0 + 2.0 * order.groups[it.group].n_phases;
+            continue;
+        }
+        const tnp::Step &S = P.steps[it.step];
+        const tnp::Node &nd = P.nodes[S.node];
+        double bytes = S.bytes, flops = S.flops, rate = 60e6;  // flops a us
+        if (o->chain_fused(S.chain)) {
+            const tnp::Chain &c = P.chains[S.chain];
+            const tnp::Node &A = P.nodes[P.steps[c.steps[0]].a];
+            bytes = 8.0 * (std::ldexp(double(A.n_inst), A.rank) + std::ldexp(double(nd.n_inst), nd.rank));
+            flops = 0.0;
+            for (int q : c.steps) flops += P.steps[q].flops;
+        } else if (effective_config(o, it.step) >= 2 && !tnk::step_skinny_takes(o->desc[it.step])) {
+            if (precision != TN_FP32 && tnk::gemm_tc_supports(o->desc[it.step])) rate = precision == TN_TF32 ? 500e6 : 320e6;
+        }
+        const double part = narrow ? std::ldexp(1.0, -(int)nd.slices_low.size()) : 1.0;
+        t += std::max(5.0, part * std::max(bytes / 6e6, flops / rate));
+    }
+    return t;
 }
 
 // One pass over slice batch b: the steps of level <= lv (64: all), the
@@ -949,28 +981,39 @@ int tn_contract_slices(tn_plan_t plan, int precision, const int64_t *slice_ids, 
     const float2 *root = at<const float2>(o, R.buf.data);
     const int32_t *E = at<const int32_t>(o, R.buf.E);
     const int32_t *uniq = at<const int32_t>(o, P.off_uniq);
-    // A pass computes the 2^m_low slices of a batch side by side; where at
-    // most half of them are asked for, a pass per slice computes just the
-    // instances of that slice (a step's time goes with its instances: 16
-    // slices of grid6x7_m10, 8 to a pass, took 19 ms each as whole passes).
-    // Steps that no value of a sliced edge changed for since the last pass
-    // keep their results: pass p re-runs the levels up to the highest of a
-    // node that depends on a changed one.
+    // A pass computes the 2^m_low slices of a batch side by side; a pass per
+    // slice computes just the instances of that slice (a step's time goes with
+    // its instances: 16 slices of grid6x7_m10, 8 to a pass, took 19 ms each as
+    // whole passes, 1.8 alone), but where launches and merged steps set the
+    // time it is as long as a whole one.  Steps that no value of a sliced edge
+    // changed for since the last pass keep their results: pass p re-runs the
+    // levels up to the highest of a node that depends on a changed one.
     start_launches(o);
-    int64_t b_prev = -1, s_prev = -1;  // s_prev = -1: a whole pass
-    auto pass = [&](int64_t b, int64_t sigma) -> int {
-        int lv = 64;
-        if (b_prev >= 0) {
-            lv = b == b_prev ? -1 : 63 - __builtin_clzll((unsigned long long)(b ^ b_prev));
-            for (const tnp::Node &nd : P.nodes) {
-                if (nd.slices_low.empty()) continue;
-                const bool same = sigma < 0 ? s_prev < 0
-                                            : s_prev >= 0 && slice_instance(nd, sigma) == slice_instance(nd, s_prev);
-                if (!same) lv = std::max(lv, nd.level);
-            }
+    struct Pos {
+        int64_t b = -1, sigma = -1;  // batch, and slice of it (-1: a whole pass)
+    } at_pos;
+    auto level = [&](const Pos &prev, const Pos &next) -> int {
+        if (prev.b < 0) return 64;
+        int lv = next.b == prev.b ? -1 : 63 - __builtin_clzll((unsigned long long)(next.b ^ prev.b));
+        for (const tnp::Node &nd : P.nodes) {
+            if (nd.slices_low.empty()) continue;
+            const bool same = next.sigma < 0 ? prev.sigma < 0
+                                             : prev.sigma >= 0 && slice_instance(nd, next.sigma) ==
+                                                                      slice_instance(nd, prev.sigma);
+            if (!same) lv = std::max(lv, nd.level);
         }
-        b_prev = b;
-        s_prev = sigma;
+        return lv;
+    };
+    std::map<std::pair<int, bool>, double> us;  // of a pass, by level and width
+    auto estimate = [&](int lv, bool narrow) {
+        auto it = us.find({lv, narrow});
+        if (it == us.end()) it = us.emplace(std::make_pair(lv, narrow), pass_us(o, precision, lv, narrow)).first;
+        return it->second;
+    };
+    auto pass = [&](int64_t b, int64_t sigma) -> int {
+        const Pos next{b, sigma};
+        const int lv = level(at_pos, next);
+        at_pos = next;
         return lv >= 0 ? run_pass(o, precision, b, lv, sigma, st) : TN_OK;
     };
     auto extract = [&](int32_t i) -> int {
@@ -982,7 +1025,14 @@ int tn_contract_slices(tn_plan_t plan, int precision, const int64_t *slice_ids, 
     for (auto &kv : by_batch) {
         std::map<int64_t, std::vector<int32_t>> by_slice;
         for (int32_t i : kv.second) by_slice[internal[i] % per].push_back(i);
-        const bool whole = 2 * (int64_t)by_slice.size() > per;
+        double narrow_us = 0.0;
+        Pos p = at_pos;
+        for (auto &ks : by_slice) {
+            const Pos next{kv.first, ks.first};
+            narrow_us += estimate(level(p, next), true);
+            p = next;
+        }
+        const bool whole = narrow_us > estimate(level(at_pos, Pos{kv.first, -1}), false);
         if (whole)
             if (int rc = pass(kv.first, -1)) return rc;
         for (auto &ks : by_slice) {

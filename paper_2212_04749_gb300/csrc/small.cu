@@ -275,19 +275,19 @@ bool step_few_takes(const StepDesc &d, bool tc) {
 }
 
 cudaError_t launch_step_few(const StepDesc &d, cudaStream_t s) {
-    if (!step_few_takes(d, false) || d.inst0 != 0) return cudaErrorInvalidValue;
+    if (!step_few_takes(d, false)) return cudaErrorInvalidValue;
     SmallDesc r;
     std::memset(&r, 0, sizeof(r));
     r.A = d.A;
     r.B = d.B;
-    r.C = d.C;
-    r.instab = d.instab;
+    r.C = d.C + d.inst0 * d.sC;
+    r.instab = d.instab + d.inst0;
     r.EA = d.EA;
     r.EB = d.EB;
-    r.EC = d.EC;
+    r.EC = d.EC + d.inst0;
     r.mxA = d.mxA;
     r.mxB = d.mxB;
-    r.mxC = d.mxC;
+    r.mxC = d.mxC ? d.mxC + d.inst0 : nullptr;
     r.sA = d.sA;
     r.sB = d.sB;
     r.sC = d.sC;

@@ -39,6 +39,7 @@ def _partials(tn, torch, c, bits, ssa, sl, ids, prec, low, force=None, calls=1, 
 @pytest.mark.parametrize("prec,config", [("fp32", None), ("fp32", 1), ("fp32", 3), ("bf16x3", 2), ("bf16x3", 3)])
 @pytest.mark.parametrize("layout,cycles,rows,tree,n_sliced,low,opts", [
     ((4, 4), 10, 300, 1, 5, 3, {}), ((4, 5), 10, 90, 2, 4, 2, {"rescale": 0}),
+    ((4, 5), 14, 60, 1, 4, 3, {}),  # steps long enough that two slices of eight still run one by one
     ((4, 4), 10, 40, 3, 4, 4, {"open_qubits": [0, 15]}), ((4, 4), 10, 200, 0, 5, 2, {"fuse": 1, "fuse_max_bits": 8})])
 def test_slices_alone_match_whole_passes(layout, cycles, rows, tree, n_sliced, low, opts, prec, config):
     torch, tn = require_cuda()
@@ -62,3 +63,35 @@ def test_slices_alone_match_whole_passes(layout, cycles, rows, tree, n_sliced, l
     few = ids[:3]  # a call whose slices lie far apart
     got, _ = _partials(tn, torch, c, bits, ssa, sl, few, prec, low, force, **opts)
     assert rel_l2(got, ref[:3]) <= tol
+
+
+@pytest.mark.parametrize("layout,cycles,rows,tree", [((3, 4), 8, 64, 1), ((4, 4), 10, 300, 1), ((4, 5), 10, 90, 2)])
+def test_some_slices_of_a_small_plan_take_no_longer_than_all(layout, cycles, rows, tree):
+    # launches and merged steps set the time of these plans: a pass per slice
+    # would take as often as long as a whole pass
+    torch, tn = require_cuda()
+    import time
+    c = random_circuit(grid_layout(*layout), cycles, seed=21)
+    st = network_structure(c)
+    bits = uniform_bitstrings(c.n_qubits, rows, seed=5)
+    ssa = candidate_trees(st, rows, seed=2, trials=3)[tree]
+    sl = choose_slices(st, ContractionTree(ssa=ssa), rows, n_sliced=3)
+    p = tn.Plan(c, bits, ssa, sl, slice_batch_log2=3)
+    ws = torch.empty(p.info["workspace_bytes"], dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.current_stream()
+    p.tn_plan_bind(ws, stream=stream)
+    out = torch.zeros(8, 2 * rows, dtype=torch.float64, device="cuda")
+
+    def seconds(n):
+        t = []
+        for _ in range(20):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            p.tn_contract_slices(np.arange(n), out[:n], "fp32", stream=stream)
+            torch.cuda.synchronize()
+            t.append(time.perf_counter() - t0)
+        return float(np.median(t))
+
+    whole = seconds(8)
+    assert seconds(4) <= 1.3 * whole and seconds(2) <= 1.3 * whole and seconds(1) <= 1.3 * whole
+    assert layout == (3, 4) or tn.TN_FORM_FEW in p.tn_plan_step_forms()  # on one slice's instances
