@@ -398,8 +398,10 @@ int tn_plan_get_choices(tn_plan_t plan, int32_t *choice, int32_t n);
  * Host only.  Features, all O(1): the operand and output bit counts
  * (mb, kb, nb, ranks), log2 of the instance, group and column counts, the
  * contiguous address runs of A, B and C (the permutation class), log2 of
- * flops and bytes per pass, one-hot precision, kernel family, schedule, and
- * log2 of the output rows. */
+ * flops and bytes per pass, one-hot precision, kernel family (per-row
+ * configuration; grouped and on the tensor cores, FP32's BF16x6 among them;
+ * grouped otherwise, as tn_contract would run the step), schedule, and log2
+ * of the output rows. */
 #define TN_NFEAT 24
 int tn_plan_features(tn_plan_t plan, int precision, int32_t config, float *feat, int32_t *eligible, int32_t n);
 

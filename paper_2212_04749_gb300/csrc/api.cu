@@ -105,14 +105,40 @@ T *at(PlanObj *o, int64_t off) {
     return reinterpret_cast<T *>(o->ws + off);
 }
 
+// A step's shape as the dispatch sees it: a descriptor without addresses
+// (maxima and packed B only present or absent).
+tnk::StepDesc shape_desc(const PlanObj *o, const tnp::Step &st) {
+    static uint32_t present;
+    const tnp::Plan &P = o->P;
+    const tnp::Node &nd = P.nodes[st.node], &B = P.nodes[st.b];
+    tnk::StepDesc d;
+    std::memset(&d, 0, sizeof(d));
+    d.mb = st.mb;
+    d.kb = st.kb;
+    d.nb = st.nb;
+    d.nInst = nd.n_inst;
+    d.nInstB = d.packBn = B.n_inst;
+    d.n_groups = st.n_groups;
+    d.max_group = (int32_t)st.max_group;
+    d.n_ctab = (int64_t)st.col_tiles.size();
+    d.n_ptab = st.n_pair_tiles;
+    if (P.opt.rescale) d.mxA = d.mxB = d.mxC = &present;
+    if (P.bpack32_bytes > 0) d.bpack = reinterpret_cast<uint8_t *>(&present);
+    d.bpack_bytes = P.bpack_bytes;
+    d.bpack32_bytes = P.bpack32_bytes;
+    d.tc_fp32 = o->tc_fp32 ? 1 : 0;
+    d.tc_resident_b = o->tc_resident_b ? 1 : 0;
+    d.tc_pair = o->tc_pair ? 1 : 0;
+    return d;
+}
+
 void build_descs(PlanObj *o) {
     tnp::Plan &P = o->P;
     o->desc.clear();
     for (const tnp::Step &st : P.steps) {
         const tnp::Node &nd = P.nodes[st.node];
         const tnp::Node &A = P.nodes[st.a], &B = P.nodes[st.b];
-        tnk::StepDesc d;
-        std::memset(&d, 0, sizeof(d));
+        tnk::StepDesc d = shape_desc(o, st);
         d.A = at<const float2>(o, A.buf.data);
         d.B = at<const float2>(o, B.buf.data);
         d.C = at<float2>(o, nd.buf.data);
@@ -129,8 +155,6 @@ void build_descs(PlanObj *o) {
         d.nOutA = A.n_out;
         d.nOutB = B.n_out;
         d.nOut = nd.n_out;
-        d.nInst = nd.n_inst;
-        d.nInstB = d.packBn = B.n_inst;
         d.EA = at<const int32_t>(o, A.buf.E);
         d.EB = at<const int32_t>(o, B.buf.E);
         d.EC = at<int32_t>(o, nd.buf.E);
@@ -138,9 +162,6 @@ void build_descs(PlanObj *o) {
         d.mxA = rs ? at<const uint32_t>(o, A.buf.mx) : nullptr;
         d.mxB = rs ? at<const uint32_t>(o, B.buf.mx) : nullptr;
         d.mxC = rs ? at<uint32_t>(o, nd.buf.mx) : nullptr;
-        d.mb = st.mb;
-        d.kb = st.kb;
-        d.nb = st.nb;
         for (int j = 0; j < st.mb; ++j) {
             d.pAm[j] = st.pAm[j];
             d.pCm[j] = st.pCm[j];
@@ -150,20 +171,11 @@ void build_descs(PlanObj *o) {
             d.pCn[j] = st.pCn[j];
         }
         d.gfirst = at<const int64_t>(o, st.off_groups);
-        d.n_groups = st.n_groups;
         d.ctab = at<const int64_t>(o, st.off_col_tiles);
-        d.n_ctab = (int64_t)st.col_tiles.size();
         d.trec = at<const int4>(o, st.off_tile_rec);
         d.ptab = st.n_pair_tiles > 0 ? at<const int2>(o, st.off_pair_tab) : nullptr;
-        d.n_ptab = st.n_pair_tiles;
         d.instab = at<const int2>(o, st.off_inst_ab);
         d.bpack = P.bpack32_bytes > 0 ? at<uint8_t>(o, P.off_bpack) : nullptr;
-        d.bpack_bytes = P.bpack_bytes;
-        d.bpack32_bytes = P.bpack32_bytes;
-
-        int64_t mg = 0;
-        for (int64_t g = 0; g < st.n_groups; ++g) mg = std::max(mg, st.group_first[g + 1] - st.group_first[g]);
-        d.max_group = (int32_t)mg;
         o->desc.push_back(d);
     }
     // fused chains
@@ -542,7 +554,8 @@ const PlanObj::Sched &schedule(PlanObj *o, int lv) {
 }
 
 // Cost-model features of step s under configuration c (tn.h, TN_NFEAT).
-void step_features(const tnp::Plan &P, int s, int precision, int c, float *f) {
+void step_features(const PlanObj *o, int s, int precision, int c, float *f) {
+    const tnp::Plan &P = o->P;
     const tnp::Step &S = P.steps[s];
     const tnp::Node &nd = P.nodes[S.node], &A = P.nodes[S.a], &B = P.nodes[S.b];
     auto lg = [](double x) { return float(std::log2(x > 1.0 ? x : 1.0)); };
@@ -553,13 +566,9 @@ void step_features(const tnp::Plan &P, int s, int precision, int c, float *f) {
     };
     int crun = 0;  // lowest C address bits held by consecutive m bits
     while (crun < S.mb && S.pCm[crun] == crun) ++crun;
-    tnk::StepDesc t;
-    std::memset(&t, 0, sizeof(t));
-    t.mb = S.mb;
-    t.kb = S.kb;
-    t.nb = S.nb;
-    const bool gemm = c >= 2;
-    const bool tc = gemm && precision != TN_FP32 && tnk::gemm_tc_supports(t);
+    tnk::StepDesc t = shape_desc(o, S);
+    const int form = step_form(t, c, false, precision, true, true);
+    const bool gemm = c >= 2, tc = form == TN_FORM_TC || form == TN_FORM_TC_FP32;
     const double ng = double(S.n_groups > 0 ? S.n_groups : 1);
     int i = 0;
     f[i++] = S.mb / 32.f;
@@ -846,9 +855,7 @@ int tn_plan_steps(tn_plan_t plan, tn_step_info *out, int32_t n) {
         r.chain_last = P.opt.fuse && st.chain_last ? 1 : 0;
         for (int j = 0; j < 40; ++j) r.c_pos_m[j] = j < st.mb ? st.pCm[j] : -1;
         for (int j = 0; j < 24; ++j) r.c_pos_n[j] = j < st.nb ? st.pCn[j] : -1;
-        int64_t mg = 0;
-        for (int64_t g = 0; g < st.n_groups; ++g) mg = std::max(mg, st.group_first[g + 1] - st.group_first[g]);
-        r.max_group = mg;
+        r.max_group = st.max_group;
         r.n_pair_tiles = st.n_pair_tiles;
     }
     return TN_OK;
@@ -1263,9 +1270,10 @@ int tn_plan_features(tn_plan_t plan, int precision, int32_t config, float *feat,
     if (!plan || (n > 0 && !feat)) return set_err(TN_EINVAL, "tn_plan_features: null argument");
     if (precision < TN_FP32 || precision > TN_BF16X3) return set_err(TN_EINVAL, "tn_plan_features: bad precision");
     if (config < 0 || config >= TN_NCONFIG) return set_err(TN_EINVAL, "tn_plan_features: bad configuration");
-    const tnp::Plan &P = reinterpret_cast<PlanObj *>(plan)->P;
+    const PlanObj *o = reinterpret_cast<const PlanObj *>(plan);
+    const tnp::Plan &P = o->P;
     for (int32_t s = 0; s < n && s < (int32_t)P.steps.size(); ++s) {
-        step_features(P, s, precision, config, feat + int64_t(s) * TN_NFEAT);
+        step_features(o, s, precision, config, feat + int64_t(s) * TN_NFEAT);
         if (eligible) eligible[s] = config_allowed(P.steps[s], config) ? 1 : 0;
     }
     return TN_OK;
@@ -1407,7 +1415,7 @@ int tn_plan_select(tn_plan_t plan, int precision, const uint16_t *params16, floa
         return set_err(TN_ENOMEM, "tn_plan_select: scratch needs " + std::to_string(need) + " bytes");
     std::vector<float> X(size_t(rows) * TN_NFEAT), y(rows);
     for (int s = 0; s < ns; ++s)
-        for (int c = 0; c < TN_NCONFIG; ++c) step_features(P, s, precision, c, &X[(size_t(s) * TN_NCONFIG + c) * TN_NFEAT]);
+        for (int c = 0; c < TN_NCONFIG; ++c) step_features(o, s, precision, c, &X[(size_t(s) * TN_NCONFIG + c) * TN_NFEAT]);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     float *dX = static_cast<float *>(scratch), *dy = dX + rows * TN_NFEAT;
     CU(cudaMemcpyAsync(dX, X.data(), X.size() * sizeof(float), cudaMemcpyHostToDevice, st));
@@ -1437,14 +1445,8 @@ int tn_plan_select(tn_plan_t plan, int precision, const uint16_t *params16, floa
         o->config_override[s] = b1;
         // (a small step that shares a launch, one of a fused chain and one of few
         // multiply-adds run the same whatever is chosen)
-        tnk::StepDesc t;
-        std::memset(&t, 0, sizeof(t));
-        t.mb = P.steps[s].mb;
-        t.kb = P.steps[s].kb;
-        t.nb = P.steps[s].nb;
-        t.nInst = P.nodes[P.steps[s].node].n_inst;
         const bool same = merges(o, s) || o->chain_fused(P.steps[s].chain) ||
-                          tnk::step_few_takes(t, precision != TN_FP32);
+                          tnk::step_few_takes(shape_desc(o, P.steps[s]), precision != TN_FP32);
         if (uncertain) uncertain[s] = (have2 && y2 - y1 < margin && !same) ? 1 : 0;
     }
     o->drop_graphs();

@@ -465,8 +465,10 @@ struct Builder {
             // GEMM column tiles of 64 complex columns over each group's
             // concatenated instances (N columns each)
             st.col_tiles.clear();
+            st.max_group = 0;
             for (int64_t g = 0; g < st.n_groups; ++g) {
-                const int64_t cols = (st.group_first[g + 1] - st.group_first[g]) << st.nb;
+                const int64_t size = st.group_first[g + 1] - st.group_first[g], cols = size << st.nb;
+                st.max_group = std::max(st.max_group, size);
                 for (int64_t t = 0; t * 64 < cols; ++t) st.col_tiles.push_back((g << 20) | t);
             }
             // kernel family: the per-row kernel takes a small B (N <= 16,

@@ -95,6 +95,7 @@ struct Step {
     int level = 64;          // recomputed in batch b > first iff level <= ctz(b)
     double runs = 1;         // passes over all 2^h batches
     int64_t n_groups = 0;    // runs of consecutive output instances sharing an A instance
+    int64_t max_group = 0;   // instances of the largest
     std::vector<int64_t> group_first;  // n_groups + 1 boundaries
     int64_t off_groups = -1;           // workspace offset of group_first
     std::vector<int64_t> col_tiles;    // non-empty (group, 64-column tile) pairs: g * 2^20 + tile

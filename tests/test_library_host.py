@@ -231,11 +231,31 @@ def test_features_and_config_eligibility(tn, name):
             assert np.all(f[:, 19] + f[:, 20] + f[:, 21] == 1.0)  # exactly one kernel family
             assert np.all(f[:, 22] == (c & 1))
             assert np.all(f[:, 17] == (prec == "tf32")) and np.all(f[:, 18] == (prec == "bf16x3"))
-            if prec == "fp32":
-                assert not np.any(f[:, 20])  # no tensor cores in FP32
+            if prec == "fp32":  # the tensor cores only where configuration 2 takes BF16x6
+                big = np.array([st["kb"] >= 6 and st["mb"] >= 6 for st in steps])
+                assert not np.any(f[~big if c == 2 else slice(None), 20])
             np.testing.assert_allclose(f[:, 0] * 32, [st["mb"] for st in steps])
             np.testing.assert_allclose(f[:, 1] * 32, [st["kb"] for st in steps])
             np.testing.assert_allclose(f[:, 2] * 32, [st["nb"] for st in steps])
+
+
+def test_features_name_the_kernel_that_runs(tn):
+    # the 53-qubit plan: in FP32 its large steps are on the tensor cores under
+    # configuration 2, on FMAs under 3 and with that form switched off; steps
+    # of few columns leave the tensor cores where B would be streamed
+    w = make_workload("diamond53_m12")
+    p = tn.Plan(w.circuit, w.bits, w.tree.ssa, w.tree.sliced)
+    steps = p.tn_plan_steps()
+
+    def tc(prec, c):
+        return p.tn_plan_features(prec, c)[0][:, 20].astype(bool)
+
+    macs = np.array([st["n_inst"] << (st["mb"] + st["kb"] + st["nb"]) for st in steps])
+    on = tc("fp32", 2)
+    assert on.sum() >= 10 and on[np.argmax(macs)] and not np.any(tc("fp32", 3))
+    assert not np.any(tc("fp32", 0)) and np.all(tc("bf16x3", 2)[on])
+    p.tn_plan_set_tc_fp32(False)
+    assert not np.any(tc("fp32", 2))
 
 
 def test_config_override_rules(tn):
