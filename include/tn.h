@@ -425,7 +425,7 @@ int tn_plan_autotune(tn_plan_t plan, int precision, int32_t reps, const uint8_t 
 /* Cost-model selection: predict log2(ms per pass) of every (step, allowed
  * configuration) with the FP16 network params16 (device, TN_MLP_NPARAMS
  * halves, see tn_mlp_to_half), set each step to its predicted fastest
- * configuration, and flag in uncertain (host, n_steps int32, may be NULL)
+ * configuration (TN_FP32: not 3 where 2 takes the tensor cores), and flag in uncertain (host, n_steps int32, may be NULL)
  * the steps, other than small ones that share launches, whose two best
  * predictions lie within `margin` (log2 units):
  * those are the steps to hand to tn_plan_autotune (its step_mask) as the
