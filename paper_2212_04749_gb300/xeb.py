@@ -11,6 +11,7 @@ over the amplitudes per iteration); the scalar update runs here.  The error bar 
 square root of the Fisher information sum g^2 at the maximum.
 """
 
+import contextlib
 import math
 
 import numpy as np
@@ -18,16 +19,21 @@ import numpy as np
 from . import tn
 
 
-def _torch_stream(torch, stream, device):
-    """`stream` (a torch stream, a raw handle, None: the current stream) as a
-    torch stream.  Torch's streams do not order themselves against one
-    another, so buffers are made, kernels launched and results read with it
-    as the current stream."""
-    if stream is None:
-        return torch.cuda.current_stream(device)
+@contextlib.contextmanager
+def _on(stream, device):
+    """Make `stream` (a torch stream, a raw handle, None: the current stream)
+    torch's current one.  Torch's streams do not order themselves against one
+    another, so buffers are made, kernels launched and results read on one."""
+    import torch
+
+    cur = torch.cuda.current_stream(device)
+    if stream is None or stream == cur or stream == cur.cuda_stream:
+        yield cur
+        return
     if isinstance(stream, int):
-        return torch.cuda.ExternalStream(stream, device=device) if stream else torch.cuda.default_stream(device)
-    return stream
+        stream = torch.cuda.ExternalStream(stream, device=device) if stream else torch.cuda.default_stream(device)
+    with torch.cuda.stream(stream):
+        yield stream
 
 
 def porter_thomas_fit(amps, k, n_qubits, stream=None, iters=60, tol=1e-13):
@@ -36,17 +42,19 @@ def porter_thomas_fit(amps, k, n_qubits, stream=None, iters=60, tol=1e-13):
     Returns a dict: fidelity (maximum likelihood, kept in [0, 1 - 1e-12]),
     stderr, loglik (up to the constant), linear (N <p> - 1), linear_stderr,
     iterations."""
+    with _on(stream, amps.device) as st:
+        return _fit(amps, k, n_qubits, st, iters, tol)
+
+
+def _fit(amps, k, n_qubits, st, iters, tol):
     import torch
 
-    st = _torch_stream(torch, stream, amps.device)
-    with torch.cuda.stream(st):
-        out = torch.empty(5, dtype=torch.float64, device=amps.device)
-        scratch = torch.empty(tn.tn_pt_moments_scratch_bytes(k), dtype=torch.uint8, device=amps.device)
+    out = torch.empty(5, dtype=torch.float64, device=amps.device)
+    scratch = torch.empty(tn.tn_pt_moments_scratch_bytes(k), dtype=torch.uint8, device=amps.device)
 
     def moments(f, log=False):
-        with torch.cuda.stream(st):
-            tn.tn_pt_moments_scratch(amps, k, n_qubits, f, out, scratch, want_log=log, stream=st)
-            return out.cpu().numpy()  # copied on st, after the launch
+        tn.tn_pt_moments_scratch(amps, k, n_qubits, f, out, scratch, want_log=log, stream=st)
+        return out.cpu().numpy()  # copied on st, the current stream, after the launch
 
     top = 1.0 - 1e-12
     s = moments(0.0)
@@ -72,8 +80,7 @@ def porter_thomas_histogram(amps, k, n_qubits, x_max=8.0, nbins=64, stream=None)
     stream as for porter_thomas_fit."""
     import torch
 
-    st = _torch_stream(torch, stream, amps.device)
-    with torch.cuda.stream(st):
+    with _on(stream, amps.device) as st:
         counts = torch.zeros(nbins + 1, dtype=torch.int64, device=amps.device)
         tn.tn_pt_histogram(amps, k, n_qubits, x_max, nbins, counts, stream=st)
         return counts.cpu().numpy()
