@@ -1152,11 +1152,12 @@ __global__ void __launch_bounds__(RED_THREADS) k_pt_moments(const double2 *__res
         const double x = pt_x(amps[p], n_states);
         const double x1 = x - 1.0;
         const double d = 1.0 + fid * x1;
-        const double g = fid == 0.0 ? x1 : x1 / d;
+        const double g = fid == 0.0 ? x1 * d : x1 / d;  // (d = 1 there, NaN for an infinite x)
         a[0] += g;
         a[1] += g * g;
         a[3] += x;
         a[4] += x * x;
+        if (fid == 0.0) a[2] += d - 1.0;
         return d;
     };
     int64_t p = int64_t(blockIdx.x) * RED_THREADS + threadIdx.x;
@@ -1175,6 +1176,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_pt_moments(const double2 *__res
         const double d = add(p);
         if (want_log && fid != 0.0) a[2] += log(d);
     }
+    if (!want_log) a[2] = 0.0;
     const double s = block_sums<5, RED_THREADS>(a, part);
     if (CLUSTER) {
         const double t = cluster_sums<5>(s, slot);

@@ -143,3 +143,26 @@ def test_analysis_on_a_stream_that_is_still_busy(kind):
         with torch.cuda.stream(side if kind == "current" else torch.cuda.default_stream()):
             got = f(late, k, n, stream=arg)
         assert np.array_equal(got, want) if isinstance(want, np.ndarray) else got == want
+
+
+@pytest.mark.parametrize("f", [0.0, 0.37])
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_moments_of_amplitudes_that_are_no_numbers(f, bad):
+    # as the formulas have it: x infinite gives NaN in g and, at F = 0, in the
+    # logarithm (0 times infinity)
+    torch, tn = require_cuda()
+    k, n = 9001, 20
+    a = _amps(k, n, 3)
+    a[4321] = bad
+    d = _dev(torch, a)
+    with np.errstate(all="ignore"):
+        ref = oxeb.pt_moments(oxeb.x_values(a, n), f)
+    out = torch.empty(5, dtype=torch.float64, device="cuda")
+    scratch = torch.empty(tn.tn_pt_moments_scratch_bytes(k), dtype=torch.uint8, device="cuda")
+    tn.tn_pt_moments(d, k, n, f, out)
+    got = [out.cpu().numpy()]
+    tn.tn_pt_moments_scratch(d, k, n, f, out, scratch)
+    for g in got + [out.cpu().numpy()]:
+        assert np.array_equal(np.isnan(g), np.isnan(ref)) and np.array_equal(np.isinf(g), np.isinf(ref)), (g, ref)
+    tn.tn_pt_moments_scratch(d, k, n, f, out, scratch, want_log=False)
+    assert out[2].item() == 0.0
