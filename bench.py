@@ -17,7 +17,7 @@ value      amplitudes/s over all ranks: bitstrings / max-over-ranks device
 e2e        the same metric through the public pipeline from host data:
            host plan (overlapped), table upload, contraction, amplitudes
            back to pinned host memory.
-roofline   the kernel family with the largest share of device time:
+roofline   the kernel with the largest share of device time:
            algorithmic bytes or flops / its measured launch time, against
            the measured peak that binds it.
 peaks      denominators measured in this run on this device: the FP32 FMA
@@ -52,7 +52,10 @@ import numpy as np  # noqa: E402
 
 METRIC = "amplitudes/sec & TFLOP/s (frac of peak), mixed vs FP32 at stated amp error"
 UNIT = "amplitudes/s"
-FAMILIES = {0: "k_step_row", 1: "k_step_gemm_simt", 2: "k_step_gemm_tc", 3: "k_chain", 4: "k_small_steps"}
+# kernels by TN_FORM_* code (tn_plan_step_forms)
+FORMS = ("k_step_row", "k_step_gemm_simt", "k_step_gemm_tc", "k_chain", "k_small_steps", "k_step_narrow", "k_step_outer",
+         "k_step_skinny", "k_step_few", "k_step_gemm_tc_bf16x6")
+ROW, TC, CHAIN, SMALL, TC_FP32 = 0, 2, 3, 4, 9
 TOL = {"fp32": 1e-5, "bf16x3": 1e-3, "tf32": 1e-3}
 
 
@@ -298,6 +301,8 @@ def traffic_record(kernel):
 
 
 def family_breakdown(steps, step_ms, kernels):
+    """Sums per kernel; several steps of a fused chain or of the merged small
+    steps share a launch, whose time is booked on one of them."""
     fam = {}
     for s, st in enumerate(steps):
         f = int(kernels[s]) if kernels is not None else 0
@@ -305,29 +310,33 @@ def family_breakdown(steps, step_ms, kernels):
         r["ms"] += float(step_ms[s])
         r["bytes"] += st["bytes"] * st["runs"]
         r["flops"] += st["flops"] * st["runs"]
-        r["launches"] += int(st["runs"])
+        if f not in (CHAIN, SMALL) or step_ms[s] > 0:
+            r["launches"] += int(st["runs"])
         r["steps"].append(s)
     return fam
 
 
 def compute_peak(family, precision, peaks):
-    """Compute-rate peak (TFLOP/s, algorithmic) of a kernel family at a
-    precision and its source: tensor-core BF16x3 = measured BF16 (sustained)
-    / 3 products; TF32 = measured TF32; SIMT = measured FP32 FMA."""
-    if family == 2:
+    """Compute-rate peak (TFLOP/s, algorithmic) of a kernel at a precision
+    and its source: tensor-core BF16x3 = measured BF16 (sustained) / 3
+    products, FP32's BF16x6 / 6; TF32 = measured TF32; the others measured
+    FP32 FMA."""
+    if family == TC_FP32:
+        return peaks["bf16_tflops_sustained"] / 6.0, "measured bf16 sustained / 6"
+    if family == TC:
         if precision == "bf16x3":
             return peaks["bf16_tflops_sustained"] / 3.0, "measured bf16 sustained / 3"
         return peaks.get("tf32_tflops"), "measured tf32"
-    if family in (0, 1, 3):
-        return peaks.get("fp32_fma_tflops"), "measured fp32 fma"
-    return None, None
+    if family == SMALL:
+        return None, None
+    return peaks.get("fp32_fma_tflops"), "measured fp32 fma"
 
 
 def roofline_of(steps, step_ms, kernels, precision, peaks):
-    """Roofline of the dominant kernel family, the per-step bound fraction
+    """Roofline of the dominant kernel, the per-step bound fraction
     and the whole path's bound fraction.  A step's bound time is the longer
-    of its algorithmic bytes at the HBM peak and its flops at its family's
-    compute peak; a family is reported HBM-bound when its summed bytes at
+    of its algorithmic bytes at the HBM peak and its flops at its kernel's
+    compute peak; a kernel is reported HBM-bound when its summed bytes at
     the HBM peak take longer than its summed flops at the compute peak."""
     fam = family_breakdown(steps, step_ms, kernels)
     hbm = peaks["hbm_gbs"]
@@ -335,7 +344,7 @@ def roofline_of(steps, step_ms, kernels, precision, peaks):
     def bound_time(s, st, f):
         tb = st["bytes"] * st["runs"] / (hbm * 1e9)
         pk, _ = compute_peak(f, precision, peaks)
-        if pk and f in (1, 2):
+        if pk and f not in (ROW, CHAIN):
             tb = max(tb, st["flops"] * st["runs"] / (pk * 1e12))
         return tb
 
@@ -345,29 +354,29 @@ def roofline_of(steps, step_ms, kernels, precision, peaks):
     sec = r["ms"] / 1e3
     pk, pk_src = compute_peak(dom, precision, peaks)
     t_hbm = r["bytes"] / (hbm * 1e9)
-    t_cmp = r["flops"] / (pk * 1e12) if pk and dom in (1, 2) else 0.0
+    t_cmp = r["flops"] / (pk * 1e12) if pk and dom not in (ROW, CHAIN) else 0.0
     if t_hbm >= t_cmp:
         roof = {"bound": "hbm", "achieved": r["bytes"] / sec / 1e9, "peak": hbm, "unit": "GB/s"}
         if pk:
-            roof["tensor_tflops" if dom == 2 else "alu_tflops"] = r["flops"] / sec / 1e12
-            roof["tensor_frac" if dom == 2 else "alu_frac"] = r["flops"] / sec / 1e12 / pk
+            roof["tensor_tflops" if dom in (TC, TC_FP32) else "alu_tflops"] = r["flops"] / sec / 1e12
+            roof["tensor_frac" if dom in (TC, TC_FP32) else "alu_frac"] = r["flops"] / sec / 1e12 / pk
     else:
-        roof = {"bound": "tensor" if dom == 2 else "alu", "achieved": r["flops"] / sec / 1e12, "peak": pk,
+        roof = {"bound": "tensor" if dom in (TC, TC_FP32) else "alu", "achieved": r["flops"] / sec / 1e12, "peak": pk,
                 "unit": "TFLOP/s", "peak_source": pk_src}
     roof["frac"] = roof["achieved"] / roof["peak"]
     roof["step_bound_frac"] = sum(bound_time(s, steps[s], dom) for s in r["steps"]) / sec
-    roof["kernel"] = FAMILIES[dom]
+    roof["kernel"] = FORMS[dom]
     roof["launches_per_step"] = r["launches"]
     roof["algorithmic_bytes_per_launch"] = r["bytes"] / max(r["launches"], 1)
     roof["share_of_step_time"] = r["ms"] / max(total_ms, 1e-12)
-    roof["per_kernel_ms"] = {FAMILIES[f]: fam[f]["ms"] for f in fam}
+    roof["per_kernel_ms"] = {FORMS[f]: fam[f]["ms"] for f in fam}
     path_bound = sum(bound_time(s, steps[s], f) for f in fam for s in fam[f]["steps"])
-    # HBM fraction of every other family (the row kernel: bandwidth steps)
+    # HBM fraction of every other kernel (the row kernel: bandwidth steps)
     others = {}
     for f, rr in fam.items():
         if f == dom or rr["ms"] <= 0:
             continue
-        others[FAMILIES[f]] = {"ms": rr["ms"], "hbm_frac": rr["bytes"] / (rr["ms"] / 1e3) / 1e9 / hbm,
+        others[FORMS[f]] = {"ms": rr["ms"], "hbm_frac": rr["bytes"] / (rr["ms"] / 1e3) / 1e9 / hbm,
                                "launches": rr["launches"]}
     roof["other_families"] = others
     return roof, path_bound / (total_ms / 1e3), dom
@@ -611,8 +620,8 @@ def run_ours(args, world, rank, local):
         kernels = None
         for _ in range(runs):
             one_step(prec, profile=True)
-            ms, kernels = plan.tn_plan_step_times()
-            step_ms += ms / runs
+            step_ms += plan.tn_plan_step_times()[0] / runs
+            kernels = plan.tn_plan_step_forms()
         plan.tn_plan_profile(False)
         return step_ms, kernels
 
@@ -661,7 +670,7 @@ def run_ours(args, world, rank, local):
             r = dict(st)
             r["config"] = int(cfgs[s_])
             r["ms_per_call"] = float(step_ms[s_])
-            r["family"] = int(kernels[s_]) if kernels is not None else -1
+            r["form"] = int(kernels[s_]) if kernels is not None else -1
             rows.append(r)
         with open(args.dump_steps, "w") as f:
             json.dump({"precision": args.precision, "workload": args.workload, "steps": rows}, f)
