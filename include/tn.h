@@ -89,9 +89,11 @@ typedef struct {
     int32_t fuse;             /* 1: non-branching chains of steps with small
                                  side operands run as one kernel each, their
                                  intermediates never stored (SM Sec. V.C) */
-    int32_t fuse_max_bits;    /* d^t: a fused chain's tile holds at most
-                                 2^d^t complex entries (SM Sec. V.C);
-                                 0: default 7 */
+    int32_t fuse_max_bits;    /* d^t: a fused chain's steps touch at most d^t
+                                 address bits of the tensor they are applied
+                                 to (2^d^t complex entries, SM Sec. V.C); the
+                                 kernel's tiles take in further untouched
+                                 bits, up to 2^12 entries; 0: default 7 */
     int32_t graphs;           /* 1: tn_contract captures its launch sequence in
                                  a CUDA graph on first use of a (precision,
                                  batch range, output buffer) and replays it */

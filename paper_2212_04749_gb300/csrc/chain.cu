@@ -23,7 +23,8 @@
 //
 // Bound: one read of A_1 and one write of C_L at HBM (L2) speed against L
 // passes of 4 N fused multiply-adds and one shared-memory round trip an entry;
-// from three steps of K = N = 4 on it is the instruction issue.  Six such
+// six steps of K = N = 4 issue in 62 % of the cycles (FMA pipe 33 %, shared
+// memory 45 %, DRAM 13 %), the rest waits at the barriers between steps.  Six such
 // steps on 2^23 entries (134 MB, 20 us of HBM) take 85 us, 33-43 us each as
 // separate row kernels; the kernel before, a warp per tile of at most 2^10
 // with 8-byte loads through per-entry index tables, took 570 us (2^7) to 6 ms

@@ -800,7 +800,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
     // registers, rounded to nearest: the error is below the FMA kernel's (0.8
     // of it over 45 random plans of 16 to 20 qubits, also where entries 2^-80
     // of an instance's largest decide; 1.53e-6 and 1.68e-6 on 53 qubits).
-    // 53-qubit circuit, FP32, all of it: 230 ms on the FMA kernel, 64.5 here.
+    // Bound by the tensor pipe (49 % of cycles busy on a step of 2^11 x 2^8 x
+    // 2^8) and a unit's chain of load, split, twelve MMAs a chunk and drain over
+    // two accumulators.  53-qubit circuit, FP32, all of it by the plan's rule:
+    // 230 ms on the FMA kernel, 64.5 here.
     constexpr int EPI_REGS = epi_regs(PREC);
     constexpr bool ASPLIT = PREC >= 2;  // A split into TMEM
     static_assert(PREC != 3 || MODE == 3, "BF16x6: packed B");

@@ -685,7 +685,8 @@ __global__ void __launch_bounds__(128) k_step_gemm_simt2(const StepDesc d, int c
 // shared memory) and 256 RX `passes` rows; a thread holds RX rows of A in
 // registers and walks the columns, B's entries as broadcasts, so that a
 // warp's 32 rows, neighbours in C where the layout allows, are stored by one
-// instruction.  Bound by HBM (C), from K = 16 on by the FMA rate.  The GEMM
+// instruction.  Bound by C's stores, from K = 16 on by the instruction issue
+// (67 % of the slots, FMA pipe 52 %) and the shared-memory reads of B.  The GEMM
 // kernel stages 16 k a chunk, stores 16 rows an instruction and pads 32
 // columns to 64: 7.36 ms for 2^15 x 4 x 32 with 1024 instances (9.7 GB, 1.43
 // ms), 1.69 here; 2^10 x 32 x 32 with 8192 (1.1 ms of FMA) and 2^14 x 16 x 32
@@ -791,9 +792,10 @@ __global__ void __launch_bounds__(256) k_step_outer(const StepDesc d, int rlog, 
 // take tiles of 8, on which all four warps work; with tiles of 16 two of them
 // would only copy (38.3 against 39.8 ms of the step below).  In tiles of 16
 // the four columns of a warp rotate with the block, so that tiles with fewer
-// load all four schedulers.  Bound by HBM (A) and the FMA rate at about the
-// same time for 8 columns; a block lives for little more than its latencies,
-// so six of them share an SM.  The per-row kernel held a row of 64 in two
+// load all four schedulers.  Bound by the instruction issue in tiles of 16 (77 %
+// of the slots, FMA pipe 55 %, DRAM 38 % on 2^14 x 64 x 2 with 505 instances on
+// 64), in tiles of 8 by its latencies (issue 53 %, DRAM 45 %); a block lives for
+// little more than those, so six of them share an SM.  The per-row kernel held a row of 64 in two
 // lanes' registers, read B from shared memory for every row and instance
 // again and loaded 32 bytes a row at a time: 4.47 ms on 2^8 x 64 x 2 with
 // 64448 A instances of 1 to 10 (9.5 GB, 1.40 ms of HBM), 2.40 ms here (1.9
@@ -1138,8 +1140,9 @@ __device__ __forceinline__ double pt_x(double2 a, double n_states) {
 //   CLUSTER: the grid is one cluster, out holds the sums;
 //   else: any grid, block b writes its sums to out[5 b .. 5 b + 4], which
 //   k_pt_final adds up (every SM).
-// The fit of 3 M amplitudes with XEB and histogram: 1.10 ms, about 0.13 ms a
-// pass; with one block of 1024 threads and a logarithm each 205.7 ms.
+// The fit of 3 M amplitudes with XEB and histogram: 1.10 ms (a pass 0.10 ms at
+// F = 0, 0.12 otherwise, 0.19 with the logarithms); with one block of 1024
+// threads and a logarithm each 205.7 ms.
 template <bool CLUSTER>
 __global__ void __launch_bounds__(RED_THREADS) k_pt_moments(const double2 *__restrict__ amps, int64_t k,
                                                             double n_states, double fid, int want_log,

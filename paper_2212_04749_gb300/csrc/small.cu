@@ -8,7 +8,7 @@
 // phases on the host, a phase's steps depend on earlier phases only and run
 // side by side, and a cluster barrier between phases takes the place of the
 // launch.  A phase costs its barrier and one round trip to L2 (maxima,
-// exponents, A and B together); a warp looks up its part of the next phase and
+// exponents, A and B together), about 2.5 us of ten with the launch; a warp looks up its part of the next phase and
 // the instances there between its arrival at the barrier and the wait.
 // 64 amplitudes of 3x4 with 8 cycles: 34.9 us with the look-up and the
 // exponents' loads behind the barrier, 32.6 so; as separate launches 177.
