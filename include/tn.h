@@ -317,7 +317,7 @@ int tn_plan_set_kernel(tn_plan_t plan, int32_t step, int32_t kernel);
  * allows (K >= 8, 64 <= M < 2^31), on the CUDA cores otherwise.  For TN_FP32
  * configuration 2 takes the tensor cores as well where a step has K >= 64,
  * 64 <= M < 2^31, N >= 64 or groups of 32 columns on average, maxima for both
- * operands (tn_options.rescale, no leaf) and room for its packed B (BF16x6):
+ * operands (tn_options.rescale) and room for its packed B (BF16x6):
  * each operand value split into three bf16 parts, which hold all of its 24
  * bits, and the six products of parts down to 2^-16 of the whole, in units of
  * 32 or 64 real k whose sums are added in FP32 registers.  (An infinity in

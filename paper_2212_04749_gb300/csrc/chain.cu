@@ -30,10 +30,11 @@
 // with 8-byte loads through per-entry index tables, took 570 us (2^7) to 6 ms
 // (2^10) for chains of this size.
 //
-// Rescale: the intermediates are not rescaled (the chain is short and the
-// operands come normalised); C_L is multiplied by 2^-(ea + sum_j eb_j), the
-// exponents of the operands' largest components, and its exponent is
-// E_A + ea + sum_j (E_Bj + eb_j).  Power-of-two factors are exact.
+// Rescale: B_j is multiplied by 2^-eb_j, the exponent of its largest component,
+// as it is staged, C_L by 2^-ea, and its exponent is
+// E_A + ea + sum_j (E_Bj + eb_j).  So the intermediates, which are not rescaled
+// themselves, stay in range whatever the side operands' scale.  Power-of-two
+// factors are exact.
 #include "kernels.cuh"
 
 namespace tnk {
@@ -228,24 +229,22 @@ __global__ void __launch_bounds__(CH_MAX_THREADS, 3) k_chain(const __grid_consta
     float2 *Bs = reinterpret_cast<float2 *>(ch_raw);
     float2 *X0 = Bs + s_boff[L], *X1 = X0 + (int64_t(1) << d.tmax);
     if (t == 0) {
-        float sc = 1.f;
         int ec = 0;
-        for (int q = 0; q <= L; ++q) {
-            sc *= ch_pow2(-s_e[q]);
-            ec += s_E[q];
-        }
-        s_sc = sc;
+        for (int q = 0; q <= L; ++q) ec += s_E[q];
+        s_sc = ch_pow2(-s_e[0]);
         if (ob == 0) d.EC[inst] = ec;
     }
     for (int j = 0; j < L; ++j) {
         const int kn = 1 << (d.kb[j] + d.nb[j]);
         const float2 *src = d.B[j] + int64_t(s_tab[1 + j]) * kn;
+        const float sb = ch_pow2(-s_e[1 + j]);
         // column n in the kernel's order (its bit b: B's n bit nperm[b])
         for (int e = t; e < kn; e += TH) {
             const int n = e >> d.kb[j];
             int m = 0;
             for (int b = 0; b < d.nb[j]; ++b) m |= ((n >> b) & 1) << d.nperm[j][b];
-            Bs[s_boff[j] + e] = __ldg(src + ((m << d.kb[j]) | (e & ((1 << d.kb[j]) - 1))));
+            const float2 v = __ldg(src + ((m << d.kb[j]) | (e & ((1 << d.kb[j]) - 1))));
+            Bs[s_boff[j] + e] = make_float2(v.x * sb, v.y * sb);
         }
     }
     const int64_t n_o = int64_t(1) << d.no;

@@ -25,8 +25,8 @@
 //                    sample from a batch, main text on Fig. 3(b), SM Sec. II);
 //                    k_sample_rows: batches of at most 32 completions
 //
-// Power-of-two rescaling: every produced instance records the largest
-// |component| of its entries (as float bits, atomicMax of non-negative
+// Power-of-two rescaling: every instance, leaves among them, has the largest
+// |component| of its entries recorded (as float bits, atomicMax of non-negative
 // floats); its consumer multiplies the loaded values by 2^-e, e the
 // exponent of that maximum, and adds e to the output's exponent E.  Scaling
 // by a power of two is exact, so with and without it the FP32 results of
@@ -83,7 +83,15 @@ __global__ void k_fill(const FillJobD *__restrict__ jobs, int64_t njobs, const L
     const LeafHighD H = highs[J.leaf_high];
     int64_t src = J.src;
     for (int c = 0; c < H.cnt; ++c) src += ((batch >> H.j[c]) & 1) * int64_t(H.stride[c]);
-    for (int e = lane; e < J.n; e += 32) ws[J.dst + e] = ws[src + e];
+    uint32_t mx = 0u;
+    for (int e = lane; e < J.n; e += 32) {
+        const float2 v = ws[src + e];
+        ws[J.dst + e] = v;
+        mx = max(mx, absmax_bits(v));
+    }
+    if (J.mx < 0) return;
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) reinterpret_cast<uint32_t *>(ws)[J.mx] = mx;
 }
 
 constexpr int ROW_THREADS = 256;

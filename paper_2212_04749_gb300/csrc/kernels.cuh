@@ -64,6 +64,7 @@ struct StepDesc {
 struct FillJobD {
     int64_t dst, src;
     int32_t leaf_high, n;
+    int64_t mx;
 };
 
 struct LeafHighD {

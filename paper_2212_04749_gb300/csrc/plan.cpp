@@ -806,6 +806,7 @@ struct Builder {
                     j.src = (p.off_leaf_full / 8) + full_off[v] + (block << nd.rank);
                     j.leaf_high = hidx;
                     j.n = int32_t(1) << nd.rank;
+                    j.mx = p.opt.rescale ? nd.buf.mx / 4 + inst : -1;
                     jobs.push_back(j);
                     job_leaf.push_back(v);
                 }

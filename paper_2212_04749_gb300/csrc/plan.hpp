@@ -218,6 +218,7 @@ struct FillJob {          // one leaf instance block
     int64_t src;          // element offset in the full-leaf region, high-slice bits = 0
     int32_t leaf_high;    // index into the LeafHigh table
     int32_t n;            // elements
+    int64_t mx;           // its max word (uint32 offset in the workspace), -1: no rescale
 };
 
 struct LeafHigh {         // sliced legs of a leaf that vary across batches

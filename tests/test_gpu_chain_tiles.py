@@ -83,3 +83,18 @@ def test_streaming_steps_without_the_fuse_option(layout, cycles, rows, tree, n_s
     if (layout, tree) == ((4, 5), 0):
         assert np.sum(p.tn_plan_step_times()[1] == 3) >= 4
     assert np.array_equal(base, p.tn_plan_get_configs())
+
+
+@pytest.mark.parametrize("fuse", [0, 1])
+@pytest.mark.parametrize("layout,cycles,rows,tree,n_sliced", [((4, 5), 12, 700, 0, 0), ((4, 5), 12, 700, 1, 2)])
+def test_chains_of_operands_of_any_scale(layout, cycles, rows, tree, n_sliced, fuse):
+    # gates of 2^-30 in two layers and of 2^30 in the next two: five of them
+    # leave the range of FP32.  Step by step the rescale keeps every
+    # intermediate in range; a fused chain does as well
+    c, bits, ssa, sl = _case(layout, cycles, rows, tree, n_sliced)
+    for g in c.two_qubit_gates:
+        g.matrix = g.matrix * 2.0 ** (30 if (g.layer // 4) % 2 else -30)
+    ref = sv.amplitudes(c, bits)
+    got, p = run_plan(c, bits, ssa, sl, fuse=fuse)
+    assert np.any(p.tn_plan_step_forms() == 3)
+    assert rel_l2(got, ref) <= 1e-5
