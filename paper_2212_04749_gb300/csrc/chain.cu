@@ -43,14 +43,6 @@ namespace {
 
 constexpr int CH_MAX_THREADS = 256;
 
-__device__ __forceinline__ int ch_exp(uint32_t bits) {
-    if (bits == 0u) return 0;
-    const int e = int((bits >> 23) & 0xffu) - 127;
-    return max(-126, min(126, e));
-}
-
-__device__ __forceinline__ float ch_pow2(int e) { return __int_as_float((127 + e) << 23); }
-
 __device__ __forceinline__ void ch_record_max(uint32_t *slot, uint32_t v) {
     asm volatile("red.relaxed.gpu.global.max.u32 [%0], %1;" ::"l"(slot), "r"(v) : "memory");
 }
@@ -207,7 +199,7 @@ __global__ void __launch_bounds__(CH_MAX_THREADS, 3) k_chain(const __grid_consta
         const int id = __ldg(d.tab + inst * (L + 1) + t);
         const uint32_t *mx = t == 0 ? d.mxA : d.mxB[t - 1];
         const int32_t *E = t == 0 ? d.EA : d.EB[t - 1];
-        const int e = mx ? ch_exp(mx[id]) : 0;
+        const int e = mx ? exp_of(mx[id]) : 0;
         s_tab[t] = id;
         s_e[t] = e;
         s_E[t] = E[id] + e;
@@ -231,13 +223,13 @@ __global__ void __launch_bounds__(CH_MAX_THREADS, 3) k_chain(const __grid_consta
     if (t == 0) {
         int ec = 0;
         for (int q = 0; q <= L; ++q) ec += s_E[q];
-        s_sc = ch_pow2(-s_e[0]);
+        s_sc = pow2f(-s_e[0]);
         if (ob == 0) d.EC[inst] = ec;
     }
     for (int j = 0; j < L; ++j) {
         const int kn = 1 << (d.kb[j] + d.nb[j]);
         const float2 *src = d.B[j] + int64_t(s_tab[1 + j]) * kn;
-        const float sb = ch_pow2(-s_e[1 + j]);
+        const float sb = pow2f(-s_e[1 + j]);
         // column n in the kernel's order (its bit b: B's n bit nperm[b])
         for (int e = t; e < kn; e += TH) {
             const int n = e >> d.kb[j];

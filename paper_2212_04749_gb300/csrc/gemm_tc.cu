@@ -63,14 +63,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-__device__ __forceinline__ int exp_of(uint32_t bits) {
-    if (bits == 0u) return 0;
-    int e = int((bits >> 23) & 0xffu) - 127;
-    return max(-126, min(126, e));
-}
-
-__device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }
-
 __device__ __forceinline__ int64_t dep(int64_t x, const int8_t *pos, int nbits) {
     int64_t r = 0;
     for (int j = 0; j < nbits; ++j) r |= ((x >> j) & 1) << pos[j];

@@ -39,16 +39,6 @@ namespace tnk {
 
 namespace {
 
-__device__ __forceinline__ int exp_of(uint32_t bits) {
-    if (bits == 0u) return 0;
-    int e = int((bits >> 23) & 0xffu) - 127;
-    return max(-126, min(126, e));
-}
-
-__device__ __forceinline__ float pow2f(int e) {  // 2^e, |e| <= 126
-    return __int_as_float((127 + e) << 23);
-}
-
 __device__ __forceinline__ uint32_t absmax_bits(float2 v) {
     return __float_as_uint(fmaxf(fabsf(v.x), fabsf(v.y)));
 }

@@ -8,6 +8,20 @@
 
 namespace tnk {
 
+// Rescale exponent of an operand from its max word: the exponent of the largest
+// |component|, within +-63, so that two operands' exponents add up to one normal
+// power of two in every kernel (products of operands beyond that leave FP32's
+// range before any factor).
+__device__ __forceinline__ int exp_of(uint32_t bits) {
+    if (bits == 0u) return 0;
+    const int e = int((bits >> 23) & 0xffu) - 127;
+    return max(-63, min(63, e));
+}
+
+__device__ __forceinline__ float pow2f(int e) {  // 2^e, |e| <= 126
+    return __int_as_float((127 + e) << 23);
+}
+
 // One pairwise contraction step, passed by value to every step kernel.
 //   C[i](m, n) = sum_k  A[a(i)](m, k) * B[b(i)](k, n)       (complex)
 // Instance i = sigma * nOut + beta;  a(i) = sigA[sigma] * nOutA + outA[beta],

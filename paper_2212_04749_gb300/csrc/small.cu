@@ -33,12 +33,6 @@ namespace {
 constexpr int SM_THREADS = 512, SM_WARPS = SM_THREADS / 32;
 constexpr int SM_CLUSTER = 16;
 
-__device__ __forceinline__ int sm_exp(uint32_t bits) {
-    if (bits == 0u) return 0;
-    const int e = int((bits >> 23) & 0xffu) - 127;
-    return max(-126, min(126, e));
-}
-
 __device__ __forceinline__ void sm_cfma(float2 &acc, float2 a, float2 b) {
     acc.x = fmaf(a.x, b.x, acc.x);
     acc.x = fmaf(-a.y, b.y, acc.x);
@@ -118,16 +112,9 @@ __device__ __forceinline__ void small_outputs(const SmallDesc &d, int lg, int fi
             acc[u].x += __shfl_xor_sync(0xffffffffu, acc[u].x, s);
             acc[u].y += __shfl_xor_sync(0xffffffffu, acc[u].y, s);
         }
-        const int ea = sm_exp(ma[u]), eb = sm_exp(mb[u]);
-        // 2^-(ea + eb), in two factors where it is no normal number
-        const int e1 = max(-126, min(126, ea + eb)), e2 = ea + eb - e1;
-        const float sc = __int_as_float((127 - e1) << 23);
-        float2 v = make_float2(acc[u].x * sc, acc[u].y * sc);
-        if (e2) {
-            const float s2 = __int_as_float((127 - e2) << 23);
-            v.x *= s2;
-            v.y *= s2;
-        }
+        const int ea = exp_of(ma[u]), eb = exp_of(mb[u]);
+        const float sc = pow2f(-(ea + eb));
+        const float2 v = make_float2(acc[u].x * sc, acc[u].y * sc);
         uint32_t mx = 0u;
         if (valid[u] && sub == 0) {
             int64_t c = int64_t(i[u]) * d.sC;
@@ -238,10 +225,9 @@ __global__ void __launch_bounds__(FEW_THREADS) k_step_few(const __grid_constant_
         acc.x += __shfl_xor_sync(0xffffffffu, acc.x, s);
         acc.y += __shfl_xor_sync(0xffffffffu, acc.y, s);
     }
-    const int ea = sm_exp(ma), eb = sm_exp(mb);
-    const int e1 = max(-126, min(126, ea + eb)), e2 = ea + eb - e1;
-    const float sc = __int_as_float((127 - e1) << 23), s2 = __int_as_float((127 - e2) << 23);
-    const float2 v = make_float2(acc.x * sc * s2, acc.y * sc * s2);
+    const int ea = exp_of(ma), eb = exp_of(mb);
+    const float sc = pow2f(-(ea + eb));
+    const float2 v = make_float2(acc.x * sc, acc.y * sc);
     uint32_t mx = 0u;
     if (valid && sub == 0) {
         d.C[c] = v;

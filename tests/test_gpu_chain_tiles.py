@@ -85,16 +85,18 @@ def test_streaming_steps_without_the_fuse_option(layout, cycles, rows, tree, n_s
     assert np.array_equal(base, p.tn_plan_get_configs())
 
 
-@pytest.mark.parametrize("fuse", [0, 1])
+@pytest.mark.parametrize("log2,layers", [(30, 2), (60, 1)])
+@pytest.mark.parametrize("fuse,config", [(0, None), (1, None), (0, 0), (0, 2)])
 @pytest.mark.parametrize("layout,cycles,rows,tree,n_sliced", [((4, 5), 12, 700, 0, 0), ((4, 5), 12, 700, 1, 2)])
-def test_chains_of_operands_of_any_scale(layout, cycles, rows, tree, n_sliced, fuse):
-    # gates of 2^-30 in two layers and of 2^30 in the next two: five of them
-    # leave the range of FP32.  Step by step the rescale keeps every
-    # intermediate in range; a fused chain does as well
+def test_operands_of_any_scale(layout, cycles, rows, tree, n_sliced, fuse, config, log2, layers):
+    # gates of 2^-log2 in some layers and of 2^log2 in the next: a few of them
+    # leave the range of FP32.  The rescale keeps every intermediate in range,
+    # step by step and within a fused chain
     c, bits, ssa, sl = _case(layout, cycles, rows, tree, n_sliced)
     for g in c.two_qubit_gates:
-        g.matrix = g.matrix * 2.0 ** (30 if (g.layer // 4) % 2 else -30)
+        g.matrix = g.matrix * 2.0 ** (log2 if (g.layer // 2 // layers) % 2 else -log2)
     ref = sv.amplitudes(c, bits)
-    got, p = run_plan(c, bits, ssa, sl, fuse=fuse)
-    assert np.any(p.tn_plan_step_forms() == 3)
+    row = lambda st: config if config != 0 or st["nb"] <= 4 and st["kb"] + st["nb"] <= 8 else 2  # noqa: E731
+    got, p = run_plan(c, bits, ssa, sl, fuse=fuse, force_config=None if config is None else row)
+    assert np.any(p.tn_plan_step_forms() == 3) == (config is None)
     assert rel_l2(got, ref) <= 1e-5
