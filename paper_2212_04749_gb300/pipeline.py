@@ -17,6 +17,7 @@ running batch: a batch then costs about max(planning / (w - 1),
 contraction).
 """
 
+import threading
 from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
@@ -60,7 +61,10 @@ def contract_batches(circ, batches, tree_ssa, sliced, precision, workspace, stre
     ahead = max(1, nws - 1)  # batches planned while one runs
     sides = [torch.cuda.Stream(device=stream.device) for _ in range(ahead)] if nws >= 2 else None
     check = torch.cuda.Stream(device=stream.device)  # reads a finished batch's error word
-    done = {}  # workspace index -> event after the last contraction that used it
+    # workspace index -> (event after the last contraction that used it, set
+    # once its error word, which lies in the workspace, has been read)
+    done = {}
+    read = [threading.Event() for _ in range(n)]
 
     def plan_of(i, prev):
         p = tn.Plan(circ, batches[i], tree_ssa, sliced, **opts)
@@ -70,7 +74,10 @@ def contract_batches(circ, batches, tree_ssa, sliced, precision, workspace, stre
                 raise ValueError(f"batch {i}: plan needs {p.info['workspace_bytes']} workspace bytes, "
                                  f"workspace holds {ws.numel()}")
             if prev is not None:
-                prev.synchronize()
+                prev[0].synchronize()
+                prev[1].wait()
+                if stop.is_set():
+                    return None
             side = sides[i % ahead]
             p.tn_plan_bind(ws, stream=side)
             side.synchronize()
@@ -80,54 +87,61 @@ def contract_batches(circ, batches, tree_ssa, sliced, precision, workspace, stre
     # launched before batch i's result is read
     amps, host = [None, None], [None, None]
     pending = None  # (index, plan, pinned result, event after its copy)
+    stop = threading.Event()  # the caller has left, or a batch failed
 
     def finish(item):
         j, pj, hj, ev = item
         ev.synchronize()
         pj.tn_plan_check(stream=check)  # its contraction has finished; syncs `check` only
+        read[j].set()
         return j, hj.numpy().view(np.complex128).copy()
 
     with ThreadPoolExecutor(max_workers=ahead) as ex:
-        futs = {j: ex.submit(plan_of, j, None) for j in range(min(ahead, n))}
-        for i in range(n):
-            p = futs.pop(i).result()
-            # batch i + ahead binds into the buffer of batch i - 1 once that finishes
-            if i + ahead < n:
-                j = i + ahead
-                futs[j] = ex.submit(plan_of, j, done.get(j % nws))
-            if configs is not None:
-                for s, c in enumerate(configs):
-                    p.tn_plan_set_config(s, int(c) + (TN_CONFIG_TUNED if 0 <= c < TN_CONFIG_TUNED else 0))
-            if chains is not None:
-                for c, on in enumerate(chains):
-                    p.tn_plan_set_chain(c, int(on))
-            m = len(batches[i]) * p.info["amps_per_row"]
-            if sides is None:
-                # one workspace: the previous batch finishes before this one binds
+        try:
+            futs = {j: ex.submit(plan_of, j, None) for j in range(min(ahead, n))}
+            for i in range(n):
+                p = futs.pop(i).result()
+                # batch i + ahead binds into the buffer of batch i - 1 once that finishes
+                if i + ahead < n:
+                    j = i + ahead
+                    futs[j] = ex.submit(plan_of, j, done.get(j % nws))
+                if configs is not None:
+                    for s, c in enumerate(configs):
+                        p.tn_plan_set_config(s, int(c) + (TN_CONFIG_TUNED if 0 <= c < TN_CONFIG_TUNED else 0))
+                if chains is not None:
+                    for c, on in enumerate(chains):
+                        p.tn_plan_set_chain(c, int(on))
+                m = len(batches[i]) * p.info["amps_per_row"]
+                if sides is None:
+                    # one workspace: the previous batch finishes before this one binds
+                    if pending is not None:
+                        yield finish(pending)
+                        pending = None
+                    if p.info["workspace_bytes"] > spaces[0].numel():
+                        raise ValueError(f"batch {i}: plan needs {p.info['workspace_bytes']} workspace bytes, "
+                                         f"workspace holds {spaces[0].numel()}")
+                    p.tn_plan_bind(spaces[0], stream=stream)
+                b = i % 2
+                with torch.cuda.stream(stream):
+                    if amps[b] is None or amps[b].numel() < 2 * m:
+                        amps[b] = torch.zeros(2 * max(m, 1), dtype=torch.float64, device=stream.device)
+                        host[b] = torch.empty(2 * max(m, 1), dtype=torch.float64, pin_memory=True)
+                    a = amps[b][:2 * m]
+                    a.zero_()
+                    p.tn_contract(a, precision, stream=stream)
+                    h = host[b][:2 * m]
+                    h.copy_(a, non_blocking=True)
+                    ev = torch.cuda.Event()
+                    ev.record(stream)
+                if sides is not None:
+                    done[i % nws] = ev, read[i]
                 if pending is not None:
                     yield finish(pending)
-                    pending = None
-                if p.info["workspace_bytes"] > spaces[0].numel():
-                    raise ValueError(f"batch {i}: plan needs {p.info['workspace_bytes']} workspace bytes, "
-                                     f"workspace holds {spaces[0].numel()}")
-                p.tn_plan_bind(spaces[0], stream=stream)
-            b = i % 2
-            with torch.cuda.stream(stream):
-                if amps[b] is None or amps[b].numel() < 2 * m:
-                    amps[b] = torch.zeros(2 * max(m, 1), dtype=torch.float64, device=stream.device)
-                    host[b] = torch.empty(2 * max(m, 1), dtype=torch.float64, pin_memory=True)
-                a = amps[b][:2 * m]
-                a.zero_()
-                p.tn_contract(a, precision, stream=stream)
-                h = host[b][:2 * m]
-                h.copy_(a, non_blocking=True)
-                ev = torch.cuda.Event()
-                ev.record(stream)
-            if sides is not None:
-                done[i % nws] = ev
+                pending = (i, p, h, ev)
+                del p
             if pending is not None:
                 yield finish(pending)
-            pending = (i, p, h, ev)
-            del p
-        if pending is not None:
-            yield finish(pending)
+        finally:  # no planning thread waits for a batch that nobody reads any more
+            stop.set()
+            for e in read:
+                e.set()

@@ -10,6 +10,8 @@ is logged, so the test sees:
   batch that used it last has been waited for, and batch i + 1 is launched
   before batch i's result is read (the overlap the pipeline exists for);
 * with one workspace, a batch binds only after the previous one was read;
+* a workspace is bound again only after its last batch's error word, which
+  lies in it, has been read;
 * every result is read after its batch's event, in input order, and holds
   that batch's values although the next batch was launched before it was
   read (two amplitude buffers in turn).
@@ -17,6 +19,7 @@ is logged, so the test sees:
 
 import sys
 import threading
+import time
 import types
 
 import numpy as np
@@ -135,6 +138,7 @@ def _fake_tn(log):
             log.last_contract = self.i
 
         def tn_plan_check(self, stream=None):
+            time.sleep(0.02)  # a worker that does not wait for it gets ahead
             log.add("check", self.i)
 
     return types.SimpleNamespace(Plan=Plan)
@@ -168,5 +172,32 @@ def test_pipeline_orders_binds_launches_and_reads(monkeypatch, nws):
         else:
             if j >= nws:  # the binding thread waited for the workspace's last batch
                 assert log.waited_before(j - nws, bind, log.items[bind][-1])
+                assert log.index("check", j - nws) < bind
             if j + 1 < n:  # the next batch runs before this one is read
                 assert log.index("contract", j + 1) < chk
+
+
+@pytest.mark.parametrize("nws", [1, 2, 3])
+@pytest.mark.parametrize("fails", [False, True])
+def test_pipeline_ends_where_the_caller_or_a_batch_stops_it(monkeypatch, nws, fails):
+    # the planning threads end too, whatever they wait for
+    log = _Log()
+    monkeypatch.setitem(sys.modules, "torch", _fake_torch(log))
+    fake = _fake_tn(log)
+    if fails:
+        def check(self, stream=None):
+            if self.i == 2:
+                raise RuntimeError("batch 2")
+        fake.Plan.tn_plan_check = check
+    monkeypatch.setattr(pipeline, "tn", fake)
+    batches = [np.full((2, 1), i, np.uint8) for i in range(9)]
+    spaces = [_Workspace(w) for w in range(nws)]
+    it = pipeline.contract_batches(None, batches, None, (), "bf16x3", spaces if nws > 1 else spaces[0])
+    before = threading.active_count()
+    assert [next(it)[0], next(it)[0]] == [0, 1]
+    if fails:
+        with pytest.raises(RuntimeError):
+            next(it)
+    else:
+        it.close()
+    assert threading.active_count() <= before
