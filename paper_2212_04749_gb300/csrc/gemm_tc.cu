@@ -1944,7 +1944,8 @@ cudaError_t launch_step_gemm_tc(const StepDesc &d, const CUtensorMap *a_map, int
         const int64_t blocks = d.nb >= 6 ? (d.packBn * nch) << (d.nb - 6) : d.n_ctab * nch;
         // column tiles dealt in twos: the CTAs that walk one row tile run side
         // by side, and their A and B at any time fit L2 (a row tile's column
-        // tiles per CTA: 11.2 against 8.3 ms on 2^10 x 2^9 x 64, groups of 32)
+        // tiles per CTA: 11.2 against 8.3 ms on 2^10 x 2^9 x 64, groups of 32);
+        // singly where twos would leave CTAs idle
         const int64_t b = ((int64_t(d.max_group) << d.nb) + TBN - 1) / TBN;
         if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
         if (d.nb >= 6)
@@ -1955,7 +1956,7 @@ cudaError_t launch_step_gemm_tc(const StepDesc &d, const CUtensorMap *a_map, int
         // (53-qubit circuit, relative L2 error over 320 oracle amplitudes and
         // time: FMA 1.68e-6, 230 ms; two from K = 128 on 1.53e-6, 64.5; from
         // K = 256 on 1.45e-6, 67.2; one always 1.34e-6, 72.3)
-        const int step = b >= 2 ? 2 : 1;
+        const int step = b >= 2 && tiles >= 8 * grid ? 2 : 1;
         if (d.kb >= 7)
             k_step_gemm_tc<3, 3, 2><<<g, NTHREADS, smem_bytes<3, true>(), s>>>(d, mtiles, err, *a_map, PACK_ST6, TBN,
                                                                                TBN, step);
@@ -2028,10 +2029,12 @@ cudaError_t launch_step_gemm_tc(const StepDesc &d, const CUtensorMap *a_map, int
                                                                             block_of());
         } else {
             // schedule 0: a row tile's column tiles dealt in twos, so that the
-            // CTAs of one row tile run side by side (as for the pairs above)
+            // CTAs of one row tile run side by side (as for the pairs above);
+            // not of few tiles, where it would leave CTAs idle (2^12 x 2^11 x
+            // 2^6, 32 tiles: 127 us in twos, 73 a tile a CTA)
             k_pack_b<2><<<dim3((unsigned)blocks), 256, 0, s>>>(d, nch);
             k_step_gemm_tc<2, 3><<<g, NTHREADS, smem_bytes<2, true>(), s>>>(d, mtiles, err, *a_map, PACK_ST, acw, ow,
-                                                                            d.sched ? block_of() : 2);
+                                                                            d.sched || tiles < 8 * grid ? block_of() : 2);
         }
         return cudaGetLastError();
     }
