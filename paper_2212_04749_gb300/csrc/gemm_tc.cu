@@ -927,8 +927,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
         // lane stores its row's columns from its registers, one instruction a
         // column, without the staging's shared-memory traffic (2^15 x 32 x 64:
         // 5.00 -> 4.46 ms, 2^17 x 16 x 8: 2.49 -> 2.07; 2^12 x 64 x 4, bound
-        // by its stores, 2.60 -> 2.69)
-        mp.rows = d.pCm[0] == 0 && d.pCm[1] == 1 ? 1 : 0;
+        // by its stores, 2.60 -> 2.69).  Not for many tiles of 16 columns,
+        // whose halves drain alternate tiles: 2^18 x 8 x 16 with 37 instances
+        // 802 us from registers, 662 staged; of few tiles (2^14 x 16 x 16)
+        // 13.2 and 15.2
+        mp.rows = d.pCm[0] == 0 && d.pCm[1] == 1 && !(ow == 16 && n_tiles >= 8 * int64_t(gridDim.x)) ? 1 : 0;
         for (int j = 0; j < 4; ++j) mp.cbit[j] = colkey(j);
         for (int c = 0; c < 16; ++c)
             mp.coff[c] = c < (1 << d.nb) * d.max_group
