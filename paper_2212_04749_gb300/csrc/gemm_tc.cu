@@ -930,8 +930,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)  // 20 warps: 96 registers (5 war
         // by its stores, 2.60 -> 2.69).  Not for many tiles of 16 columns,
         // whose halves drain alternate tiles: 2^18 x 8 x 16 with 37 instances
         // 802 us from registers, 662 staged; of few tiles (2^14 x 16 x 16)
-        // 13.2 and 15.2
-        mp.rows = d.pCm[0] == 0 && d.pCm[1] == 1 && !(ow == 16 && n_tiles >= 8 * int64_t(gridDim.x)) ? 1 : 0;
+        // 13.2 and 15.2, with 4 of the 16 columns on average (2^14 x 8 x 4, 497
+        // instances on 459) 495 and 705
+        mp.rows = d.pCm[0] == 0 && d.pCm[1] == 1 &&
+                          !(ow == 16 && n_tiles >= 8 * int64_t(gridDim.x) && (d.nInst << d.nb) >= 12 * d.n_groups)
+                      ? 1
+                      : 0;
         for (int j = 0; j < 4; ++j) mp.cbit[j] = colkey(j);
         for (int c = 0; c < 16; ++c)
             mp.coff[c] = c < (1 << d.nb) * d.max_group
