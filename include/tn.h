@@ -327,10 +327,11 @@ int tn_plan_set_kernel(tn_plan_t plan, int32_t step, int32_t kernel);
  * shape leaves the GEMM's tiles empty (few outputs or few columns per
  * instance, K <= 4 or, in TN_FP32, <= 32) take kernels of their own under
  * configurations 2 and 3, in FP32 (family 1 of tn_plan_step_times).  A step of
- * at most 2^20 outputs and 2^23 complex multiply-adds (2^21 where it would run
- * on the tensor cores) runs an output per thread in FP32 under every
- * configuration that the caller did not set for it; the autotuner then times
- * that under each. */
+ * few multiply-adds (at most 2^16 outputs and 2^23 complex multiply-adds, or
+ * 2^18 and 2^21; 2^21 where it would run on the tensor cores) runs an output per
+ * thread in FP32 under every configuration that the caller did not set for it,
+ * one of up to 2^20 outputs with a short K in the place of the plan's own
+ * configuration; the autotuner times what runs under each. */
 #define TN_NCONFIG 4
 
 /* Set step `step` to configuration `config` (-1: the plan's own choice: 0 or

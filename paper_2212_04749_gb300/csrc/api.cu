@@ -294,9 +294,12 @@ bool config_allowed(const tnp::Step &S, int c) {
     return c >= 2 || (S.nb <= 4 && S.kb + S.nb <= 8);
 }
 
+// The configuration that the plan takes by itself.
+int own_config(const tnp::Step &S) { return S.kernel == 0 ? 0 : 2; }
+
 int effective_config(const PlanObj *o, int s) {
     if (s < (int)o->config_override.size() && o->config_override[s] >= 0) return o->config_override[s];
-    return o->P.steps[s].kernel == 0 ? 0 : 2;
+    return own_config(o->P.steps[s]);
 }
 
 // The slice instance of node nd that low slice bits sigma select: the bits
@@ -343,13 +346,14 @@ void apply_window(const PlanObj *o, const tnp::Step &S, int64_t sigma, tnk::Step
 
 // The kernel (TN_FORM_*) of a step under configuration cfg, and its schedule
 // (d.sched).  ruled: nobody chose the configuration; few: an output per
-// thread is allowed; map_ok: A has a TMA descriptor (FP32; the other
+// thread is not allowed (0), where it is the faster under every configuration
+// (1), also where only the plan's own, cfg, is slower (2); map_ok: A has a TMA descriptor (FP32; the other
 // precisions fail without one).
-int step_form(tnk::StepDesc &d, int cfg, bool ruled, int precision, bool few, bool map_ok) {
+int step_form(tnk::StepDesc &d, int cfg, bool ruled, int precision, int few, bool map_ok) {
     d.sched = cfg & 1;
     const bool skinny = tnk::step_skinny_takes(d);
     const bool on_tc = cfg >= 2 && precision != TN_FP32 && tnk::gemm_tc_supports(d) && !skinny;
-    if (few && tnk::step_few_takes(d, on_tc)) return TN_FORM_FEW;
+    if (few && tnk::step_few_takes(d, on_tc, few == 2)) return TN_FORM_FEW;
     if (cfg < 2) return tnk::step_row_narrow(d) ? TN_FORM_NARROW : TN_FORM_ROW;
     if (skinny) return TN_FORM_SKINNY;  // few outputs per instance and a long K (e.g. the root)
     if (on_tc) {
@@ -400,7 +404,7 @@ int run_step(PlanObj *o, int s, int precision, int64_t sigma, cudaStream_t st) {
     d.tc_pair = o->tc_pair ? 1 : 0;
     const bool chosen = s < (int)o->pinned.size() && o->pinned[s];  // by the caller: runs as it is
     const bool ruled = !(s < (int)o->config_override.size() && o->config_override[s] >= 0);
-    const int form = step_form(d, cfg, ruled, precision, !chosen, o->amap[s].ok);
+    const int form = step_form(d, cfg, ruled, precision, chosen ? 0 : (cfg == own_config(S) ? 2 : 1), o->amap[s].ok);
     cudaError_t e;
     switch (form) {
         case TN_FORM_FEW: e = tnk::launch_step_few(d, st); break;
@@ -567,7 +571,7 @@ void step_features(const PlanObj *o, int s, int precision, int c, float *f) {
     int crun = 0;  // lowest C address bits held by consecutive m bits
     while (crun < S.mb && S.pCm[crun] == crun) ++crun;
     tnk::StepDesc t = shape_desc(o, S);
-    const int form = step_form(t, c, false, precision, true, true);
+    const int form = step_form(t, c, false, precision, c == own_config(S) ? 2 : 1, true);
     const bool gemm = c >= 2, tc = form == TN_FORM_TC || form == TN_FORM_TC_FP32;
     const double ng = double(S.n_groups > 0 ? S.n_groups : 1);
     int i = 0;
@@ -1431,7 +1435,7 @@ int tn_plan_select(tn_plan_t plan, int precision, const uint16_t *params16, floa
         // FMAs (3) are at most 5 % faster where BF16x6 (2) applies (one of 70
         // measured steps; the median takes 3.1 times as long), and its rows
         // are rare in a corpus: not left to the network
-        const bool split = precision == TN_FP32 && step_form(t, 2, false, precision, true, true) == TN_FORM_TC_FP32;
+        const bool split = precision == TN_FP32 && step_form(t, 2, false, precision, 1, true) == TN_FORM_TC_FP32;
         for (int c = 0; c < TN_NCONFIG; ++c) {
             if (!config_allowed(P.steps[s], c) || (split && c == 3)) continue;
             const float v = y[size_t(s) * TN_NCONFIG + c];
@@ -1451,7 +1455,7 @@ int tn_plan_select(tn_plan_t plan, int precision, const uint16_t *params16, floa
         // (a small step that shares a launch, one of a fused chain and one of few
         // multiply-adds run the same whatever is chosen)
         const bool same = merges(o, s) || o->chain_fused(P.steps[s].chain) ||
-                          tnk::step_few_takes(shape_desc(o, P.steps[s]), precision != TN_FP32);
+                          tnk::step_few_takes(shape_desc(o, P.steps[s]), precision != TN_FP32, false);
         if (uncertain) uncertain[s] = (have2 && y2 - y1 < margin && !same) ? 1 : 0;
     }
     o->drop_graphs();

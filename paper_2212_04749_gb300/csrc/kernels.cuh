@@ -229,8 +229,9 @@ struct SmallArgs {
 static_assert(sizeof(SmallArgs) <= 4096, "kernel parameters");
 cudaError_t init_small_kernel();
 // A single step of few multiply-adds, a thread or a few lanes per output
-// (FP32; tc: it would run on the tensor cores otherwise).
-bool step_few_takes(const StepDesc &d, bool tc);
+// (FP32; tc: it would run on the tensor cores otherwise; own: under the
+// plan's own configuration).
+bool step_few_takes(const StepDesc &d, bool tc, bool own);
 cudaError_t launch_step_few(const StepDesc &d, cudaStream_t s);
 cudaError_t launch_small(const SmallArgs &a, cudaStream_t s);
 

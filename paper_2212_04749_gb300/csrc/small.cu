@@ -250,18 +250,29 @@ __global__ void __launch_bounds__(FEW_THREADS) k_step_few(const __grid_constant_
 
 }  // namespace
 
-bool step_few_takes(const StepDesc &d, bool tc) {
+bool step_few_takes(const StepDesc &d, bool tc, bool own) {
     // 2^23 multiply-adds (128 MB through L1, 4 us); against the tensor cores,
     // whose persistent kernel takes 14 us for any small step, 2^21: 2^14 x 16 x
-    // 16 takes 16.3 us here and 14.2 there, 2^11 x 32 x 32 8.2 and 16.3
-    // (outputs: 2^20 take 16 to 17 us here, 18 to 22 on the row kernel)
-    if (d.kb > 10 || d.mb + d.nb > 20) return false;
-    return (d.nInst << (d.mb + d.nb)) <= (int64_t(1) << 20) &&
-           (d.nInst << (d.mb + d.nb + d.kb)) <= (int64_t(1) << (tc ? 21 : 23));
+    // 16 takes 16.3 us here and 14.2 there, 2^11 x 32 x 32 8.2 and 16.3.
+    // Single outputs of K = 2^9 and more are the skinny kernel's: 12.1 us here
+    // against 8.0 at K = 2^10
+    if (d.kb > 10 || d.mb + d.nb > 20 || (d.kb >= 9 && step_skinny_takes(d))) return false;
+    const int64_t out = d.nInst << (d.mb + d.nb), macs = out << d.kb, one = 1;
+    if (out > (one << 20) || macs > (one << (tc ? 21 : 23))) return false;
+    // 2^18 outputs and more: K <= 8, 2^22 multiply-adds where the row kernel
+    // cannot take it (2^18 outputs of K = 32 in a GEMM: 26.5 us here, 20.4
+    // there; 2^20 of K = 8 19.6 and 18.0)
+    const bool row = d.nb <= 4 && d.kb + d.nb <= 8;
+    if (out > (one << 17) && (d.kb > 3 || macs > (one << (row ? 23 : 22)))) return false;
+    // Beyond this the row kernel's second schedule is often faster (2^18 x 4 x 4
+    // 18.5 us here, 15.7 under configuration 0, 9.8 under 1; 2^15 x 32 x 8 24.4,
+    // 24.4 and 12.1), so there only in the place of the plan's own
+    // configuration: tuning tells them apart
+    return own || out <= (one << 16) || (out <= (one << 18) && macs <= (one << 21));
 }
 
 cudaError_t launch_step_few(const StepDesc &d, cudaStream_t s) {
-    if (!step_few_takes(d, false)) return cudaErrorInvalidValue;
+    if (!step_few_takes(d, false, true)) return cudaErrorInvalidValue;
     SmallDesc r;
     std::memset(&r, 0, sizeof(r));
     r.A = d.A;

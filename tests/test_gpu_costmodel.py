@@ -216,8 +216,8 @@ def test_masked_autotuning_leaves_the_other_steps_choices(case20):
 
 
 def test_masked_autotuning_times_the_kernel_that_runs_afterwards():
-    # a step of few multiply-adds takes k_step_few whatever is chosen, in the
-    # timed runs too
+    # a step of few multiply-adds and at most 2^16 outputs takes k_step_few
+    # whatever is chosen, in the timed runs too
     torch, tn = require_cuda()
     from rqc import grid_layout, network_structure, random_circuit
     from rqc.bitstrings import uniform_bitstrings
@@ -232,6 +232,7 @@ def test_masked_autotuning_times_the_kernel_that_runs_afterwards():
     amps = torch.zeros(2 * len(bits), dtype=torch.float64, device="cuda")
     p.tn_contract(amps, "fp32", stream=st)
     few = p.tn_plan_step_forms() == tn.TN_FORM_FEW
+    few &= np.array([st["n_inst"] << (st["mb"] + st["nb"]) <= 1 << 16 for st in p.tn_plan_steps()])
     assert np.any(few)
     p.tn_plan_autotune("fp32", amps, reps=1, step_mask=few, stream=st)
     assert np.all(p.tn_plan_step_forms()[few] == tn.TN_FORM_FEW)
