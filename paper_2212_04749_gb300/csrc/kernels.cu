@@ -1443,11 +1443,24 @@ cudaError_t launch_step_gemm_simt(const StepDesc &d, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-bool step_outer_takes(const StepDesc &d) { return d.kb <= 5 && d.nb >= 5 && d.mb >= 5 && d.mb <= 40; }
+// Rows side by side of a block (log2) and rows of a thread.
+static int outer_rlog(const StepDesc &d) { return d.mb < 8 ? d.mb : 8; }
+static int outer_rx(const StepDesc &d) { return d.mb >= 9 && d.kb <= 4 ? 2 : 1; }
+
+bool step_outer_takes(const StepDesc &d) {
+    if (d.kb > 5 || d.nb < 5 || d.mb < 5 || d.mb > 40) return false;
+    if (d.kb <= 2) return true;
+    // A block walks 64 columns whatever K is: with few blocks the GEMM tiles,
+    // which split them, are faster (K = 16: 8 blocks 24.4 against 16.3 us, 32
+    // 25 and 20, 64 25 and 27; K = 8: 37 blocks 19 and 18, 64 14 and 18; K =
+    // 32: 16 blocks 24 and 20, 32 17 and 21)
+    const int64_t blocks = d.n_ctab * ((int64_t(1) << d.mb) / (outer_rx(d) << outer_rlog(d)));
+    return blocks >= (d.kb == 5 ? 32 : 48);
+}
 
 cudaError_t launch_step_outer(const StepDesc &d, cudaStream_t s) {
     if (!step_outer_takes(d)) return cudaErrorInvalidValue;
-    const int rlog = d.mb < 8 ? d.mb : 8, rx = d.mb >= 9 && d.kb <= 4 ? 2 : 1;
+    const int rlog = outer_rlog(d), rx = outer_rx(d);
     // up to four passes of rows for one B tile, while that leaves eight blocks an SM
     int passes = 1;
     const int64_t tiles = (int64_t(1) << d.mb) / (rx << rlog);
