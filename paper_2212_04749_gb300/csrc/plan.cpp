@@ -670,7 +670,9 @@ struct Builder {
         if ((P.nodes[st.node].n_inst << st.nb) < 32 * int64_t(st.n_groups)) return 0;
         return int64_t(st.col_tiles.size()) * chunks;
     }
-    bool pack32 = false;  // room for them
+    int64_t pack32 = 0;  // room for the steps that need at most this (half as
+                         // much again as for TF32 and BF16x3 with N >= 64)
+    int64_t bpack_cap() const { return std::max(int64_t(256) << 20, P.opt.workspace_limit / 16); }
 
     // Workspace layout; returns total bytes.  own_slots: the outputs of small
     // steps share no memory with other intermediates.
@@ -900,19 +902,13 @@ struct Builder {
         // so one region serves all; steps above the cap (256 MiB, or 1/16 of
         // the workspace limit if that is more) keep B resident or stream it
         p.bpack_bytes = 0;
-        const int64_t bpack_cap = std::max(int64_t(256) << 20, p.opt.workspace_limit / 16);
         for (const Step &st : p.steps) {
             if (st.nb < 6 || st.kb < 3 || st.kb > 24 || st.mb < 6 || st.mb > 30) continue;
             const int64_t nch = ((int64_t(1) << st.kb) + 15) / 16;
             const int64_t bytes = p.nodes[st.b].n_inst * (int64_t(1) << (st.nb - 6)) * nch * 16384;
-            if (bytes <= bpack_cap) p.bpack_bytes = std::max(p.bpack_bytes, bytes);
+            if (bytes <= bpack_cap()) p.bpack_bytes = std::max(p.bpack_bytes, bytes);
         }
-        p.bpack32_bytes = p.bpack_bytes;
-        if (pack32)  // half as much again as the 16 KB a chunk above
-            for (const Step &st : p.steps) {
-                const int64_t bytes = pack32_bytes(st);
-                if (bytes <= bpack_cap / 2 * 3) p.bpack32_bytes = std::max(p.bpack32_bytes, bytes);
-            }
+        p.bpack32_bytes = std::max(p.bpack_bytes, pack32);
         p.off_bpack = p.bpack32_bytes > 0 ? take(p.bpack32_bytes) : -1;
         for (Chain &c : p.chains) {
             const Step &last = p.steps[c.steps.back()];
@@ -1348,13 +1344,20 @@ bool make_plan(const tn_circuit *circ, const uint8_t *bits, int64_t k, const int
         if (!P.opt.fuse && crosses(plain, with)) B.drop_chains();
         else plain = with;
     }
-    // room for B packed for FP32: the same
-    if (P.opt.rescale)
-        for (const Step &st : P.steps) B.pack32 = B.pack32 || B.pack32_bytes(st) > 0;
-    if (B.pack32) {
-        const int64_t with = layout(false, false);
-        if (crosses(plain, with)) B.pack32 = false;
-        else plain = with;
+    // Room for B packed for FP32: as many of the steps as cross no limit (the
+    // region only moves what lies behind it).
+    std::vector<int64_t> needs;
+    for (const Step &st : P.steps) {
+        const int64_t n = P.opt.rescale ? B.pack32_bytes(st) : 0;
+        if (n > P.bpack_bytes && n <= B.bpack_cap() / 2 * 3) needs.push_back(n);
+    }
+    std::sort(needs.rbegin(), needs.rend());
+    for (int64_t n : needs) {
+        const int64_t with = plain + Arena::align(n) - Arena::align(P.bpack_bytes);
+        if (crosses(plain, with)) continue;
+        B.pack32 = n;
+        plain = with;
+        break;
     }
     int64_t slots = 0;
     for (const Step &st : P.steps)

@@ -258,6 +258,22 @@ def test_features_name_the_kernel_that_runs(tn):
     assert not np.any(tc("fp32", 2))
 
 
+def test_packed_region_for_fp32_crosses_no_limit(tn):
+    # a limit below the plan with all of it: the steps that still fit stay on
+    # the tensor cores, TF32's and BF16x3's do not depend on it
+    w = make_workload("diamond53_m12")
+
+    def plan(**kw):
+        p = tn.Plan(w.circuit, w.bits, w.tree.ssa, w.tree.sliced, **kw)
+        return p.info["workspace_bytes"], [p.tn_plan_features(prec, 2)[0][:, 20] for prec in ("fp32", "bf16x3")]
+
+    full, (fp32, bf16) = plan()
+    limit = full - (100 << 20)
+    ws, (some, same) = plan(workspace_limit=limit)
+    assert ws <= limit and 0 < some.sum() < fp32.sum() and np.all(fp32[some == 1] == 1)
+    assert np.array_equal(bf16, same)
+
+
 def test_config_override_rules(tn):
     w = make_workload("grid5x6_m14")
     p = tn.Plan(w.circuit, w.bits, w.tree.ssa, w.tree.sliced)
